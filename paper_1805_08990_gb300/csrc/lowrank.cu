@@ -729,7 +729,7 @@ dme_status dme_lr_plan(const dme_plan_desc* desc, const double* A, const double*
         // the dense plan only supplies E_t, S and their slices: no slice-pair probe
         dme_plan_desc d2 = *desc;
         if (d2.prec == DME_SPLIT_BF16) d2.pairs = 14;
-        DME_TRY(plan_create(&d2, A, C, B, R, S, cuda_stream, &lr->P));
+        DME_TRY(plan_create(&d2, A, C, B, R, S, cuda_stream, &lr->P, false, false));
         lr->st = lr->P->st;
         lr->status = lr->P->status;
         lr->Bt = lr->P->Bt;

@@ -132,6 +132,36 @@ dme_status cong64(int n, const double* P, const double* E, double* X, double* ou
     return DME_OK;
 }
 
+// FP64 plans from this size on run their products as residue products (k_mod.cu).
+constexpr int kModMinN = 192;
+
+// Planes of a rows x k operand in the plan; *ok = false (and no error) if they do not fit.
+dme_status mod_alloc(dme_plan_t p, ModBuf* b, int rows, int k, bool* ok) {
+    b->rows = rows;
+    b->k = k;
+    b->Kp = mod_kpad(k);
+    *ok = palloc(p, reinterpret_cast<void**>(&b->data), mod_plane_bytes(rows, k)) == DME_OK &&
+          palloc(p, reinterpret_cast<void**>(&b->row), mod_row_bytes(rows)) == DME_OK;
+    if (!*ok) {
+        b->data = nullptr;
+        set_error("");
+        return DME_OK;
+    }
+    return mod_make_maps(*b);
+}
+
+// cong64 by residue products: with G = op(Gp) (its planes in G), X = G P^T and
+// out = G X^T + addends, i.e. G P G^T without a transposed operand.
+dme_status cong_mod(dme_plan_t p, const ModBuf& G, const double* Gp, int tG, const double* P, double* out, double alpha,
+                    const double* D1, double b1, const double* D2, double b2, const double* D3, double b3) {
+    const int n = p->n;
+    launch_mod_convert(P, n, n, n, p->mstep, p->st);
+    DME_TRY(launch_mod_gemm(G, p->mstep, gp(n, n, n, Gp, n, tG, P, n, 1, p->X, n, 1.0), p->mws, true, p->status, p->st));
+    launch_mod_convert(p->X, n, n, n, p->mstep, p->st);
+    return launch_mod_gemm(G, p->mstep, gp(n, n, n, Gp, n, tG, p->X, n, 1, out, n, alpha, 1, D1, b1, D2, b2, D3, b3),
+                           p->mws, true, p->status, p->st);
+}
+
 dme_status check_status(dme_plan_t p, const char* where) {
     DME_CUDA_TRY(cudaStreamSynchronize(p->st));
     int hs = 0;
@@ -803,6 +833,7 @@ dme_status compile_seq(dme_plan_t p, const std::vector<std::pair<int, double>>& 
             case DME_F12: {
                 int idx;
                 DME_TRY(compute_ew(p, ft.second, &idx));
+                DME_TRY(plan_mod_planes(p, idx));
                 o.kind = OP_CONG;
                 o.ew = idx;
                 o.wcoef = (ft.first == DME_F12) ? 1.0 : 0.0;
@@ -854,6 +885,22 @@ void drop_graph(GraphSlot& g) {
 }
 
 }  // namespace
+
+dme_status dme::plan_mod_planes(dme_plan_t p, int idx) {
+    EWEntry& e = p->ew[idx];
+    if (!p->mod || e.Gm.data) return DME_OK;
+    const int n = p->n;
+    bool ok = false;
+    DME_TRY(mod_alloc(p, &e.Gm, n, n, &ok));
+    if (!ok) return DME_OK;
+    TmpPool tp(p->st);
+    double* Et = nullptr;
+    DME_TRY(tp.get(&Et, (size_t)n * n));
+    launch_transpose(e.E, Et, n, n, n, n, p->st);
+    launch_mod_convert(Et, n, n, n, e.Gm, p->st);
+    DME_CUDA_TRY(cudaGetLastError());
+    return DME_OK;
+}
 
 // Compile one step of size h into ops (and, with fsal, its head / interior /
 // closing parts).  Extrapolated scheme of order 2q, one step:
@@ -913,6 +960,12 @@ dme_status run_sflow(dme_plan_t p, double* P, double tau, int rule, double qcoef
     const int n = p->n;
     cudaStream_t st = p->st;
     const double* Qd = qcoef != 0.0 ? p->Q : nullptr;
+    if (p->mod && p->mS.data) {
+        if (rule == DME_T4_EULER)
+            return cong_mod(p, p->mS, p->S, 0, P, P, tau, P, 1.0, Qd, qcoef, nullptr, 0.0);
+        DME_TRY(cong_mod(p, p->mS, p->S, 0, P, p->Xs, 1.0, nullptr, 0.0, nullptr, 0.0, nullptr, 0.0));   // S P S^T
+        return cong_mod(p, p->mS, p->S, 0, p->Xs, P, 0.5 * tau * tau, P, 1.0, p->Xs, tau, Qd, qcoef);
+    }
     // X1 = P S^T ; Xs = S X1  (= S P S^T, symmetric)
     DME_TRY(gemm1(gp(n, n, n, P, n, 0, p->S, n, 1, p->X, n, 1.0), st));
     if (rule == DME_T4_EULER) {
@@ -960,6 +1013,9 @@ dme_status dme::run_op(dme_plan_t p, const Op& o, double* Pcaller) {
         case OP_CONG: {
             const EWEntry& e = p->ew[o.ew];
             ProfScope ps(p, DME_KIND_FP64_GEMM);
+            if (p->mod && e.Gm.data)
+                return cong_mod(p, e.Gm, e.E, 1, P, P, 1.0, o.wcoef != 0.0 ? e.W : nullptr, o.wcoef,
+                                o.qcoef != 0.0 ? p->Q : nullptr, o.qcoef, nullptr, 0.0);
             return cong64(n, P, e.E, p->X, P, o.wcoef != 0.0 ? e.W : nullptr, o.wcoef,
                           o.qcoef != 0.0 ? p->Q : nullptr, o.qcoef, nullptr, 0.0, st);
         }
@@ -1064,7 +1120,8 @@ namespace {
 }  // namespace
 
 dme_status dme::plan_create(const dme_plan_desc* d, const double* A, const double* QorC, const double* B,
-                            const double* R, const double* S, void* stream, dme_plan_t* out, bool serving) {
+                            const double* R, const double* S, void* stream, dme_plan_t* out, bool serving,
+                            bool dense_steps) {
     DME_TRY(validate(d, A, QorC, B, R, S));
     if (d->prec == DME_SPLIT_BF16 && d->n > OZ_MAX_K) {
         set_error("DME_SPLIT_BF16 supports n <= 4096 (exact slice accumulation over K <= 4096)");
@@ -1164,6 +1221,15 @@ dme_status dme::plan_create(const dme_plan_desc* d, const double* A, const doubl
             DME_TRY(alloc_slices(p, &p->Ssl, n, n, OZ_SLICES_FIXED));
             launch_slice_rows_f64(p->S, n, n, n, p->Ssl, st);
         }
+    }
+    if (!p->split && !serving && dense_steps && n >= kModMinN) {
+        bool ok = false, oks = true;
+        DME_TRY(mod_alloc(p, &p->mstep, n, n, &ok));
+        if (ok) ok = palloc_t(p, &p->mws, mod_ws_bytes(n, n)) == DME_OK;
+        if (ok && gen) DME_TRY(mod_alloc(p, &p->mS, n, n, &oks));
+        if (ok && gen && oks) launch_mod_convert(p->S, n, n, n, p->mS, st);
+        p->mod = ok;
+        if (!ok) set_error("");
     }
     // ||[[-A^T, Q], [0, A]]||_1 for the scaling of every t
     launch_block_norm1(p->A, p->Q, n, p->small, st);
@@ -1388,6 +1454,7 @@ static dme_status apply_impl(dme_plan_t plan, int flow, double t, double* P, boo
             case DME_F12: {
                 int idx;
                 DME_TRY(compute_ew(plan, t, &idx));
+                DME_TRY(plan_mod_planes(plan, idx));
                 o.kind = OP_CONG;
                 o.ew = idx;
                 o.wcoef = flow == DME_F12 ? 1.0 : 0.0;

@@ -4,8 +4,10 @@
 #include <vector>
 
 #include "dme_internal.h"
+#include "mod_internal.h"
 #include "split_internal.h"
 
+using dme::ModBuf;
 using dme::SliceBuf;
 using dme::GemmProb;
 
@@ -15,6 +17,7 @@ struct EWEntry {
     double* W;
     int s;
     SliceBuf Gsl;   // split path: slices of E^T (rows of E^T = columns of E)
+    ModBuf Gm;      // FP64 path: residue planes of E^T, made on the first congruence
 };
 
 enum OpKind { OP_CONG = 0, OP_AXPY = 1, OP_RICC = 2, OP_SFLOW = 3, OP_COPY = 4, OP_COMBINE = 5 };
@@ -79,6 +82,11 @@ struct dme_plan_s {
     float2* U = nullptr;       // split path: G P as normalised (hi, lo) pairs
     float2* kws = nullptr;     // split path: split-K workspace of the tail tiles
     int* kcnt = nullptr;       // split path: split-K arrival counters
+    // FP64 path from kModMinN on: products as residue products (planes of the per-step
+    // operand, P or G P; of S; and the products' workspace)
+    bool mod = false;
+    ModBuf mstep, mS;
+    uint8_t* mws = nullptr;
     // split path with n > 1536 and T3: the Riccati products on the tensor cores
     bool tric = false;
     SliceBuf btsl;             // slices of Bt^T (m rows, 5 slices)
@@ -99,9 +107,11 @@ namespace dme {
 
 // Build a plan (validated descriptor; pointers host or device).  A serving plan
 // (grouped launches, which never split K: at the server's loads splitting only adds
-// units and tail work to launches that are already full) holds no split-K workspace.
+// units and tail work to launches that are already full) holds no split-K workspace
+// and no residue planes; nor has the plan under a factored path (dense_steps = false).
 dme_status plan_create(const dme_plan_desc* d, const double* A, const double* QorC, const double* B,
-                       const double* R, const double* S, void* stream, dme_plan_t* out, bool serving = false);
+                       const double* R, const double* S, void* stream, dme_plan_t* out, bool serving = false,
+                       bool dense_steps = true);
 // Free a plan and everything it owns (synchronises its stream).
 void free_plan(dme_plan_t p);
 // Compile one step of size h into p->ops (computes missing E_t, W_t).
@@ -112,6 +122,9 @@ dme_status run_op(dme_plan_t p, const Op& o, double* P);
 size_t plan_estimate_bytes(const dme_plan_desc& d, bool serving = false);
 // E_t, W_t of the plan for step t (computed and cached on first use): index into p->ew.
 dme_status plan_ew(dme_plan_t p, double t, int* idx);
+// Residue planes of E_t^T of p->ew[idx] (FP64 plans on residue products; none if they do
+// not fit in memory: the products with this E then stay on the FP64 pipe).
+dme_status plan_mod_planes(dme_plan_t p, int idx);
 // Report (and clear) the plan's device status word after synchronising its stream.
 dme_status plan_check(dme_plan_t p, const char* where);
 // The descriptor and pointer checks of dme_plan.

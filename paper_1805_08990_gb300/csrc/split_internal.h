@@ -114,6 +114,9 @@ struct SliceDesc {
 
 int slice_kpad(int k);
 size_t slice_buf_bytes(int rows, int k, int ns);
+// Encode a tensor map of bf16 data (strides of dimensions 1 .. rank - 1 in bytes).
+dme_status encode_bf16_map(CUtensorMap* out, const void* data, int rank, const cuuint64_t* dims,
+                           const cuuint64_t* strides, const cuuint32_t* box, CUtensorMapSwizzle swizzle);
 // Encode sb.tmap and (ns > 4) sb.tmap4.
 dme_status make_slice_tmaps(SliceBuf& sb);
 // The tensor map of A's (or B's) slices whose box spans the planes configuration cfg reads.

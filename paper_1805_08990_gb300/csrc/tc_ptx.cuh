@@ -168,6 +168,18 @@ __device__ __forceinline__ uint64_t desc_kmajor_sw64(uint32_t saddr) {
     return d;
 }
 
+// As desc_kmajor_sw64 for rows of 128 bytes (64 bf16) with the 128-byte swizzle,
+// 8-row groups 1024 bytes apart (swizzle mode 2).
+__device__ __forceinline__ uint64_t desc_kmajor_sw128(uint32_t saddr) {
+    uint64_t d = 0;
+    d |= static_cast<uint64_t>((saddr >> 4) & 0x3FFFu);
+    d |= static_cast<uint64_t>(1u) << 16;
+    d |= static_cast<uint64_t>(1024u >> 4) << 32;
+    d |= static_cast<uint64_t>(1u) << 46;
+    d |= static_cast<uint64_t>(2u) << 61;
+    return d;
+}
+
 // Instruction descriptor of kind::f16 with bf16 A and B (K-major), fp32 D:
 // D format bits 4-5 (1 = f32), A format 7-9 and B format 10-12 (1 = bf16),
 // N >> 3 in bits 17-22, M >> 4 in bits 24-28.
