@@ -94,8 +94,10 @@ void launch_transpose(const double* X, double* Y, int rows, int cols, int ldx, i
 void launch_lincomb(double* Y, int n, int ld, const double* X1, double c1, const double* X2, double c2,
                     const double* X3, double c3, double cI, cudaStream_t st);  // Y = c1X1+c2X2+c3X3+cI I
 void launch_symmetrize(double* X, int n, int ld, cudaStream_t st);   // X = (X + X^T)/2
-void launch_block_norm1(const double* A, const double* Q, int n, double* colsum_out, cudaStream_t st);
-void launch_max_reduce(const double* x, int len, double* out, cudaStream_t st);
+// out[0] = ||[[-A^T, Q], [0, A]]||_1; out[1] = max_i |log2(row sum i / column sum i)| of
+// |A| (indices where both are zero left out; infinite where one is).
+void launch_block_norm1(const double* A, const double* Q, int n, double* work, double* out, cudaStream_t st);
+size_t block_norm1_work_doubles(int n);
 
 // B (n x nrhs, ldb) <- M^{-1} B by Gauss-Jordan elimination with partial
 // pivoting, blocked by panels of 16 columns (n <= 4096: stream-ordered

@@ -326,38 +326,87 @@ void launch_symmetrize(double* X, int n, int ld, cudaStream_t st) {
     symmetrize_kernel<<<std::min(n, 152 * 16), 256, 0, st>>>(X, n, ld);
 }
 
-// Column abs-sums of the Van Loan matrix [[-A^T, Q], [0, A]] (2n columns).
-__global__ void block_norm1_kernel(const double* A, const double* Q, int n, double* colsum) {
-    int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= n) return;
-    double s1 = 0.0, s2 = 0.0;
-    for (int i = 0; i < n; ++i) {
-        s1 += fabs(A[(size_t)j * n + i]);                                  // column j of -A^T = row j of A
-        s2 += fabs(Q[(size_t)i * n + j]) + fabs(A[(size_t)i * n + j]);    // column n+j
+// Column abs-sums of the Van Loan matrix [[-A^T, Q], [0, A]]: column j of -A^T is row j of
+// A, column n + j holds those of Q and A.  Block (strip of 32 columns, chunk of NORM_ROWS
+// rows): partial column sums in row order, then a fixed tree; the row sums a warp per row.
+// One thread per column over all rows took 443 us at n = 1024 (a serial chain of n loads).
+constexpr int NORM_ROWS = 128;
+
+__global__ void __launch_bounds__(256) colsum_partial_kernel(const double* __restrict__ A, const double* __restrict__ Q,
+                                                             int n, double* __restrict__ pa, double* __restrict__ pq) {
+    __shared__ double sa[8][33], sq[8][33];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int j = blockIdx.x * 32 + lane, r0 = blockIdx.y * NORM_ROWS;
+    double a = 0.0, q = 0.0;
+    if (j < n)
+        for (int i = r0 + w; i < min(n, r0 + NORM_ROWS); i += 8) {
+            a += fabs(A[(size_t)i * n + j]);
+            q += fabs(Q[(size_t)i * n + j]);
+        }
+    sa[w][lane] = a;
+    sq[w][lane] = q;
+    __syncthreads();
+    if (w == 0 && j < n) {
+        for (int k = 1; k < 8; ++k) {
+            a += sa[k][lane];
+            q += sq[k][lane];
+        }
+        pa[(size_t)blockIdx.y * n + j] = a;
+        pq[(size_t)blockIdx.y * n + j] = q;
     }
-    colsum[j] = s1;
-    colsum[n + j] = s2;
 }
 
-void launch_block_norm1(const double* A, const double* Q, int n, double* colsum_out, cudaStream_t st) {
-    block_norm1_kernel<<<(n + 127) / 128, 128, 0, st>>>(A, Q, n, colsum_out);
+__global__ void __launch_bounds__(256) rowsum_kernel(const double* __restrict__ A, int n, double* __restrict__ rs) {
+    const int i = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (i >= n) return;
+    double a = 0.0;
+    for (int k = lane; k < n; k += 32) a += fabs(A[(size_t)i * n + k]);
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) a += __shfl_xor_sync(0xffffffffu, a, off);
+    if (lane == 0) rs[i] = a;
 }
 
-__global__ void max_reduce_kernel(const double* x, int len, double* out) {
-    __shared__ double red[1024];
-    double m = 0.0;
-    for (int i = threadIdx.x; i < len; i += blockDim.x) m = fmax(m, x[i]);
+__global__ void __launch_bounds__(1024) norm1_final_kernel(const double* __restrict__ rs, const double* __restrict__ pa,
+                                                           const double* __restrict__ pq, int n, int chunks,
+                                                           double* __restrict__ out) {
+    __shared__ double red[1024], rat[1024];
+    double m = 0.0, f = 0.0;
+    for (int j = threadIdx.x; j < n; j += blockDim.x) {
+        double a = 0.0, q = 0.0;
+        for (int c = 0; c < chunks; ++c) {
+            a += pa[(size_t)c * n + j];
+            q += pq[(size_t)c * n + j];
+        }
+        m = fmax(m, fmax(rs[j], a + q));
+        if (rs[j] != 0.0 || a != 0.0) f = fmax(f, fabs(log2(rs[j] / a)));
+    }
     red[threadIdx.x] = m;
+    rat[threadIdx.x] = f;
     __syncthreads();
     for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-        if (threadIdx.x < s) red[threadIdx.x] = fmax(red[threadIdx.x], red[threadIdx.x + s]);
+        if (threadIdx.x < s) {
+            red[threadIdx.x] = fmax(red[threadIdx.x], red[threadIdx.x + s]);
+            rat[threadIdx.x] = fmax(rat[threadIdx.x], rat[threadIdx.x + s]);
+        }
         __syncthreads();
     }
-    if (threadIdx.x == 0) *out = red[0];
+    if (threadIdx.x == 0) {
+        out[0] = red[0];
+        out[1] = rat[0];
+    }
 }
 
-void launch_max_reduce(const double* x, int len, double* out, cudaStream_t st) {
-    max_reduce_kernel<<<1, 1024, 0, st>>>(x, len, out);
+size_t block_norm1_work_doubles(int n) {
+    return (size_t)n * (1 + 2 * (size_t)((n + NORM_ROWS - 1) / NORM_ROWS));
+}
+
+void launch_block_norm1(const double* A, const double* Q, int n, double* work, double* out, cudaStream_t st) {
+    const int chunks = (n + NORM_ROWS - 1) / NORM_ROWS;
+    double* pa = work + n;
+    double* pq = pa + (size_t)chunks * n;
+    rowsum_kernel<<<(n + 7) / 8, 256, 0, st>>>(A, n, work);
+    colsum_partial_kernel<<<dim3((n + 31) / 32, chunks), 256, 0, st>>>(A, Q, n, pa, pq);
+    norm1_final_kernel<<<1, 1024, 0, st>>>(work, pa, pq, n, chunks, out);
 }
 
 // ============================================================== small Cholesky

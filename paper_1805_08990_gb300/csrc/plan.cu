@@ -132,9 +132,6 @@ dme_status cong64(int n, const double* P, const double* E, double* X, double* ou
     return DME_OK;
 }
 
-// FP64 plans from this size on run their products as residue products (k_mod.cu).
-constexpr int kModMinN = 192;
-
 // Planes of a rows x k operand in the plan; *ok = false (and no error) if they do not fit.
 dme_status mod_alloc(dme_plan_t p, ModBuf* b, int rows, int k, bool* ok) {
     b->rows = rows;
@@ -251,20 +248,88 @@ dme_status acc_setup(TmpPool& tp, int n, int* status, AccWork* w) {
     return DME_OK;
 }
 
-// C = alpha op(L) op(R) + b1 D1 (n x n): the accurate tensor mode with aw, else FP64.
-dme_status prod(int n, AccWork* aw, const double* L, int tL, const double* R, int tR, double* C, double alpha,
-                const double* D1, double b1, cudaStream_t st, double* skw = nullptr, size_t skl = 0) {
-    if (aw) return acc_prod(n, *aw, L, tL, R, tR, C, alpha, D1, b1, st);
-    return gemm64_splitk(gp(n, n, n, L, n, tL, R, n, tR, C, n, alpha, 0, D1, b1), skw, skl, st);
+// Plans from this size on run their FP64 products as residue products (k_mod.cu): the
+// steps' of an FP64 plan, and the exponential's (squarings included) of any plan that is
+// not built inside a serving budget.
+constexpr int kModMinN = 192;
+
+// The exponential's residue products: planes of the left and the right operand,
+// transpose scratch, workspace.
+struct ModWork {
+    ModBuf a, b;
+    double* t = nullptr;
+    uint8_t* ws = nullptr;
+    int* status = nullptr;
+    bool balanced = false;
+};
+
+dme_status mod_setup(TmpPool& tp, int n, int* status, ModWork* w) {
+    for (ModBuf* b : {&w->a, &w->b}) {
+        double *pl, *rw;
+        DME_TRY(tp.get(&pl, mod_plane_bytes(n, n) / 8 + 1));
+        DME_TRY(tp.get(&rw, mod_row_bytes(n) / 8 + 1));
+        b->data = reinterpret_cast<__nv_bfloat16*>(pl);
+        b->row = reinterpret_cast<dme::ModRow*>(rw);
+        b->rows = n;
+        b->k = n;
+        b->Kp = mod_kpad(n);
+        DME_TRY(mod_make_maps(*b));
+    }
+    double* ws;
+    DME_TRY(tp.get(&ws, mod_ws_bytes(n, n) / 8 + 1));
+    DME_TRY(tp.get(&w->t, (size_t)n * n));
+    w->ws = reinterpret_cast<uint8_t*>(ws);
+    w->status = status;
+    return DME_OK;
+}
+
+// Planes of the rows of X (or of X^T with t) into b.
+void mod_rows(int n, ModWork& w, const double* X, int t, const ModBuf& b, cudaStream_t st) {
+    if (t) launch_transpose(X, w.t, n, n, n, n, st);
+    launch_mod_convert(t ? w.t : X, n, n, n, b, st);
+}
+
+// Where the exponential's products run: the accurate slice mode, residue products, or
+// (both null) the FP64 pipe, with K split for small n (skw).
+struct ProdPath {
+    AccWork* acc = nullptr;
+    ModWork* mod = nullptr;
+    double* skw = nullptr;
+    size_t skl = 0;
+};
+
+// C = alpha op(L) op(R) + b1 D1 (n x n).  On residue products `certify` is false for the
+// products of A alone when A is balanced: the exponential of a balanced matrix is only
+// normwise accurate in FP64 too (its solves are), so its entries far below the row and
+// column maxima, which no certificate covers, carry no digits that FP64 sums would keep.
+dme_status prod(int n, const ProdPath& w, const double* L, int tL, const double* R, int tR, double* C, double alpha,
+                const double* D1, double b1, cudaStream_t st, int tri = 0, bool certify = true) {
+    if (w.acc) return acc_prod(n, *w.acc, L, tL, R, tR, C, alpha, D1, b1, st);
+    const GemmProb g = gp(n, n, n, L, n, tL, R, n, tR, C, n, alpha, tri, D1, b1);
+    if (w.mod) {
+        mod_rows(n, *w.mod, L, tL, w.mod->a, st);
+        mod_rows(n, *w.mod, R, !tR, w.mod->b, st);
+        return launch_mod_gemm(w.mod->a, w.mod->b, g, w.mod->ws, certify, w.mod->status, st);
+    }
+    return gemm64_splitk(g, w.skw, w.skl, st);
 }
 
 // (O22, O12) = (L, L11 = ls L22^T) * (R):  O22 = L22 R22, O12 = ls L22^T R12 + L12 R22.
-dme_status bprod(int n, AccWork* aw, const double* L22, const double* L12, double ls, const double* R22,
-                 const double* R12, double* O22, double* O12, cudaStream_t st, double* skw = nullptr,
-                 size_t skl = 0) {
-    DME_TRY(prod(n, aw, L22, 0, R22, 0, O22, 1.0, nullptr, 0.0, st, skw, skl));
-    DME_TRY(prod(n, aw, L22, 1, R12, 0, O12, ls, nullptr, 0.0, st, skw, skl));
-    DME_TRY(prod(n, aw, L12, 0, R22, 0, O12, 1.0, O12, 1.0, st, skw, skl));
+dme_status bprod(int n, const ProdPath& w, const double* L22, const double* L12, double ls, const double* R22,
+                 const double* R12, double* O22, double* O12, cudaStream_t st) {
+    if (w.mod && !w.acc) {
+        // R22's planes serve two products
+        ModWork& m = *w.mod;
+        mod_rows(n, m, R22, 1, m.b, st);
+        mod_rows(n, m, L22, 0, m.a, st);
+        DME_TRY(launch_mod_gemm(m.a, m.b, gp(n, n, n, L22, n, 0, R22, n, 0, O22, n, 1.0), m.ws, !m.balanced, m.status, st));
+        mod_rows(n, m, L12, 0, m.a, st);
+        DME_TRY(launch_mod_gemm(m.a, m.b, gp(n, n, n, L12, n, 0, R22, n, 0, O12, n, 1.0), m.ws, true, m.status, st));
+        return prod(n, w, L22, 1, R12, 0, O12, ls, O12, 1.0, st);
+    }
+    DME_TRY(prod(n, w, L22, 0, R22, 0, O22, 1.0, nullptr, 0.0, st));
+    DME_TRY(prod(n, w, L22, 1, R12, 0, O12, ls, nullptr, 0.0, st));
+    DME_TRY(prod(n, w, L12, 0, R22, 0, O12, 1.0, O12, 1.0, st));
     return DME_OK;
 }
 
@@ -445,32 +510,44 @@ dme_status compute_ew(dme_plan_t p, double tau, int* idx) {
     }
     // split plans of n >= kAccMinN: the Pade products on the tensor cores (accurate mode)
     AccWork accw;
-    AccWork* aw = nullptr;
+    ProdPath pp;                          // the [13/13] chain
     if (p->split && n >= kAccMinN) {
         DME_TRY(acc_setup(tp, n, p->status, &accw));
-        aw = &accw;
+        pp.acc = &accw;
     }
+    // residue products, if their planes fit in memory
+    ModWork modw;
+    if (p->mod_ew) {
+        if (mod_setup(tp, n, p->status, &modw) == DME_OK) {
+            modw.balanced = p->balanced;
+            pp.mod = &modw;
+        } else {
+            set_error("");
+        }
+    }
+    pp.skw = skw;
+    pp.skl = skl;
 
     // X = sc M:  X22 = sc A, X12 = sc Q, X11 = -X22^T (implicit)
     launch_lincomb(X22, n, n, p->A, sc, nullptr, 0, nullptr, 0, 0.0, st);
     launch_lincomb(X12, n, n, p->Q, sc, nullptr, 0, nullptr, 0, 0.0, st);
     // X2 = X X (odd * odd -> even), X4 = X2 X2, X6 = X4 X2
-    DME_TRY(bprod(n, aw, X22, X12, -1.0, X22, X12, A22, A12, st, skw, skl));
-    DME_TRY(bprod(n, aw, A22, A12, 1.0, A22, A12, B22, B12, st, skw, skl));
-    DME_TRY(bprod(n, aw, B22, B12, 1.0, A22, A12, C22, C12, st, skw, skl));
+    DME_TRY(bprod(n, pp, X22, X12, -1.0, X22, X12, A22, A12, st));
+    DME_TRY(bprod(n, pp, A22, A12, 1.0, A22, A12, B22, B12, st));
+    DME_TRY(bprod(n, pp, B22, B12, 1.0, A22, A12, C22, C12, st));
     // odd part: U = X (X6 (c13 X6 + c11 X4 + c9 X2) + c7 X6 + c5 X4 + c3 X2 + c1 I)
     launch_lincomb(Y22, n, n, C22, c[13], B22, c[11], A22, c[9], 0.0, st);
     launch_lincomb(Y12, n, n, C12, c[13], B12, c[11], A12, c[9], 0.0, st);
-    DME_TRY(bprod(n, aw, C22, C12, 1.0, Y22, Y12, T22, T12, st, skw, skl));
+    DME_TRY(bprod(n, pp, C22, C12, 1.0, Y22, Y12, T22, T12, st));
     launch_lincomb(U22, n, n, C22, c[7], B22, c[5], A22, c[3], c[1], st);
     launch_lincomb(U12, n, n, C12, c[7], B12, c[5], A12, c[3], 0.0, st);
     launch_lincomb(T22, n, n, T22, 1.0, U22, 1.0, nullptr, 0, 0.0, st);
     launch_lincomb(T12, n, n, T12, 1.0, U12, 1.0, nullptr, 0, 0.0, st);
-    DME_TRY(bprod(n, aw, X22, X12, -1.0, T22, T12, U22, U12, st, skw, skl));
+    DME_TRY(bprod(n, pp, X22, X12, -1.0, T22, T12, U22, U12, st));
     // even part: V = X6 (c12 X6 + c10 X4 + c8 X2) + c6 X6 + c4 X4 + c2 X2 + c0 I
     launch_lincomb(Y22, n, n, C22, c[12], B22, c[10], A22, c[8], 0.0, st);
     launch_lincomb(Y12, n, n, C12, c[12], B12, c[10], A12, c[8], 0.0, st);
-    DME_TRY(bprod(n, aw, C22, C12, 1.0, Y22, Y12, V22, V12, st, skw, skl));
+    DME_TRY(bprod(n, pp, C22, C12, 1.0, Y22, Y12, V22, V12, st));
     launch_lincomb(T22, n, n, C22, c[6], B22, c[4], A22, c[2], c[0], st);
     launch_lincomb(T12, n, n, C12, c[6], B12, c[4], A12, c[2], 0.0, st);
     launch_lincomb(V22, n, n, V22, 1.0, T22, 1.0, nullptr, 0, 0.0, st);
@@ -492,7 +569,7 @@ dme_status compute_ew(dme_plan_t p, double tau, int* idx) {
     DME_TRY(launch_gj_solve(LUq, n, n, R22, n, n, gjw, p->status, st));
     // R12 = p22^{-T} (p12 - q12 R22)
     R12 = C12;
-    DME_TRY(prod(n, aw, q12, 0, R22, 0, R12, -1.0, p12, 1.0, st, skw, skl));
+    DME_TRY(prod(n, pp, q12, 0, R22, 0, R12, -1.0, p12, 1.0, st));
     LUp = C22;
     launch_transpose(p22, LUp, n, n, n, n, st);
     DME_TRY(launch_gj_solve(LUp, n, n, R12, n, n, gjw, p->status, st));
@@ -502,12 +579,25 @@ dme_status compute_ew(dme_plan_t p, double tau, int* idx) {
     double* tmp = T22;
     double* E2 = T12;
     launch_lincomb(E, n, n, R22, 1.0, nullptr, 0, nullptr, 0, 0.0, st);
-    DME_TRY(prod(n, aw, R22, 1, R12, 0, Wm, 1.0, nullptr, 0.0, st, skw, skl));
+    DME_TRY(prod(n, pp, R22, 1, R12, 0, Wm, 1.0, nullptr, 0.0, st));
     launch_symmetrize(Wm, n, n, st);
     for (int i = 0; i < s; ++i) {
-        DME_TRY(gemm64_splitk(gp(n, n, n, Wm, n, 0, E, n, 0, tmp, n, 1.0), skw, skl, st));   // tmp = W E
-        DME_TRY(gemm64_splitk(gp(n, n, n, E, n, 1, tmp, n, 0, Wm, n, 1.0, 1, Wm, 1.0), skw, skl, st));   // W = E^T tmp + W
-        DME_TRY(gemm64_splitk(gp(n, n, n, E, n, 0, E, n, 0, E2, n, 1.0), skw, skl, st));     // E2 = E E
+        // tmp = W E, E2 = E E, W = E^T tmp + W
+        const GemmProb g1 = gp(n, n, n, Wm, n, 0, E, n, 0, tmp, n, 1.0);
+        const GemmProb g2 = gp(n, n, n, E, n, 0, E, n, 0, E2, n, 1.0);
+        const GemmProb g3 = gp(n, n, n, E, n, 1, tmp, n, 0, Wm, n, 1.0, 1, Wm, 1.0);
+        if (pp.mod) {
+            // the planes of E^T serve all three
+            mod_rows(n, modw, E, 1, modw.b, st);
+            mod_rows(n, modw, Wm, 0, modw.a, st);
+            DME_TRY(launch_mod_gemm(modw.a, modw.b, g1, modw.ws, true, p->status, st));
+            mod_rows(n, modw, E, 0, modw.a, st);
+            DME_TRY(launch_mod_gemm(modw.a, modw.b, g2, modw.ws, !p->balanced, p->status, st));
+            mod_rows(n, modw, tmp, 1, modw.a, st);
+            DME_TRY(launch_mod_gemm(modw.b, modw.a, g3, modw.ws, true, p->status, st));
+        } else {
+            for (const GemmProb* g : {&g1, &g2, &g3}) DME_TRY(gemm64_splitk(*g, skw, skl, st));
+        }
         std::swap(E, E2);
     }
     EWEntry ent;
@@ -739,10 +829,10 @@ dme_status choose_pairs(dme_plan_t p) {
     // FP64, or from n = kAccMinN on the accurate tensor mode (about 2^-39 of the row
     // scales per product, two orders below the errors measured against it)
     AccWork accw;
-    AccWork* aw = nullptr;
+    ProdPath aw;
     if (n >= kAccMinN) {
         DME_TRY(acc_setup(tp, n, p->status, &accw));
-        aw = &accw;
+        aw.acc = &accw;
     }
     std::vector<double*> refs;
     std::vector<const SliceBuf*> gs;
@@ -1232,10 +1322,18 @@ dme_status dme::plan_create(const dme_plan_desc* d, const double* A, const doubl
         if (!ok) set_error("");
     }
     // ||[[-A^T, Q], [0, A]]||_1 for the scaling of every t
-    launch_block_norm1(p->A, p->Q, n, p->small, st);
-    launch_max_reduce(p->small, 2 * n, p->small + 2 * n, st);
-    DME_CUDA_TRY(cudaMemcpyAsync(&p->normM, p->small + 2 * n, sizeof(double), cudaMemcpyDeviceToHost, st));
+    double norms[2] = {0.0, 0.0};
+    {
+        TmpPool tp(st);
+        double* work = nullptr;
+        DME_TRY(tp.get(&work, block_norm1_work_doubles(n)));
+        launch_block_norm1(p->A, p->Q, n, work, p->small, st);
+    }
+    DME_CUDA_TRY(cudaMemcpyAsync(norms, p->small, sizeof(norms), cudaMemcpyDeviceToHost, st));
     DME_CUDA_TRY(cudaStreamSynchronize(st));
+    p->normM = norms[0];
+    p->balanced = norms[1] <= 8.0;
+    p->mod_ew = !serving && n >= kModMinN;
     DME_TRY(build_ops(p, d->h));
     DME_TRY(check_status(p, "dme_plan"));
     DME_TRY(choose_pairs(p));

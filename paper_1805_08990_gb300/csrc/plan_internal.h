@@ -84,7 +84,9 @@ struct dme_plan_s {
     int* kcnt = nullptr;       // split path: split-K arrival counters
     // FP64 path from kModMinN on: products as residue products (planes of the per-step
     // operand, P or G P; of S; and the products' workspace)
-    bool mod = false;
+    bool mod = false;          // the steps' products
+    bool mod_ew = false;       // the exponential's products (its transients fit no serving budget)
+    bool balanced = false;     // A's row and column sums agree within 2^8 at every index
     ModBuf mstep, mS;
     uint8_t* mws = nullptr;
     // split path with n > 1536 and T3: the Riccati products on the tensor cores
