@@ -78,6 +78,8 @@ struct DescArena {
 // (at most the resident CTA count; CTAs stride over the tiles).
 dme_status gemm64_grouped(std::vector<GemmProb>& probs, GemmProb* dev_desc, cudaStream_t st,
                           DescArena* arena = nullptr, int tile = 64);
+// One product in 8-wide tiles, for few 32-wide ones; the same bits as gemm64_grouped.
+dme_status gemm64_small(const GemmProb& g, cudaStream_t st);
 // Query the persistent grid sizes ahead of any stream capture.
 void gemm64_prepare();
 // One product of fewer 32-wide tiles than half the SMs (the plan's products for
@@ -141,6 +143,18 @@ dme_status launch_jacobi_eig(const double* G, int ldg, int r, double* Vt, int ld
 // also times sqrt(rowscale[a]) when rowscale is given, which may alias d_out).
 void launch_lr_select(const double* lam, const double* Vt, int ldv, int r, double tol, int inv_sqrt, double* T,
                       int ldt, double* d_out, int* k_out, cudaStream_t st, const double* rowscale = nullptr);
+// Pivoted Cholesky diag(d)^{1/2} G diag(d)^{1/2} = R^T R (R r x r, rows from *k on zero, its
+// columns in the order of G's), stopping at pivots <= tol * the first.
+dme_status launch_chol_pivot(const double* G, int ldg, int r, const double* d, double tol, double* R, int ldr, int* k,
+                             int* status, cudaStream_t st);
+// H = R R^T = T^T T over its leading *k rows (*k lowered to the first pivot that is not
+// positive), nrm[j] the squared norm of row j of T, X = T^{-T} R (rows from *k on zero).
+dme_status launch_qlp_rows(const double* H, int ldh, int r, const double* R, int ldr, int* k, double* T, int ldt,
+                           double* rinv, double* nrm, double* X, int ldx, cudaStream_t st);
+// The basis of the kept rows j of X (nrm[j] > tol * max): T[a][rank] = X[j][a] sqrt(d[a]),
+// d_out = 1 (may alias d), *k_out their count.
+void launch_qlp_select(const double* X, int ldx, const double* nrm, const int* k, int r, double tol, const double* d,
+                       double* T, int ldt, double* d_out, int* k_out, cudaStream_t st);
 // G_ij *= sqrt(d_i d_j) for the r x r matrix G.
 void launch_sym_scale(double* G, int ldg, int r, const double* d, cudaStream_t st);
 // F = V diag(psi(lam)) V^T (m x m) for the factored Riccati flow over t.

@@ -23,9 +23,10 @@
 
 namespace dme {
 
-constexpr int RZ_ROWS = 8;      // rows of P per block in kernel (1): one per warp
+constexpr int RZ_ROWS = 4;      // rows of P per block in kernel (1): two warps each
 constexpr int RZ_MB = 8;        // columns of Bt per pass
-constexpr int RU_TILE = 64;     // update tile
+constexpr int RU_TILE = 32;     // update tile
+constexpr int RU_FUSE = 8;      // largest m whose Y the update forms itself
 
 __host__ __device__ __forceinline__ int rz_blocks(int n) { return (n + RZ_ROWS - 1) / RZ_ROWS; }
 
@@ -72,81 +73,81 @@ __device__ __forceinline__ int ric_find(const RicDesc* d, int nd, int blk) {
     return lo;
 }
 
-// (1) Z[r][c] = sum_k P[r][k] Bt[k][c] for the block's 8 rows (one per warp),
-// in passes of 8 columns; Bt chunks staged in shared memory; then the block's
-// partial Gram sums Gpart[b][i][c] = sum_{r in block} Bt[r][i] Z[r][c] in a
-// fixed order (deterministic, no atomics).
+// (1) Z[r][c] = sum_k P[r][k] Bt[k][c] for the block's RZ_ROWS rows, two warps a row
+// (each half of the row's 64-column steps, the halves added in order), then the
+// block's partial Gram sums Gpart[b][i][c] = sum_{r in block} Bt[r][i] Z[r][c] in a
+// fixed order (deterministic, no atomics).  MB columns per pass.
+// Bound: the FP64 pipe (two FMAs per SM and cycle): n^2 m FMAs, so a pass computes no
+// column that is not there, and four rows a block give n / 4 blocks.
+template <int MB>
+__device__ __forceinline__ void riccati_z_pass(const RicDesc& d, int row, int half, int lane, int c0,
+                                               double (&acc)[RZ_MB]) {
+    const int n = d.n, m = d.m;
+    const double* __restrict__ prow = d.P + (size_t)row * n;
+    const double* __restrict__ Bt = d.Bt + c0;
+    const bool vec = (n % 2) == 0;
+#pragma unroll 2
+    for (int k = 2 * lane + 64 * half; k < n; k += 128) {
+        const bool two = k + 1 < n;
+        double p0, p1 = 0.0;
+        if (vec) {
+            const double2 v = *reinterpret_cast<const double2*>(prow + k);
+            p0 = v.x;
+            p1 = v.y;
+        } else {
+            p0 = prow[k];
+            if (two) p1 = prow[k + 1];
+        }
+#pragma unroll
+        for (int c = 0; c < MB; ++c) {
+            const double b0 = Bt[(size_t)k * m + c], b1 = two ? Bt[(size_t)(k + 1) * m + c] : 0.0;
+            acc[c] = fma(p1, b1, fma(p0, b0, acc[c]));
+        }
+    }
+}
+
 __global__ void __launch_bounds__(256) riccati_z_kernel(const __grid_constant__ RicBatch batch) {
-    constexpr int KC = 512;
-    // Bt chunk stored column-major in pairs: sB2[c][k/2] = (Bt[k][c], Bt[k+1][c]), so the lanes of a
-    // warp (consecutive k pairs) read consecutive 16-byte words of one column
-    __shared__ double2 sB2[RZ_MB][KC / 2];
+    __shared__ double sH[2 * RZ_ROWS][RZ_MB];
     __shared__ double sZ[RZ_ROWS][RZ_MB];
     const RicDesc* ds = ric_descs(batch);
     const int ip = ric_find<0>(ds, batch.nd, blockIdx.x);
     const RicDesc& d = ds[ip];
     const int lb = blockIdx.x - d.sz;
     const int n = d.n, m = d.m;
-    const double* __restrict__ P = d.P;
     const double* __restrict__ Bt = d.Bt;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int row = lb * RZ_ROWS + warp;
-    const bool vec = (n % 2) == 0;
+    const int row = lb * RZ_ROWS + (warp >> 1);
     for (int c0 = 0; c0 < m; c0 += RZ_MB) {
         const int mb = min(RZ_MB, m - c0);
         double acc[RZ_MB];
 #pragma unroll
         for (int c = 0; c < RZ_MB; ++c) acc[c] = 0.0;
-        for (int k0 = 0; k0 < n; k0 += KC) {
-            __syncthreads();
-            for (int e = threadIdx.x; e < (KC / 2) * RZ_MB; e += blockDim.x) {
-                const int c = e / (KC / 2), kp = e % (KC / 2), k = 2 * kp;
-                double2 v;
-                v.x = (k0 + k < n && c < mb) ? Bt[(size_t)(k0 + k) * m + c0 + c] : 0.0;
-                v.y = (k0 + k + 1 < n && c < mb) ? Bt[(size_t)(k0 + k + 1) * m + c0 + c] : 0.0;
-                sB2[c][kp] = v;
-            }
-            __syncthreads();
-            if (row >= n) continue;
-            const int kend = min(KC, n - k0);
-            const double* prow = P + (size_t)row * n + k0;
-            // 2 consecutive doubles per lane per iteration: a warp covers 64 columns
-            for (int k = 2 * lane; k < kend; k += 64) {
-                double p0, p1 = 0.0;
-                if (vec && k + 1 < kend) {
-                    double2 v = *reinterpret_cast<const double2*>(prow + k);
-                    p0 = v.x;
-                    p1 = v.y;
-                } else {
-                    p0 = prow[k];
-                    if (k + 1 < kend) p1 = prow[k + 1];
-                }
-                // k is even; past the row end p1 = 0 and the staged Bt is zero-filled
-#pragma unroll
-                for (int c = 0; c < RZ_MB; ++c) {
-                    const double2 b = sB2[c][k >> 1];
-                    acc[c] = fma(p1, b.y, fma(p0, b.x, acc[c]));
-                }
+        if (row < n) {
+            switch (mb) {
+                case 1: riccati_z_pass<1>(d, row, warp & 1, lane, c0, acc); break;
+                case 2: riccati_z_pass<2>(d, row, warp & 1, lane, c0, acc); break;
+                case 3: riccati_z_pass<3>(d, row, warp & 1, lane, c0, acc); break;
+                case 4: riccati_z_pass<4>(d, row, warp & 1, lane, c0, acc); break;
+                case 5: riccati_z_pass<5>(d, row, warp & 1, lane, c0, acc); break;
+                case 6: riccati_z_pass<6>(d, row, warp & 1, lane, c0, acc); break;
+                case 7: riccati_z_pass<7>(d, row, warp & 1, lane, c0, acc); break;
+                default: riccati_z_pass<8>(d, row, warp & 1, lane, c0, acc); break;
             }
         }
 #pragma unroll
         for (int c = 0; c < RZ_MB; ++c) {
+            if (c >= mb) break;
             double v = acc[c];
 #pragma unroll
             for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-            acc[c] = v;
+            if (lane == 0) sH[warp][c] = v;
         }
         __syncthreads();
-        if (lane == 0) {
-#pragma unroll
-            for (int c = 0; c < RZ_MB; ++c) sZ[warp][c] = (row < n) ? acc[c] : 0.0;
-        }
-        if (row < n && lane < mb) {
-            double v = 0.0;
-#pragma unroll
-            for (int c = 0; c < RZ_MB; ++c)
-                if (c == lane) v = acc[c];
-            d.Z[(size_t)row * m + c0 + lane] = v;
+        for (int e = threadIdx.x; e < RZ_ROWS * mb; e += blockDim.x) {
+            const int r = e / mb, c = e % mb, rr = lb * RZ_ROWS + r;
+            const double v = rr < n ? sH[2 * r][c] + sH[2 * r + 1][c] : 0.0;
+            sZ[r][c] = v;
+            if (rr < n) d.Z[(size_t)rr * m + c0 + c] = v;
         }
         __syncthreads();
         for (int e = threadIdx.x; e < m * mb; e += blockDim.x) {
@@ -158,6 +159,7 @@ __global__ void __launch_bounds__(256) riccati_z_kernel(const __grid_constant__ 
             }
             d.Gpart[(size_t)lb * m * m + (size_t)i * m + c0 + jj] = sacc;
         }
+        __syncthreads();
     }
 }
 
@@ -248,40 +250,38 @@ __global__ void riccati_gpart_kernel(const __grid_constant__ RicBatch batch) {
 
 // (3) Y[i][r] = sum_{c <= r} Linv[r][c] Z[i][c]   (Y = Z L^{-T}); Y = 0 when the
 // m x m matrix was not SPD (an update with Y then leaves P as it is).
+__device__ __forceinline__ double riccati_y_entry(const RicDesc& d, int i, int r) {
+    double s = 0.0;
+    for (int c = 0; c <= r; ++c) s = fma(d.Linv[r * d.m + c], d.Z[(size_t)i * d.m + c], s);
+    return s;
+}
+
 __global__ void riccati_y_kernel(const __grid_constant__ RicBatch batch) {
     const RicDesc* ds = ric_descs(batch);
     const RicDesc& d = ds[ric_find<1>(ds, batch.nd, blockIdx.x)];
     const int i = (blockIdx.x - d.sy) * blockDim.x + threadIdx.x;
     const int m = d.m;
     if (i >= d.n) return;
-    if (*d.status & DEV_NOTSPD) {
-        for (int r = 0; r < m; ++r) d.Y[(size_t)i * m + r] = 0.0;
-        return;
-    }
-    for (int r = 0; r < m; ++r) {
-        double s = 0.0;
-        for (int c = 0; c <= r; ++c) s = fma(d.Linv[r * m + c], d.Z[(size_t)i * m + c], s);
-        d.Y[(size_t)i * m + r] = s;
-    }
+    const bool skip = (*d.status & DEV_NOTSPD) != 0;
+    for (int r = 0; r < m; ++r) d.Y[(size_t)i * m + r] = skip ? 0.0 : riccati_y_entry(d, i, r);
 }
 
 // (4) P[i][j] <- P[i][j] - t sum_r Y[i][r] Y[j][r] (+ q Q[i][j]).  The result is
 // symmetric (the sum is taken in the same order for (i, j) and (j, i)), so only
-// the 64 x 64 tiles on or above the diagonal are computed: each reads its
+// the 32 x 32 tiles on or above the diagonal are computed: each reads its
 // upper block of P, writes it, and for an off-diagonal tile also writes the
 // transposed block below the diagonal from a shared-memory copy (coalesced).
-// Half of the FP64 work and of the traffic on P of a full update.
-constexpr int RU_LD = RU_TILE + 1;
-constexpr size_t RU_SMEM = sizeof(double) * (2 * RU_TILE * 33 + RU_TILE * RU_LD);
-
+// Half of the FP64 work and of the traffic on P of a full update.  Problems of
+// m <= RU_FUSE form the Y rows of the tile from Z and Linv here (m (m + 1) FMAs per
+// row against 32 m of the tile's own), which saves them a launch.  The tile's entries
+// of P (and Q) are loaded together before the first is stored: one by one, each load
+// waited behind the store before it (64-wide tiles, n = 81: 16 us).
 __global__ void __launch_bounds__(256) riccati_update_kernel(const __grid_constant__ RicBatch batch) {
     const RicDesc* ds = ric_descs(batch);
     const RicDesc& d = ds[ric_find<2>(ds, batch.nd, blockIdx.x)];
     if (*d.status & DEV_NOTSPD) return;
-    extern __shared__ double ru_smem[];
-    double(*Yi)[33] = reinterpret_cast<double(*)[33]>(ru_smem);
-    double(*Yj)[33] = reinterpret_cast<double(*)[33]>(ru_smem + RU_TILE * 33);
-    double* Vt = ru_smem + 2 * RU_TILE * 33;           // [RU_TILE][RU_LD]
+    __shared__ double Yi[RU_TILE][33], Yj[RU_TILE][33];
+    __shared__ double Vt[RU_TILE][RU_TILE + 1];
     const int n = d.n, m = d.m;
     const int T = (n + RU_TILE - 1) / RU_TILE;
     // upper-triangle tile (ti <= tj), row by row
@@ -292,41 +292,42 @@ __global__ void __launch_bounds__(256) riccati_update_kernel(const __grid_consta
     }
     const int tj = ti + rem;
     const int i0 = ti * RU_TILE, j0 = tj * RU_TILE;
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;   // 32 x 8
+    double pv[4], qv[4];
+#pragma unroll
+    for (int h = 0; h < 4; ++h) {
+        const int i = i0 + ty + 8 * h, j = j0 + tx;
+        const bool in = i < n && j < n;
+        const size_t off = (size_t)i * n + j;
+        pv[h] = in ? d.P[off] : 0.0;
+        qv[h] = in && d.Qadd ? d.Qadd[off] : 0.0;
+    }
+    const bool fuse = m <= RU_FUSE;
     for (int e = threadIdx.x; e < RU_TILE * m; e += blockDim.x) {
-        int r = e / m, c = e % m;
-        Yi[r][c] = (i0 + r < n) ? d.Y[(size_t)(i0 + r) * m + c] : 0.0;
-        Yj[r][c] = (j0 + r < n) ? d.Y[(size_t)(j0 + r) * m + c] : 0.0;
+        const int r = e / m, c = e % m;
+        const int gi = i0 + r, gj = j0 + r;
+        Yi[r][c] = gi < n ? (fuse ? riccati_y_entry(d, gi, c) : d.Y[(size_t)gi * m + c]) : 0.0;
+        Yj[r][c] = gj < n ? (fuse ? riccati_y_entry(d, gj, c) : d.Y[(size_t)gj * m + c]) : 0.0;
     }
     __syncthreads();
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;   // 32 x 8
-    for (int di = ty; di < RU_TILE; di += 8) {
-        const int i = i0 + di;
-        if (i >= n) break;
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int dj = tx + 32 * h, j = j0 + dj;
-            if (j >= n) continue;
-            double s = 0.0;
-            for (int c = 0; c < m; ++c) s = fma(Yi[di][c], Yj[dj][c], s);
-            const size_t off = (size_t)i * n + j;
-            double v = d.P[off] - d.t * s;
-            if (d.Qadd) v += d.q * d.Qadd[off];
-            d.P[off] = v;
-            Vt[di * RU_LD + dj] = v;
-        }
+    for (int h = 0; h < 4; ++h) {
+        const int di = ty + 8 * h, i = i0 + di, j = j0 + tx;
+        if (i >= n || j >= n) continue;
+        double s = 0.0;
+        for (int c = 0; c < m; ++c) s = fma(Yi[di][c], Yj[tx][c], s);
+        double v = pv[h] - d.t * s;
+        if (d.Qadd) v += d.q * qv[h];
+        d.P[(size_t)i * n + j] = v;
+        Vt[di][tx] = v;
     }
     if (ti == tj) return;
     __syncthreads();
     // mirror: P[j][i] = V[i][j] for the block below the diagonal
-    for (int dj = ty; dj < RU_TILE; dj += 8) {
-        const int j = j0 + dj;
-        if (j >= n) break;
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int di = tx + 32 * h, i = i0 + di;
-            if (i >= n) continue;
-            d.P[(size_t)j * n + i] = Vt[di * RU_LD + dj];
-        }
+    for (int h = 0; h < 4; ++h) {
+        const int dj = ty + 8 * h, j = j0 + dj, i = i0 + tx;
+        if (j < n && i < n) d.P[(size_t)j * n + i] = Vt[tx][dj];
     }
 }
 
@@ -418,11 +419,10 @@ dme_status launch_riccati_grouped(const std::vector<RicItem>& items, void* dev_d
     }
     riccati_z_kernel<<<sz, 256, 0, st>>>(b);
     riccati_small_kernel<<<b.nd, 1024, 0, st>>>(b);
-    riccati_y_kernel<<<sy, 128, 0, st>>>(b);
-    static const cudaError_t attr =
-        cudaFuncSetAttribute(riccati_update_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RU_SMEM);
-    DME_CUDA_TRY(attr);
-    riccati_update_kernel<<<su, 256, RU_SMEM, st>>>(b);
+    bool wide = false;
+    for (const RicItem& it : items) wide = wide || it.m > RU_FUSE;
+    if (wide) riccati_y_kernel<<<sy, 128, 0, st>>>(b);
+    riccati_update_kernel<<<su, 256, 0, st>>>(b);
     DME_CUDA_TRY(cudaGetLastError());
     return DME_OK;
 }

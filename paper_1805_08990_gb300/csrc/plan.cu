@@ -115,13 +115,16 @@ GemmProb gp(int M, int N, int K, const double* A, int lda, int tA, const double*
     return g;
 }
 
-// One FP64 product; 32-wide output tiles when 64-wide ones would not fill one
-// wave of the SMs (both tile shapes give bit-identical results).
+// One FP64 product: 64-wide output tiles when they fill one wave of the SMs, else 32-wide
+// ones, else (fewer 32-wide tiles than SMs) 8-wide ones; all give bit-identical results.
 dme_status gemm1(const GemmProb& g, cudaStream_t st) {
     std::vector<GemmProb> v{g};
-    long tiles64 = (long)((g.M + 63) / 64) * ((g.N + 63) / 64);
-    if (g.tri) tiles64 = (tiles64 + (g.M + 63) / 64) / 2;
-    return gemm64_grouped(v, nullptr, st, nullptr, tiles64 < 152 ? 32 : 64);
+    auto tiles = [&](long w) {
+        const long t = ((g.M + w - 1) / w) * ((g.N + w - 1) / w);
+        return g.tri ? (t + (g.M + w - 1) / w) / 2 : t;
+    };
+    if (tiles(32) < 152) return gemm64_small(g, st);
+    return gemm64_grouped(v, nullptr, st, nullptr, tiles(64) < 152 ? 32 : 64);
 }
 
 // out = G^T P G + addends, symmetric, with G = E (so out = E^T P E); X is n x n work.
@@ -923,7 +926,7 @@ dme_status compile_seq(dme_plan_t p, const std::vector<std::pair<int, double>>& 
             case DME_F12: {
                 int idx;
                 DME_TRY(compute_ew(p, ft.second, &idx));
-                DME_TRY(plan_mod_planes(p, idx));
+                if (p->mod) DME_TRY(plan_mod_planes(p, idx));
                 o.kind = OP_CONG;
                 o.ew = idx;
                 o.wcoef = (ft.first == DME_F12) ? 1.0 : 0.0;
@@ -978,7 +981,7 @@ void drop_graph(GraphSlot& g) {
 
 dme_status dme::plan_mod_planes(dme_plan_t p, int idx) {
     EWEntry& e = p->ew[idx];
-    if (!p->mod || e.Gm.data) return DME_OK;
+    if (!p->mod_ew || e.Gm.data) return DME_OK;
     const int n = p->n;
     bool ok = false;
     DME_TRY(mod_alloc(p, &e.Gm, n, n, &ok));
@@ -1202,7 +1205,8 @@ size_t dme::plan_estimate_bytes(const dme_plan_desc& d, bool serving) {
         split = (5 * (size_t)taus + 5 + 8) * sl + nn;                   // E^T / S slices, P and U slices, U pairs
         if (d.n >= kSplitKMinN && (!serving || d.n > 1536)) split += OZ_SPLIT_WS_FLOAT2 * sizeof(float2);
     }
-    return persistent + transient + split + (size_t)d.n * 64 * sizeof(double) + (1u << 20);
+    return persistent + transient + split + (1u << 20) +
+           std::max<size_t>((size_t)d.n * 64, riccati_work_doubles(d.n, d.m)) * sizeof(double);
 }
 
 namespace {
@@ -1552,7 +1556,7 @@ static dme_status apply_impl(dme_plan_t plan, int flow, double t, double* P, boo
             case DME_F12: {
                 int idx;
                 DME_TRY(compute_ew(plan, t, &idx));
-                DME_TRY(plan_mod_planes(plan, idx));
+                if (plan->mod) DME_TRY(plan_mod_planes(plan, idx));
                 o.kind = OP_CONG;
                 o.ew = idx;
                 o.wcoef = flow == DME_F12 ? 1.0 : 0.0;
