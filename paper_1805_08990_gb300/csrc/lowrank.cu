@@ -83,6 +83,13 @@ struct dme_lr_s {
     std::vector<WFactor> wf;
     std::vector<void*> allocs;
     int r = 0;
+    bool loose = false;            // the factor's last compression was a QLP one
+    int* k0dev = nullptr;
+    // FP64 with n >= 192: E_t^T L and S L as residue products (planes of L^T and of S,
+    // L^T itself, the products' workspace)
+    bool mod = false;
+    ModBuf ml, ms;
+    uint8_t* mws = nullptr;
 };
 
 namespace {
@@ -149,6 +156,8 @@ dme_status gemm(dme_lr_t lr, const GemmProb& g, cudaStream_t st) {
     }
     const long tiles64 = (long)((g.M + 63) / 64) * ((g.N + 63) / 64);
     if (tiles64 <= 16 && g.K >= 1024) return gemm_ws(lr, g, st);
+    // few 32-wide tiles (the r x r products): 8-wide ones, over all SMs
+    if ((long)((g.M + 31) / 32) * ((g.N + 31) / 32) <= 76) return gemm64_small(g, st);
     std::vector<GemmProb> v{g};
     return gemm64_grouped(v, nullptr, st, nullptr, g.N <= 64 ? 32 : 64);
 }
@@ -226,12 +235,55 @@ dme_status compress(dme_lr_t lr, double*& L, double*& L2, double* d, int ld, int
     return DME_OK;
 }
 
+// The same factor with fewer or as many columns as `compress` keeps and up to a few more,
+// for the compressions that another one of the same solve follows: pivoted QLP instead
+// of the eigen-decomposition (launch_chol_pivot), L <- Lt X_k^T, d <- 1.
+dme_status compress_qlp(dme_lr_t lr) {
+    int& r = lr->r;
+    if (r == 0) return DME_OK;
+    cudaStream_t st = lr->st;
+    const int n = lr->n, rc = lr->rcap;
+    double *R = lr->J1, *X = lr->J2, *T = lr->J3, *H = lr->J4;
+    double *rinv = lr->lam, *nrm = lr->d2;
+    DME_TRY(gemm(lr, mk(r, r, n, lr->L, rc, 1, lr->L, rc, 0, lr->G, rc, 1.0, 1), st));         // L^T L
+    DME_TRY(launch_chol_pivot(lr->G, rc, r, lr->d, std::max(0.01 * lr->tol, 4e-16), R, rc, lr->k0dev, lr->status, st));
+    DME_TRY(gemm(lr, mk(r, r, r, R, rc, 0, R, rc, 1, H, rc, 1.0, 1), st));                     // R R^T
+    DME_TRY(launch_qlp_rows(H, rc, r, R, rc, lr->k0dev, T, rc, rinv, nrm, X, rc, st));
+    // one Newton-Schulz step: the rows of X orthonormal to rounding
+    DME_TRY(gemm(lr, mk(r, r, r, X, rc, 0, X, rc, 1, H, rc, 1.0, 1), st));
+    DME_TRY(gemm(lr, mk(r, r, r, H, rc, 0, X, rc, 0, R, rc, -0.5, 0, X, 1.5), st));
+    launch_qlp_select(R, rc, nrm, lr->k0dev, r, lr->tol, lr->d, lr->T, rc, lr->d, lr->kdev, st);
+    int k = 0;
+    DME_CUDA_TRY(cudaMemcpyAsync(&k, lr->kdev, sizeof(int), cudaMemcpyDeviceToHost, st));
+    DME_CUDA_TRY(cudaStreamSynchronize(st));
+    DME_TRY(gemm(lr, mk(n, k, r, lr->L, rc, 0, lr->T, rc, 0, lr->L2, rc, 1.0), st));           // Lt X_k^T
+    std::swap(lr->L, lr->L2);
+    r = k;
+    lr->loose = true;
+    return DME_OK;
+}
+
+// After an appending flow: `last` for the last compression of a solve, whose factor is the
+// eigen-decomposition of P.
+dme_status compress_state(dme_lr_t lr, bool last) {
+    if (!last) return compress_qlp(lr);
+    lr->loose = false;
+    return compress(lr, lr->L, lr->L2, lr->d, lr->rcap, lr->r);
+}
+
 dme_status need_cols(dme_lr_t lr, int cols) {
     if (cols > lr->rcap)
         return set_error("low-rank path: " + std::to_string(cols) + " columns exceed the capacity " +
                          std::to_string(lr->rcap) + " (raise rmax up to 224, or tol)"),
                DME_ENOMEM;
     return DME_OK;
+}
+
+// Room for r + extra columns with r the state's (blocks = 1), or blocks * r: a factor that
+// QLP left with a few columns more is first brought to its eigen-decomposition.
+dme_status make_room(dme_lr_t lr, int blocks, int extra) {
+    if (lr->loose && blocks * lr->r + extra > lr->rcap) DME_TRY(compress_state(lr, true));
+    return need_cols(lr, blocks * lr->r + extra);
 }
 
 // Gauss-Legendre nodes and weights on [0, t] (Newton on the Legendre recurrence).
@@ -480,6 +532,18 @@ dme_status apply_split(dme_lr_t lr, const SliceBuf& Msl, const double* X, int ld
     return launch_ozaki_gemm(oz_tmap_a(Msl, OZ_P14), oz_tmap_b(lr->xsl, OZ_P14), p, st);
 }
 
+// FP64 by residue products: C (n x k, ldc) = alpha op(M) X for X (n x k, ldx), op(M)'s planes
+// in Mm; the planes of X^T's rows are made here.
+dme_status apply_mod(dme_lr_t lr, const ModBuf& Mm, const double* M, int tM, const double* X, int ldx, int k, double* C,
+                     int ldc, double alpha) {
+    if (k == 0) return DME_OK;
+    cudaStream_t st = lr->st;
+    const int n = lr->n;
+    launch_transpose(X, lr->Xtr, n, k, ldx, n, st);
+    launch_mod_convert(lr->Xtr, k, n, n, lr->ml, st);
+    return launch_mod_gemm(Mm, lr->ml, mk(n, k, n, M, n, tM, X, ldx, 0, C, ldc, alpha), lr->mws, true, lr->status, st);
+}
+
 dme_status lr_T1(dme_lr_t lr, double tau) {
     if (lr->r == 0) return DME_OK;
     if (lr->sparse) {
@@ -490,8 +554,12 @@ dme_status lr_T1(dme_lr_t lr, double tau) {
     int idx;
     DME_TRY(plan_ew(lr->P, tau, &idx));
     const EWEntry& e = lr->P->ew[idx];
+    if (lr->mod) DME_TRY(plan_mod_planes(lr->P, idx));
+    const ModBuf& Gm = lr->P->ew[idx].Gm;
     if (lr->split)
         DME_TRY(apply_split(lr, e.Gsl, lr->L, lr->rcap, lr->r, lr->L2, lr->rcap, 1.0));
+    else if (lr->mod && Gm.data)
+        DME_TRY(apply_mod(lr, Gm, e.E, 1, lr->L, lr->rcap, lr->r, lr->L2, lr->rcap, 1.0));
     else
         DME_TRY(gemm(lr, mk(lr->n, lr->r, lr->n, e.E, lr->n, 1, lr->L, lr->rcap, 0, lr->L2, lr->rcap, 1.0),
                      lr->st));
@@ -500,7 +568,7 @@ dme_status lr_T1(dme_lr_t lr, double tau) {
 }
 
 dme_status lr_append(dme_lr_t lr, const double* X, int ldx, int k, const double* dsrc, double dval) {
-    DME_TRY(need_cols(lr, lr->r + k));
+    DME_TRY(make_room(lr, 1, k));
     cudaStream_t st = lr->st;
     launch_copy_cols(lr->L + lr->r, lr->rcap, X, ldx, lr->n, k, 1.0, nullptr, st);
     if (dsrc) DME_CUDA_TRY(cudaMemcpyAsync(lr->d + lr->r, dsrc, sizeof(double) * k, cudaMemcpyDeviceToDevice, st));
@@ -509,17 +577,17 @@ dme_status lr_append(dme_lr_t lr, const double* X, int ldx, int k, const double*
     return DME_OK;
 }
 
-dme_status lr_T2(dme_lr_t lr, double tau) {
+dme_status lr_T2(dme_lr_t lr, double tau, bool last) {
     DME_TRY(lr_append(lr, lr->LQ, lr->p, lr->p, nullptr, tau));
-    return compress(lr, lr->L, lr->L2, lr->d, lr->rcap, lr->r);
+    return compress_state(lr, last);
 }
 
-dme_status lr_T12(dme_lr_t lr, double tau) {
+dme_status lr_T12(dme_lr_t lr, double tau, bool last) {
     const WFactor* f = nullptr;
     DME_TRY(wfactor(lr, tau, &f));
     DME_TRY(lr_T1(lr, tau));
     if (f->k > 0) DME_TRY(lr_append(lr, f->L, f->k, f->k, f->d, 0.0));
-    return compress(lr, lr->L, lr->L2, lr->d, lr->rcap, lr->r);
+    return compress_state(lr, last);
 }
 
 dme_status lr_T3(dme_lr_t lr, double tau) {
@@ -538,12 +606,12 @@ dme_status lr_T3(dme_lr_t lr, double tau) {
     return DME_OK;
 }
 
-dme_status lr_T4(dme_lr_t lr, double tau, int rule) {
+dme_status lr_T4(dme_lr_t lr, double tau, int rule, bool last) {
     if (lr->r == 0) return DME_OK;
     cudaStream_t st = lr->st;
-    const int n = lr->n, r = lr->r, rc = lr->rcap;
     const int blocks = rule == DME_T4_EULER ? 2 : 3;
-    DME_TRY(need_cols(lr, blocks * r));
+    DME_TRY(make_room(lr, blocks, 0));
+    const int n = lr->n, r = lr->r, rc = lr->rcap;
     if (lr->sparse) {
         launch_spmm(lr->s_ptr, lr->s_idx, lr->s_val, n, r, lr->L, rc, lr->L + r, rc, std::sqrt(tau), st);
         if (blocks == 3)
@@ -552,12 +620,15 @@ dme_status lr_T4(dme_lr_t lr, double tau, int rule) {
         for (int b = 1; b < blocks; ++b)
             DME_CUDA_TRY(cudaMemcpyAsync(lr->d + b * r, lr->d, sizeof(double) * r, cudaMemcpyDeviceToDevice, st));
         lr->r = blocks * r;
-        return compress(lr, lr->L, lr->L2, lr->d, rc, lr->r);
+        return compress_state(lr, last);
     }
     const double* S = lr->P->S;
     if (lr->split) {
         DME_TRY(apply_split(lr, lr->P->Ssl, lr->L, rc, r, lr->L + r, rc, std::sqrt(tau)));
         if (blocks == 3) DME_TRY(apply_split(lr, lr->P->Ssl, lr->L + r, rc, r, lr->L + 2 * r, rc, std::sqrt(0.5 * tau)));
+    } else if (lr->mod && lr->ms.data) {
+        DME_TRY(apply_mod(lr, lr->ms, S, 0, lr->L, rc, r, lr->L + r, rc, std::sqrt(tau)));
+        if (blocks == 3) DME_TRY(apply_mod(lr, lr->ms, S, 0, lr->L + r, rc, r, lr->L + 2 * r, rc, std::sqrt(0.5 * tau)));
     } else {
         DME_TRY(gemm(lr, mk(n, r, n, S, n, 0, lr->L, rc, 0, lr->L + r, rc, std::sqrt(tau)), st));          // sqrt(t) S L
         if (blocks == 3)
@@ -566,7 +637,7 @@ dme_status lr_T4(dme_lr_t lr, double tau, int rule) {
     for (int b = 1; b < blocks; ++b)
         DME_CUDA_TRY(cudaMemcpyAsync(lr->d + b * r, lr->d, sizeof(double) * r, cudaMemcpyDeviceToDevice, st));
     lr->r = blocks * r;
-    return compress(lr, lr->L, lr->L2, lr->d, rc, lr->r);
+    return compress_state(lr, last);
 }
 
 int t4_rule(const dme_plan_desc& d) {
@@ -574,13 +645,13 @@ int t4_rule(const dme_plan_desc& d) {
     return d.comp == DME_STRANG ? DME_T4_MIDPOINT : DME_T4_EULER;
 }
 
-dme_status lr_apply(dme_lr_t lr, int flow, double tau) {
+dme_status lr_apply(dme_lr_t lr, int flow, double tau, bool last) {
     switch (flow) {
         case DME_F1: return lr_T1(lr, tau);
-        case DME_F2: return lr_T2(lr, tau);
-        case DME_F12: return lr_T12(lr, tau);
+        case DME_F2: return lr_T2(lr, tau, last);
+        case DME_F12: return lr_T12(lr, tau, last);
         case DME_F3: return lr_T3(lr, tau);
-        case DME_F4: return lr_T4(lr, tau, t4_rule(lr->desc));
+        case DME_F4: return lr_T4(lr, tau, t4_rule(lr->desc), last);
     }
     set_error("low-rank path: unknown flow");
     return DME_EINVAL;
@@ -639,6 +710,39 @@ dme_status lr_opts(const dme_lr_opts* opts, int* q, int* rmax, double* tol) {
     return DME_OK;
 }
 
+// Planes of L^T (and of S) and the workspace of E_t^T L on residue products; without them
+// (not enough memory) the products stay on the FP64 pipe.
+dme_status lr_mod_setup(dme_lr_t lr, int n, int rc) {
+    auto planes = [&](ModBuf* b, int rows) -> bool {
+        double *pl = nullptr, *rw = nullptr;
+        b->rows = rows;
+        b->k = n;
+        b->Kp = mod_kpad(n);
+        if (lr_alloc(lr, &pl, mod_plane_bytes(rows, n) / 8 + 1) != DME_OK ||
+            lr_alloc(lr, &rw, mod_row_bytes(rows) / 8 + 1) != DME_OK)
+            return false;
+        b->data = reinterpret_cast<__nv_bfloat16*>(pl);
+        b->row = reinterpret_cast<ModRow*>(rw);
+        return mod_make_maps(*b) == DME_OK;
+    };
+    double* ws = nullptr;
+    if (!planes(&lr->ml, rc) || lr_alloc(lr, &ws, mod_ws_bytes(n, rc) / 8 + 1) != DME_OK ||
+        lr_alloc(lr, &lr->Xtr, (size_t)rc * n) != DME_OK) {
+        set_error("");
+        return DME_OK;
+    }
+    lr->mws = reinterpret_cast<uint8_t*>(ws);
+    lr->mod = true;
+    if (lr->P->S) {
+        if (planes(&lr->ms, n)) launch_mod_convert(lr->P->S, n, n, n, lr->ms, lr->st);
+        else {
+            lr->ms.data = nullptr;
+            set_error("");
+        }
+    }
+    return DME_OK;
+}
+
 // Buffers shared by the dense and the sparse forms, and L_Q = C^T.
 dme_status lr_setup(dme_lr_t lr, const dme_plan_desc* desc, const double* C, int q, int rmax, double tol) {
     lr->desc = *desc;
@@ -693,9 +797,11 @@ dme_status lr_setup(dme_lr_t lr, const dme_plan_desc* desc, const double* C, int
         DME_CUDA_TRY(cudaMemsetAsync(xs, 0, sizeof(float) * rc, st));
         DME_TRY(make_slice_tmaps(lr->xsl));
     }
+    if (!lr->split && lr->P && lr->P->mod_ew) DME_TRY(lr_mod_setup(lr, (int)n, (int)rc));
     double* kd = nullptr;
     DME_TRY(lr_alloc(lr, &kd, 1));
     lr->kdev = reinterpret_cast<int*>(kd);
+    lr->k0dev = lr->kdev + 1;
     double* Cd = nullptr;
     DME_TRY(lr_alloc(lr, &Cd, (size_t)desc->p * n));
     DME_CUDA_TRY(cudaMemcpyAsync(Cd, C, sizeof(double) * desc->p * n, cudaMemcpyDefault, st));
@@ -904,6 +1010,7 @@ dme_status dme_lr_solve(dme_lr_t lr, const double* L0, const double* D0, int r0,
         cudaStream_t st = lr->st;
         const int n = lr->n, rc = lr->rcap;
         lr->r = 0;
+        lr->loose = false;
         if (r0 > 0) {
             // P0 = L0 D0 L0^T with D0 symmetric: L0 V, d = eigenvalues (> 0), then compress
             DME_CUDA_TRY(cudaMemcpy2DAsync(lr->L2, sizeof(double) * rc, L0, sizeof(double) * r0, sizeof(double) * r0, n,
@@ -921,8 +1028,13 @@ dme_status dme_lr_solve(dme_lr_t lr, const double* L0, const double* D0, int r0,
         }
         const double h = T / nsteps;
         const auto seq = plan_step_sequence(lr->desc, h);
+        // the last flow of a step that compresses
+        int lastc = -1;
+        for (int i = 0; i < (int)seq.size(); ++i)
+            if (seq[i].first == DME_F2 || seq[i].first == DME_F12 || seq[i].first == DME_F4) lastc = i;
         for (int s = 0; s < nsteps; ++s)
-            for (auto& ft : seq) DME_TRY(lr_apply(lr, ft.first, ft.second));
+            for (int i = 0; i < (int)seq.size(); ++i)
+                DME_TRY(lr_apply(lr, seq[i].first, seq[i].second, s == nsteps - 1 && i == lastc));
         if (P_out && n > 16384) return set_error("dme_lr_solve: P_out needs n <= 16384 (use dme_lr_factors)"), DME_EINVAL;
         if (P_out) {
             const size_t nn = (size_t)n * n;
