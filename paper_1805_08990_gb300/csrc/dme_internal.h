@@ -157,9 +157,9 @@ void launch_qlp_select(const double* X, int ldx, const double* nrm, const int* k
                        double* T, int ldt, double* d_out, int* k_out, cudaStream_t st);
 // G_ij *= sqrt(d_i d_j) for the r x r matrix G.
 void launch_sym_scale(double* G, int ldg, int r, const double* d, cudaStream_t st);
-// F = V diag(psi(lam)) V^T (m x m) for the factored Riccati flow over t.
-void launch_ric_weights(const double* lam, const double* Vt, int ldv, int m, double t, double* F, int ldf,
-                        cudaStream_t st);
+// Y = G F^T for the factored Riccati flow over t: (I + G F G^T)(I + G F G^T)^T =
+// (I + t G G^T)^{-1}, G and Y r x m, m <= 32.
+void launch_ric_factor(const double* G, int r, int m, double t, double* Y, int* status, cudaStream_t st);
 // Y = alpha X (n x k block), columns scaled by sqrt(d[j]) when d is given.
 void launch_copy_cols(double* Y, int ldy, const double* X, int ldx, int n, int k, double alpha, const double* d,
                       cudaStream_t st);
@@ -187,7 +187,7 @@ void launch_spmm(const int* ptr, const int* idx, const double* val, int n, int r
 // (val holds the values of A^T already multiplied by invg = 1/g),
 // stopping after two consecutive terms with |d_k| |w_k|_F <= tol |p|_F (at most
 // `terms` - 1 terms), then v = scale p.  Y may be X.  Wa, Wb: n x r scratch
-// (ldw); part: 4 leja_grid_max() doubles; sums: 4 doubles; bar: 2 unsigned.
+// (ldw); part: 4 leja_grid_max() floats; sums: 4 floats; bar: 4 unsigned.
 struct LejaCall {
     const int* ptr;
     const int* idx;

@@ -12,6 +12,10 @@
 // by a grid barrier (grid_sync.cuh) whose last arriving block sums the
 // partials in a fixed order, so every block takes the same, reproducible
 // stopping decision.
+// Bound: FP64 issue (nnz + 2 FMAs per entry and term, two per SM and cycle) and the
+// barrier.  The norms of the stopping test are formed in fp32 from the top bits of the
+// entries: as FP64 sums, the shuffles and the block sums alone were 830 FP64 warp
+// instructions per SM and term, more than the recurrence itself.
 #include "dme_internal.h"
 #include "grid_sync.cuh"
 
@@ -23,8 +27,8 @@ namespace {
 
 constexpr int LJ_THREADS = 256;
 
-// Block sum of two values; the result is valid in every thread.
-__device__ __forceinline__ void block_sum2(double& a, double& b, double* sh) {
+// Block sum of two values; the result is valid in thread 0.
+__device__ __forceinline__ void block_sum2(float& a, float& b, float* sh) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) {
@@ -37,26 +41,28 @@ __device__ __forceinline__ void block_sum2(double& a, double& b, double* sh) {
         sh[2 * warp + 1] = b;
     }
     __syncthreads();
-    a = 0.0;
-    b = 0.0;
-    for (int w = 0; w < LJ_THREADS / 32; ++w) {   // fixed order
-        a += sh[2 * w];
-        b += sh[2 * w + 1];
+    if (threadIdx.x == 0) {
+        a = 0.0f;
+        b = 0.0f;
+        for (int w = 0; w < LJ_THREADS / 32; ++w) {   // fixed order
+            a += sh[2 * w];
+            b += sh[2 * w + 1];
+        }
     }
 }
 
 // Grid barrier number `b`.  If part != nullptr the last block to arrive first
 // sums part[2i], part[2i+1] over the grid (fixed order) into sums[0..1].
 // Returns false after a timeout (status set).
-__device__ bool grid_barrier(unsigned* bar, unsigned b, const double* part, double* sums, int* status,
-                             double* sh) {
+__device__ bool grid_barrier(unsigned* bar, unsigned b, const float* part, float* sums, int* status, float* sh) {
     __shared__ int s_last, s_ok;
     if (gs_arrive(bar, b, &s_last)) {
         if (part) {
-            double a = 0.0, p = 0.0;
+            float a = 0.0f, p = 0.0f;
             for (int i = threadIdx.x; i < (int)gridDim.x; i += LJ_THREADS) {
-                a += __ldcg(part + 2 * i);
-                p += __ldcg(part + 2 * i + 1);
+                const float2 v = __ldcg(reinterpret_cast<const float2*>(part) + i);
+                a += v.x;
+                p += v.y;
             }
             block_sum2(a, p, sh);
             if (threadIdx.x == 0) {
@@ -69,6 +75,19 @@ __device__ bool grid_barrier(unsigned* bar, unsigned b, const double* part, doub
         return true;
     }
     return gs_wait(bar, b, status, &s_ok);
+}
+
+// The exponent field of |x| (0 for zero and subnormals).
+__device__ __forceinline__ int exp_field(double x) { return (__double2hiint(x) >> 20) & 0x7FF; }
+
+// |x| 2^(1023 - e0) as a float (20 mantissa bits), from the bits of x: the stopping test's
+// norms need a few digits and run beside the FP64 pipe.  Saturates at 2^60.
+__device__ __forceinline__ float mag(double x, int e0) {
+    const int h = __double2hiint(x) & 0x7FFFFFFF;
+    const int e = (h >> 20) - e0;
+    if (e < -100 || (h >> 20) == 0) return 0.0f;
+    if (e > 60) return 1.152921504606847e18f;
+    return __int_as_float(((e + 127) << 23) | ((h & 0xFFFFF) << 3));
 }
 
 struct LejaArgs {
@@ -85,9 +104,10 @@ struct LejaArgs {
     int ldw;
     double c, invg, scale, tol;
     int substeps, terms;
-    double* part;       // 2 buffers x 2 gridDim doubles
-    double* sums;       // 2 buffers x 2 doubles
-    unsigned* bar;      // arrival counter, release generation (zeroed before the launch)
+    float* part;        // 2 buffers x 2 gridDim floats
+    float* sums;        // 2 buffers x 2 floats
+    unsigned* bar;      // arrival counter, release generation, largest exponent field of the
+                        // substep's v (two, by parity); zeroed before the launch
     int* status;
     double xi[80];
     double dd[80];
@@ -116,16 +136,25 @@ struct Entries {
 };
 
 __global__ void __launch_bounds__(LJ_THREADS) leja_persistent_kernel(const LejaArgs a) {
-    __shared__ double sh[2 * (LJ_THREADS / 32)];
+    __shared__ float sh[2 * (LJ_THREADS / 32)];
     const Entries it(a.n, a.r);
     unsigned b = 0;
     // v = X (Y may be X: every entry is read and written by its own thread)
     for (int row = it.row0, j = it.j0; row < a.n; it.next(row, j))
         a.Wa[(size_t)row * a.ldw + j] = a.X[(size_t)row * a.ldx + j];
     for (int sub = 0; sub < a.substeps; ++sub) {
-        for (int row = it.row0, j = it.j0; row < a.n; it.next(row, j))   // p = d_0 v
-            a.Y[(size_t)row * a.ldy + j] = a.dd[0] * a.Wa[(size_t)row * a.ldw + j];
+        int em = 0;
+        for (int row = it.row0, j = it.j0; row < a.n; it.next(row, j)) {   // p = d_0 v
+            const double v = a.Wa[(size_t)row * a.ldw + j];
+            a.Y[(size_t)row * a.ldy + j] = a.dd[0] * v;
+            em = max(em, exp_field(v));
+        }
+        em = __reduce_max_sync(0xffffffffu, em);
+        if ((threadIdx.x & 31) == 0) atomicMax(a.bar + 2 + (sub & 1), (unsigned)em);
         if (!grid_barrier(a.bar, ++b, nullptr, nullptr, a.status, sh)) return;
+        const int e0 = (int)__ldcg(a.bar + 2 + (sub & 1));
+        // the other parity's word is read again only after the barriers of this substep
+        if (blockIdx.x == 0 && threadIdx.x == 0) atomicExch(a.bar + 2 + ((sub + 1) & 1), 0u);
         const double* W = a.Wa;
         double* Wn = a.Wb;
         int small = 0;
@@ -133,7 +162,7 @@ __global__ void __launch_bounds__(LJ_THREADS) leja_persistent_kernel(const LejaA
             // val holds A^T / g, so w_{k+1} = val w_k - (c/g + x_k) w_k: one FP64
             // FMA per stored entry plus one (FP64 issue is the bound on this part)
             const double beta = a.c * a.invg + a.xi[k - 1], dk = a.dd[k];
-            double aw = 0.0, ap = 0.0;
+            float aw = 0.0f, ap = 0.0f;
             for (int row = it.row0, j = it.j0; row < a.n; it.next(row, j)) {
                 double wn = -beta * __ldcg(W + (size_t)row * a.ldw + j);
                 for (int q = a.ptr[row]; q < a.ptr[row + 1]; ++q)
@@ -141,12 +170,13 @@ __global__ void __launch_bounds__(LJ_THREADS) leja_persistent_kernel(const LejaA
                 Wn[(size_t)row * a.ldw + j] = wn;
                 const double pv = fma(dk, wn, a.Y[(size_t)row * a.ldy + j]);
                 a.Y[(size_t)row * a.ldy + j] = pv;
-                aw = fma(wn, wn, aw);
-                ap = fma(pv, pv, ap);
+                const float fw = mag(wn, e0), fp = mag(pv, e0);
+                aw = fmaf(fw, fw, aw);
+                ap = fmaf(fp, fp, ap);
             }
             block_sum2(aw, ap, sh);
-            double* part = a.part + (size_t)(k & 1) * 2 * gridDim.x;
-            double* sums = a.sums + 2 * (k & 1);
+            float* part = a.part + (size_t)(k & 1) * 2 * gridDim.x;
+            float* sums = a.sums + 2 * (k & 1);
             if (threadIdx.x == 0) {
                 part[2 * blockIdx.x] = aw;
                 part[2 * blockIdx.x + 1] = ap;
@@ -154,7 +184,7 @@ __global__ void __launch_bounds__(LJ_THREADS) leja_persistent_kernel(const LejaA
             if (!grid_barrier(a.bar, ++b, part, sums, a.status, sh)) return;
             const double nw = __ldcg(sums), np = __ldcg(sums + 1);
             // stop after two consecutive terms |d_k| |w_k| <= tol |p|
-            if (fabs(dk) * sqrt(nw) <= a.tol * sqrt(np)) ++small;
+            if (dk * dk * nw <= a.tol * a.tol * np) ++small;
             else small = 0;
             double* t = const_cast<double*>(W);
             W = Wn;
@@ -238,8 +268,8 @@ dme_status launch_leja_apply(const LejaCall& c, cudaStream_t st) {
     a.tol = c.tol;
     a.substeps = c.substeps;
     a.terms = c.terms;
-    a.part = c.part;
-    a.sums = c.sums;
+    a.part = reinterpret_cast<float*>(c.part);
+    a.sums = reinterpret_cast<float*>(c.sums);
     a.bar = c.bar;
     a.status = c.status;
     for (int i = 0; i < 80; ++i) {
@@ -257,7 +287,7 @@ dme_status launch_leja_apply(const LejaCall& c, cudaStream_t st) {
             a.X = c.Y;
             a.ldx = c.ldy;
         }
-        DME_CUDA_TRY(cudaMemsetAsync(c.bar, 0, 2 * sizeof(unsigned), st));
+        DME_CUDA_TRY(cudaMemsetAsync(c.bar, 0, 4 * sizeof(unsigned), st));
         void* args[] = {&a};
         DME_TRY(coop_launch(reinterpret_cast<const void*>(leja_persistent_kernel), dim3(grid), dim3(LJ_THREADS),
                             args, 0, st, leja_per_sm()));

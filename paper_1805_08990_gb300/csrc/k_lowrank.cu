@@ -446,20 +446,71 @@ __global__ void __launch_bounds__(256) select_kernel(const double* __restrict__ 
     if (tid == 0) *k_out = kcount;
 }
 
-// F = V diag(psi) V^T, psi_i = -t / (sqrt(1 + t l_i) (1 + sqrt(1 + t l_i))), l_i >= 0:
-// the matrix function with G F G^T = (I + t G G^T)^{-1/2} - I.
-__global__ void ric_weights_kernel(const double* __restrict__ lam, const double* __restrict__ Vt, int ldv, int m,
-                                   double t, double* __restrict__ F, int ldf) {
-    for (int e = threadIdx.x; e < m * m; e += blockDim.x) {
-        const int a = e / m, b = e % m;
-        double acc = 0.0;
-        for (int i = 0; i < m; ++i) {
-            const double l = fmax(lam[i], 0.0);
-            const double sq = sqrt(1.0 + t * l);
-            const double psi = -t / (sq * (1.0 + sq));
-            acc += Vt[(size_t)i * ldv + a] * psi * Vt[(size_t)i * ldv + b];
+// Y = G F^T (r x m) with F = -t K^{-T} (K + I)^{-1}, K the Cholesky factor of
+// I + t G^T G (m x m): (I + G F G^T)(I + G F G^T)^T = (I + t G G^T)^{-1} (Andrews' square
+// root of the rank-m downdate).  One block: H = G^T G a warp per entry of its upper
+// triangle, then the m x m part in one warp, Y by all threads.
+__global__ void __launch_bounds__(256) ric_factor_kernel(const double* __restrict__ G, int r, int m, double t,
+                                                         double* __restrict__ Y, int* status) {
+    __shared__ double K[32][33], F[32][33];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    int bad = 0;
+    for (int e = warp; e < m * m; e += 8) {
+        const int i = e / m, j = e % m;
+        if (i > j) continue;
+        double s = 0.0;
+        for (int q = lane; q < r; q += 32) s = fma(G[(size_t)q * m + i], G[(size_t)q * m + j], s);
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+        if (!isfinite(s)) bad = 1;
+        if (lane == 0) {
+            const double v = (i == j ? 1.0 : 0.0) + t * s;
+            K[i][j] = v;
+            K[j][i] = v;
         }
-        F[(size_t)a * ldf + b] = acc;
+    }
+    if (__syncthreads_or(bad)) {
+        if (tid == 0) atomicOr(status, DEV_NONFINITE);
+        return;
+    }
+    if (warp == 0) {
+        // Cholesky in place (lower): I + t G^T G is positive definite
+        for (int j = 0; j < m; ++j) {
+            double dj = K[j][j];
+            for (int k = 0; k < j; ++k) dj -= K[j][k] * K[j][k];
+            dj = sqrt(dj);
+            __syncwarp();
+            if (lane > j && lane < m) {
+                double s = K[lane][j];
+                for (int k = 0; k < j; ++k) s -= K[lane][k] * K[j][k];
+                K[lane][j] = s / dj;
+            }
+            __syncwarp();
+            if (lane == 0) K[j][j] = dj;
+            __syncwarp();
+        }
+        // column `lane` of F: (K + I) x = e, then K^T y = x
+        if (lane < m) {
+            double x[32];
+            for (int i = 0; i < m; ++i) {
+                double s = i == lane ? 1.0 : 0.0;
+                for (int k = 0; k < i; ++k) s -= K[i][k] * x[k];
+                x[i] = s / (K[i][i] + 1.0);
+            }
+            for (int i = m - 1; i >= 0; --i) {
+                double s = x[i];
+                for (int k = i + 1; k < m; ++k) s -= K[k][i] * x[k];
+                x[i] = s / K[i][i];
+                F[i][lane] = -t * x[i];
+            }
+        }
+    }
+    __syncthreads();
+    for (int e = tid; e < r * m; e += blockDim.x) {
+        const int q = e / m, i = e % m;
+        double s = 0.0;
+        for (int k = 0; k < m; ++k) s = fma(G[(size_t)q * m + k], F[i][k], s);
+        Y[(size_t)q * m + i] = s;
     }
 }
 
@@ -711,9 +762,9 @@ void launch_sym_scale(double* G, int ldg, int r, const double* d, cudaStream_t s
     sym_scale_kernel<<<std::min(1024, (r * r + 255) / 256), 256, 0, st>>>(G, ldg, r, d);
 }
 
-void launch_ric_weights(const double* lam, const double* Vt, int ldv, int m, double t, double* F, int ldf,
-                        cudaStream_t st) {
-    ric_weights_kernel<<<1, 256, 0, st>>>(lam, Vt, ldv, m, t, F, ldf);
+void launch_ric_factor(const double* G, int r, int m, double t, double* Y, int* status, cudaStream_t st) {
+    if (r <= 0 || m <= 0) return;
+    ric_factor_kernel<<<1, 256, 0, st>>>(G, r, m, t, Y, status);
 }
 
 void launch_copy_cols(double* Y, int ldy, const double* X, int ldx, int n, int k, double alpha, const double* d,

@@ -8,8 +8,8 @@
 //   T_12(t): L <- [E_t^T L, L_I], d <- [d, d_I]   then compression; (L_I, d_I) is the
 //            compressed Gauss-Legendre factor of W_t (Alg. 2), built once per t
 //   T_3(t):  with Lt = L diag(d)^{1/2} and G = Lt^T Bt (r x m):
-//            L <- Lt (I + t G G^T)^{-1/2} = Lt + (Lt G) F(G^T G) G^T, d <- 1, where
-//            F(x) = -t / (sqrt(1 + t x)(1 + sqrt(1 + t x))); equal to the §2.2 form
+//            L <- Lt (I + G F G^T), d <- 1, F = -t K^{-T} (K + I)^{-1} with
+//            K K^T = I + t G^T G: a square root of (I + t G G^T)^{-1}; equal to the §2.2 form
 //            L (I + t D L^T B R^{-1} B^T L)^{-1} D L^T by the push-through identity
 //   T_4(t):  L <- [L, sqrt(t) S L, sqrt(t/2) S (sqrt(t) S L)], d <- [d, d, d] (midpoint)
 //            or [L, sqrt(t) S L], [d, d] (Euler), then compression
@@ -71,7 +71,7 @@ struct dme_lr_s {
     double* LQ = nullptr;                                            // C^T, n x p
     double *G = nullptr, *Vt = nullptr, *lam = nullptr, *T = nullptr;  // rcap x rcap work
     double *J1 = nullptr, *J2 = nullptr, *J3 = nullptr, *J4 = nullptr;  // rcap x rcap eigensolver work
-    double *Gm = nullptr, *H = nullptr, *VtH = nullptr, *lamH = nullptr, *F = nullptr, *Y = nullptr, *Z = nullptr;
+    double *Gm = nullptr, *Y = nullptr, *Z = nullptr;
     double* Pout = nullptr;   // n x n, allocated on the first dense output
     int* kdev = nullptr;
     bool split = false;            // the products with E_t and S on the tensor cores
@@ -596,10 +596,7 @@ dme_status lr_T3(dme_lr_t lr, double tau) {
     const int n = lr->n, m = lr->m, r = lr->r, rc = lr->rcap;
     launch_copy_cols(lr->L2, rc, lr->L, rc, n, r, 1.0, lr->d, st);                              // Lt
     DME_TRY(gemm(lr, mk(r, m, n, lr->L2, rc, 1, lr->Bt, m, 0, lr->Gm, m, 1.0), st));              // G = Lt^T Bt
-    DME_TRY(gemm(lr, mk(m, m, r, lr->Gm, m, 1, lr->Gm, m, 0, lr->H, m, 1.0, 1), st));                // G^T G
-    DME_TRY(launch_jacobi_eig(lr->H, m, m, lr->VtH, m, lr->lamH, lr->status, st));
-    launch_ric_weights(lr->lamH, lr->VtH, m, m, tau, lr->F, m, st);                               // F(G^T G)
-    DME_TRY(gemm(lr, mk(r, m, m, lr->Gm, m, 0, lr->F, m, 0, lr->Y, m, 1.0), st));                    // Y = G F
+    launch_ric_factor(lr->Gm, r, m, tau, lr->Y, lr->status, st);                                   // Y = G F^T
     DME_TRY(gemm(lr, mk(n, m, r, lr->L2, rc, 0, lr->Gm, m, 0, lr->Z, m, 1.0), st));                  // Z = Lt G
     DME_TRY(gemm(lr, mk(n, r, m, lr->Z, m, 0, lr->Y, m, 1, lr->L, rc, 1.0, 0, lr->L2, 1.0), st));    // L = Lt + Z Y^T
     launch_fill(lr->d, r, 1.0, st);
@@ -768,10 +765,6 @@ dme_status lr_setup(dme_lr_t lr, const dme_plan_desc* desc, const double* C, int
     DME_TRY(lr_alloc(lr, &lr->J3, rc * rc));
     DME_TRY(lr_alloc(lr, &lr->J4, rc * rc));
     DME_TRY(lr_alloc(lr, &lr->Gm, rc * m));
-    DME_TRY(lr_alloc(lr, &lr->H, m * m));
-    DME_TRY(lr_alloc(lr, &lr->VtH, m * m));
-    DME_TRY(lr_alloc(lr, &lr->lamH, m));
-    DME_TRY(lr_alloc(lr, &lr->F, m * m));
     DME_TRY(lr_alloc(lr, &lr->Y, rc * m));
     DME_TRY(lr_alloc(lr, &lr->Z, n * m));
     lr->ws_doubles = std::max<size_t>((size_t)8 * rc * rc, (size_t)kSplitMax * rc * m);
