@@ -46,28 +46,31 @@ using namespace tc;
 
 constexpr int OZ_BM = 128, OZ_BN = 128, OZ_BK = 32;
 constexpr int OZ_SLICE_BYTES = OZ_BM * OZ_BK * 2;                 // 8 KB per slice tile
-constexpr int OZ_NACC = 4;                                        // accumulators: levels 0, 1, 2, >= 3
 constexpr uint64_t OZ_TIMEOUT_NS = 2000000000ull;                 // 2 s per wait
 constexpr int OZ_EPI_WARPS = 8;                                  // two per TMEM lane quadrant
 constexpr int OZ_THREADS = 64 + 32 * OZ_EPI_WARPS;               // producer + MMA warps + epilogue
-constexpr int OZ_EPI_COLS = OZ_BN / (OZ_EPI_WARPS / 4);          // columns per epilogue warp (64)
-constexpr uint32_t OZ_IDESC = idesc_bf16_f32(OZ_BM, OZ_BN);
 
 // Epilogue staging buffer: 32 tile columns x 128 rows of 8-byte outputs (row
 // stride 129 words), through which the epilogue writes row segments coalesced.
 constexpr int OZ_EPI_STAGE_BYTES = 32 * (OZ_BM + 1) * 8;
 
-template <int SA_, int SB_, int L_, int STAGES_, bool ACC_, int NACC_ = 4>
+// BN: tile columns.  128, or for products of few tiles 64 or 32: a 128 x 128 tile's FP64
+// epilogue alone keeps one SM's FP64 pipe busy for 16 us, so a product of fewer tiles
+// than SMs is cut into narrower ones (the MMAs of an output are the same in any width).
+template <int SA_, int SB_, int L_, int STAGES_, bool ACC_, int NACC_ = 4, int BN_ = OZ_BN>
 struct OzCfg {
-    static constexpr int SA = SA_, SB = SB_, L = L_, STAGES = STAGES_;
+    static constexpr int SA = SA_, SB = SB_, L = L_, STAGES = STAGES_, BN = BN_;
+    static constexpr int EC = BN / (OZ_EPI_WARPS / 4);              // columns per epilogue warp
+    static constexpr int B_SLICE_BYTES = BN * OZ_BK * 2;
+    static constexpr uint32_t IDESC = idesc_bf16_f32(OZ_BM, BN);
     static constexpr bool ACC = ACC_;                                // accurate mode (exact chunks)
     // TMEM accumulators: levels 0, 1, 2, >= 3 (4), or level 0 and levels >= 1 (2: products
     // of at most 64 K, where the shared accumulator rounds at most four times)
     static constexpr int NACC = NACC_;
-    static constexpr int TMEM_COLS = NACC * OZ_BN;
+    static constexpr int TMEM_COLS = NACC * BN;
     static constexpr int MIN_BLOCKS = NACC == 2 ? 2 : 1;            // CTAs per SM the registers allow
     static constexpr int A_BYTES = SA * OZ_SLICE_BYTES;
-    static constexpr int STAGE_BYTES = (SA + SB) * OZ_SLICE_BYTES;
+    static constexpr int STAGE_BYTES = SA * OZ_SLICE_BYTES + SB * B_SLICE_BYTES;
     // the staged epilogue when the buffer fits beside the stage ring
     static constexpr bool STAGED_EPI = !ACC && STAGES * STAGE_BYTES + OZ_EPI_STAGE_BYTES + 1024 + 256 <= 232448;
     static constexpr int EPI_BYTES = STAGED_EPI ? OZ_EPI_STAGE_BYTES : 0;
@@ -86,6 +89,13 @@ using CfgP13s = OzCfg<4, 4, 4, 1, false, 2>;
 using CfgP14s = OzCfg<5, 4, 4, 1, false, 2>;
 using CfgP14 = OzCfg<5, 4, 4, 3, false>;
 using CfgA21 = OzCfg<6, 6, 5, 2, true>;
+// narrow tiles
+using CfgP13n64 = OzCfg<4, 4, 4, 4, false, 4, 64>;
+using CfgP13n32 = OzCfg<4, 4, 4, 4, false, 4, 32>;
+using CfgP14n64 = OzCfg<5, 4, 4, 3, false, 4, 64>;
+using CfgP14n32 = OzCfg<5, 4, 4, 4, false, 4, 32>;
+static_assert(CfgP13n64::STAGED_EPI && CfgP13n32::STAGED_EPI && CfgP14n64::STAGED_EPI && CfgP14n32::STAGED_EPI,
+              "narrow tiles stage their epilogue");
 static_assert(CfgP14::SMEM <= 232448 && CfgA21::SMEM <= 232448, "shared memory per CTA");
 static_assert(2 * CfgP14s::SMEM <= 232448 && 2 * CfgP10s::SMEM <= 232448, "two short CTAs per SM");
 static_assert(CfgP14e::STAGED_EPI, "the two-stage 14-product form stages its epilogue");
@@ -441,6 +451,27 @@ __device__ __forceinline__ void oz_tile_coords(const OzParams& p, int t, int& tm
     }
 }
 
+// Tiles of BN < 128 columns: column by column, for a triangle only the tiles with an entry
+// on or above the diagonal (oz_tile_count of them).
+__host__ __device__ __forceinline__ int oz_narrow_rows(const OzParams& p, int bn, int c) {
+    const int all = (p.M + OZ_BM - 1) / OZ_BM;
+    if (!p.tri) return all;
+    const int r = (c * bn + bn - 1) / OZ_BM + 1;
+    return r < all ? r : all;
+}
+
+__device__ __forceinline__ void oz_narrow_coords(const OzParams& p, int bn, int t, int& tm, int& tn) {
+    int c = 0;
+    while (true) {
+        const int r = oz_narrow_rows(p, bn, c);
+        if (t < r) break;
+        t -= r;
+        ++c;
+    }
+    tm = t;
+    tn = c;
+}
+
 // Exact float -> double conversion of a normal or zero float by bit moves
 // (subnormal floats are flushed to zero; the epilogue never produces them
 // for in-range data).
@@ -464,6 +495,7 @@ struct OzUnit {
     int tm, tn, kb0, nk, part, nparts, widx, chunk;
 };
 
+template <int BN>
 __device__ __forceinline__ void oz_single_unit(const OzParams* p, const CUtensorMap* tA, const CUtensorMap* tB,
                                                bool acc, int u, OzUnit& o) {
     o.p = p;
@@ -482,7 +514,8 @@ __device__ __forceinline__ void oz_single_unit(const OzParams* p, const CUtensor
         nparts = p->split_parts;
         widx = j / p->split_parts;
     }
-    oz_tile_coords(*p, tile, o.tm, o.tn);
+    if (BN == OZ_BN) oz_tile_coords(*p, tile, o.tm, o.tn);
+    else oz_narrow_coords(*p, BN, tile, o.tm, o.tn);
     if (acc) {
         o.kb0 = chunk * OZ_ACC_CHUNK_KB;
         o.nk = min(OZ_ACC_CHUNK_KB, nk_all - o.kb0);
@@ -496,6 +529,7 @@ __device__ __forceinline__ void oz_single_unit(const OzParams* p, const CUtensor
     o.chunk = chunk;
 }
 
+template <int BN>
 __device__ __forceinline__ void oz_group_unit(const OzGroupDesc* __restrict__ d, int nd, int u, OzUnit& o) {
     int lo = 0, hi = nd - 1;
     while (lo < hi) {
@@ -503,64 +537,69 @@ __device__ __forceinline__ void oz_group_unit(const OzGroupDesc* __restrict__ d,
         if (d[mid].start <= u) lo = mid;
         else hi = mid - 1;
     }
-    oz_single_unit(&d[lo].p, &d[lo].tmA, &d[lo].tmB, false, u - d[lo].start, o);
+    oz_single_unit<BN>(&d[lo].p, &d[lo].tmA, BN == OZ_BN ? &d[lo].tmB : (BN == 64 ? &d[lo].tmB64 : &d[lo].tmB32), false,
+                       u - d[lo].start, o);
 }
 
-// Load 32 columns of the four accumulators of TMEM lane quadrant q at column c0
-// into h (level 0, raw fp32 bits) and l (levels 1 + 2 + 3.., as fp32 bits).
-// (The levels 2 and 3 come through a 16-column temporary: the epilogue warps
+// Load EC columns of the four accumulators (BN columns apart) of TMEM lane quadrant q at
+// column c0 into h (level 0, raw fp32 bits) and l (levels 1 + 2 + 3.., as fp32 bits).
+// (The levels 2 and 3 come through a 16-column temporary: at EC = 64 the epilogue warps
 // hold 128 values each and the kernel's register budget is 168.)
-__device__ __forceinline__ void oz_load_half(uint32_t tmem, int q, int c0, uint32_t (&h)[32], uint32_t (&l)[32]) {
+template <int BN, int EC>
+__device__ __forceinline__ void oz_load_cols(uint32_t tmem, int q, int c0, uint32_t (&h)[EC], uint32_t (&l)[EC]) {
     const uint32_t ta = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)c0;
-    tmem_ld_32x32b_x32(ta, h);
-    tmem_ld_32x32b_x32(ta + OZ_BN, l);
 #pragma unroll
-    for (int g = 0; g < 2; ++g) {
+    for (int g = 0; g < EC; g += 16) {
         uint32_t t[16];
-        tmem_ld_32x32b_x16(ta + 2 * OZ_BN + 16 * g, t);
+        tmem_ld_32x32b_x16(ta + g, h + g);
+        tmem_ld_32x32b_x16(ta + BN + g, l + g);
+        tmem_ld_32x32b_x16(ta + 2 * BN + g, t);
         tmem_ld_wait();
 #pragma unroll
         for (int jj = 0; jj < 16; ++jj)
-            l[16 * g + jj] = __float_as_uint(__uint_as_float(l[16 * g + jj]) + __uint_as_float(t[jj]));
-        tmem_ld_32x32b_x16(ta + 3 * OZ_BN + 16 * g, t);
+            l[g + jj] = __float_as_uint(__uint_as_float(l[g + jj]) + __uint_as_float(t[jj]));
+        tmem_ld_32x32b_x16(ta + 3 * BN + g, t);
         tmem_ld_wait();
 #pragma unroll
         for (int jj = 0; jj < 16; ++jj)
-            l[16 * g + jj] = __float_as_uint(__uint_as_float(l[16 * g + jj]) + __uint_as_float(t[jj]));
+            l[g + jj] = __float_as_uint(__uint_as_float(l[g + jj]) + __uint_as_float(t[jj]));
     }
 }
 
-// Epilogue of 32 columns (tile columns c0 .. c0+31) of row i from registers.
-__device__ __forceinline__ void oz_store_half(const OzParams& p, int m0, int n0, int i, int c0, bool diag,
-                                              const uint32_t (&h)[32], const uint32_t (&l)[32]) {
-    if (i >= p.M) return;
-    const float sA = p.sa[i];
-    if (p.mode == OZ_OUT_PAIR) {
+// The column scales of the EC columns from c0 of a warp, lane l holding those of the columns
+// l, l + 32 (handed out by shuffles: a load per output would wait for each store before it).
+template <int EC>
+struct OzColScale {
+    float s[EC > 32 ? 2 : 1];
+    __device__ __forceinline__ OzColScale(const OzParams& p, int j0, int lane) {
 #pragma unroll
-        for (int jj = 0; jj < 32; ++jj) {
-            const int j = n0 + c0 + jj;
-            if (j >= p.N) break;
-            const float s = sA * p.sb[j];
-            const float hv = __uint_as_float(h[jj]), lv = __uint_as_float(l[jj]);
-            // TwoSum: (sh, sl) = hi + lo exactly
-            const float sh = hv + lv;
-            const float bb = sh - hv;
-            const float sl = (hv - (sh - bb)) + (lv - bb);
-            p.Cp[(size_t)i * p.ldc + j] = make_float2(sh * s, sl * s);
-        }
-        return;
+        for (int g = 0; g < (EC > 32 ? 2 : 1); ++g) s[g] = j0 + 32 * g + lane < p.N ? p.sb[j0 + 32 * g + lane] : 0.0f;
     }
+    __device__ __forceinline__ float at(int jj) const { return __shfl_sync(0xffffffffu, s[jj / 32], jj % 32); }
+};
+
+// Epilogue of one row (thread) and EC columns from tile column c0 straight from registers.
+template <int EC>
+__device__ __forceinline__ void oz_store_direct(const OzParams& p, int n0, int i, int c0, bool diag,
+                                                const OzColScale<EC>& sc, const uint32_t (&h)[EC],
+                                                const uint32_t (&l)[EC]) {
+    const float sA = i < p.M ? p.sa[i] : 0.0f;
     const double alpha = p.alpha;
 #pragma unroll
-    for (int jj = 0; jj < 32; ++jj) {
+    for (int jj = 0; jj < EC; ++jj) {
         const int j = n0 + c0 + jj;
-        if (j >= p.N) break;
-        if (diag && i > j) continue;                   // lower half of a diagonal tile: its mirror owns it
-        const float s = sA * p.sb[j];
+        const float s = sA * sc.at(jj);
+        if (j >= p.N || i >= p.M) continue;
         const float hv = __uint_as_float(h[jj]), lv = __uint_as_float(l[jj]);
+        // TwoSum: (sh, sl) = hi + lo exactly
         const float sh = hv + lv;
         const float bb = sh - hv;
         const float sl = (hv - (sh - bb)) + (lv - bb);
+        if (p.mode == OZ_OUT_PAIR) {
+            p.Cp[(size_t)i * p.ldc + j] = make_float2(sh * s, sl * s);
+            continue;
+        }
+        if (diag && i > j) continue;                   // lower half of a diagonal tile: its mirror owns it
         double v = f2d_bits(sh * s) + f2d_bits(sl * s);
         if (alpha != 1.0) v *= alpha;
         if (p.tri) {
@@ -583,7 +622,8 @@ __device__ __forceinline__ void oz_store_half(const OzParams& p, int m0, int n0,
 }
 
 // Staged epilogue of one 16-column round: the thread of tile row il holds the
-// level sums of columns c0 + h0 .. c0 + h0 + 15 (entries h0 .. h0 + 15 of h, l).
+// level sums of columns c0 + h0 .. c0 + h0 + 15 (entries h0 .. h0 + 15 of h, l; c0 the first
+// column of its warp).
 // Phase 1: each thread forms its 16 outputs (FP64 value or normalised pair);
 // a triangle output also goes straight to its mirror (j, i), coalesced over the
 // warp's rows, with the symmetric addends read at (j, i); every output is put
@@ -591,64 +631,64 @@ __device__ __forceinline__ void oz_store_half(const OzParams& p, int m0, int n0,
 // T holds 32 tile columns).  Phase 2: the 256 epilogue threads write the 128
 // staged row segments (i, j) coalesced (non-triangle F64 outputs add their
 // addends here, read at (i, j)).  Two named-barrier syncs per round.
-__device__ __forceinline__ void oz_store_staged(const OzParams& p, int m0, int n0, int il, int c0, int h0, bool diag,
-                                                const uint32_t (&h)[32], const uint32_t (&l)[32], uint64_t* T,
-                                                int ew, int lane) {
+// (EC: columns held; EW: columns per warp, the distance of the two warps' columns; o0: the
+// round's first column within the warp's.)
+template <int EC, int EW>
+__device__ __forceinline__ void oz_store_staged_at(const OzParams& p, int m0, int n0, int il, int c0, int h0, int o0,
+                                                bool diag, const OzColScale<EC>& sc, const uint32_t (&h)[EC],
+                                                const uint32_t (&l)[EC], uint64_t* __restrict__ T, int ew, int lane) {
     const int i = m0 + il;
     const int slot = (ew / 4) * 16;                        // T columns of this warp pair: 0..15 or 16..31
-    if (i < p.M) {
-        const float sA = p.sa[i];
-        // four columns at a time: their addends are loaded before any of the four
-        // stores (an in-place update may alias Cd and D1, which would otherwise
-        // serialise every load behind the previous store)
+    const float sA = i < p.M ? p.sa[i] : 0.0f;
+    // DG columns at a time: their addends are loaded before any of the stores (an in-place
+    // update may alias Cd and D1, which would otherwise serialise every load behind the
+    // previous store)
+    constexpr int DG = EW > 32 ? 4 : 8;
 #pragma unroll
-        for (int g = 0; g < 16; g += 4) {
-            double a1[4], a2[4], a3[4];
+    for (int g = 0; g < 16; g += DG) {
+        double a1[DG], a2[DG], a3[DG];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int j = n0 + c0 + h0 + g + u;
-                const bool in = p.mode == OZ_OUT_F64 && p.tri && j < p.N && !(diag && i > j);
-                const size_t tof = (size_t)j * p.ldc + i;
-                a1[u] = (in && p.D1) ? p.D1[tof] : 0.0;
-                a2[u] = (in && p.D2) ? p.D2[tof] : 0.0;
-                a3[u] = (in && p.D3) ? p.D3[tof] : 0.0;
-            }
+        for (int u = 0; u < DG; ++u) {
+            const int j = n0 + c0 + h0 + g + u;
+            const bool in = p.mode == OZ_OUT_F64 && p.tri && j < p.N && i < p.M && !(diag && i > j);
+            const size_t tof = (size_t)j * p.ldc + i;
+            a1[u] = (in && p.D1) ? p.D1[tof] : 0.0;
+            a2[u] = (in && p.D2) ? p.D2[tof] : 0.0;
+            a3[u] = (in && p.D3) ? p.D3[tof] : 0.0;
+        }
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int jj = g + u;
-                const int j = n0 + c0 + h0 + jj;
-                if (j >= p.N) break;
-                const float s = sA * p.sb[j];
-                const float hv = __uint_as_float(h[h0 + jj]), lv = __uint_as_float(l[h0 + jj]);
-                const float sh = hv + lv;
-                const float bb = sh - hv;
-                const float sl = (hv - (sh - bb)) + (lv - bb);
-                uint64_t word;
-                if (p.mode == OZ_OUT_PAIR) {
-                    const float2 v = make_float2(sh * s, sl * s);
-                    word = *reinterpret_cast<const uint64_t*>(&v);
-                } else {
-                    double v = f2d_bits(sh * s) + f2d_bits(sl * s);
-                    if (p.alpha != 1.0) v *= p.alpha;
-                    if (p.tri) {
-                        if (diag && i > j) continue;           // its mirror (j, i) owns this entry
-                        if (p.D1) v += p.b1 * a1[u];
-                        if (p.D2) v += p.b2 * a2[u];
-                        if (p.D3) v += p.b3 * a3[u];
-                        p.Cd[(size_t)j * p.ldc + i] = v;
-                    }
-                    word = (uint64_t)__double_as_longlong(v);
+        for (int u = 0; u < DG; ++u) {
+            const int jj = g + u;
+            const int j = n0 + c0 + h0 + jj;
+            const float s = sA * sc.at(h0 + jj);
+            if (j >= p.N || i >= p.M) continue;
+            const float hv = __uint_as_float(h[h0 + jj]), lv = __uint_as_float(l[h0 + jj]);
+            const float sh = hv + lv;
+            const float bb = sh - hv;
+            const float sl = (hv - (sh - bb)) + (lv - bb);
+            uint64_t word;
+            if (p.mode == OZ_OUT_PAIR) {
+                word = (uint64_t)__float_as_uint(sh * s) | ((uint64_t)__float_as_uint(sl * s) << 32);
+            } else {
+                double v = f2d_bits(sh * s) + f2d_bits(sl * s);
+                if (p.alpha != 1.0) v *= p.alpha;
+                if (p.tri) {
+                    if (diag && i > j) continue;           // its mirror (j, i) owns this entry
+                    if (p.D1) v += p.b1 * a1[u];
+                    if (p.D2) v += p.b2 * a2[u];
+                    if (p.D3) v += p.b3 * a3[u];
+                    p.Cd[(size_t)j * p.ldc + i] = v;
                 }
-                T[(slot + jj) * (OZ_BM + 1) + il] = word;
+                word = (uint64_t)__double_as_longlong(v);
             }
+            T[(slot + jj) * (OZ_BM + 1) + il] = word;
         }
     }
     asm volatile("bar.sync 1, 256;" ::: "memory");
     // phase 2: warp ew writes tile rows 16 ew .. 16 ew + 15; lanes 0-15 the first warp
-    // pair's 16 columns (tile columns c0' + h0 ..), lanes 16-31 the second pair's (c0' + 64)
+    // pair's 16 columns, lanes 16-31 the second pair's (EC columns on)
     const int half = lane >> 4, jl = lane & 15;
-    const int cbase = (c0 - (ew / 4) * 64) + half * 64 + h0;   // tile column of this lane's slot
-    const int j = n0 + cbase + jl;
+    const int j = n0 + half * EW + o0 + jl;
 #pragma unroll 4
     for (int r = 0; r < 16; ++r) {
         const int rl = 16 * ew + r;
@@ -658,7 +698,7 @@ __device__ __forceinline__ void oz_store_staged(const OzParams& p, int m0, int n
         const uint64_t word = T[(half * 16 + jl) * (OZ_BM + 1) + rl];
         const size_t off = (size_t)gi * p.ldc + j;
         if (p.mode == OZ_OUT_PAIR) {
-            p.Cp[off] = *reinterpret_cast<const float2*>(&word);
+            p.Cp[off] = make_float2(__uint_as_float((uint32_t)word), __uint_as_float((uint32_t)(word >> 32)));
         } else {
             double v = __longlong_as_double((long long)word);
             if (!p.tri) {
@@ -747,7 +787,7 @@ __device__ __forceinline__ void oz_persistent(int units, Resolve resolve) {
                 const OzParams& p = *w.p;
                 tma_prefetch_desc(w.tA);
                 tma_prefetch_desc(w.tB);
-                const int m0 = w.tm * OZ_BM, n0 = w.tn * OZ_BN;
+                const int m0 = w.tm * OZ_BM, n0 = w.tn * Cfg::BN;
                 for (int it = 0; it < w.nk; ++it, ++kit) {
                     if (*abort_flag) {
                         ok = false;
@@ -775,16 +815,18 @@ __device__ __forceinline__ void oz_persistent(int units, Resolve resolve) {
                     // of them at the last k block of a short one (full 128-column segments
                     // only, 16-byte aligned; transposed for tri outputs)
                     if (!Cfg::ACC && p.mode == OZ_OUT_F64 && (p.ldc % 2) == 0 && (p.D1 || p.D2)) {
-                        const int r0 = it, r1 = (it == w.nk - 1) ? OZ_BM : min(it + 1, OZ_BM);
+                        // rows of the addend tile (transposed for tri outputs) and their length
+                        const int nr = p.tri ? Cfg::BN : OZ_BM, seg = p.tri ? OZ_BM : Cfg::BN;
+                        const int r0 = it, r1 = (it == w.nk - 1) ? nr : min(it + 1, nr);
                         for (int rr = r0; rr < r1; ++rr) {
                             const int ra = (p.tri ? n0 : m0) + rr, ca = p.tri ? m0 : n0;
                             const int rmax = p.tri ? p.N : p.M, cmax = p.tri ? p.M : p.N;
-                            if (ra >= rmax || ca + OZ_BN > cmax) continue;
+                            if (ra >= rmax || ca + seg > cmax) continue;
                             const size_t off = (size_t)ra * p.ldc + ca;
                             if (p.D1 && ((reinterpret_cast<uintptr_t>(p.D1 + off) & 15) == 0))
-                                prefetch_l2_bulk(p.D1 + off, OZ_BN * sizeof(double));
+                                prefetch_l2_bulk(p.D1 + off, seg * sizeof(double));
                             if (p.D2 && ((reinterpret_cast<uintptr_t>(p.D2 + off) & 15) == 0))
-                                prefetch_l2_bulk(p.D2 + off, OZ_BN * sizeof(double));
+                                prefetch_l2_bulk(p.D2 + off, seg * sizeof(double));
                         }
                     }
                 }
@@ -836,11 +878,18 @@ __device__ __forceinline__ void oz_persistent(int units, Resolve resolve) {
                                 if (sa + sb > Cfg::L || sa + sb > Lu) continue;
                                 const int lvl = (sa + sb < Cfg::NACC - 1) ? sa + sb : Cfg::NACC - 1;
                                 const uint64_t ad = desc_kmajor_sw64(a0 + sa * OZ_SLICE_BYTES + kk * 32);
-                                const uint64_t bd = desc_kmajor_sw64(b0 + sb * OZ_SLICE_BYTES + kk * 32);
+                                const uint64_t bd = desc_kmajor_sw64(b0 + sb * Cfg::B_SLICE_BYTES + kk * 32);
                                 // the pairs (0, t), t <= 3, come first and open accumulator t at the
                                 // unit's first k step; everything else accumulates
                                 const uint32_t acc = (it == 0 && kk == 0 && sa == 0 && sb < Cfg::NACC) ? 0u : 1u;
-                                mma_bf16(tmem + (uint32_t)(lvl * OZ_BN), ad, bd, OZ_IDESC, acc);
+                                // the pairs of one A slice follow one another: its operand is read from
+                                // shared memory once and kept in the collector
+                                const uint32_t dt = tmem + (uint32_t)(lvl * Cfg::BN);
+                                const int nb = min(Cfg::SB - 1, Cfg::L - sa);      // this A slice's last pair
+                                if (nb == 0) mma_bf16(dt, ad, bd, Cfg::IDESC, acc);
+                                else if (sb == 0) mma_bf16_keep_a<MMA_A_FILL>(dt, ad, bd, Cfg::IDESC, acc);
+                                else if (sb < nb) mma_bf16_keep_a<MMA_A_USE>(dt, ad, bd, Cfg::IDESC, acc);
+                                else mma_bf16_keep_a<MMA_A_LASTUSE>(dt, ad, bd, Cfg::IDESC, acc);
                             }
                         }
                     }
@@ -861,7 +910,7 @@ __device__ __forceinline__ void oz_persistent(int units, Resolve resolve) {
         // [cq, cq + 64) with cq = 64 * ((w - 2) / 4)
         const int q = warp & 3;
         const int ew = warp - 2;                                   // 0 .. OZ_EPI_WARPS-1
-        const int cq = OZ_EPI_COLS * (ew / 4);
+        const int cq = Cfg::EC * (ew / 4);
         int li = 0;
         for (int u = blockIdx.x; u < units; u += gridDim.x, ++li) {
             OzUnit w;
@@ -886,7 +935,7 @@ __device__ __forceinline__ void oz_persistent(int units, Resolve resolve) {
                 break;
             }
             fence_after_sync();
-            const int m0 = w.tm * OZ_BM, n0 = w.tn * OZ_BN;
+            const int m0 = w.tm * OZ_BM, n0 = w.tn * Cfg::BN;
             const int il = 32 * q + lane;                          // tile row of this thread
             const int i = m0 + il;
             if (Cfg::ACC) {
@@ -897,62 +946,55 @@ __device__ __forceinline__ void oz_persistent(int units, Resolve resolve) {
                 if (lane == 0) mbar_arrive(acc_empty);
                 continue;
             }
+            // tri: whether the tile holds entries below the diagonal
+            const bool diag = p.tri && n0 < m0 + OZ_BM;
             if (Cfg::NACC == 2) {
                 // short products (never split in K): 32 columns at a time, TMEM released at
                 // the end (the next unit's product is as short), so that the registers allow
                 // two CTAs per SM
-                const bool diag = p.tri && w.tm == w.tn;
 #pragma unroll
-                for (int hh = 0; hh < 2; ++hh) {
+                for (int hh = 0; hh < Cfg::EC / 32; ++hh) {
                     uint32_t hs[32], ls[32];
                     const uint32_t ta = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(cq + 32 * hh);
                     tmem_ld_32x32b_x32(ta, hs);
-                    tmem_ld_32x32b_x32(ta + OZ_BN, ls);
+                    tmem_ld_32x32b_x32(ta + Cfg::BN, ls);
                     tmem_ld_wait();
-                    oz_store_staged(p, m0, n0, il, cq + 32 * hh, 0, diag, hs, ls, stage_T, ew, lane);
-                    oz_store_staged(p, m0, n0, il, cq + 32 * hh, 16, diag, hs, ls, stage_T, ew, lane);
+                    const OzColScale<32> sc(p, n0 + cq + 32 * hh, lane);
+                    // (the second half's columns of the other warp pair lie EC on as well)
+                    oz_store_staged_at<32, Cfg::EC>(p, m0, n0, il, cq + 32 * hh, 0, 32 * hh, diag, sc, hs, ls, stage_T, ew,
+                                                    lane);
+                    oz_store_staged_at<32, Cfg::EC>(p, m0, n0, il, cq + 32 * hh, 16, 32 * hh + 16, diag, sc, hs, ls, stage_T,
+                                                    ew, lane);
                 }
                 fence_before_sync();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(acc_empty);
                 continue;
             }
-            uint32_t h0[32], l0[32], h1[32], l1[32];
-            if (Cfg::NACC == 4) {
-                oz_load_half(tmem, q, cq, h0, l0);
-                oz_load_half(tmem, q, cq + 32, h1, l1);
-            } else {
-                const uint32_t ta = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)cq;
-                tmem_ld_32x32b_x32(ta, h0);
-                tmem_ld_32x32b_x32(ta + OZ_BN, l0);
-                tmem_ld_32x32b_x32(ta + 32, h1);
-                tmem_ld_32x32b_x32(ta + OZ_BN + 32, l1);
-                tmem_ld_wait();
-            }
+            constexpr int EC = Cfg::EC;
+            uint32_t h[EC], l[EC];
+            oz_load_cols<Cfg::BN, EC>(tmem, q, cq, h, l);
             // the accumulators are in registers: hand TMEM back to the MMA warp
             fence_before_sync();
             __syncwarp();
             if (lane == 0) mbar_arrive(acc_empty);
             if (w.nparts > 1) {
-                // split K: publish this part's level sums; oz_tail_kernel adds the parts
+                // split K: publish this part's level sums (column-major, so that a warp's rows
+                // are contiguous); oz_tail_kernel adds the parts
                 constexpr size_t tile_elems = (size_t)OZ_BM * OZ_BN;
-                float2* mine = p.ws + ((size_t)w.widx * w.nparts + w.part) * tile_elems + (size_t)il * OZ_BN + cq;
+                float2* mine = p.ws + ((size_t)w.widx * w.nparts + w.part) * tile_elems + (size_t)cq * OZ_BM + il;
 #pragma unroll
-                for (int jj = 0; jj < 32; ++jj) {
-                    mine[jj] = make_float2(__uint_as_float(h0[jj]), __uint_as_float(l0[jj]));
-                    mine[32 + jj] = make_float2(__uint_as_float(h1[jj]), __uint_as_float(l1[jj]));
-                }
+                for (int jj = 0; jj < EC; ++jj)
+                    mine[(size_t)jj * OZ_BM] = make_float2(__uint_as_float(h[jj]), __uint_as_float(l[jj]));
                 continue;
             }
-            const bool diag = p.tri && w.tm == w.tn;
+            const OzColScale<EC> sc(p, n0 + cq, lane);
             if (Cfg::STAGED_EPI) {
-                oz_store_staged(p, m0, n0, il, cq, 0, diag, h0, l0, stage_T, ew, lane);
-                oz_store_staged(p, m0, n0, il, cq, 16, diag, h0, l0, stage_T, ew, lane);
-                oz_store_staged(p, m0, n0, il, cq + 32, 0, diag, h1, l1, stage_T, ew, lane);
-                oz_store_staged(p, m0, n0, il, cq + 32, 16, diag, h1, l1, stage_T, ew, lane);
+#pragma unroll
+                for (int r0 = 0; r0 < EC; r0 += 16)
+                    oz_store_staged_at<EC, EC>(p, m0, n0, il, cq, r0, r0, diag, sc, h, l, stage_T, ew, lane);
             } else {
-                oz_store_half(p, m0, n0, i, cq, diag, h0, l0);
-                oz_store_half(p, m0, n0, i, cq + 32, diag, h1, l1);
+                oz_store_direct<EC>(p, n0, i, cq, diag, sc, h, l);
             }
         }
     }
@@ -966,7 +1008,7 @@ template <class Cfg>
 __global__ void __launch_bounds__(OZ_THREADS, Cfg::MIN_BLOCKS) ozaki_gemm_kernel(const __grid_constant__ CUtensorMap tmA,
                                                                    const __grid_constant__ CUtensorMap tmB,
                                                                    const __grid_constant__ OzParams p) {
-    oz_persistent<Cfg>(p.units, [&](int u, OzUnit& o) { oz_single_unit(&p, &tmA, &tmB, Cfg::ACC, u, o); });
+    oz_persistent<Cfg>(p.units, [&](int u, OzUnit& o) { oz_single_unit<Cfg::BN>(&p, &tmA, &tmB, Cfg::ACC, u, o); });
 }
 
 // Grouped form: the tiles of every problem laid end to end; a unit finds its
@@ -976,33 +1018,35 @@ __global__ void __launch_bounds__(OZ_THREADS, Cfg::MIN_BLOCKS) ozaki_gemm_kernel
 template <class Cfg>
 __global__ void __launch_bounds__(OZ_THREADS, 1) ozaki_gemm_grouped_kernel(const OzGroupDesc* __restrict__ d, int nd,
                                                                            int units) {
-    oz_persistent<Cfg>(units, [&](int u, OzUnit& o) { oz_group_unit(d, nd, u, o); });
+    oz_persistent<Cfg>(units, [&](int u, OzUnit& o) { oz_group_unit<Cfg::BN>(d, nd, u, o); });
 }
 
 // Split K of the tail: the parts' level sums added in part order (the level-0
 // parts are exact integers, so their sum is exact), then the epilogue of one
-// element.  Block (tail tile, group of 8 tile rows) of 8 warps: warp w takes
-// tile row 8 g + w and its lanes 32 consecutive columns at a time, so the
-// workspace reads, the addend reads (at (i, j): tri addends are symmetric)
-// and the row-direction stores are coalesced; the element arithmetic is
-// oz_store_half's, so a split tile gives what an unsplit one would from the
-// same level sums.
+// element.  Block (tail tile, 32 x 32 part of it): the workspace is read with the lanes
+// over its rows, the values staged in shared memory, and the addends read and the outputs
+// written with the lanes over the columns (tri: the mirror over the rows again), so every
+// access is coalesced; the element arithmetic is the GEMM epilogue's, so a split tile
+// gives what an unsplit one would from the same level sums.
 __device__ __forceinline__ void oz_tail_tile(const OzParams& p, int widx) {
     constexpr size_t tile_elems = (size_t)OZ_BM * OZ_BN;
-    const int il = blockIdx.y * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    __shared__ uint64_t T[32][33];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int r0 = (blockIdx.y & 3) * 32, c0 = (blockIdx.y >> 2) * 32;
     int tm, tn;
     oz_tile_coords(p, p.split_first + widx, tm, tn);
-    const int i = tm * OZ_BM + il;
-    if (i >= p.M) return;
-    const bool diag = p.tri && tm == tn;
-    const float sA = p.sa[i];
-    const float2* base = p.ws + (size_t)widx * p.split_parts * tile_elems + (size_t)il * OZ_BN;
-    for (int c0 = 0; c0 < OZ_BN; c0 += 32) {
-        const int jl = c0 + lane, j = tn * OZ_BN + jl;
-        if (j >= p.N || (diag && i > j)) continue;
+    const int i0 = tm * OZ_BM + r0, j0 = tn * OZ_BN + c0;
+    if (i0 >= p.M || j0 >= p.N || (p.tri && i0 >= j0 + 32)) return;      // the whole block
+    const int il = i0 + lane;
+    const float sA = il < p.M ? p.sa[il] : 0.0f;
+    const float2* base = p.ws + (size_t)widx * p.split_parts * tile_elems + r0 + lane;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        const int cl = w + 8 * u, j = j0 + cl;
+        if (il >= p.M || j >= p.N) continue;
         float hv = 0.f, lv = 0.f;
         for (int pp = 0; pp < p.split_parts; ++pp) {
-            const float2 v = base[(size_t)pp * tile_elems + jl];
+            const float2 v = base[(size_t)pp * tile_elems + (size_t)(c0 + cl) * OZ_BM];
             hv += v.x;
             lv += v.y;
         }
@@ -1010,18 +1054,39 @@ __device__ __forceinline__ void oz_tail_tile(const OzParams& p, int widx) {
         const float sh = hv + lv;
         const float bb = sh - hv;
         const float sl = (hv - (sh - bb)) + (lv - bb);
-        const size_t off = (size_t)i * p.ldc + j;
         if (p.mode == OZ_OUT_PAIR) {
-            p.Cp[off] = make_float2(sh * s, sl * s);
+            T[lane][cl] = (uint64_t)__float_as_uint(sh * s) | ((uint64_t)__float_as_uint(sl * s) << 32);
+        } else {
+            double v = f2d_bits(sh * s) + f2d_bits(sl * s);
+            if (p.alpha != 1.0) v *= p.alpha;
+            T[lane][cl] = (uint64_t)__double_as_longlong(v);
+        }
+    }
+    __syncthreads();
+    const int j = j0 + lane;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        const int r = w + 8 * u, i = i0 + r;
+        if (i >= p.M || j >= p.N || (p.tri && i > j)) continue;
+        const size_t off = (size_t)i * p.ldc + j;
+        const uint64_t word = T[r][lane];
+        if (p.mode == OZ_OUT_PAIR) {
+            p.Cp[off] = make_float2(__uint_as_float((uint32_t)word), __uint_as_float((uint32_t)(word >> 32)));
             continue;
         }
-        double v = f2d_bits(sh * s) + f2d_bits(sl * s);
-        if (p.alpha != 1.0) v *= p.alpha;
+        double v = __longlong_as_double((long long)word);
         if (p.D1) v += p.b1 * p.D1[off];
         if (p.D2) v += p.b2 * p.D2[off];
         if (p.D3) v += p.b3 * p.D3[off];
         p.Cd[off] = v;
-        if (p.tri && i != j) p.Cd[(size_t)j * p.ldc + i] = v;
+        T[r][lane] = (uint64_t)__double_as_longlong(v);
+    }
+    if (!p.tri) return;
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        const int c = w + 8 * u, jr = j0 + c, i = i0 + lane;
+        if (jr < p.N && i < p.M && i < jr) p.Cd[(size_t)jr * p.ldc + i] = __longlong_as_double((long long)T[lane][c]);
     }
 }
 
@@ -1092,10 +1157,10 @@ dme_status encode_bf16_map(CUtensorMap* out, const void* data, int rank, const c
     return DME_OK;
 }
 
-static dme_status make_slice_tmap(const SliceBuf& sb, int planes, CUtensorMap* out) {
+static dme_status make_slice_tmap(const SliceBuf& sb, int planes, CUtensorMap* out, int box_rows = OZ_BM) {
     cuuint64_t dims[3] = {(cuuint64_t)sb.Kp, (cuuint64_t)sb.rows, (cuuint64_t)sb.ns};
     cuuint64_t strides[2] = {(cuuint64_t)sb.Kp * 2, (cuuint64_t)sb.rows * sb.Kp * 2};
-    cuuint32_t box[3] = {(cuuint32_t)OZ_BK, (cuuint32_t)OZ_BM, (cuuint32_t)planes};
+    cuuint32_t box[3] = {(cuuint32_t)OZ_BK, (cuuint32_t)box_rows, (cuuint32_t)planes};
     return encode_bf16_map(out, sb.data, 3, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_64B);
 }
 
@@ -1103,6 +1168,10 @@ dme_status make_slice_tmaps(SliceBuf& sb) {
     if (sb.ns < 1 || sb.ns > 8) return set_error("slice buffer: 1 to 8 planes"), DME_EINVAL;
     DME_TRY(make_slice_tmap(sb, sb.ns, &sb.tmap));
     if (sb.ns > 4) DME_TRY(make_slice_tmap(sb, 4, &sb.tmap4));
+    if (sb.ns >= 4 && sb.scheme == OZ_DIG9) {
+        DME_TRY(make_slice_tmap(sb, 4, &sb.tmap64, 64));
+        DME_TRY(make_slice_tmap(sb, 4, &sb.tmap32, 32));
+    }
     return DME_OK;
 }
 
@@ -1184,7 +1253,19 @@ static void oz_split_rule(OzParams& p, int nsm) {
     p.units = p.split_first + (tiles - p.split_first) * p.split_parts;
 }
 
-dme_status launch_ozaki_gemm(const CUtensorMap& tA, const CUtensorMap& tB, OzParams p, cudaStream_t st) {
+// Tile width of a launch of `tiles` 128-wide tiles, none split in K: narrower ones while
+// they are at most one wave (n = 256: 4 tiles of 128 columns took 26 and 46 us a product,
+// 16 of 32 columns 9 and 13).
+static int oz_tile_width(int tiles, int nsm) { return 4 * tiles <= nsm ? 32 : (2 * tiles <= nsm ? 64 : 128); }
+
+static int oz_narrow_tiles(const OzParams& p, int bn) {
+    int t = 0;
+    for (int c = 0; c < (p.N + bn - 1) / bn; ++c) t += oz_narrow_rows(p, bn, c);
+    return t;
+}
+
+dme_status launch_ozaki_gemm(const SliceBuf& A, const SliceBuf& B, OzParams p, cudaStream_t st) {
+    const CUtensorMap &tA = oz_tmap_a(A, p.cfg), &tB = oz_tmap_b(B, p.cfg);
     if (p.M <= 0 || p.N <= 0) return DME_OK;
     if (p.Kp % OZ_BK != 0 || p.Kp > OZ_MAX_K) {
         set_error("ozaki gemm: K must be a multiple of 32 and at most 4096");
@@ -1218,6 +1299,17 @@ dme_status launch_ozaki_gemm(const CUtensorMap& tA, const CUtensorMap& tB, OzPar
     // products round exactly as the grouped serving kernel's.
     const bool shortk = !acc && p.Kp <= 2 * OZ_BK && tiles > nsm;
     const int grid = std::min(p.units, shortk ? 2 * nsm : nsm);
+    const int bn = acc || shortk || p.split_parts > 1 ? OZ_BN : oz_tile_width(tiles, nsm);
+    if (bn < OZ_BN) {
+        p.tiles_n = (p.N + bn - 1) / bn;
+        p.tiles = p.units = p.split_first = oz_narrow_tiles(p, bn);
+        const int g = std::min(p.units, nsm);
+        if (p.cfg == OZ_P14)
+            return bn == 64 ? oz_launch_single<CfgP14n64>(tA, B.tmap64, p, g, st)
+                            : oz_launch_single<CfgP14n32>(tA, B.tmap32, p, g, st);
+        return bn == 64 ? oz_launch_single<CfgP13n64>(tA, B.tmap64, p, g, st)     // (cuts 10 products itself)
+                        : oz_launch_single<CfgP13n32>(tA, B.tmap32, p, g, st);
+    }
     switch (p.cfg) {
         case OZ_P10:
             DME_TRY(shortk ? oz_launch_single<CfgP10s>(tA, tB, p, grid, st) : oz_launch_single<CfgP10>(tA, tB, p, grid, st));
@@ -1234,7 +1326,7 @@ dme_status launch_ozaki_gemm(const CUtensorMap& tA, const CUtensorMap& tB, OzPar
         default: return set_error("ozaki gemm: unknown configuration"), DME_EINVAL;
     }
     if (p.split_parts > 1) {
-        oz_tail_kernel<<<dim3(tiles - p.split_first, OZ_BM / 8), 256, 0, st>>>(p);
+        oz_tail_kernel<<<dim3(tiles - p.split_first, 16), 256, 0, st>>>(p);
         DME_CUDA_TRY(cudaGetLastError());
     }
     if (acc) {
@@ -1256,7 +1348,11 @@ static dme_status oz_grouped_attr() {
 
 dme_status ozaki_grouped_prepare() {
     DME_TRY(oz_grouped_attr<CfgP13>());
+    DME_TRY(oz_grouped_attr<CfgP13n64>());
+    DME_TRY(oz_grouped_attr<CfgP13n32>());
     DME_TRY(oz_grouped_attr<CfgP14e>());
+    DME_TRY(oz_grouped_attr<CfgP14n64>());
+    DME_TRY(oz_grouped_attr<CfgP14n32>());
     return DME_OK;
 }
 
@@ -1286,8 +1382,18 @@ dme_status launch_ozaki_grouped(std::vector<OzGroupDesc>& items, OzGroupDesc* de
     std::stable_sort(live.begin(), live.end(), [](const OzGroupDesc& x, const OzGroupDesc& y) {
         return x.p.Kp / x.p.split_parts > y.p.Kp / y.p.split_parts;
     });
-    int tail_total = 0;
+    int tail_total = 0, tiles128 = 0;
+    bool split = false;
     for (auto& it : live) {
+        tiles128 += it.p.tiles;
+        split = split || it.p.split_parts > 1;
+    }
+    const int bn = split ? OZ_BN : oz_tile_width(tiles128, sm_count());
+    for (auto& it : live) {
+        if (bn < OZ_BN) {
+            it.p.tiles_n = (it.p.N + bn - 1) / bn;
+            it.p.tiles = it.p.units = it.p.split_first = oz_narrow_tiles(it.p, bn);
+        }
         it.start = total;
         total += it.p.units;
         it.tail_start = tail_total;
@@ -1304,18 +1410,19 @@ dme_status launch_ozaki_grouped(std::vector<OzGroupDesc>& items, OzGroupDesc* de
     }
     const int grid = std::min(total, sm_count());
     const int nd = (int)live.size();
-    switch (cfg) {
-        case OZ_P13:
-            ozaki_gemm_grouped_kernel<CfgP13><<<grid, OZ_THREADS, CfgP13::SMEM, st>>>(d, nd, total);
-            break;
-        default:   // serving problems are small: the staged two-stage form of 14 products
-            ozaki_gemm_grouped_kernel<CfgP14e><<<grid, OZ_THREADS, CfgP14e::SMEM, st>>>(d, nd, total);
-            break;
+    if (cfg == OZ_P13) {
+        if (bn == 32) ozaki_gemm_grouped_kernel<CfgP13n32><<<grid, OZ_THREADS, CfgP13n32::SMEM, st>>>(d, nd, total);
+        else if (bn == 64) ozaki_gemm_grouped_kernel<CfgP13n64><<<grid, OZ_THREADS, CfgP13n64::SMEM, st>>>(d, nd, total);
+        else ozaki_gemm_grouped_kernel<CfgP13><<<grid, OZ_THREADS, CfgP13::SMEM, st>>>(d, nd, total);
+    } else {   // serving problems are small: the staged two-stage form of 14 products
+        if (bn == 32) ozaki_gemm_grouped_kernel<CfgP14n32><<<grid, OZ_THREADS, CfgP14n32::SMEM, st>>>(d, nd, total);
+        else if (bn == 64) ozaki_gemm_grouped_kernel<CfgP14n64><<<grid, OZ_THREADS, CfgP14n64::SMEM, st>>>(d, nd, total);
+        else ozaki_gemm_grouped_kernel<CfgP14e><<<grid, OZ_THREADS, CfgP14e::SMEM, st>>>(d, nd, total);
     }
     DME_CUDA_TRY(cudaGetLastError());
     // the parts of the split problems added and their epilogues run, in one launch
     if (tail_total > 0) {
-        oz_tail_grouped_kernel<<<dim3(tail_total, OZ_BM / 8), 256, 0, st>>>(d, nd);
+        oz_tail_grouped_kernel<<<dim3(tail_total, 16), 256, 0, st>>>(d, nd);
         DME_CUDA_TRY(cudaGetLastError());
     }
     return DME_OK;
@@ -1412,7 +1519,7 @@ extern "C" dme_status dme_gemm_split_noalloc(int M, int N, int K, const double* 
         o.ldc = N;
         o.Cd = C;
         o.status = status;
-        DME_TRY(launch_ozaki_gemm(oz_tmap_a(sa, OZ_P14), oz_tmap_b(sb, OZ_P14), o, st));
+        DME_TRY(launch_ozaki_gemm(sa, sb, o, st));
         int hs = 0;
         DME_CUDA_TRY(cudaMemcpyAsync(&hs, status, sizeof(int), cudaMemcpyDeviceToHost, st));
         DME_CUDA_TRY(cudaStreamSynchronize(st));

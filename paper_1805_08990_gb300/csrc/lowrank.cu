@@ -529,7 +529,7 @@ dme_status apply_split(dme_lr_t lr, const SliceBuf& Msl, const double* X, int ld
     p.status = lr->status;
     p.ws = lr->P->kws;
     p.ws_cnt = lr->P->kcnt;
-    return launch_ozaki_gemm(oz_tmap_a(Msl, OZ_P14), oz_tmap_b(lr->xsl, OZ_P14), p, st);
+    return launch_ozaki_gemm(Msl, lr->xsl, p, st);
 }
 
 // FP64 by residue products: C (n x k, ldc) = alpha op(M) X for X (n x k, ldx), op(M)'s planes

@@ -221,7 +221,7 @@ dme_status acc_prod(int n, AccWork& w, const double* L, int tL, const double* R,
     o.b1 = b1;
     o.wsd = w.wsd;
     o.status = w.status;
-    return launch_ozaki_gemm(oz_tmap_a(w.a, OZ_A21), oz_tmap_b(w.b, OZ_A21), o, st);
+    return launch_ozaki_gemm(w.a, w.b, o, st);
 }
 
 // Scratch of the accurate mode for n x n products, from a plan-time pool.
@@ -399,7 +399,7 @@ dme_status split_cong(dme_plan_t p, const double* P, const SliceBuf& G, double* 
     a.ws_cnt = p->kcnt;
     {
         ProfScope ps(p, DME_KIND_SPLIT_GEMM);
-        DME_TRY(launch_ozaki_gemm(oz_tmap_a(G, cfg), oz_tmap_b(p->psl, cfg), a, st));
+        DME_TRY(launch_ozaki_gemm(G, p->psl, a, st));
     }
     {
         ProfScope ps(p, DME_KIND_SLICE);
@@ -422,7 +422,7 @@ dme_status split_cong(dme_plan_t p, const double* P, const SliceBuf& G, double* 
     b.ws = p->kws;
     b.ws_cnt = p->kcnt;
     ProfScope ps(p, DME_KIND_SPLIT_GEMM);
-    return launch_ozaki_gemm(oz_tmap_a(G, cfg), oz_tmap_b(p->usl, cfg), b, st);
+    return launch_ozaki_gemm(G, p->usl, b, st);
 }
 
 // T3 on the split path for n > 1536: Z^T = Bt^T P (P symmetric) on the tensor
@@ -445,7 +445,7 @@ dme_status split_riccati(dme_plan_t p, double* P, double tau, double qcoef) {
     a.status = p->status;
     a.ws = p->kws;
     a.ws_cnt = p->kcnt;
-    DME_TRY(launch_ozaki_gemm(oz_tmap_a(p->btsl, p->cfg), oz_tmap_b(p->psl, p->cfg), a, st));
+    DME_TRY(launch_ozaki_gemm(p->btsl, p->psl, a, st));
     launch_transpose(p->Zt, Z, m, n, n, m, st);
     DME_TRY(launch_riccati_from_z(p->Bt, n, m, tau, p->rwork, p->status, st));
     launch_slice_rows_f64(Y, n, m, m, p->ysla, st);
@@ -464,7 +464,7 @@ dme_status split_riccati(dme_plan_t p, double* P, double tau, double qcoef) {
         b.b2 = qcoef;
     }
     b.status = p->status;
-    return launch_ozaki_gemm(oz_tmap_a(p->ysla, p->cfg), oz_tmap_b(p->yslb, p->cfg), b, st);
+    return launch_ozaki_gemm(p->ysla, p->yslb, b, st);
 }
 
 dme_status compute_ew(dme_plan_t p, double tau, int* idx) {
@@ -1744,7 +1744,7 @@ static dme_status gemm_split_impl(int M, int N, int K, const double* A, const do
         o.Cd = C;
         o.status = status;
         o.wsd = wsd;
-        if (s == DME_OK) s = launch_ozaki_gemm(oz_tmap_a(sa, o.cfg), oz_tmap_b(sb, o.cfg), o, st);
+        if (s == DME_OK) s = launch_ozaki_gemm(sa, sb, o, st);
         int hs = 0;
         if (s == DME_OK) {
             cudaError_t e = cudaMemcpyAsync(&hs, status, sizeof(int), cudaMemcpyDeviceToHost, st);

@@ -438,6 +438,8 @@ dme_status run_lane(dme_server_t s, std::vector<Req*>& res, int lane) {
                 std::memset(&a, 0, sizeof(a));
                 a.tmA = oz_tmap_a(e.Gsl, p->cfg);
                 a.tmB = oz_tmap_b(p->psl, p->cfg);
+                a.tmB64 = p->psl.tmap64;
+                a.tmB32 = p->psl.tmap32;
                 DME_TRY(oz_params(e.Gsl, p->psl, p->cfg, &a.p));
                 a.p.mode = OZ_OUT_PAIR;
                 a.p.ldc = n;
@@ -449,6 +451,8 @@ dme_status run_lane(dme_server_t s, std::vector<Req*>& res, int lane) {
                 std::memset(&b, 0, sizeof(b));
                 b.tmA = oz_tmap_a(e.Gsl, p->cfg);
                 b.tmB = oz_tmap_b(p->usl, p->cfg);
+                b.tmB64 = p->usl.tmap64;
+                b.tmB32 = p->usl.tmap32;
                 DME_TRY(oz_params(e.Gsl, p->usl, p->cfg, &b.p));
                 b.p.mode = OZ_OUT_F64;
                 b.p.tri = 1;

@@ -54,6 +54,7 @@ struct SliceBuf {
     int scheme = OZ_DIG9;
     CUtensorMap tmap;
     CUtensorMap tmap4;
+    CUtensorMap tmap64, tmap32;   // DIG9: four planes in boxes of 64 and 32 rows (narrow tiles)
 };
 
 struct OzParams {
@@ -78,7 +79,7 @@ struct OzParams {
     // split-K of the last partial wave (single-problem launches only): tiles with index
     // >= split_first run as split_parts units over consecutive K ranges; each writes its
     // level sums to ws, and a second kernel adds them in part order and runs the
-    // epilogue.  ws: [tail tile][part][128 x 128] (level 0, levels >= 1).
+    // epilogue.  ws: [tail tile][part][128 columns][128 rows] (level 0, levels >= 1).
     float2* ws;
     int* ws_cnt;          // unused (kept for the layout of the grouped descriptors)
     int split_first;      // set by the launcher
@@ -95,7 +96,7 @@ constexpr size_t OZ_SPLIT_WS_FLOAT2 = (size_t)OZ_SPLIT_MAX_TAIL * 2 * 128 * 128;
 // One problem of a grouped split GEMM (tensor maps live in global memory).
 struct OzGroupDesc {
     CUtensorMap tmA;
-    CUtensorMap tmB;
+    CUtensorMap tmB, tmB64, tmB32;
     OzParams p;
     int start;            // first unit index (set by the launcher)
     int tail_start;       // first split tile in the launch's tail kernel (set by the launcher)
@@ -139,7 +140,7 @@ dme_status launch_slice_grouped(std::vector<SliceDesc>& items, bool pair, cudaSt
 dme_status oz_params(const SliceBuf& A, const SliceBuf& B, int cfg, OzParams* p);
 // The accurate mode's chunk workspace in doubles for an M x N product over K.
 size_t oz_acc_ws_doubles(int M, int N, int K);
-dme_status launch_ozaki_gemm(const CUtensorMap& tA, const CUtensorMap& tB, OzParams p, cudaStream_t st);
+dme_status launch_ozaki_gemm(const SliceBuf& A, const SliceBuf& B, OzParams p, cudaStream_t st);
 // Grouped launch over independent problems: items of 10 and 13 slice products
 // together, or of 14 alone (not the accurate mode), ordered by K per unit,
 // largest first, so that the longest units start in the first wave.  A problem
