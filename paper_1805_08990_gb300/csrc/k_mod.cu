@@ -288,20 +288,27 @@ struct ModGemmArgs {
     int* status;
 };
 
-template <int BN_>
+// CL: CTAs of a cluster, one below the other on CL row tiles of the same column tile; each
+// loads its own A tile and 1 / CL of the B tile, which it multicasts to all of them.  One
+// plane pair gives one MMA, so a 128 x 128 tile wants 32 KB from L2 per 256 cycles and SM,
+// and L2 delivered about 47 bytes per cycle and SM; 128 x 256 tiles in clusters of four
+// want 24 KB per 512.
+template <int BN_, int CL_>
 struct ModCfg {
-    static constexpr int BN = BN_;
+    static constexpr int BN = BN_, CL = CL_;
     static constexpr int A_BYTES = MG_BM * MOD_BK * 2, B_BYTES = BN * MOD_BK * 2;
     static constexpr int STAGE = A_BYTES + B_BYTES;
-    static constexpr int STAGES = BN == 64 ? 8 : 6;
+    static constexpr int STAGES = BN == 64 ? 8 : (BN == 128 ? 6 : 4);
+    static constexpr int TM = MG_BM * CL;                     // rows of a unit's tile
     static constexpr int SMEM = STAGES * STAGE + 1024 + 256;
     static constexpr uint32_t IDESC = idesc_bf16_f32(MG_BM, BN);
 };
-static_assert(ModCfg<128>::SMEM <= 232448 && ModCfg<64>::SMEM <= 232448, "shared memory per CTA");
+static_assert(ModCfg<256, 4>::SMEM <= 232448 && ModCfg<128, 1>::SMEM <= 232448 && ModCfg<64, 1>::SMEM <= 232448,
+              "shared memory per CTA");
 
 // Tiles in groups of eight tile rows, column by column inside a group; a triangle
 // product has only the tiles with an entry on or above the diagonal.
-template <int BN>
+template <int BN, int TM>
 __device__ __forceinline__ void mod_tile(const ModGemmArgs& p, int t, int& tm, int& tn) {
     int first = 0;
     while (true) {
@@ -315,8 +322,8 @@ __device__ __forceinline__ void mod_tile(const ModGemmArgs& p, int t, int& tm, i
             }
             t -= in_group;
         } else {
-            for (int c = first * MG_BM / BN; c < p.tiles_n; ++c) {
-                const int cnt = min(rows, (c * BN + BN - 1) / MG_BM + 1 - first);
+            for (int c = first * TM / BN; c < p.tiles_n; ++c) {
+                const int cnt = min(rows, (c * BN + BN - 1) / TM + 1 - first);
                 if (t < cnt) {
                     tm = first + t;
                     tn = c;
@@ -336,15 +343,19 @@ __device__ __forceinline__ float mod_reduce(float x, float p, float inv) {
     return r < 0.0f ? r + p : r;
 }
 
-// Persistent, one CTA per SM: a unit is one tile of one plane.  Warp 0 loads (TMA, a
+// Persistent, one CTA per SM: a unit is one tile (TM x BN) of one plane, worked on by the
+// CTAs of a cluster.  Warp 0 loads (TMA, a
 // ring of stages), warp 1 issues the MMAs into two TMEM accumulators in turn (one per
 // K pass), warps 2-9 reduce the finished one to bytes meanwhile.
-template <int BN, bool MULTI>
+template <int BN, int CL, bool MULTI>
 __global__ void __launch_bounds__(MG_THREADS, 1) mod_gemm_kernel(const __grid_constant__ CUtensorMap tA,
                                                                  const __grid_constant__ CUtensorMap tB,
                                                                  const __grid_constant__ ModGemmArgs p) {
-    using Cfg = ModCfg<BN>;
-    constexpr int S = Cfg::STAGES;
+    using Cfg = ModCfg<BN, CL>;
+    constexpr int S = Cfg::STAGES, TM = Cfg::TM;
+    constexpr uint16_t ALL = (uint16_t)((1 << CL) - 1);
+    const int rank = CL > 1 ? (int)cluster_ctarank() : 0;
+    const int first_unit = blockIdx.x / CL, unit_step = gridDim.x / CL;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     // full[S], empty[S], accumulator full[2], accumulator empty[2], drain
@@ -353,7 +364,10 @@ __global__ void __launch_bounds__(MG_THREADS, 1) mod_gemm_kernel(const __grid_co
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
-        for (int s = 0; s < 2 * S; ++s) mbar_init(smem_u32(&bars[s]), 1);
+        for (int s = 0; s < S; ++s) {
+            mbar_init(smem_u32(&bars[s]), 1);
+            mbar_init(smem_u32(&bars[S + s]), CL);         // every CTA that this one's B part went to
+        }
         for (int a = 0; a < 2; ++a) {
             mbar_init(smem_u32(&bars[2 * S + a]), 1);
             mbar_init(smem_u32(&bars[2 * S + 2 + a]), MG_EPI_WARPS);
@@ -368,6 +382,7 @@ __global__ void __launch_bounds__(MG_THREADS, 1) mod_gemm_kernel(const __grid_co
     }
     fence_before_sync();
     __syncthreads();
+    if (CL > 1) cluster_sync();                                // the barriers are ready in every CTA
     fence_after_sync();
     const uint32_t tmem = *tmem_slot;
     const int nk = p.Kp / MOD_BK;
@@ -381,10 +396,10 @@ __global__ void __launch_bounds__(MG_THREADS, 1) mod_gemm_kernel(const __grid_co
             bool ok = true;
             tma_prefetch_desc(&tA);
             tma_prefetch_desc(&tB);
-            for (int u = blockIdx.x; u < p.units && ok; u += gridDim.x) {
+            for (int u = first_unit; u < p.units && ok; u += unit_step) {
                 const int m = u / p.tiles;
                 int tm, tn;
-                mod_tile<BN>(p, u - m * p.tiles, tm, tn);
+                mod_tile<BN, TM>(p, u - m * p.tiles, tm, tn);
                 for (int it = 0; it < nk; ++it, ++kit) {
                     const int s = kit % S;
                     const uint32_t ph = (kit / S) & 1;
@@ -397,8 +412,12 @@ __global__ void __launch_bounds__(MG_THREADS, 1) mod_gemm_kernel(const __grid_co
                     const uint32_t full = smem_u32(&bars[s]);
                     uint8_t* st = smem + s * Cfg::STAGE;
                     mbar_arrive_expect_tx(full, Cfg::STAGE);
-                    tma_load_3d(smem_u32(st), &tA, full, it * MOD_BK, tm * MG_BM, m);
-                    tma_load_3d(smem_u32(st + Cfg::A_BYTES), &tB, full, it * MOD_BK, tn * BN, m);
+                    tma_load_3d(smem_u32(st), &tA, full, it * MOD_BK, tm * TM + rank * MG_BM, m);
+                    if (CL > 1)
+                        tma_load_3d_multicast(smem_u32(st + Cfg::A_BYTES + rank * (Cfg::B_BYTES / CL)), &tB, full,
+                                              it * MOD_BK, tn * BN + rank * (BN / CL), m, ALL);
+                    else
+                        tma_load_3d(smem_u32(st + Cfg::A_BYTES), &tB, full, it * MOD_BK, tn * BN, m);
                     issued |= 1u << s;
                     last_ph = (last_ph & ~(1u << s)) | (ph << s);
                 }
@@ -412,7 +431,7 @@ __global__ void __launch_bounds__(MG_THREADS, 1) mod_gemm_kernel(const __grid_co
         if (lane == 0) {
             int kit = 0, ai = 0;
             bool ok = true;
-            for (int u = blockIdx.x; u < p.units && ok; u += gridDim.x) {
+            for (int u = first_unit; u < p.units && ok; u += unit_step) {
                 // the magnitudes' sum needs no exact passes
                 const bool one = !MULTI || u / p.tiles == MOD_NM;
                 for (int it = 0; it < nk; ++it, ++kit) {
@@ -436,7 +455,8 @@ __global__ void __launch_bounds__(MG_THREADS, 1) mod_gemm_kernel(const __grid_co
                     for (int kk = 0; kk < MOD_BK / 16; ++kk)
                         mma_bf16(acc, desc_kmajor_sw128(a0 + kk * 32), desc_kmajor_sw128(b0 + kk * 32), Cfg::IDESC,
                                  (kc == 0 && kk == 0) ? 0u : 1u);
-                    mma_commit(smem_u32(&bars[S + s]));
+                    if (CL > 1) mma_commit_multicast(smem_u32(&bars[S + s]), ALL);
+                    else mma_commit(smem_u32(&bars[S + s]));
                     if (it == nk - 1 || (!one && kc == CH - 1)) {
                         mma_commit(smem_u32(&bars[2 * S + (ai & 1)]));
                         ++ai;
@@ -456,11 +476,11 @@ __global__ void __launch_bounds__(MG_THREADS, 1) mod_gemm_kernel(const __grid_co
         const int c0 = NC * (ew / 4);
         int ai = 0;
         bool ok = true;
-        for (int u = blockIdx.x; u < p.units && ok; u += gridDim.x) {
+        for (int u = first_unit; u < p.units && ok; u += unit_step) {
             const int m = u / p.tiles;
             int tm, tn;
-            mod_tile<BN>(p, u - m * p.tiles, tm, tn);
-            const int i = tm * MG_BM + 32 * q + lane, j0 = tn * BN + c0;
+            mod_tile<BN, TM>(p, u - m * p.tiles, tm, tn);
+            const int i = tm * TM + rank * MG_BM + 32 * q + lane, j0 = tn * BN + c0;
             const bool mag = m == MOD_NM;
             const int passes = (!MULTI || mag) ? 1 : nch;
             const float pm = mag ? 1.0f : c_mod.p[m], inv = mag ? 1.0f : c_mod.inv[m];
@@ -547,6 +567,7 @@ __global__ void __launch_bounds__(MG_THREADS, 1) mod_gemm_kernel(const __grid_co
     __syncthreads();
     fence_after_sync();
     if (warp == 1) tmem_dealloc(tmem, 2 * BN);
+    if (CL > 1) cluster_sync();                                // no CTA leaves while another may still write to it
 }
 
 // ------------------------------------------------------------------ 3. combine
@@ -703,14 +724,65 @@ dme_status mod_map(const ModBuf& b, int box_rows, CUtensorMap* out) {
     return encode_bf16_map(out, b.data, 3, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_128B);
 }
 
-template <int BN, bool MULTI>
-dme_status mod_gemm_launch(const CUtensorMap& tA, const CUtensorMap& tB, const ModGemmArgs& a, cudaStream_t st) {
+template <int BN, int CL, bool MULTI>
+dme_status mod_gemm_launch(const CUtensorMap& tA, const CUtensorMap& tB, const ModGemmArgs& a, int clusters, cudaStream_t st) {
+    using Cfg = ModCfg<BN, CL>;
     static const cudaError_t attr = cudaFuncSetAttribute(
-        mod_gemm_kernel<BN, MULTI>, cudaFuncAttributeMaxDynamicSharedMemorySize, ModCfg<BN>::SMEM);
+        mod_gemm_kernel<BN, CL, MULTI>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::SMEM);
     DME_CUDA_TRY(attr);
-    mod_gemm_kernel<BN, MULTI><<<std::min(a.units, mod_sms()), MG_THREADS, ModCfg<BN>::SMEM, st>>>(tA, tB, a);
-    DME_CUDA_TRY(cudaGetLastError());
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(std::min(a.units, clusters) * CL);
+    cfg.blockDim = dim3(MG_THREADS);
+    cfg.dynamicSmemBytes = Cfg::SMEM;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = CL;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = CL > 1 ? 1 : 0;
+    DME_CUDA_TRY(cudaLaunchKernelEx(&cfg, mod_gemm_kernel<BN, CL, MULTI>, tA, tB, a));
     return DME_OK;
+}
+
+// Clusters of four 192 KB CTAs that the device holds at once (0: none).
+int mod_clusters() {
+    static const int n = [] {
+        if (cudaFuncSetAttribute(mod_gemm_kernel<256, 4, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 ModCfg<256, 4>::SMEM) != cudaSuccess) {
+            cudaGetLastError();
+            return 0;
+        }
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(4 * mod_sms());
+        cfg.blockDim = dim3(MG_THREADS);
+        cfg.dynamicSmemBytes = ModCfg<256, 4>::SMEM;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = 4;
+        at[0].val.clusterDim.y = 1;
+        at[0].val.clusterDim.z = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        int c = 0;
+        if (cudaOccupancyMaxActiveClusters(&c, mod_gemm_kernel<256, 4, true>, &cfg) != cudaSuccess) {
+            cudaGetLastError();
+            return 0;
+        }
+        return std::min(c, mod_sms() / 4);
+    }();
+    return n;
+}
+
+// Tiles of TM x BN of an M x N product (a triangle: those with an entry on or above the
+// diagonal).
+int mod_tile_count(int M, int N, int tri, int tm, int bn) {
+    const int rows = (M + tm - 1) / tm, cols = (N + bn - 1) / bn;
+    if (!tri) return rows * cols;
+    int t = 0;
+    for (int c = 0; c < cols; ++c) t += std::min(rows, (c * bn + bn - 1) / tm + 1);
+    return t;
 }
 
 }  // namespace
@@ -744,23 +816,33 @@ dme_status launch_mod_gemm(const ModBuf& A, const ModBuf& B, const GemmProb& g, 
     a.rb = B.row;
     a.kfac = 9007199254740992.0f / (float)g.K;
     a.status = status;
-    const int bn = g.N <= 64 ? 64 : 128;
-    a.tiles_m = (g.M + MG_BM - 1) / MG_BM;
-    a.tiles_n = (g.N + bn - 1) / bn;
-    if (g.tri) {
-        a.tiles = 0;
-        for (int c = 0; c < a.tiles_n; ++c) a.tiles += std::min(a.tiles_m, (c * bn + bn - 1) / MG_BM + 1);
-    } else {
-        a.tiles = a.tiles_m * a.tiles_n;
-    }
-    a.units = a.tiles * (certify ? MOD_PLANES : MOD_NM);
+    const int planes = certify ? MOD_PLANES : MOD_NM;
     const bool multi = a.Kp > MOD_CHUNK;
-    if (bn == 64)
-        DME_TRY(multi ? (mod_gemm_launch<64, true>(A.t128, B.t64, a, st))
-                      : (mod_gemm_launch<64, false>(A.t128, B.t64, a, st)));
-    else
-        DME_TRY(multi ? (mod_gemm_launch<128, true>(A.t128, B.t128, a, st))
-                      : (mod_gemm_launch<128, false>(A.t128, B.t128, a, st)));
+    auto shape = [&](int tm, int bn) {
+        a.tiles_m = (g.M + tm - 1) / tm;
+        a.tiles_n = (g.N + bn - 1) / bn;
+        a.tiles = mod_tile_count(g.M, g.N, g.tri, tm, bn);
+        a.units = a.tiles * planes;
+    };
+    if (g.N <= 64) {
+        shape(MG_BM, 64);
+        DME_TRY(multi ? (mod_gemm_launch<64, 1, true>(A.t128, B.t64, a, mod_sms(), st))
+                      : (mod_gemm_launch<64, 1, false>(A.t128, B.t64, a, mod_sms(), st)));
+    } else {
+        // the shape with the shorter run: waves x measured cycles per K block of 64
+        const int nc = mod_clusters();
+        const long w1 = ((long)mod_tile_count(g.M, g.N, g.tri, 128, 128) * planes + mod_sms() - 1) / mod_sms();
+        const long w4 = nc > 0 ? ((long)mod_tile_count(g.M, g.N, g.tri, 512, 256) * planes + nc - 1) / nc : 0;
+        if (nc > 0 && w4 * 560 < w1 * 690) {
+            shape(512, 256);
+            DME_TRY(multi ? (mod_gemm_launch<256, 4, true>(A.t128, B.t64, a, nc, st))
+                          : (mod_gemm_launch<256, 4, false>(A.t128, B.t64, a, nc, st)));
+        } else {
+            shape(MG_BM, 128);
+            DME_TRY(multi ? (mod_gemm_launch<128, 1, true>(A.t128, B.t128, a, mod_sms(), st))
+                          : (mod_gemm_launch<128, 1, false>(A.t128, B.t128, a, mod_sms(), st)));
+        }
+    }
     const int tn = (g.N + 31) / 32, tm = (g.M + 31) / 32;
     const int blocks = g.tri ? tn * (tn + 1) / 2 : tm * tn;
     mod_combine_kernel<<<blocks, 256, 0, st>>>(g, a.R, a.plane, a.ldr, a.ra, a.rb, certify ? 1 : 0, tn);

@@ -35,7 +35,7 @@ inline int mod_kpad(int k) { return (k + MOD_BK - 1) / MOD_BK * MOD_BK; }
 inline size_t mod_plane_bytes(int rows, int k) { return (size_t)MOD_PLANES * rows * mod_kpad(k) * 2; }
 inline size_t mod_row_bytes(int rows) { return (size_t)rows * sizeof(ModRow); }
 // Workspace of an M x N product: a byte per residue and output, and the certificate.
-inline int mod_ldr(int N) { return (N + 127) / 128 * 128; }
+inline int mod_ldr(int N) { return (N + 255) / 256 * 256; }
 inline size_t mod_ws_bytes(int M, int N) { return (size_t)MOD_PLANES * M * mod_ldr(N); }
 
 // Encode the tensor maps of buf (data, rows, k, Kp set).
