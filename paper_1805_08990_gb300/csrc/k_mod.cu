@@ -63,6 +63,7 @@ struct ModConst {
     float p[MOD_NM], inv[MOD_NM];
     float c1[MOD_NM], c2[MOD_NM], c3[MOD_NM];     // 2^16, 2^32, 2^48 mod p, centred
     uint32_t w0[MOD_NM], w1[MOD_NM], w2[MOD_NM];  // (P / p) inverse(P / p) mod P, without its low 32 bits
+    uint32_t o0, o1, o2;                          // -128 sum_m w_m mod P (bytes hold residue + 128)
     uint64_t plo;                                 // P without its low 32 bits
     uint32_t phi;
     float qscale;                                 // 2^(64 + 10) / (P / 2^32)
@@ -90,13 +91,18 @@ constexpr ModConst make_mod_const() {
         c.w2[m] = (uint32_t)(h >> 64);
     }
     const u128 ph = (P + ((u128)1 << 31)) >> 32;
+    u128 sw = 0;
+    for (int m = 0; m < MOD_NM; ++m) sw += ((u128)c.w2[m] << 64) + ((u128)c.w1[m] << 32) + (u128)c.w0[m];
+    const u128 o = ph - (sw * 128) % ph;
+    c.o0 = (uint32_t)o;
+    c.o1 = (uint32_t)(o >> 32);
+    c.o2 = (uint32_t)(o >> 64);
     c.plo = (uint64_t)ph;
     c.phi = (uint32_t)(ph >> 64);
     c.qscale = (float)(18889465931478580854784.0 / ((double)c.phi * 18446744073709551616.0 + (double)c.plo));
     return c;
 }
 
-constexpr ModConst kModConst = make_mod_const();
 __constant__ ModConst c_mod = make_mod_const();
 static_assert(mod_product() >> 125 != 0 && mod_product() >> 126 == 0, "2^122 < P / 8: the quotient is never ambiguous");
 
@@ -248,9 +254,9 @@ __global__ void __launch_bounds__(T) mod_convert_kernel(const double* __restrict
         r.pad = 0;
         info[row] = r;
     }
-    const size_t plane = (size_t)prow * Kp;
-    __nv_bfloat16* o = out + (size_t)row * Kp;
+    const size_t plane = (size_t)prow * Kp, kblock = (size_t)prow * MOD_BK;
     for (int k = 4 * tid; k < Kp; k += 4 * T) {
+        __nv_bfloat16* o = out + (k / MOD_BK) * kblock + (size_t)row * MOD_BK + k % MOD_BK;
         long long V[4] = {0, 0, 0, 0};
         uint32_t f[4] = {0, 0, 0, 0};
         if (!zero && !bad && k < cols) {
@@ -261,19 +267,17 @@ __global__ void __launch_bounds__(T) mod_convert_kernel(const double* __restrict
                 f[u] = __float_as_uint(mag_scaled(b[u], E));
             }
         }
-        store_residues4(V, o + k, plane);
+        store_residues4(V, o, plane);
         uint2 w;
         w.x = __byte_perm(f[0], f[1], 0x7632);                 // truncated to bf16
         w.y = __byte_perm(f[2], f[3], 0x7632);
-        *reinterpret_cast<uint2*>(o + k + MOD_NM * plane) = w;
+        *reinterpret_cast<uint2*>(o + MOD_NM * plane) = w;
     }
 }
 
 // ------------------------------------------------------------------ 2. multiply
 constexpr int MG_BM = 128;
 constexpr uint64_t MG_TIMEOUT_NS = 2000000000ull;
-constexpr int MG_EPI_WARPS = 8;
-constexpr int MG_THREADS = 64 + 32 * MG_EPI_WARPS;
 
 struct ModGemmArgs {
     int M, N, Kp;
@@ -288,22 +292,28 @@ struct ModGemmArgs {
     int* status;
 };
 
-// CL: CTAs of a cluster, one below the other on CL row tiles of the same column tile; each
-// loads its own A tile and 1 / CL of the B tile, which it multicasts to all of them.  One
-// plane pair gives one MMA, so a 128 x 128 tile wants 32 KB from L2 per 256 cycles and SM,
-// and L2 delivered about 47 bytes per cycle and SM; 128 x 256 tiles in clusters of four
-// want 24 KB per 512.
-template <int BN_, int CL_>
+// PAIR: two CTAs work on a 256 x 256 tile (tcgen05 cta_group::2: each loads its 128 rows of
+// A and 128 of B, and holds its 128 rows of the result).  One plane pair gives one MMA per
+// K step, so what a stage of shared memory is good for decides: 32 KB buy 256 cycles of
+// MMA in a 128 x 128 tile, 512 in a pair's, and loads came back 3900 cycles after they were
+// issued at K = 2048 (six stages of the former: 690 cycles per K block; 128 x 256 tiles in
+// clusters of four with a multicast B, four stages of 48 KB: 970 per 512 of MMA; pairs,
+// seven stages: 860, and 800 with no load at all, where cuBLAS runs at 640).
+template <int BN_, bool PAIR_>
 struct ModCfg {
-    static constexpr int BN = BN_, CL = CL_;
-    static constexpr int A_BYTES = MG_BM * MOD_BK * 2, B_BYTES = BN * MOD_BK * 2;
+    static constexpr int BN = BN_, CL = PAIR_ ? 2 : 1;
+    static constexpr int B_ROWS = BN / CL;                    // rows of B in one CTA
+    static constexpr int A_BYTES = MG_BM * MOD_BK * 2, B_BYTES = B_ROWS * MOD_BK * 2;
     static constexpr int STAGE = A_BYTES + B_BYTES;
-    static constexpr int STAGES = BN == 64 ? 8 : (BN == 128 ? 6 : 4);
+    static constexpr int STAGES = BN == 64 ? 8 : (BN == 128 ? 6 : 7);
     static constexpr int TM = MG_BM * CL;                     // rows of a unit's tile
+    // epilogue warps: 64 (BN = 64: 32) columns each.  Eight warps on 128 columns each took
+    // longer over a pass than its MMAs (17 instructions an output then, 5 now)
+    static constexpr int EPI = BN == 256 ? 16 : 8, THREADS = 64 + 32 * EPI, NC = 4 * BN / EPI;
     static constexpr int SMEM = STAGES * STAGE + 1024 + 256;
-    static constexpr uint32_t IDESC = idesc_bf16_f32(MG_BM, BN);
+    static constexpr uint32_t IDESC = idesc_bf16_f32(TM, BN);
 };
-static_assert(ModCfg<256, 4>::SMEM <= 232448 && ModCfg<128, 1>::SMEM <= 232448 && ModCfg<64, 1>::SMEM <= 232448,
+static_assert(ModCfg<256, true>::SMEM <= 232448 && ModCfg<128, false>::SMEM <= 232448 && ModCfg<64, false>::SMEM <= 232448,
               "shared memory per CTA");
 
 // Tiles in groups of eight tile rows, column by column inside a group; a triangle
@@ -336,25 +346,27 @@ __device__ __forceinline__ void mod_tile(const ModGemmArgs& p, int t, int& tm, i
     }
 }
 
-// x mod p in [0, p) of an integer |x| <= 2^24 in fp32
-__device__ __forceinline__ float mod_reduce(float x, float p, float inv) {
+// The centred residue of an integer |x| <= 2^24 in fp32: in [-128, 127] for every modulus
+// but 256, and [-128, 128] there (the fma's only error is 1 / p's own rounding).
+__device__ __forceinline__ float mod_centred(float x, float p, float inv) {
     const float q = fmaf(x, inv, 12582912.0f) - 12582912.0f;
-    const float r = fmaf(-q, p, x);
-    return r < 0.0f ? r + p : r;
+    return fmaf(-q, p, x);
 }
+
+// Bits whose low byte (low half for sums) is r + 128 (a residue 128 modulo 256 wraps to 0).
+__device__ __forceinline__ uint32_t mod_bits(float r) { return __float_as_uint(r + 8388736.0f); }
 
 // Persistent, one CTA per SM: a unit is one tile (TM x BN) of one plane, worked on by the
 // CTAs of a cluster.  Warp 0 loads (TMA, a
 // ring of stages), warp 1 issues the MMAs into two TMEM accumulators in turn (one per
-// K pass), warps 2-9 reduce the finished one to bytes meanwhile.
-template <int BN, int CL, bool MULTI>
-__global__ void __launch_bounds__(MG_THREADS, 1) mod_gemm_kernel(const __grid_constant__ CUtensorMap tA,
+// K pass), the others reduce the finished one to bytes meanwhile.
+template <int BN, bool PAIR, bool MULTI>
+__global__ void __launch_bounds__(ModCfg<BN, PAIR>::THREADS, 1) mod_gemm_kernel(const __grid_constant__ CUtensorMap tA,
                                                                  const __grid_constant__ CUtensorMap tB,
                                                                  const __grid_constant__ ModGemmArgs p) {
-    using Cfg = ModCfg<BN, CL>;
-    constexpr int S = Cfg::STAGES, TM = Cfg::TM;
-    constexpr uint16_t ALL = (uint16_t)((1 << CL) - 1);
-    const int rank = CL > 1 ? (int)cluster_ctarank() : 0;
+    using Cfg = ModCfg<BN, PAIR>;
+    constexpr int S = Cfg::STAGES, TM = Cfg::TM, CL = Cfg::CL;
+    const int rank = PAIR ? (int)cluster_ctarank() : 0;
     const int first_unit = blockIdx.x / CL, unit_step = gridDim.x / CL;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -366,23 +378,28 @@ __global__ void __launch_bounds__(MG_THREADS, 1) mod_gemm_kernel(const __grid_co
     if (threadIdx.x == 0) {
         for (int s = 0; s < S; ++s) {
             mbar_init(smem_u32(&bars[s]), 1);
-            mbar_init(smem_u32(&bars[S + s]), CL);         // every CTA that this one's B part went to
+            mbar_init(smem_u32(&bars[S + s]), 1);
         }
         for (int a = 0; a < 2; ++a) {
             mbar_init(smem_u32(&bars[2 * S + a]), 1);
-            mbar_init(smem_u32(&bars[2 * S + 2 + a]), MG_EPI_WARPS);
+            mbar_init(smem_u32(&bars[2 * S + 2 + a]), Cfg::EPI * CL);      // (the even CTA's is used)
         }
         mbar_init(smem_u32(&bars[2 * S + 4]), 1);
         *abort_flag = 0;
         fence_mbar_init();
     }
     if (warp == 1) {
-        tmem_alloc(smem_u32(tmem_slot), 2 * BN);
-        tmem_relinquish();
+        if (PAIR) {
+            tmem_alloc_pair(smem_u32(tmem_slot), 2 * BN);
+            tmem_relinquish_pair();
+        } else {
+            tmem_alloc(smem_u32(tmem_slot), 2 * BN);
+            tmem_relinquish();
+        }
     }
     fence_before_sync();
     __syncthreads();
-    if (CL > 1) cluster_sync();                                // the barriers are ready in every CTA
+    if (PAIR) cluster_sync();                                  // the barriers are ready in both CTAs
     fence_after_sync();
     const uint32_t tmem = *tmem_slot;
     const int nk = p.Kp / MOD_BK;
@@ -411,24 +428,30 @@ __global__ void __launch_bounds__(MG_THREADS, 1) mod_gemm_kernel(const __grid_co
                     }
                     const uint32_t full = smem_u32(&bars[s]);
                     uint8_t* st = smem + s * Cfg::STAGE;
-                    mbar_arrive_expect_tx(full, Cfg::STAGE);
-                    tma_load_3d(smem_u32(st), &tA, full, it * MOD_BK, tm * TM + rank * MG_BM, m);
-                    if (CL > 1)
-                        tma_load_3d_multicast(smem_u32(st + Cfg::A_BYTES + rank * (Cfg::B_BYTES / CL)), &tB, full,
-                                              it * MOD_BK, tn * BN + rank * (BN / CL), m, ALL);
-                    else
-                        tma_load_3d(smem_u32(st + Cfg::A_BYTES), &tB, full, it * MOD_BK, tn * BN, m);
+                    if (PAIR) {
+                        // both CTAs' loads complete on the even one's barrier
+                        const uint32_t lead = cluster_map(full, 0);
+                        if (rank == 0) mbar_arrive_expect_tx(full, 2 * Cfg::STAGE);
+                        tma_load_3d_pair(smem_u32(st), &tA, lead, 0, tm * TM + rank * MG_BM, m * nk + it);
+                        tma_load_3d_pair(smem_u32(st + Cfg::A_BYTES), &tB, lead, 0, tn * BN + rank * Cfg::B_ROWS, m * nk + it);
+                        if (rank != 0) continue;
+                    } else {
+                        mbar_arrive_expect_tx(full, Cfg::STAGE);
+                        tma_load_3d(smem_u32(st), &tA, full, 0, tm * TM, m * nk + it);
+                        tma_load_3d(smem_u32(st + Cfg::A_BYTES), &tB, full, 0, tn * BN, m * nk + it);
+                    }
                     issued |= 1u << s;
                     last_ph = (last_ph & ~(1u << s)) | (ph << s);
                 }
             }
-            // every load this thread issued has landed before the CTA may exit
+            // every load has landed before the CTA may exit (a pair's loads: the even CTA waits,
+            // the odd one for it at the cluster barrier below)
             for (int s = 0; s < S; ++s)
                 if (((issued >> s) & 1u) && !mbar_wait(smem_u32(&bars[s]), (last_ph >> s) & 1u, MG_TIMEOUT_NS))
                     *abort_flag = 1;
         }
     } else if (warp == 1) {
-        if (lane == 0) {
+        if (lane == 0 && rank == 0) {
             int kit = 0, ai = 0;
             bool ok = true;
             for (int u = first_unit; u < p.units && ok; u += unit_step) {
@@ -452,27 +475,35 @@ __global__ void __launch_bounds__(MG_THREADS, 1) mod_gemm_kernel(const __grid_co
                     fence_after_sync();
                     const uint32_t a0 = smem_u32(smem + s * Cfg::STAGE), b0 = a0 + Cfg::A_BYTES;
 #pragma unroll
-                    for (int kk = 0; kk < MOD_BK / 16; ++kk)
-                        mma_bf16(acc, desc_kmajor_sw128(a0 + kk * 32), desc_kmajor_sw128(b0 + kk * 32), Cfg::IDESC,
-                                 (kc == 0 && kk == 0) ? 0u : 1u);
-                    if (CL > 1) mma_commit_multicast(smem_u32(&bars[S + s]), ALL);
-                    else mma_commit(smem_u32(&bars[S + s]));
-                    if (it == nk - 1 || (!one && kc == CH - 1)) {
-                        mma_commit(smem_u32(&bars[2 * S + (ai & 1)]));
-                        ++ai;
+                    for (int kk = 0; kk < MOD_BK / 16; ++kk) {
+                        const uint64_t ad = desc_kmajor_sw128(a0 + kk * 32), bd = desc_kmajor_sw128(b0 + kk * 32);
+                        const uint32_t add = (kc == 0 && kk == 0) ? 0u : 1u;
+                        if (PAIR) mma_bf16_pair(acc, ad, bd, Cfg::IDESC, add);
+                        else mma_bf16(acc, ad, bd, Cfg::IDESC, add);
                     }
+                    const bool done = it == nk - 1 || (!one && kc == CH - 1);
+                    if (PAIR) {
+                        mma_commit_pair(smem_u32(&bars[S + s]));
+                        if (done) mma_commit_pair(smem_u32(&bars[2 * S + (ai & 1)]));
+                    } else {
+                        mma_commit(smem_u32(&bars[S + s]));
+                        if (done) mma_commit(smem_u32(&bars[2 * S + (ai & 1)]));
+                    }
+                    if (done) ++ai;
                 }
             }
             // every MMA issued has completed before TMEM is released
-            mma_commit(smem_u32(&bars[2 * S + 4]));
-            if (!mbar_wait(smem_u32(&bars[2 * S + 4]), 0, MG_TIMEOUT_NS)) {
-                atomicOr(p.status, DEV_TIMEOUT);
-                *abort_flag = 1;
-            }
+            if (PAIR) mma_commit_pair(smem_u32(&bars[2 * S + 4]));
+            else mma_commit(smem_u32(&bars[2 * S + 4]));
+        }
+        // (both CTAs of a pair wait: the odd one's barriers have then had every arrival)
+        if (lane == 0 && !mbar_wait(smem_u32(&bars[2 * S + 4]), 0, MG_TIMEOUT_NS)) {
+            atomicOr(p.status, DEV_TIMEOUT);
+            *abort_flag = 1;
         }
     } else {
         const int q = warp & 3, ew = warp - 2;
-        constexpr int NC = BN / 2;                             // columns per thread
+        constexpr int NC = Cfg::NC;                            // columns per thread
         const int c0 = NC * (ew / 4);
         int ai = 0;
         bool ok = true;
@@ -484,6 +515,7 @@ __global__ void __launch_bounds__(MG_THREADS, 1) mod_gemm_kernel(const __grid_co
             const bool mag = m == MOD_NM;
             const int passes = (!MULTI || mag) ? 1 : nch;
             const float pm = mag ? 1.0f : c_mod.p[m], inv = mag ? 1.0f : c_mod.inv[m];
+            const float bias = 8388608.0f + 128.0f * (float)passes;
             uint32_t sum[MULTI ? NC / 2 : 1];                  // two 16-bit sums of passes a word
             if (MULTI) {
 #pragma unroll
@@ -526,9 +558,8 @@ __global__ void __launch_bounds__(MG_THREADS, 1) mod_gemm_kernel(const __grid_co
                     if (MULTI) {
 #pragma unroll
                         for (int c = 0; c < 32; c += 2) {
-                            const uint32_t r0 = __float_as_uint(mod_reduce(__uint_as_float(v[c]), pm, inv) + 8388608.0f);
-                            const uint32_t r1 =
-                                __float_as_uint(mod_reduce(__uint_as_float(v[c + 1]), pm, inv) + 8388608.0f);
+                            const uint32_t r0 = mod_bits(mod_centred(__uint_as_float(v[c]), pm, inv));
+                            const uint32_t r1 = mod_bits(mod_centred(__uint_as_float(v[c + 1]), pm, inv));
                             sum[MULTI ? 16 * h + c / 2 : 0] += __byte_perm(r0, r1, 0x5410);
                         }
                         if (ps < passes - 1) continue;
@@ -541,13 +572,14 @@ __global__ void __launch_bounds__(MG_THREADS, 1) mod_gemm_kernel(const __grid_co
                         for (int t = 0; t < 4; ++t) {
                             float x;
                             if (MULTI) {
+                                // a half word: the passes' residues + 128 each
                                 const uint32_t s2 = sum[MULTI ? 16 * h + (c + t) / 2 : 0];
                                 const uint32_t s = (t & 1) ? (s2 >> 16) : (s2 & 0xFFFFu);
-                                x = __uint_as_float(0x4B000000u | s) - 8388608.0f;
+                                x = __uint_as_float(0x4B000000u | s) - bias;
                             } else {
                                 x = __uint_as_float(v[c + t]);
                             }
-                            r[t] = __float_as_uint(mod_reduce(x, pm, inv) + 8388608.0f);
+                            r[t] = mod_bits(mod_centred(x, pm, inv));
                         }
                         w[c / 4] = __byte_perm(__byte_perm(r[0], r[1], 0x0040), __byte_perm(r[2], r[3], 0x0040), 0x5410);
                     }
@@ -559,30 +591,45 @@ __global__ void __launch_bounds__(MG_THREADS, 1) mod_gemm_kernel(const __grid_co
                 }
                 fence_before_sync();
                 __syncwarp();
-                if (lane == 0) mbar_arrive(smem_u32(&bars[2 * S + 2 + (ai & 1)]));
+                if (lane == 0) {
+                    const uint32_t eb = smem_u32(&bars[2 * S + 2 + (ai & 1)]);
+                    if (PAIR) mbar_arrive_cluster(cluster_map(eb, 0));
+                    else mbar_arrive(eb);
+                }
             }
         }
     }
     fence_before_sync();
     __syncthreads();
     fence_after_sync();
-    if (warp == 1) tmem_dealloc(tmem, 2 * BN);
-    if (CL > 1) cluster_sync();                                // no CTA leaves while another may still write to it
+    // no CTA of a pair leaves, or frees its TMEM, while the other's loads, MMAs or arrivals may
+    // still reach it
+    if (PAIR) {
+        cluster_sync();
+        if (warp == 1) tmem_dealloc_pair(tmem, 2 * BN);
+    } else if (warp == 1) {
+        tmem_dealloc(tmem, 2 * BN);
+    }
 }
 
 // ------------------------------------------------------------------ 3. combine
-// The signed 128-bit integer v times 2^e as a double, rounded once (64 leading bits).
+// The signed 128-bit integer v times 2^e as a double: its 64 leading bits, rounded to the
+// nearest (ties to even), all in integers (a conversion per output on the FP64 pipe, two a
+// cycle and SM, would cost as much as the rest).
 __device__ __forceinline__ double int_scaled(__int128 v, int e) {
     const bool neg = v < 0;
     const u128 a = neg ? (u128)(-v) : (u128)v;
     const unsigned long long hi = (unsigned long long)(a >> 64), lo = (unsigned long long)a;
     if ((hi | lo) == 0) return 0.0;
     const int z = hi ? __clzll((long long)hi) : 64 + __clzll((long long)lo);
-    const unsigned long long t = (unsigned long long)((a << z) >> 64);
-    double d = __ull2double_rn(t);                              // [2^63, 2^64]
-    long long b = __double_as_longlong(d) + ((long long)(64 - z + e) << 52);
-    if (neg) b |= (long long)(1ull << 63);
-    return __longlong_as_double(b);
+    const unsigned long long t = (unsigned long long)((a << z) >> 64);      // top bit set
+    unsigned long long m = t >> 11;
+    const unsigned rem = (unsigned)t & 0x7FFu;
+    m += rem > 0x400u || (rem == 0x400u && (m & 1));
+    // m in [2^52, 2^53]: its top bit adds one to the exponent field below
+    const unsigned long long b =
+        m + ((unsigned long long)(1023 + 126 - z + e) << 52) + (neg ? 1ull << 63 : 0ull);
+    return __longlong_as_double((long long)b);
 }
 
 // FP64 sums of a 32 x 32 tile from the operands (k in increasing order, fma).
@@ -639,7 +686,7 @@ __global__ void __launch_bounds__(256) mod_combine_kernel(const __grid_constant_
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 if (j + u >= pb.N) break;
-                unsigned long long a0 = 0, a1 = 0, a2 = 0;
+                unsigned long long a0 = c_mod.o0, a1 = c_mod.o1, a2 = c_mod.o2;
 #pragma unroll
                 for (int m = 0; m < MOD_NM; ++m) {
                     const uint32_t v = (y[m] >> (8 * u)) & 0xFFu;
@@ -689,7 +736,8 @@ __global__ void __launch_bounds__(256) mod_combine_kernel(const __grid_constant_
         const int r = (threadIdx.x >> 5) + 8 * h, i = i0 + r, j = j0 + cc;
         if (i < pb.M && j < pb.N && !(pb.tri && i > j)) {
             const size_t off = (size_t)i * pb.ldd + j;
-            double v = pb.alpha * sS[r][cc];
+            double v = sS[r][cc];
+            if (pb.alpha != 1.0) v *= pb.alpha;
             if (pb.D1) v += pb.b1 * pb.D1[off];
             if (pb.D2) v += pb.b2 * pb.D2[off];
             if (pb.D3) v += pb.b3 * pb.D3[off];
@@ -718,59 +766,56 @@ int mod_sms() {
 }
 
 dme_status mod_map(const ModBuf& b, int box_rows, CUtensorMap* out) {
-    cuuint64_t dims[3] = {(cuuint64_t)b.Kp, (cuuint64_t)b.rows, (cuuint64_t)MOD_PLANES};
-    cuuint64_t strides[2] = {(cuuint64_t)b.Kp * 2, (cuuint64_t)b.rows * b.Kp * 2};
+    cuuint64_t dims[3] = {(cuuint64_t)MOD_BK, (cuuint64_t)b.rows, (cuuint64_t)MOD_PLANES * (b.Kp / MOD_BK)};
+    cuuint64_t strides[2] = {(cuuint64_t)MOD_BK * 2, (cuuint64_t)b.rows * MOD_BK * 2};
     cuuint32_t box[3] = {(cuuint32_t)MOD_BK, (cuuint32_t)box_rows, 1};
     return encode_bf16_map(out, b.data, 3, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_128B);
 }
 
-template <int BN, int CL, bool MULTI>
-dme_status mod_gemm_launch(const CUtensorMap& tA, const CUtensorMap& tB, const ModGemmArgs& a, int clusters, cudaStream_t st) {
-    using Cfg = ModCfg<BN, CL>;
+template <int BN, bool PAIR, bool MULTI>
+dme_status mod_gemm_launch(const CUtensorMap& tA, const CUtensorMap& tB, const ModGemmArgs& a, int groups, cudaStream_t st) {
+    using Cfg = ModCfg<BN, PAIR>;
     static const cudaError_t attr = cudaFuncSetAttribute(
-        mod_gemm_kernel<BN, CL, MULTI>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::SMEM);
+        mod_gemm_kernel<BN, PAIR, MULTI>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::SMEM);
     DME_CUDA_TRY(attr);
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(std::min(a.units, clusters) * CL);
-    cfg.blockDim = dim3(MG_THREADS);
+    cfg.gridDim = dim3(std::min(a.units, groups) * Cfg::CL);
+    cfg.blockDim = dim3(Cfg::THREADS);
     cfg.dynamicSmemBytes = Cfg::SMEM;
     cfg.stream = st;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = CL;
+    at[0].val.clusterDim.x = Cfg::CL;
     at[0].val.clusterDim.y = 1;
     at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
-    cfg.numAttrs = CL > 1 ? 1 : 0;
-    DME_CUDA_TRY(cudaLaunchKernelEx(&cfg, mod_gemm_kernel<BN, CL, MULTI>, tA, tB, a));
+    cfg.numAttrs = PAIR ? 1 : 0;
+    DME_CUDA_TRY(cudaLaunchKernelEx(&cfg, mod_gemm_kernel<BN, PAIR, MULTI>, tA, tB, a));
     return DME_OK;
 }
 
-// Clusters of four 192 KB CTAs that the device holds at once (0: none).
-int mod_clusters() {
+// CTA pairs that the device holds at once (0: none).
+int mod_pairs() {
     static const int n = [] {
-        if (cudaFuncSetAttribute(mod_gemm_kernel<256, 4, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 ModCfg<256, 4>::SMEM) != cudaSuccess) {
-            cudaGetLastError();
-            return 0;
-        }
         cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(4 * mod_sms());
-        cfg.blockDim = dim3(MG_THREADS);
-        cfg.dynamicSmemBytes = ModCfg<256, 4>::SMEM;
+        cfg.gridDim = dim3(2 * mod_sms());
+        cfg.blockDim = dim3(ModCfg<256, true>::THREADS);
+        cfg.dynamicSmemBytes = ModCfg<256, true>::SMEM;
         cudaLaunchAttribute at[1];
         at[0].id = cudaLaunchAttributeClusterDimension;
-        at[0].val.clusterDim.x = 4;
+        at[0].val.clusterDim.x = 2;
         at[0].val.clusterDim.y = 1;
         at[0].val.clusterDim.z = 1;
         cfg.attrs = at;
         cfg.numAttrs = 1;
         int c = 0;
-        if (cudaOccupancyMaxActiveClusters(&c, mod_gemm_kernel<256, 4, true>, &cfg) != cudaSuccess) {
+        if (cudaFuncSetAttribute(mod_gemm_kernel<256, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 ModCfg<256, true>::SMEM) != cudaSuccess ||
+            cudaOccupancyMaxActiveClusters(&c, mod_gemm_kernel<256, true, true>, &cfg) != cudaSuccess) {
             cudaGetLastError();
             return 0;
         }
-        return std::min(c, mod_sms() / 4);
+        return std::min(c, mod_sms() / 2);
     }();
     return n;
 }
@@ -826,21 +871,24 @@ dme_status launch_mod_gemm(const ModBuf& A, const ModBuf& B, const GemmProb& g, 
     };
     if (g.N <= 64) {
         shape(MG_BM, 64);
-        DME_TRY(multi ? (mod_gemm_launch<64, 1, true>(A.t128, B.t64, a, mod_sms(), st))
-                      : (mod_gemm_launch<64, 1, false>(A.t128, B.t64, a, mod_sms(), st)));
+        DME_TRY(multi ? (mod_gemm_launch<64, false, true>(A.t128, B.t64, a, mod_sms(), st))
+                      : (mod_gemm_launch<64, false, false>(A.t128, B.t64, a, mod_sms(), st)));
     } else {
-        // the shape with the shorter run: waves x measured cycles per K block of 64
-        const int nc = mod_clusters();
+        // the shape with the shorter run: waves x measured cycles per K block of 64 (pairs:
+        // 860 in the steady state, less by what the first and last waves overlap).  Below
+        // K = 512 a unit is all latency and the smaller tile is faster (n = 256: 8.4 us
+        // against 12.1)
+        const int np = mod_pairs();
         const long w1 = ((long)mod_tile_count(g.M, g.N, g.tri, 128, 128) * planes + mod_sms() - 1) / mod_sms();
-        const long w4 = nc > 0 ? ((long)mod_tile_count(g.M, g.N, g.tri, 512, 256) * planes + nc - 1) / nc : 0;
-        if (nc > 0 && w4 * 560 < w1 * 690) {
-            shape(512, 256);
-            DME_TRY(multi ? (mod_gemm_launch<256, 4, true>(A.t128, B.t64, a, nc, st))
-                          : (mod_gemm_launch<256, 4, false>(A.t128, B.t64, a, nc, st)));
+        const long w2 = np > 0 ? ((long)mod_tile_count(g.M, g.N, g.tri, 256, 256) * planes + np - 1) / np : 0;
+        if (np > 0 && a.Kp >= 512 && w2 * 600 < w1 * 690) {
+            shape(256, 256);
+            DME_TRY(multi ? (mod_gemm_launch<256, true, true>(A.t128, B.t128, a, np, st))
+                          : (mod_gemm_launch<256, true, false>(A.t128, B.t128, a, np, st)));
         } else {
             shape(MG_BM, 128);
-            DME_TRY(multi ? (mod_gemm_launch<128, 1, true>(A.t128, B.t128, a, mod_sms(), st))
-                          : (mod_gemm_launch<128, 1, false>(A.t128, B.t128, a, mod_sms(), st)));
+            DME_TRY(multi ? (mod_gemm_launch<128, false, true>(A.t128, B.t128, a, mod_sms(), st))
+                          : (mod_gemm_launch<128, false, false>(A.t128, B.t128, a, mod_sms(), st)));
         }
     }
     const int tn = (g.N + 31) / 32, tm = (g.M + 31) / 32;

@@ -22,8 +22,8 @@ struct ModRow {
     int pad;
 };
 
-// Residue planes of a rows x k operand: [MOD_PLANES][rows][Kp] bf16, Kp = k rounded
-// up to 64 (zero padded), and the rows' scales.
+// Residue planes of a rows x k operand: [MOD_PLANES][Kp / 64][rows][64] bf16 (the rows of a
+// tile's K block are contiguous), Kp = k rounded up to 64 (zero padded), and the rows' scales.
 struct ModBuf {
     __nv_bfloat16* data = nullptr;
     ModRow* row = nullptr;
