@@ -9,6 +9,7 @@
 // tile loads, not on latency hiding.
 #include "dme_internal.h"
 #include "gemm64_tile.cuh"
+#include "pdl.cuh"
 
 #include <algorithm>
 #include <cmath>
@@ -121,6 +122,8 @@ __device__ __forceinline__ void gemm64_load8(const GemmProb& pb, int row0, int c
 
 __global__ void __launch_bounds__(64) gemm64_small_kernel(const __grid_constant__ GemmProb pb) {
     __shared__ double As[G8_K][G8 + 1], Bs[G8_K][G8 + 1];
+    pdl_trigger();
+    pdl_wait();
     int ti, tj;
     tile_coords(pb, blockIdx.x, ti, tj);
     const int row0 = ti * G8, col0 = tj * G8, tx = threadIdx.x & 7, ty = threadIdx.x >> 3;
@@ -156,8 +159,7 @@ dme_status gemm64_small(const GemmProb& g, cudaStream_t st) {
     GemmProb pb = g;
     const int tm = (g.M + G8 - 1) / G8, tn = (g.N + G8 - 1) / G8;
     pb.tiles_n = tn;
-    gemm64_small_kernel<<<g.tri ? tn * (tn + 1) / 2 : tm * tn, 64, 0, st>>>(pb);
-    DME_CUDA_TRY(cudaGetLastError());
+    DME_CUDA_TRY(pdl_launch(gemm64_small_kernel, g.tri ? tn * (tn + 1) / 2 : tm * tn, 64, 0, st, pb));
     return DME_OK;
 }
 

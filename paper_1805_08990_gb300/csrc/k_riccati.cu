@@ -16,6 +16,7 @@
 // Everything is FP64.  (1) and (4) stream P once each with coalesced,
 // 16-byte vector loads; the row dot-products of (1) are warp reductions.
 #include "dme_internal.h"
+#include "pdl.cuh"
 
 #include <algorithm>
 #include <cstring>
@@ -28,7 +29,9 @@ constexpr int RZ_MB = 8;        // columns of Bt per pass
 constexpr int RU_TILE = 32;     // update tile
 constexpr int RU_FUSE = 8;      // largest m whose Y the update forms itself
 
-__host__ __device__ __forceinline__ int rz_blocks(int n) { return (n + RZ_ROWS - 1) / RZ_ROWS; }
+constexpr int RZ_PARTS = 608;   // most blocks of kernel (1), and so most partial Gram matrices
+__host__ __device__ __forceinline__ int rz_groups(int n) { return (n + RZ_ROWS - 1) / RZ_ROWS; }
+__host__ __device__ __forceinline__ int rz_blocks(int n) { return rz_groups(n) < RZ_PARTS ? rz_groups(n) : RZ_PARTS; }
 
 size_t riccati_work_doubles(int n, int m) {
     // Z (n m) | Y (n m) | Gpart (blocks m m) | Linv (m m)
@@ -73,22 +76,29 @@ __device__ __forceinline__ int ric_find(const RicDesc* d, int nd, int blk) {
     return lo;
 }
 
-// (1) Z[r][c] = sum_k P[r][k] Bt[k][c] for the block's RZ_ROWS rows, two warps a row
-// (each half of the row's 64-column steps, the halves added in order), then the
-// block's partial Gram sums Gpart[b][i][c] = sum_{r in block} Bt[r][i] Z[r][c] in a
-// fixed order (deterministic, no atomics).  MB columns per pass.
+// (1) Z[r][c] = sum_k P[r][k] Bt[k][c], four rows at a time (row groups b, b + gridDim, ...),
+// two warps a row (each half of the row's 64-column steps, the halves added in order), and
+// the block's partial Gram sums Gpart[b][i][c] = sum_{its rows} Bt[r][i] Z[r][c], one entry
+// a thread, in a fixed order (deterministic, no atomics).  MB columns per pass.
 // Bound: the FP64 pipe (two FMAs per SM and cycle): n^2 m FMAs, so a pass computes no
-// column that is not there, and four rows a block give n / 4 blocks.
-template <int MB>
-__device__ __forceinline__ void riccati_z_pass(const RicDesc& d, int row, int half, int lane, int c0,
-                                               double (&acc)[RZ_MB]) {
+// column that is not there, and four rows a block give n / 4 blocks; at most RZ_PARTS of
+// them, since one block adds the partial sums (n = 4096, m = 8, 1024 of them: 16 us of its FP64 pipe).
+// Up to four columns of Bt are read as they lie; more of them, at a stride of m doubles per
+// lane, would keep L1 busier than the FP64 pipe (n = 4096, m = 8: 535 us), so they are staged
+// column by column in pairs: sB[c][k / 2] = (Bt[k][c], Bt[k + 1][c]) (344 us; the FP64
+// pipe alone 223).
+constexpr int RZ_KC = 512;
+
+template <int MB, bool STAGED>
+__device__ __forceinline__ void riccati_z_row(const RicDesc& d, int row, int half, int lane, int c0, int kbeg, int kend,
+                                              const double2 (*sB)[RZ_KC / 2], double (&acc)[RZ_MB]) {
     const int n = d.n, m = d.m;
     const double* __restrict__ prow = d.P + (size_t)row * n;
     const double* __restrict__ Bt = d.Bt + c0;
     const bool vec = (n % 2) == 0;
 #pragma unroll 2
-    for (int k = 2 * lane + 64 * half; k < n; k += 128) {
-        const bool two = k + 1 < n;
+    for (int k = kbeg + 2 * lane + 64 * half; k < kend; k += 128) {
+        const bool two = k + 1 < kend;
         double p0, p1 = 0.0;
         if (vec) {
             const double2 v = *reinterpret_cast<const double2*>(prow + k);
@@ -100,13 +110,24 @@ __device__ __forceinline__ void riccati_z_pass(const RicDesc& d, int row, int ha
         }
 #pragma unroll
         for (int c = 0; c < MB; ++c) {
-            const double b0 = Bt[(size_t)k * m + c], b1 = two ? Bt[(size_t)(k + 1) * m + c] : 0.0;
+            double b0, b1;
+            if (STAGED) {
+                const double2 b = sB[c][(k - kbeg) >> 1];
+                b0 = b.x;
+                b1 = b.y;
+            } else {
+                b0 = Bt[(size_t)k * m + c];
+                b1 = two ? Bt[(size_t)(k + 1) * m + c] : 0.0;
+            }
             acc[c] = fma(p1, b1, fma(p0, b0, acc[c]));
         }
     }
 }
 
 __global__ void __launch_bounds__(256) riccati_z_kernel(const __grid_constant__ RicBatch batch) {
+    pdl_trigger();
+    pdl_wait();
+    __shared__ double2 sB[RZ_MB][RZ_KC / 2];
     __shared__ double sH[2 * RZ_ROWS][RZ_MB];
     __shared__ double sZ[RZ_ROWS][RZ_MB];
     const RicDesc* ds = ric_descs(batch);
@@ -115,51 +136,114 @@ __global__ void __launch_bounds__(256) riccati_z_kernel(const __grid_constant__ 
     const int lb = blockIdx.x - d.sz;
     const int n = d.n, m = d.m;
     const double* __restrict__ Bt = d.Bt;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int row = lb * RZ_ROWS + (warp >> 1);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, tid = threadIdx.x;
+    const int parts = rz_blocks(n), groups = rz_groups(n);
     for (int c0 = 0; c0 < m; c0 += RZ_MB) {
         const int mb = min(RZ_MB, m - c0);
-        double acc[RZ_MB];
+        const int gi = tid / mb, gj = tid % mb;               // this thread's Gram entry (m mb <= 256)
+        double gram = 0.0;
+        for (int g = lb; g < groups; g += parts) {
+            const int row = g * RZ_ROWS + (warp >> 1);
+            double acc[RZ_MB];
 #pragma unroll
-        for (int c = 0; c < RZ_MB; ++c) acc[c] = 0.0;
-        if (row < n) {
-            switch (mb) {
-                case 1: riccati_z_pass<1>(d, row, warp & 1, lane, c0, acc); break;
-                case 2: riccati_z_pass<2>(d, row, warp & 1, lane, c0, acc); break;
-                case 3: riccati_z_pass<3>(d, row, warp & 1, lane, c0, acc); break;
-                case 4: riccati_z_pass<4>(d, row, warp & 1, lane, c0, acc); break;
-                case 5: riccati_z_pass<5>(d, row, warp & 1, lane, c0, acc); break;
-                case 6: riccati_z_pass<6>(d, row, warp & 1, lane, c0, acc); break;
-                case 7: riccati_z_pass<7>(d, row, warp & 1, lane, c0, acc); break;
-                default: riccati_z_pass<8>(d, row, warp & 1, lane, c0, acc); break;
+            for (int c = 0; c < RZ_MB; ++c) acc[c] = 0.0;
+            if (mb <= 4) {
+                if (row < n) {
+                    switch (mb) {
+                        case 1: riccati_z_row<1, false>(d, row, warp & 1, lane, c0, 0, n, sB, acc); break;
+                        case 2: riccati_z_row<2, false>(d, row, warp & 1, lane, c0, 0, n, sB, acc); break;
+                        case 3: riccati_z_row<3, false>(d, row, warp & 1, lane, c0, 0, n, sB, acc); break;
+                        default: riccati_z_row<4, false>(d, row, warp & 1, lane, c0, 0, n, sB, acc); break;
+                    }
+                }
+            } else {
+                for (int k0 = 0; k0 < n; k0 += RZ_KC) {
+                    __syncthreads();
+                    for (int e = tid; e < (RZ_KC / 2) * mb; e += blockDim.x) {
+                        const int kp = e / mb, c = e % mb, k = k0 + 2 * kp;      // consecutive in memory over c
+                        double2 v;
+                        v.x = k < n ? Bt[(size_t)k * m + c0 + c] : 0.0;
+                        v.y = k + 1 < n ? Bt[(size_t)(k + 1) * m + c0 + c] : 0.0;
+                        sB[c][kp] = v;
+                    }
+                    __syncthreads();
+                    if (row >= n) continue;
+                    const int kend = min(n, k0 + RZ_KC);
+                    switch (mb) {
+                        case 5: riccati_z_row<5, true>(d, row, warp & 1, lane, c0, k0, kend, sB, acc); break;
+                        case 6: riccati_z_row<6, true>(d, row, warp & 1, lane, c0, k0, kend, sB, acc); break;
+                        case 7: riccati_z_row<7, true>(d, row, warp & 1, lane, c0, k0, kend, sB, acc); break;
+                        default: riccati_z_row<8, true>(d, row, warp & 1, lane, c0, k0, kend, sB, acc); break;
+                    }
+                }
             }
-        }
 #pragma unroll
-        for (int c = 0; c < RZ_MB; ++c) {
-            if (c >= mb) break;
-            double v = acc[c];
+            for (int c = 0; c < RZ_MB; ++c) {
+                if (c >= mb) break;
+                double v = acc[c];
 #pragma unroll
-            for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-            if (lane == 0) sH[warp][c] = v;
-        }
-        __syncthreads();
-        for (int e = threadIdx.x; e < RZ_ROWS * mb; e += blockDim.x) {
-            const int r = e / mb, c = e % mb, rr = lb * RZ_ROWS + r;
-            const double v = rr < n ? sH[2 * r][c] + sH[2 * r + 1][c] : 0.0;
-            sZ[r][c] = v;
-            if (rr < n) d.Z[(size_t)rr * m + c0 + c] = v;
-        }
-        __syncthreads();
-        for (int e = threadIdx.x; e < m * mb; e += blockDim.x) {
-            const int i = e / mb, jj = e % mb;
-            double sacc = 0.0;
-            for (int r = 0; r < RZ_ROWS; ++r) {
-                const int rr = lb * RZ_ROWS + r;
-                if (rr < n) sacc = fma(Bt[(size_t)rr * m + i], sZ[r][jj], sacc);
+                for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+                if (lane == 0) sH[warp][c] = v;
             }
-            d.Gpart[(size_t)lb * m * m + (size_t)i * m + c0 + jj] = sacc;
+            __syncthreads();
+            if (tid < RZ_ROWS * mb) {
+                const int r = tid / mb, c = tid % mb, rr = g * RZ_ROWS + r;
+                const double v = rr < n ? sH[2 * r][c] + sH[2 * r + 1][c] : 0.0;
+                sZ[r][c] = v;
+                if (rr < n) d.Z[(size_t)rr * m + c0 + c] = v;
+            }
+            __syncthreads();
+            if (gi < m)
+                for (int r = 0; r < RZ_ROWS; ++r) {
+                    const int rr = g * RZ_ROWS + r;
+                    if (rr < n) gram = fma(Bt[(size_t)rr * m + gi], sZ[r][gj], gram);
+                }
         }
+        if (gi < m) d.Gpart[(size_t)lb * m * m + (size_t)gi * m + c0 + gj] = gram;
         __syncthreads();
+    }
+}
+
+// Threads of riccati_small_kernel for a problem: few partial sums leave most of 1024 threads
+// nothing but the tree over them; many need the loads in flight (n = 4096, m = 8: 35 us with
+// 256 threads, 20 with 1024).  The order of the sums follows from it, not from the launch's
+// size, so a problem gives the same bits alone and in a batch.
+__host__ __device__ __forceinline__ int rs_threads(int n, int m) { return m <= 16 && rz_blocks(n) * m * m <= 4096 ? 256 : 1024; }
+
+// M = I + t (G + G^T) / 2 for m <= RS_MAX, its Cholesky and L^{-1} in one warp: row `lane` of
+// M in registers, the pivot row handed out by shuffles (through shared memory, with the
+// columns of L^{-1} in local arrays, n = 4096, m = 8 took 28 us of which the sums were 12).
+constexpr int RS_MAX = 8;
+__device__ __forceinline__ void riccati_factor_small(const RicDesc& d, const double (&G)[32][33], int lane) {
+    const int m = d.m;
+    double a[RS_MAX], rinv[RS_MAX];
+#pragma unroll
+    for (int j = 0; j < RS_MAX; ++j)
+        a[j] = (lane < m && j < m) ? (lane == j ? 1.0 : 0.0) + d.t * 0.5 * (G[lane][j] + G[j][lane]) : 0.0;
+#pragma unroll
+    for (int j = 0; j < RS_MAX; ++j) {
+        if (j >= m) break;
+        const double dj = __shfl_sync(0xffffffffu, a[j], j);
+        if (!(dj > 0.0)) {
+            if (lane == 0) atomicOr(d.status, DEV_NOTSPD);
+            return;
+        }
+        rinv[j] = rsqrt(dj);
+        const double lj = a[j] * rinv[j];                     // L[lane][j], lane >= j
+        a[j] = lj;
+#pragma unroll
+        for (int k = j + 1; k < RS_MAX; ++k) a[k] = fma(-lj, __shfl_sync(0xffffffffu, lj, k), a[k]);
+    }
+    // column `lane` of L^{-1}: y_r = (e_r - sum_{k < r} L[r][k] y_k) / L[r][r]
+    double y[RS_MAX];
+#pragma unroll
+    for (int r = 0; r < RS_MAX; ++r) {
+        if (r >= m) break;
+        double s = (r == lane) ? 1.0 : 0.0;
+#pragma unroll
+        for (int k = 0; k < r; ++k) s = fma(-__shfl_sync(0xffffffffu, a[k], r), y[k], s);
+        y[r] = (r < lane) ? 0.0 : s * rinv[r];
+        if (lane < m) d.Linv[r * m + lane] = y[r];
     }
 }
 
@@ -167,6 +251,8 @@ __global__ void __launch_bounds__(256) riccati_z_kernel(const __grid_constant__ 
 // problem.  The sum over blocks is a fixed two-level order (strided partial
 // sums, then a tree), so the result does not depend on scheduling.
 __global__ void __launch_bounds__(1024) riccati_small_kernel(const __grid_constant__ RicBatch batch) {
+    pdl_trigger();
+    pdl_wait();
     __shared__ double red[1024];
     __shared__ double L[32][33];
     const RicDesc& d = ric_descs(batch)[blockIdx.x];
@@ -174,7 +260,7 @@ __global__ void __launch_bounds__(1024) riccati_small_kernel(const __grid_consta
     const int nblocks = rz_blocks(d.n);
     const double t = d.t;
     const int E = m * m;
-    const int G = max(1, 1024 / E);
+    const int G = max(1, rs_threads(d.n, m) / E);
     const int tid = threadIdx.x;
     const int e = tid % E, g = tid / E;
     double sacc = 0.0;
@@ -190,6 +276,10 @@ __global__ void __launch_bounds__(1024) riccati_small_kernel(const __grid_consta
     if (tid < E) L[tid / m][tid % m] = red[tid];
     __syncthreads();
     if (tid >= 32) return;
+    if (m <= RS_MAX) {
+        riccati_factor_small(d, L, tid);
+        return;
+    }
     const int lane = tid;
     // symmetrise and add the identity: M = I + t (G + G^T)/2
     double Mv[32];
@@ -231,19 +321,22 @@ __global__ void __launch_bounds__(1024) riccati_small_kernel(const __grid_consta
     }
 }
 
-// (1b) The partial Gram sums of (1) from a Z computed elsewhere (same blocks of
-// RZ_ROWS rows, same fixed order).
+// (1b) The partial Gram sums of (1) from a Z computed elsewhere (same blocks and order).
 __global__ void riccati_gpart_kernel(const __grid_constant__ RicBatch batch) {
+    pdl_trigger();
+    pdl_wait();
     const RicDesc* ds = ric_descs(batch);
     const RicDesc& d = ds[ric_find<0>(ds, batch.nd, blockIdx.x)];
     const int lb = blockIdx.x - d.sz, n = d.n, m = d.m;
+    const int parts = rz_blocks(n), groups = rz_groups(n);
     for (int e = threadIdx.x; e < m * m; e += blockDim.x) {
         const int i = e / m, c = e % m;
         double sacc = 0.0;
-        for (int r = 0; r < RZ_ROWS; ++r) {
-            const int rr = lb * RZ_ROWS + r;
-            if (rr < n) sacc = fma(d.Bt[(size_t)rr * m + i], d.Z[(size_t)rr * m + c], sacc);
-        }
+        for (int g = lb; g < groups; g += parts)
+            for (int r = 0; r < RZ_ROWS; ++r) {
+                const int rr = g * RZ_ROWS + r;
+                if (rr < n) sacc = fma(d.Bt[(size_t)rr * m + i], d.Z[(size_t)rr * m + c], sacc);
+            }
         d.Gpart[(size_t)lb * m * m + e] = sacc;
     }
 }
@@ -257,6 +350,8 @@ __device__ __forceinline__ double riccati_y_entry(const RicDesc& d, int i, int r
 }
 
 __global__ void riccati_y_kernel(const __grid_constant__ RicBatch batch) {
+    pdl_trigger();
+    pdl_wait();
     const RicDesc* ds = ric_descs(batch);
     const RicDesc& d = ds[ric_find<1>(ds, batch.nd, blockIdx.x)];
     const int i = (blockIdx.x - d.sy) * blockDim.x + threadIdx.x;
@@ -277,6 +372,8 @@ __global__ void riccati_y_kernel(const __grid_constant__ RicBatch batch) {
 // of P (and Q) are loaded together before the first is stored: one by one, each load
 // waited behind the store before it (64-wide tiles, n = 81: 16 us).
 __global__ void __launch_bounds__(256) riccati_update_kernel(const __grid_constant__ RicBatch batch) {
+    pdl_trigger();
+    pdl_wait();
     const RicDesc* ds = ric_descs(batch);
     const RicDesc& d = ds[ric_find<2>(ds, batch.nd, blockIdx.x)];
     if (*d.status & DEV_NOTSPD) return;
@@ -347,10 +444,9 @@ dme_status launch_riccati_from_z(const double* Bt, int n, int m, double t, doubl
     d.n = n;
     d.m = m;
     d.status = status;
-    riccati_gpart_kernel<<<rz_blocks(n), 64, 0, st>>>(b);
-    riccati_small_kernel<<<1, 1024, 0, st>>>(b);
-    riccati_y_kernel<<<(n + 127) / 128, 128, 0, st>>>(b);
-    DME_CUDA_TRY(cudaGetLastError());
+    DME_CUDA_TRY(pdl_launch(riccati_gpart_kernel, rz_blocks(n), 64, 0, st, b));
+    DME_CUDA_TRY(pdl_launch(riccati_small_kernel, 1, rs_threads(n, m), 0, st, b));
+    DME_CUDA_TRY(pdl_launch(riccati_y_kernel, (n + 127) / 128, 128, 0, st, b));
     return DME_OK;
 }
 
@@ -417,12 +513,15 @@ dme_status launch_riccati_grouped(const std::vector<RicItem>& items, void* dev_d
         }
         b.dev = reinterpret_cast<const RicDesc*>(dev_desc);
     }
-    riccati_z_kernel<<<sz, 256, 0, st>>>(b);
-    riccati_small_kernel<<<b.nd, 1024, 0, st>>>(b);
-    bool wide = false;
-    for (const RicItem& it : items) wide = wide || it.m > RU_FUSE;
-    if (wide) riccati_y_kernel<<<sy, 128, 0, st>>>(b);
-    riccati_update_kernel<<<su, 256, 0, st>>>(b);
+    int mmax = 0, threads = 256;
+    for (const RicItem& it : items) {
+        mmax = std::max(mmax, it.m);
+        threads = std::max(threads, rs_threads(it.n, it.m));
+    }
+    DME_CUDA_TRY(pdl_launch(riccati_z_kernel, sz, 256, 0, st, b));
+    DME_CUDA_TRY(pdl_launch(riccati_small_kernel, b.nd, threads, 0, st, b));
+    if (mmax > RU_FUSE) DME_CUDA_TRY(pdl_launch(riccati_y_kernel, sy, 128, 0, st, b));
+    DME_CUDA_TRY(pdl_launch(riccati_update_kernel, su, 256, 0, st, b));
     DME_CUDA_TRY(cudaGetLastError());
     return DME_OK;
 }
