@@ -38,6 +38,7 @@
 #include <cstring>
 #include <mutex>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 namespace dme {
@@ -290,34 +291,17 @@ __global__ void __launch_bounds__(256) slice_rows_kernel(const double* __restric
     slice_row_warp<PAIR, SCHEME, NS>(X, Xp, row, cols, ldx, out, Kp, scale, prow);
 }
 
-// Grouped slicing (serving): the rows of several problems laid end to end,
-// a warp per row; warp w finds its problem by a binary search over row0.
-template <bool PAIR>
-__global__ void __launch_bounds__(256) slice_rows_grouped_kernel(const SliceDesc* __restrict__ d, int nd,
-                                                                 int total_rows) {
-    const int g = blockIdx.x * 8 + (threadIdx.x >> 5);
-    if (g >= total_rows) return;
-    int lo = 0, hi = nd - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (d[mid].row0 <= g) lo = mid;
-        else hi = mid - 1;
-    }
-    const SliceDesc& q = d[lo];
-    slice_row_warp<PAIR, OZ_DIG9, 4>(q.X, q.Xp, g - q.row0, q.cols, q.ldx, q.out, q.Kp, q.scale, q.prow);
-}
-
-// Long rows (Kp > 1024): one CTA of 256 threads per row; each thread keeps G
-// groups of 4 consecutive entries (k = 4 tid + 1024 g) in registers, so the
-// row is read from memory once; the row maximum is a block reduction.  Same
-// digits as slice_rows_kernel.
-template <bool PAIR, int SCHEME, int NS, int G>
-__global__ void __launch_bounds__(256) slice_long_rows_kernel(const double* __restrict__ X,
-                                                              const float2* __restrict__ Xp, int rows, int cols,
-                                                              int ldx, __nv_bfloat16* __restrict__ out, int Kp,
-                                                              float* __restrict__ scale, int prow) {
-    __shared__ int wmax[8];
-    const int row = blockIdx.x, tid = threadIdx.x;
+// One block of T threads per row; each thread keeps G groups of 4 consecutive entries
+// (k = 4 tid + 4 T g) in registers, so the row is read from memory once; the row maximum is
+// a block reduction.  Same digits as slice_row_warp.  A warp per row (the first form, still
+// the grouped launch's on short rows) left the SMs with seven warps each at n = 1024 and
+// walked every row in eight dependent steps: 12 (FP64) and 15 us (pairs) against 7 and 8.
+template <bool PAIR, int SCHEME, int NS, int T, int G>
+__device__ __forceinline__ void slice_row_block(const double* __restrict__ X, const float2* __restrict__ Xp, int row,
+                                                int cols, int ldx, __nv_bfloat16* __restrict__ out, int Kp,
+                                                float* __restrict__ scale, int prow) {
+    __shared__ int wmax[T / 32];
+    const int tid = threadIdx.x;
     const size_t base = (size_t)row * ldx;
     const bool vec = (ldx % 2) == 0;
     double d[G][4];
@@ -325,7 +309,7 @@ __global__ void __launch_bounds__(256) slice_long_rows_kernel(const double* __re
     int emax = -100000;
 #pragma unroll
     for (int g = 0; g < G; ++g) {
-        const int k = 4 * tid + 1024 * g;
+        const int k = 4 * tid + 4 * T * g;
         if (k < cols) {
             load4<PAIR>(X, Xp, base, k, cols, vec, d[g], f[g]);
         } else {
@@ -344,14 +328,14 @@ __global__ void __launch_bounds__(256) slice_long_rows_kernel(const double* __re
     __syncthreads();
     emax = wmax[0];
 #pragma unroll
-    for (int w = 1; w < 8; ++w) emax = max(emax, wmax[w]);
+    for (int w = 1; w < T / 32; ++w) emax = max(emax, wmax[w]);
     const bool zero_row = emax < -100 || emax > 126;
     const int E = emax + 1;
     if (tid == 0) scale[row] = zero_row ? 0.0f : ldexpf(1.0f, E);
     const size_t plane = (size_t)prow * Kp;     // planes hold prow >= rows rows
 #pragma unroll
     for (int g = 0; g < G; ++g) {
-        const int k = 4 * tid + 1024 * g;
+        const int k = 4 * tid + 4 * T * g;
         if (k >= Kp) continue;
         long long V[4] = {0, 0, 0, 0};
         if (!zero_row && k < cols) {
@@ -362,20 +346,48 @@ __global__ void __launch_bounds__(256) slice_long_rows_kernel(const double* __re
     }
 }
 
+// Grouped slicing (serving): the rows of several problems laid end to end, a block of T
+// threads per row (Kp <= 4 T G), which finds its problem by a binary search over row0.
+template <bool PAIR, int T, int G>
+__global__ void __launch_bounds__(T) slice_rows_grouped_kernel(const SliceDesc* __restrict__ d, int nd) {
+    const int g = blockIdx.x;
+    int lo = 0, hi = nd - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (d[mid].row0 <= g) lo = mid;
+        else hi = mid - 1;
+    }
+    const SliceDesc& q = d[lo];
+    slice_row_block<PAIR, OZ_DIG9, 4, T, G>(q.X, q.Xp, g - q.row0, q.cols, q.ldx, q.out, q.Kp, q.scale, q.prow);
+}
+
+template <bool PAIR, int SCHEME, int NS, int T, int G>
+__global__ void __launch_bounds__(T) slice_block_rows_kernel(const double* __restrict__ X,
+                                                             const float2* __restrict__ Xp, int cols, int ldx,
+                                                             __nv_bfloat16* __restrict__ out, int Kp,
+                                                             float* __restrict__ scale, int prow) {
+    slice_row_block<PAIR, SCHEME, NS, T, G>(X, Xp, blockIdx.x, cols, ldx, out, Kp, scale, prow);
+}
+
 template <bool PAIR, int SCHEME, int NS>
 static void slice_launch(const double* X, const float2* Xp, int rows, int cols, int ldx, const SliceBuf& sb,
                          cudaStream_t st) {
     if (rows <= 0 || rows > sb.rows) return;
     const int pr = sb.rows;
-    if (sb.Kp > 2048)
-        slice_long_rows_kernel<PAIR, SCHEME, NS, 4>
-            <<<rows, 256, 0, st>>>(X, Xp, rows, cols, ldx, sb.data, sb.Kp, sb.scale, pr);
-    else if (sb.Kp > 1024)
-        slice_long_rows_kernel<PAIR, SCHEME, NS, 2>
-            <<<rows, 256, 0, st>>>(X, Xp, rows, cols, ldx, sb.data, sb.Kp, sb.scale, pr);
+    const int k = sb.Kp;
+    if (k > 2048)
+        slice_block_rows_kernel<PAIR, SCHEME, NS, 256, 4><<<rows, 256, 0, st>>>(X, Xp, cols, ldx, sb.data, k, sb.scale, pr);
+    else if (k > 1024)
+        slice_block_rows_kernel<PAIR, SCHEME, NS, 256, 2><<<rows, 256, 0, st>>>(X, Xp, cols, ldx, sb.data, k, sb.scale, pr);
+    else if (k > 512)
+        slice_block_rows_kernel<PAIR, SCHEME, NS, 256, 1><<<rows, 256, 0, st>>>(X, Xp, cols, ldx, sb.data, k, sb.scale, pr);
+    else if (k > 256)
+        slice_block_rows_kernel<PAIR, SCHEME, NS, 128, 1><<<rows, 128, 0, st>>>(X, Xp, cols, ldx, sb.data, k, sb.scale, pr);
+    else if (k > 128)
+        slice_block_rows_kernel<PAIR, SCHEME, NS, 64, 1><<<rows, 64, 0, st>>>(X, Xp, cols, ldx, sb.data, k, sb.scale, pr);
     else
         slice_rows_kernel<PAIR, SCHEME, NS>
-            <<<(rows + 7) / 8, 256, 0, st>>>(X, Xp, rows, cols, ldx, sb.data, sb.Kp, sb.scale, pr);
+            <<<(rows + 7) / 8, 256, 0, st>>>(X, Xp, rows, cols, ldx, sb.data, k, sb.scale, pr);
 }
 
 dme_status launch_slice_grouped(std::vector<SliceDesc>& items, bool pair, cudaStream_t st, DescArena* arena) {
@@ -388,9 +400,19 @@ dme_status launch_slice_grouped(std::vector<SliceDesc>& items, bool pair, cudaSt
     if (total == 0) return DME_OK;
     const SliceDesc* dd = static_cast<const SliceDesc*>(arena->put(items.data(), items.size() * sizeof(SliceDesc)));
     if (!dd) return set_error("grouped slicing: descriptor arena full"), DME_ENOMEM;
-    const int grid = (total + 7) / 8;
-    if (pair) slice_rows_grouped_kernel<true><<<grid, 256, 0, st>>>(dd, (int)items.size(), total);
-    else slice_rows_grouped_kernel<false><<<grid, 256, 0, st>>>(dd, (int)items.size(), total);
+    int kmax = 0;
+    for (auto& it : items) kmax = std::max(kmax, it.Kp);
+    auto launch = [&](auto t, auto g) {
+        constexpr int T = decltype(t)::value, G = decltype(g)::value;
+        if (pair) slice_rows_grouped_kernel<true, T, G><<<total, T, 0, st>>>(dd, (int)items.size());
+        else slice_rows_grouped_kernel<false, T, G><<<total, T, 0, st>>>(dd, (int)items.size());
+    };
+    using std::integral_constant;
+    if (kmax <= 256) launch(integral_constant<int, 64>{}, integral_constant<int, 1>{});
+    else if (kmax <= 512) launch(integral_constant<int, 128>{}, integral_constant<int, 1>{});
+    else if (kmax <= 1024) launch(integral_constant<int, 256>{}, integral_constant<int, 1>{});
+    else if (kmax <= 2048) launch(integral_constant<int, 256>{}, integral_constant<int, 2>{});
+    else launch(integral_constant<int, 256>{}, integral_constant<int, 4>{});
     DME_CUDA_TRY(cudaGetLastError());
     return DME_OK;
 }
