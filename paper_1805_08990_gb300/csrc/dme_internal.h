@@ -109,6 +109,15 @@ size_t block_norm1_work_doubles(int n);
 dme_status launch_gj_solve(double* M, int n, int ldm, double* B, int nrhs, int ldb, double* work, int* status,
                            cudaStream_t st);
 size_t gj_work_doubles(int n, int nrhs);
+// Y = an approximate inverse of X (n x n), computed in FP32 without pivoting across its
+// blocks of 64 (it may be useless, or hold infinities: the caller finds out).  F:
+// inv32_floats(n), work: inv32_work_floats(n).
+dme_status launch_inv32(const double* X, int n, double* Y, float* F, float* work, cudaStream_t st);
+size_t inv32_floats(int n);
+size_t inv32_work_floats(int n);
+// X += C (len entries); work[0] = |C|^2, work[1] = |X|^2 (refine_work_doubles()).
+void launch_refine_update(double* X, const double* C, size_t len, double* work, cudaStream_t st);
+size_t refine_work_doubles();
 // Self-test of the bounded grid-barrier wait: one block waits for a release
 // that never comes; *timed_out = 1 once the wait gave up with DEV_TIMEOUT.
 dme_status wait_timeout_selftest(int* timed_out);

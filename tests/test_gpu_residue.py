@@ -6,8 +6,9 @@ import numpy as np
 import pytest
 import torch
 
+import oracle as O
 import paper_1805_08990_gb300 as dme
-from gpu_util import dev, host, require_gpu
+from gpu_util import FP64_TOL, dev, host, rel, require_gpu
 
 pytestmark = pytest.mark.gpu
 
@@ -98,3 +99,34 @@ def test_generalised_steps_match_fp64_sums():
         X = S.astype(q) @ P0.astype(q) @ S.astype(q).T
         ref = P0 + 0.25 * X + (0.25 ** 2 / 2 * (S.astype(q) @ X @ S.astype(q).T) if rule == dme.DME_T4_MIDPOINT else 0)
         assert np.linalg.norm((host(P) - ref).astype(np.float64)) <= 1e-15 * np.linalg.norm(ref.astype(np.float64))
+
+
+@pytest.mark.parametrize("n", [192, 257, 448])
+@pytest.mark.parametrize("kind", ["dense", "rotation", "graded"])
+def test_exponential_solves(n, kind):
+    """The exponential's solves: refined from an FP32 inverse (dense), given up for the pivoted
+    elimination where that inverse fails (rotation by pi: the leading blocks of the Pade
+    denominator are singular, the matrix is not), and not tried for an unbalanced operator."""
+    r = np.random.default_rng(n)
+    if kind == "rotation":
+        m = n // 2
+        A = np.zeros((n, n))
+        A[np.arange(m), m + np.arange(m)] = np.pi
+        A[m + np.arange(m), np.arange(m)] = -np.pi
+        ref = np.eye(n)
+        ref[: 2 * m, : 2 * m] *= -1.0
+        t = 1.0
+    else:
+        A = r.standard_normal((n, n)) / np.sqrt(n) - 2.0 * np.eye(n)
+        t = 0.4
+        ref = O.expm(t * A)
+        if kind == "graded":
+            d = np.exp2(np.linspace(-6.0, 6.0, n))
+            A = A * d[None, :] / d[:, None]
+    plan = dme.Plan(dev(A), C=dev(np.full((1, n), 1e-3)), h=t, flows=["F1", "F2"], comp="lie")
+    E = torch.empty(n, n, dtype=torch.float64, device="cuda")
+    plan.expm(t, E, None)
+    got = host(E)
+    if kind == "graded":
+        got = got * d[:, None] / d[None, :]
+    assert rel(got, ref) < FP64_TOL
