@@ -58,11 +58,16 @@ constexpr int OZ_EPI_STAGE_BYTES = 32 * (OZ_BM + 1) * 8;
 // BN: tile columns.  128, or for products of few tiles 64 or 32: a 128 x 128 tile's FP64
 // epilogue alone keeps one SM's FP64 pipe busy for 16 us, so a product of fewer tiles
 // than SMs is cut into narrower ones (the MMAs of an output are the same in any width).
-template <int SA_, int SB_, int L_, int STAGES_, bool ACC_, int NACC_ = 4, int BN_ = OZ_BN>
+// KB: K per stage, 32 (64-byte rows) or, for narrow tiles, 64: those are bound by the number
+// of rows their loads fetch (768 a K block of 32 at 14 products: 2000 cycles, with half of
+// the MMAs left out too).
+template <int SA_, int SB_, int L_, int STAGES_, bool ACC_, int NACC_ = 4, int BN_ = OZ_BN, int KB_ = OZ_BK>
 struct OzCfg {
+    static constexpr int KB = KB_;
+    static constexpr int A_SLICE_BYTES = OZ_BM * KB * 2;
     static constexpr int SA = SA_, SB = SB_, L = L_, STAGES = STAGES_, BN = BN_;
     static constexpr int EC = BN / (OZ_EPI_WARPS / 4);              // columns per epilogue warp
-    static constexpr int B_SLICE_BYTES = BN * OZ_BK * 2;
+    static constexpr int B_SLICE_BYTES = BN * KB * 2;
     static constexpr uint32_t IDESC = idesc_bf16_f32(OZ_BM, BN);
     static constexpr bool ACC = ACC_;                                // accurate mode (exact chunks)
     // TMEM accumulators: levels 0, 1, 2, >= 3 (4), or level 0 and levels >= 1 (2: products
@@ -70,8 +75,8 @@ struct OzCfg {
     static constexpr int NACC = NACC_;
     static constexpr int TMEM_COLS = NACC * BN;
     static constexpr int MIN_BLOCKS = NACC == 2 ? 2 : 1;            // CTAs per SM the registers allow
-    static constexpr int A_BYTES = SA * OZ_SLICE_BYTES;
-    static constexpr int STAGE_BYTES = SA * OZ_SLICE_BYTES + SB * B_SLICE_BYTES;
+    static constexpr int A_BYTES = SA * A_SLICE_BYTES;
+    static constexpr int STAGE_BYTES = A_BYTES + SB * B_SLICE_BYTES;
     // the staged epilogue when the buffer fits beside the stage ring
     static constexpr bool STAGED_EPI = !ACC && STAGES * STAGE_BYTES + OZ_EPI_STAGE_BYTES + 1024 + 256 <= 232448;
     static constexpr int EPI_BYTES = STAGED_EPI ? OZ_EPI_STAGE_BYTES : 0;
@@ -91,10 +96,10 @@ using CfgP14s = OzCfg<5, 4, 4, 1, false, 2>;
 using CfgP14 = OzCfg<5, 4, 4, 3, false>;
 using CfgA21 = OzCfg<6, 6, 5, 2, true>;
 // narrow tiles
-using CfgP13n64 = OzCfg<4, 4, 4, 4, false, 4, 64>;
-using CfgP13n32 = OzCfg<4, 4, 4, 4, false, 4, 32>;
+using CfgP13n64 = OzCfg<4, 4, 4, 2, false, 4, 64, 64>;
+using CfgP13n32 = OzCfg<4, 4, 4, 2, false, 4, 32, 64>;
 using CfgP14n64 = OzCfg<5, 4, 4, 3, false, 4, 64>;
-using CfgP14n32 = OzCfg<5, 4, 4, 4, false, 4, 32>;
+using CfgP14n32 = OzCfg<5, 4, 4, 2, false, 4, 32, 64>;
 static_assert(CfgP13n64::STAGED_EPI && CfgP13n32::STAGED_EPI && CfgP14n64::STAGED_EPI && CfgP14n32::STAGED_EPI,
               "narrow tiles stage their epilogue");
 static_assert(CfgP14::SMEM <= 232448 && CfgA21::SMEM <= 232448, "shared memory per CTA");
@@ -517,13 +522,13 @@ struct OzUnit {
     int tm, tn, kb0, nk, part, nparts, widx, chunk;
 };
 
-template <int BN>
+template <int BN, int KB>
 __device__ __forceinline__ void oz_single_unit(const OzParams* p, const CUtensorMap* tA, const CUtensorMap* tB,
                                                bool acc, int u, OzUnit& o) {
     o.p = p;
     o.tA = tA;
     o.tB = tB;
-    const int nk_all = p->Kp / OZ_BK;
+    const int nk_all = (p->Kp + KB - 1) / KB;          // (KB = 64 past an odd Kp / 32: zeros)
     int tile = u, part = 0, nparts = 1, widx = 0, chunk = 0;
     if (acc) {
         // chunk-major: the units working at one time share one K range
@@ -551,7 +556,7 @@ __device__ __forceinline__ void oz_single_unit(const OzParams* p, const CUtensor
     o.chunk = chunk;
 }
 
-template <int BN>
+template <int BN, int KB>
 __device__ __forceinline__ void oz_group_unit(const OzGroupDesc* __restrict__ d, int nd, int u, OzUnit& o) {
     int lo = 0, hi = nd - 1;
     while (lo < hi) {
@@ -559,8 +564,9 @@ __device__ __forceinline__ void oz_group_unit(const OzGroupDesc* __restrict__ d,
         if (d[mid].start <= u) lo = mid;
         else hi = mid - 1;
     }
-    oz_single_unit<BN>(&d[lo].p, &d[lo].tmA, BN == OZ_BN ? &d[lo].tmB : (BN == 64 ? &d[lo].tmB64 : &d[lo].tmB32), false,
-                       u - d[lo].start, o);
+    const OzGroupDesc& g = d[lo];
+    const CUtensorMap* tB = BN == OZ_BN ? &g.tmB : (KB == 64 ? (BN == 64 ? &g.tmB64w : &g.tmB32w) : &g.tmB64);
+    oz_single_unit<BN, KB>(&g.p, KB == 64 ? &g.tmAw : &g.tmA, tB, false, u - g.start, o);
 }
 
 // Load EC columns of the four accumulators (BN columns apart) of TMEM lane quadrant q at
@@ -776,7 +782,7 @@ __device__ __forceinline__ void oz_persistent(int units, Resolve resolve) {
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * S + 3);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
         for (int s = 0; s < S; ++s) {
             mbar_init(smem_u32(&bars[s]), 1);
@@ -825,7 +831,7 @@ __device__ __forceinline__ void oz_persistent(int units, Resolve resolve) {
                     }
                     const uint32_t full = smem_u32(&bars[s]);
                     uint8_t* st = smem + s * Cfg::STAGE_BYTES;
-                    const int kc = (w.kb0 + it) * OZ_BK;
+                    const int kc = (w.kb0 + it) * Cfg::KB;
                     mbar_arrive_expect_tx(full, Cfg::STAGE_BYTES);
                     // one box per operand: the 32 x 128 tile of each of its SA (SB) planes,
                     // planes 8 KB apart in the stage
@@ -859,73 +865,76 @@ __device__ __forceinline__ void oz_persistent(int units, Resolve resolve) {
                     *abort_flag = 1;
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            int kit = 0, li = 0;
-            int* status = nullptr;
-            for (int u = blockIdx.x; u < units; u += gridDim.x, ++li) {
-                if (*abort_flag) break;
-                OzUnit w;
-                resolve(u, w);
-                status = w.p->status;
-                // the epilogue has copied the previous unit's accumulators out of TMEM
-                if (li > 0 && !mbar_wait(acc_empty, (li - 1) & 1, OZ_TIMEOUT_NS)) {
-                    atomicOr(status, DEV_TIMEOUT);
+        // the whole warp walks the units, so that addresses and descriptors stay in uniform
+        // registers, and one lane issues: with the loop under `lane == 0` and a descriptor built
+        // per MMA, an issue took 60 cycles, as long as the MMA of a 128 x 128 tile and twice
+        // that of a 128 x 32 one
+        const bool leader = elect_one();
+        int kit = 0, li = 0;
+        int* status = nullptr;
+        for (int u = blockIdx.x; u < units; u += gridDim.x, ++li) {
+            if (__any_sync(0xffffffffu, *abort_flag != 0)) break;
+            OzUnit w;
+            resolve(u, w);
+            status = w.p->status;
+            // the epilogue has copied the previous unit's accumulators out of TMEM
+            bool ok = li == 0 || mbar_wait(acc_empty, (li - 1) & 1, OZ_TIMEOUT_NS);
+            if (!__all_sync(0xffffffffu, ok)) {
+                if (leader) atomicOr(status, DEV_TIMEOUT);
+                *abort_flag = 1;
+                break;
+            }
+            fence_after_sync();
+            // the unit's own level cut: a grouped launch of the 4 x 4 slice kernel also
+            // runs 10-product problems (levels <= 3), with the same MMAs in the same order
+            // as their own kernel
+            const bool cut = Cfg::L > 3 && w.p->cfg == OZ_P10;
+            for (int it = 0; it < w.nk; ++it, ++kit) {
+                const int s = kit % S;
+                const uint32_t ph = (kit / S) & 1;
+                ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars[s]), ph, OZ_TIMEOUT_NS));
+                if (!ok) {
+                    if (leader) atomicOr(status, DEV_TIMEOUT);
                     *abort_flag = 1;
                     break;
                 }
                 fence_after_sync();
-                bool ok = true;
-                // the unit's own level cut: a grouped launch of the 4 x 4 slice kernel also
-                // runs 10-product problems (levels <= 3), with the same MMAs in the same order
-                // as their own kernel
-                const int Lu = min(Cfg::L, w.p->cfg == OZ_P10 ? 3 : Cfg::L);
-                for (int it = 0; it < w.nk; ++it, ++kit) {
-                    const int s = kit % S;
-                    const uint32_t ph = (kit / S) & 1;
-                    if (!mbar_wait(smem_u32(&bars[s]), ph, OZ_TIMEOUT_NS)) {
-                        atomicOr(status, DEV_TIMEOUT);
-                        *abort_flag = 1;
-                        ok = false;
-                        break;
-                    }
-                    fence_after_sync();
-                    const uint32_t a0 = smem_u32(smem + s * Cfg::STAGE_BYTES);
-                    const uint32_t b0 = a0 + Cfg::A_BYTES;
+                const uint32_t a0 = smem_u32(smem + s * Cfg::STAGE_BYTES);
+                const uint32_t b0 = a0 + Cfg::A_BYTES;
+                // an operand's descriptor: the stage's plus the offset (in 16-byte units)
+                const uint64_t ad0 = Cfg::KB == 64 ? desc_kmajor_sw128(a0) : desc_kmajor_sw64(a0);
+                const uint64_t bd0 = Cfg::KB == 64 ? desc_kmajor_sw128(b0) : desc_kmajor_sw64(b0);
+                const uint32_t open = it == 0 ? 0u : 1u;
+                if (leader) {
 #pragma unroll
-                    for (int kk = 0; kk < OZ_BK / 16; ++kk) {
+                    for (int kk = 0; kk < Cfg::KB / 16; ++kk) {
 #pragma unroll
                         for (int sa = 0; sa < Cfg::SA; ++sa) {
 #pragma unroll
                             for (int sb = 0; sb < Cfg::SB; ++sb) {
-                                if (sa + sb > Cfg::L || sa + sb > Lu) continue;
+                                if (sa + sb > Cfg::L || (sa + sb > 3 && cut)) continue;
                                 const int lvl = (sa + sb < Cfg::NACC - 1) ? sa + sb : Cfg::NACC - 1;
-                                const uint64_t ad = desc_kmajor_sw64(a0 + sa * OZ_SLICE_BYTES + kk * 32);
-                                const uint64_t bd = desc_kmajor_sw64(b0 + sb * Cfg::B_SLICE_BYTES + kk * 32);
                                 // the pairs (0, t), t <= 3, come first and open accumulator t at the
                                 // unit's first k step; everything else accumulates
-                                const uint32_t acc = (it == 0 && kk == 0 && sa == 0 && sb < Cfg::NACC) ? 0u : 1u;
-                                // the pairs of one A slice follow one another: its operand is read from
-                                // shared memory once and kept in the collector
-                                const uint32_t dt = tmem + (uint32_t)(lvl * Cfg::BN);
-                                const int nb = min(Cfg::SB - 1, Cfg::L - sa);      // this A slice's last pair
-                                if (nb == 0) mma_bf16(dt, ad, bd, Cfg::IDESC, acc);
-                                else if (sb == 0) mma_bf16_keep_a<MMA_A_FILL>(dt, ad, bd, Cfg::IDESC, acc);
-                                else if (sb < nb) mma_bf16_keep_a<MMA_A_USE>(dt, ad, bd, Cfg::IDESC, acc);
-                                else mma_bf16_keep_a<MMA_A_LASTUSE>(dt, ad, bd, Cfg::IDESC, acc);
+                                const uint32_t acc = (kk == 0 && sa == 0 && sb < Cfg::NACC) ? open : 1u;
+                                mma_bf16(tmem + (uint32_t)(lvl * Cfg::BN), ad0 + ((sa * Cfg::A_SLICE_BYTES + kk * 32) >> 4),
+                                         bd0 + ((sb * Cfg::B_SLICE_BYTES + kk * 32) >> 4), Cfg::IDESC, acc);
                             }
                         }
                     }
                     mma_commit(smem_u32(&bars[S + s]));
+                    if (it == w.nk - 1) mma_commit(acc_full);
                 }
-                if (!ok) break;
-                mma_commit(acc_full);
+                __syncwarp();
             }
-            // every MMA issued has completed before TMEM is released
-            mma_commit(smem_u32(&bars[2 * S + 2]));
-            if (!mbar_wait(smem_u32(&bars[2 * S + 2]), 0, OZ_TIMEOUT_NS)) {
-                if (status) atomicOr(status, DEV_TIMEOUT);
-                *abort_flag = 1;
-            }
+            if (!ok) break;
+        }
+        // every MMA issued has completed before TMEM is released
+        if (leader) mma_commit(smem_u32(&bars[2 * S + 2]));
+        __syncwarp();
+        if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&bars[2 * S + 2]), 0, OZ_TIMEOUT_NS))) {
+            if (leader && status) atomicOr(status, DEV_TIMEOUT);
+            *abort_flag = 1;
         }
     } else {
         // epilogue: warp w reads TMEM lanes 32 (w % 4) .. +31 = tile rows, columns
@@ -1030,7 +1039,7 @@ template <class Cfg>
 __global__ void __launch_bounds__(OZ_THREADS, Cfg::MIN_BLOCKS) ozaki_gemm_kernel(const __grid_constant__ CUtensorMap tmA,
                                                                    const __grid_constant__ CUtensorMap tmB,
                                                                    const __grid_constant__ OzParams p) {
-    oz_persistent<Cfg>(p.units, [&](int u, OzUnit& o) { oz_single_unit<Cfg::BN>(&p, &tmA, &tmB, Cfg::ACC, u, o); });
+    oz_persistent<Cfg>(p.units, [&](int u, OzUnit& o) { oz_single_unit<Cfg::BN, Cfg::KB>(&p, &tmA, &tmB, Cfg::ACC, u, o); });
 }
 
 // Grouped form: the tiles of every problem laid end to end; a unit finds its
@@ -1040,7 +1049,7 @@ __global__ void __launch_bounds__(OZ_THREADS, Cfg::MIN_BLOCKS) ozaki_gemm_kernel
 template <class Cfg>
 __global__ void __launch_bounds__(OZ_THREADS, 1) ozaki_gemm_grouped_kernel(const OzGroupDesc* __restrict__ d, int nd,
                                                                            int units) {
-    oz_persistent<Cfg>(units, [&](int u, OzUnit& o) { oz_group_unit<Cfg::BN>(d, nd, u, o); });
+    oz_persistent<Cfg>(units, [&](int u, OzUnit& o) { oz_group_unit<Cfg::BN, Cfg::KB>(d, nd, u, o); });
 }
 
 // Split K of the tail: the parts' level sums added in part order (the level-0
@@ -1179,11 +1188,13 @@ dme_status encode_bf16_map(CUtensorMap* out, const void* data, int rank, const c
     return DME_OK;
 }
 
-static dme_status make_slice_tmap(const SliceBuf& sb, int planes, CUtensorMap* out, int box_rows = OZ_BM) {
+static dme_status make_slice_tmap(const SliceBuf& sb, int planes, CUtensorMap* out, int box_rows = OZ_BM,
+                                  int box_k = OZ_BK) {
     cuuint64_t dims[3] = {(cuuint64_t)sb.Kp, (cuuint64_t)sb.rows, (cuuint64_t)sb.ns};
     cuuint64_t strides[2] = {(cuuint64_t)sb.Kp * 2, (cuuint64_t)sb.rows * sb.Kp * 2};
-    cuuint32_t box[3] = {(cuuint32_t)OZ_BK, (cuuint32_t)box_rows, (cuuint32_t)planes};
-    return encode_bf16_map(out, sb.data, 3, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_64B);
+    cuuint32_t box[3] = {(cuuint32_t)box_k, (cuuint32_t)box_rows, (cuuint32_t)planes};
+    return encode_bf16_map(out, sb.data, 3, dims, strides, box,
+                           box_k == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B);
 }
 
 dme_status make_slice_tmaps(SliceBuf& sb) {
@@ -1192,7 +1203,10 @@ dme_status make_slice_tmaps(SliceBuf& sb) {
     if (sb.ns > 4) DME_TRY(make_slice_tmap(sb, 4, &sb.tmap4));
     if (sb.ns >= 4 && sb.scheme == OZ_DIG9) {
         DME_TRY(make_slice_tmap(sb, 4, &sb.tmap64, 64));
-        DME_TRY(make_slice_tmap(sb, 4, &sb.tmap32, 32));
+        DME_TRY(make_slice_tmap(sb, 4, &sb.tmap64w, 64, 64));
+        DME_TRY(make_slice_tmap(sb, 4, &sb.tmap32w, 32, 64));
+        DME_TRY(make_slice_tmap(sb, sb.ns, &sb.tmapw, OZ_BM, 64));
+        DME_TRY(make_slice_tmap(sb, 4, &sb.tmap4w, OZ_BM, 64));
     }
     return DME_OK;
 }
@@ -1326,11 +1340,12 @@ dme_status launch_ozaki_gemm(const SliceBuf& A, const SliceBuf& B, OzParams p, c
         p.tiles_n = (p.N + bn - 1) / bn;
         p.tiles = p.units = p.split_first = oz_narrow_tiles(p, bn);
         const int g = std::min(p.units, nsm);
+        const CUtensorMap& tAw = oz_tmap_aw(A, p.cfg);
         if (p.cfg == OZ_P14)
             return bn == 64 ? oz_launch_single<CfgP14n64>(tA, B.tmap64, p, g, st)
-                            : oz_launch_single<CfgP14n32>(tA, B.tmap32, p, g, st);
-        return bn == 64 ? oz_launch_single<CfgP13n64>(tA, B.tmap64, p, g, st)     // (cuts 10 products itself)
-                        : oz_launch_single<CfgP13n32>(tA, B.tmap32, p, g, st);
+                            : oz_launch_single<CfgP14n32>(tAw, B.tmap32w, p, g, st);
+        return bn == 64 ? oz_launch_single<CfgP13n64>(tAw, B.tmap64w, p, g, st)     // (cuts 10 products itself)
+                        : oz_launch_single<CfgP13n32>(tAw, B.tmap32w, p, g, st);
     }
     switch (p.cfg) {
         case OZ_P10:

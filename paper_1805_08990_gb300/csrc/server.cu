@@ -439,7 +439,9 @@ dme_status run_lane(dme_server_t s, std::vector<Req*>& res, int lane) {
                 a.tmA = oz_tmap_a(e.Gsl, p->cfg);
                 a.tmB = oz_tmap_b(p->psl, p->cfg);
                 a.tmB64 = p->psl.tmap64;
-                a.tmB32 = p->psl.tmap32;
+                a.tmAw = oz_tmap_aw(e.Gsl, p->cfg);
+                a.tmB64w = p->psl.tmap64w;
+                a.tmB32w = p->psl.tmap32w;
                 DME_TRY(oz_params(e.Gsl, p->psl, p->cfg, &a.p));
                 a.p.mode = OZ_OUT_PAIR;
                 a.p.ldc = n;
@@ -452,7 +454,9 @@ dme_status run_lane(dme_server_t s, std::vector<Req*>& res, int lane) {
                 b.tmA = oz_tmap_a(e.Gsl, p->cfg);
                 b.tmB = oz_tmap_b(p->usl, p->cfg);
                 b.tmB64 = p->usl.tmap64;
-                b.tmB32 = p->usl.tmap32;
+                b.tmAw = oz_tmap_aw(e.Gsl, p->cfg);
+                b.tmB64w = p->usl.tmap64w;
+                b.tmB32w = p->usl.tmap32w;
                 DME_TRY(oz_params(e.Gsl, p->usl, p->cfg, &b.p));
                 b.p.mode = OZ_OUT_F64;
                 b.p.tri = 1;

@@ -54,7 +54,9 @@ struct SliceBuf {
     int scheme = OZ_DIG9;
     CUtensorMap tmap;
     CUtensorMap tmap4;
-    CUtensorMap tmap64, tmap32;   // DIG9: four planes in boxes of 64 and 32 rows (narrow tiles)
+    // DIG9, for narrow tiles: four planes in boxes of 64 rows; and with 64 k to the box (w),
+    // of 64, 32 and 128 rows, and every plane in boxes of 128
+    CUtensorMap tmap64, tmap64w, tmap32w, tmap4w, tmapw;
 };
 
 struct OzParams {
@@ -96,7 +98,8 @@ constexpr size_t OZ_SPLIT_WS_FLOAT2 = (size_t)OZ_SPLIT_MAX_TAIL * 2 * 128 * 128;
 // One problem of a grouped split GEMM (tensor maps live in global memory).
 struct OzGroupDesc {
     CUtensorMap tmA;
-    CUtensorMap tmB, tmB64, tmB32;
+    CUtensorMap tmB, tmB64;
+    CUtensorMap tmAw, tmB64w, tmB32w;   // 64 k to the box
     OzParams p;
     int start;            // first unit index (set by the launcher)
     int tail_start;       // first split tile in the launch's tail kernel (set by the launcher)
@@ -126,6 +129,9 @@ inline const CUtensorMap& oz_tmap_a(const SliceBuf& A, int cfg) {
 }
 inline const CUtensorMap& oz_tmap_b(const SliceBuf& B, int cfg) {
     return B.ns > oz_cfg_slices_b(cfg) ? B.tmap4 : B.tmap;
+}
+inline const CUtensorMap& oz_tmap_aw(const SliceBuf& A, int cfg) {
+    return A.ns > oz_cfg_slices_a(cfg) ? A.tmap4w : A.tmapw;
 }
 // Slice the rows of X (rows x cols, leading dimension ldx; rows <= sb.rows) into sb
 // (planes and digit scheme of sb: DIG9 with 4 or 5, DIG7 with 6; each plane holds

@@ -132,39 +132,17 @@ __device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t adesc, uint64
         : "memory");
 }
 
-// As mma_bf16, with the A operand's collector buffer: `fill` keeps A for the next MMA,
-// `use` takes it from there (same A), `lastuse` takes it and lets it go.
-enum { MMA_A_FILL = 0, MMA_A_USE = 1, MMA_A_LASTUSE = 2 };
-template <int OP>
-__device__ __forceinline__ void mma_bf16_keep_a(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                                uint32_t accumulate) {
-    if (OP == MMA_A_FILL)
-        asm volatile(
-            "{\n"
-            " .reg .pred p;\n"
-            " setp.ne.b32 p, %4, 0;\n"
-            " tcgen05.mma.cta_group::1.kind::f16.collector::a::fill [%0], %1, %2, %3, p;\n"
-            "}\n" ::"r"(d_tmem),
-            "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-            : "memory");
-    else if (OP == MMA_A_USE)
-        asm volatile(
-            "{\n"
-            " .reg .pred p;\n"
-            " setp.ne.b32 p, %4, 0;\n"
-            " tcgen05.mma.cta_group::1.kind::f16.collector::a::use [%0], %1, %2, %3, p;\n"
-            "}\n" ::"r"(d_tmem),
-            "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-            : "memory");
-    else
-        asm volatile(
-            "{\n"
-            " .reg .pred p;\n"
-            " setp.ne.b32 p, %4, 0;\n"
-            " tcgen05.mma.cta_group::1.kind::f16.collector::a::lastuse [%0], %1, %2, %3, p;\n"
-            "}\n" ::"r"(d_tmem),
-            "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-            : "memory");
+// One lane of a converged warp, the same one each time.
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile(
+        "{\n"
+        " .reg .pred p;\n"
+        " elect.sync _|p, 0xffffffff;\n"
+        " selp.u32 %0, 1, 0, p;\n"
+        "}\n"
+        : "=r"(p));
+    return p != 0;
 }
 
 // Arrive on `bar` once every tcgen05.mma issued so far by this thread has completed.
