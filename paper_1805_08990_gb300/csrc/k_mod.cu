@@ -374,7 +374,7 @@ __global__ void __launch_bounds__(ModCfg<BN, PAIR>::THREADS, 1) mod_gemm_kernel(
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + S * Cfg::STAGE);
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * S + 5);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
         for (int s = 0; s < S; ++s) {
             mbar_init(smem_u32(&bars[s]), 1);
@@ -451,7 +451,9 @@ __global__ void __launch_bounds__(ModCfg<BN, PAIR>::THREADS, 1) mod_gemm_kernel(
                     *abort_flag = 1;
         }
     } else if (warp == 1) {
-        if (lane == 0 && rank == 0) {
+        // the warp together, one lane issuing: addresses and descriptors in uniform registers
+        const bool leader = elect_one();
+        if (rank == 0) {
             int kit = 0, ai = 0;
             bool ok = true;
             for (int u = first_unit; u < p.units && ok; u += unit_step) {
@@ -461,44 +463,51 @@ __global__ void __launch_bounds__(ModCfg<BN, PAIR>::THREADS, 1) mod_gemm_kernel(
                     const int kc = one ? it : it % CH;
                     const uint32_t acc = tmem + (uint32_t)((ai & 1) * BN);
                     if (kc == 0) {
-                        if (ai >= 2 && !mbar_wait(smem_u32(&bars[2 * S + 2 + (ai & 1)]), ((ai >> 1) - 1) & 1, MG_TIMEOUT_NS))
-                            ok = false;
+                        if (ai >= 2) ok = mbar_wait(smem_u32(&bars[2 * S + 2 + (ai & 1)]), ((ai >> 1) - 1) & 1, MG_TIMEOUT_NS);
                         fence_after_sync();
                     }
                     const int s = kit % S;
-                    if (!ok || !mbar_wait(smem_u32(&bars[s]), (kit / S) & 1, MG_TIMEOUT_NS)) {
-                        atomicOr(p.status, DEV_TIMEOUT);
+                    ok = ok && mbar_wait(smem_u32(&bars[s]), (kit / S) & 1, MG_TIMEOUT_NS);
+                    ok = __all_sync(0xffffffffu, ok);
+                    if (!ok) {
+                        if (leader) atomicOr(p.status, DEV_TIMEOUT);
                         *abort_flag = 1;
-                        ok = false;
                         break;
                     }
                     fence_after_sync();
-                    const uint32_t a0 = smem_u32(smem + s * Cfg::STAGE), b0 = a0 + Cfg::A_BYTES;
-#pragma unroll
-                    for (int kk = 0; kk < MOD_BK / 16; ++kk) {
-                        const uint64_t ad = desc_kmajor_sw128(a0 + kk * 32), bd = desc_kmajor_sw128(b0 + kk * 32);
-                        const uint32_t add = (kc == 0 && kk == 0) ? 0u : 1u;
-                        if (PAIR) mma_bf16_pair(acc, ad, bd, Cfg::IDESC, add);
-                        else mma_bf16(acc, ad, bd, Cfg::IDESC, add);
-                    }
+                    const uint32_t a0 = smem_u32(smem + s * Cfg::STAGE);
+                    const uint64_t ad = desc_kmajor_sw128(a0), bd = desc_kmajor_sw128(a0 + Cfg::A_BYTES);
+                    const uint32_t open = kc == 0 ? 0u : 1u;
                     const bool done = it == nk - 1 || (!one && kc == CH - 1);
-                    if (PAIR) {
-                        mma_commit_pair(smem_u32(&bars[S + s]));
-                        if (done) mma_commit_pair(smem_u32(&bars[2 * S + (ai & 1)]));
-                    } else {
-                        mma_commit(smem_u32(&bars[S + s]));
-                        if (done) mma_commit(smem_u32(&bars[2 * S + (ai & 1)]));
+                    if (leader) {
+#pragma unroll
+                        for (int kk = 0; kk < MOD_BK / 16; ++kk) {
+                            const uint32_t add = kk == 0 ? open : 1u;
+                            if (PAIR) mma_bf16_pair(acc, ad + 2 * kk, bd + 2 * kk, Cfg::IDESC, add);
+                            else mma_bf16(acc, ad + 2 * kk, bd + 2 * kk, Cfg::IDESC, add);
+                        }
+                        if (PAIR) {
+                            mma_commit_pair(smem_u32(&bars[S + s]));
+                            if (done) mma_commit_pair(smem_u32(&bars[2 * S + (ai & 1)]));
+                        } else {
+                            mma_commit(smem_u32(&bars[S + s]));
+                            if (done) mma_commit(smem_u32(&bars[2 * S + (ai & 1)]));
+                        }
                     }
+                    __syncwarp();
                     if (done) ++ai;
                 }
             }
             // every MMA issued has completed before TMEM is released
-            if (PAIR) mma_commit_pair(smem_u32(&bars[2 * S + 4]));
-            else mma_commit(smem_u32(&bars[2 * S + 4]));
+            if (leader) {
+                if (PAIR) mma_commit_pair(smem_u32(&bars[2 * S + 4]));
+                else mma_commit(smem_u32(&bars[2 * S + 4]));
+            }
+            __syncwarp();
         }
         // (both CTAs of a pair wait: the odd one's barriers have then had every arrival)
-        if (lane == 0 && !mbar_wait(smem_u32(&bars[2 * S + 4]), 0, MG_TIMEOUT_NS)) {
-            atomicOr(p.status, DEV_TIMEOUT);
+        if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&bars[2 * S + 4]), 0, MG_TIMEOUT_NS))) {
+            if (leader) atomicOr(p.status, DEV_TIMEOUT);
             *abort_flag = 1;
         }
     } else {
