@@ -197,20 +197,44 @@ __global__ void __launch_bounds__(1024) jacobi_eig_kernel(const double* __restri
 // 0.25 ms).  Both factorisations are one block (a chain of r pivots, FP64 issue of
 // one SM): the packed upper triangle in shared memory.
 
-// The rank-one update of the remaining triangle: rows a of the list idx (or a itself),
-// a warp each, lanes over b >= a.
-template <bool LIST>
-__device__ __forceinline__ void chol_update(double* A, const double* v, const int* idx, int a0, int m, int r) {
-    const int lane = threadIdx.x & 31;
-    for (int a = a0 + (threadIdx.x >> 5); a < m; a += blockDim.x >> 5) {
-        const int i = LIST ? idx[a] : a;
-        const double vi = v[i];
-        for (int b = a + lane; b < m; b += 32) {
-            const int j = LIST ? idx[b] : b;
-            const int e = LIST ? (i <= j ? pk(i, j, r) : pk(j, i, r)) : pk(i, j, r);
-            A[e] = fma(-vi, v[j], A[e]);
+//
+// Per pivot the chain is scale, update, next pivot, each FP64 instruction of a lone warp
+// about 65 cycles: warp 0 keeps the diagonal by itself and forms the next pivot and its
+// reciprocal root while the others update the triangle (as one rank-one update between
+// barriers, with the root and a divide in every warp: 82 and 60 us at r = 57 instead of
+// 42 and 36, 122 and 86 at r = 100 instead of 69 and 42).
+
+// The rank-one update of the strict triangle over positions [a0, m), by warps 1, 2, ...:
+// rows q from the front and from the back are paired, so that a pair has m - a0 - 1
+// entries and lanes idle only at its end.  col(a) is the column at position a.
+template <class Col>
+__device__ __forceinline__ void chol_update(double* A, const double* v, int a0, int m, int r, const Col& col) {
+    const int lane = threadIdx.x & 31, w = m - a0;
+    for (int q = (threadIdx.x >> 5) - 1; q < (w + 1) / 2; q += (blockDim.x >> 5) - 1) {
+        const int back = w - 1 - q;
+        const int i0 = col(a0 + q), i1 = col(a0 + back);
+        const double v0 = v[i0], v1 = v[i1];
+        const int len = back == q ? back : w - 1;
+        for (int t = lane; t < len; t += 32) {
+            const bool front = t < back;
+            const int j = col(a0 + (front ? q + 1 + t : t + 1)), i = front ? i0 : i1;
+            const int e = i <= j ? pk(i, j, r) : pk(j, i, r);
+            A[e] = fma(front ? -v0 : -v1, v[j], A[e]);
         }
     }
+}
+
+// One warp: the position of the largest diagonal entry among col(0), ..., col(m - 1) to 20
+// bits (lane l has seen l, l + 32, ...: `hi` the largest high word, `pos` its position).
+__device__ __forceinline__ int chol_argmax(int hi, int pos) {
+    const int top = __reduce_max_sync(0xffffffffu, hi);
+    return __reduce_min_sync(0xffffffffu, hi == top ? pos : 0x7fffffff);
+}
+
+// The high word of x as an ordering key; negatives, infinities and NaN sort below zero.
+__device__ __forceinline__ int chol_key(double x) {
+    const int h = __double2hiint(x);
+    return h < 0x7FF00000 ? h : -1;
 }
 
 __global__ void __launch_bounds__(512) chol_pivot_kernel(const double* __restrict__ G, int ldg, int r,
@@ -218,10 +242,11 @@ __global__ void __launch_bounds__(512) chol_pivot_kernel(const double* __restric
                                                          double* __restrict__ R, int ldr, int* __restrict__ k_out,
                                                          int* status) {
     extern __shared__ __align__(16) double csm[];
-    double* A = csm;                                  // packed upper triangle
+    double* A = csm;                                  // packed upper triangle (diagonal unused)
     double* v = A + (size_t)r * (r + 1) / 2;
     double* ds = v + r;                               // sqrt(d)
-    int* idx = reinterpret_cast<int*>(ds + r);
+    double* dg = ds + r;                              // the diagonal
+    int* idx = reinterpret_cast<int*>(dg + r);
     __shared__ int s_pos, bad;
     __shared__ double s_piv, s_rp;
     const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31;
@@ -237,6 +262,7 @@ __global__ void __launch_bounds__(512) chol_pivot_kernel(const double* __restric
         if (i <= j) {
             const double g = 0.5 * (G[(size_t)i * ldg + j] + G[(size_t)j * ldg + i]) * (ds[i] * ds[j]);
             A[pk(i, j, r)] = g;
+            if (i == j) dg[i] = g;
             if (!isfinite(g)) bad = 1;
         }
     }
@@ -248,51 +274,54 @@ __global__ void __launch_bounds__(512) chol_pivot_kernel(const double* __restric
         }
         return;
     }
-    int m = r, k = 0;
+    int m = r, k = 0, pos = -1;
     double stop = 0.0;
-    for (; m > 0; ++k) {
+    for (;; ++k) {
+        // position pos (the last pivot) now holds the last column; idx[pos] itself is only
+        // rewritten below, where nobody reads it
+        const auto col = [&](int a) { return idx[a == pos ? m : a]; };
         if (tid < 32) {
-            double best = -1.0;
-            int pos = 0;
+            int hi = -1, at = 0;
             for (int a = lane; a < m; a += 32) {
-                const int i = idx[a];
-                const double x = A[pk(i, i, r)];
-                if (x > best) {
-                    best = x;
-                    pos = a;
+                const int j = col(a);
+                double x = dg[j];
+                if (k > 0) {
+                    x = fma(-v[j], v[j], x);
+                    dg[j] = x;
+                }
+                if (chol_key(x) > hi) {
+                    hi = chol_key(x);
+                    at = a;
                 }
             }
-#pragma unroll
-            for (int off = 16; off > 0; off >>= 1) {
-                const double ov = __shfl_xor_sync(0xffffffffu, best, off);
-                const int op = __shfl_xor_sync(0xffffffffu, pos, off);
-                if (ov > best || (ov == best && op < pos)) {
-                    best = ov;
-                    pos = op;
-                }
-            }
+            at = chol_argmax(hi, at);
+            __syncwarp();
             if (lane == 0) {
-                s_piv = best;
-                s_rp = best > 0.0 ? 1.0 / sqrt(best) : 0.0;
-                s_pos = pos;
+                double x = 0.0;
+                if (m > 0 && at < m) {
+                    x = dg[col(at)];
+                    if (k > 0 && pos < m) idx[pos] = idx[m];
+                }
+                s_pos = at;
+                s_piv = x;
+                s_rp = x > 0.0 ? rsqrt(x) : 0.0;
             }
+        } else if (k > 0) {
+            chol_update(A, v, 0, m, r, col);
         }
         __syncthreads();
-        const double piv = s_piv;
+        const double piv = s_piv, rp = s_rp;
         if (k == 0) stop = tol * piv;
-        if (!(piv > stop)) break;
-        const int pos = s_pos, p = idx[pos];
+        if (m == 0 || !(piv > stop)) break;
+        pos = s_pos;
+        const int p = idx[pos];
         for (int a = tid; a < m; a += nt) {
             const int j = idx[a];
-            const double x = A[p <= j ? pk(p, j, r) : pk(j, p, r)] * s_rp;
+            const double x = (p == j ? dg[j] : A[p < j ? pk(p, j, r) : pk(j, p, r)]) * rp;
             v[j] = x;
             R[(size_t)k * ldr + j] = x;
         }
-        __syncthreads();
-        if (tid == 0) idx[pos] = idx[m - 1];
         --m;
-        __syncthreads();
-        chol_update<true>(A, v, idx, 0, m, r);
         __syncthreads();
     }
     if (tid == 0) *k_out = k;
@@ -304,102 +333,138 @@ __global__ void __launch_bounds__(512) chol_rows_kernel(const double* __restrict
                                                         double* __restrict__ T, int ldt, double* __restrict__ rinv,
                                                         double* __restrict__ nrm) {
     extern __shared__ __align__(16) double csm[];
+    __shared__ double s_rp;
     const int n = min(*k, r);
-    double* A = csm;
+    double* A = csm;                                  // packed upper triangle (diagonal unused)
     double* v = A + (size_t)r * (r + 1) / 2;
+    double* dg = v + r;
     const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31;
     for (int e = tid; e < n * n; e += nt) {
         const int i = e / n, j = e % n;
         if (i <= j) A[pk(i, j, r)] = H[(size_t)i * ldh + j];
+        if (i == j) dg[i] = H[(size_t)i * ldh + i];
     }
     __syncthreads();
     int j = 0;
-    for (; j < n; ++j) {
-        const double piv = A[pk(j, j, r)];
-        if (!(piv > 0.0)) break;
-        const double rp = 1.0 / sqrt(piv);
+    for (;; ++j) {
+        if (tid < 32) {
+            for (int a = j + lane; a < n; a += 32) {
+                double x = dg[a];
+                if (j > 0) {
+                    x = fma(-v[a], v[a], x);
+                    dg[a] = x;
+                }
+                if (a == j) s_rp = x > 0.0 ? rsqrt(x) : 0.0;
+            }
+        } else if (j > 0) {
+            if (tid >= nt - 32) {                      // the last row's norm, beside the update
+                double s = 0.0;
+                for (int a = j - 1 + lane; a < n; a += 32) s = fma(v[a], v[a], s);
+#pragma unroll
+                for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+                if (lane == 0) nrm[j - 1] = s;
+            }
+            chol_update(A, v, j, n, r, [](int a) { return a; });
+        }
+        __syncthreads();
+        if (j == n) break;
+        const double rp = s_rp;
+        if (!(rp > 0.0)) break;
+        if (tid == 0) rinv[j] = rp;
         for (int a = j + tid; a < n; a += nt) {
-            const double x = A[pk(j, a, r)] * rp;
+            const double x = (a == j ? dg[a] : A[pk(j, a, r)]) * rp;
             v[a] = x;
             T[(size_t)j * ldt + a] = x;
         }
-        __syncthreads();
-        if (tid >= nt - 32) {                          // the row's norm, beside the update
-            double s = 0.0;
-            for (int a = j + lane; a < n; a += 32) s = fma(v[a], v[a], s);
-#pragma unroll
-            for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-            if (lane == 0) {
-                nrm[j] = s;
-                rinv[j] = rp;
-            }
-        }
-        chol_update<false>(A, v, nullptr, j + 1, n, r);
         __syncthreads();
     }
     if (tid == 0) *k = j;
 }
 
 // X = T^{-T} R, a warp per column, lane l holding the entries l, l + 32, ...; rows from *k
-// on are zero.  The next row of T is loaded while the current one is applied.
+// on are zero.  The rows of T come in panels through shared memory: with a row loaded ahead
+// from L2 each of the k dependent steps took that latency (32 us at r = 56, now 20).
+constexpr int QS_ROWS = 16;
 __global__ void __launch_bounds__(128) qlp_solve_kernel(const double* __restrict__ T, int ldt,
                                                         const double* __restrict__ rinv, const double* __restrict__ R,
                                                         int ldr, int r, const int* __restrict__ k, double* __restrict__ X,
                                                         int ldx) {
     constexpr int Q = LR_MAX_RANK / 32;
+    __shared__ double Ts[QS_ROWS][LR_MAX_RANK], ri[QS_ROWS];
     const int c = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-    if (c >= r) return;
+    const bool on = c < r;
     const int n = *k;
-    double b[Q], t[Q];
+    double b[Q];
 #pragma unroll
     for (int q = 0; q < Q; ++q) {
         const int i = lane + 32 * q;
-        b[q] = i < n ? R[(size_t)i * ldr + c] : 0.0;
-        t[q] = i < n ? T[i] : 0.0;
+        b[q] = on && i < n ? R[(size_t)i * ldr + c] : 0.0;
     }
 #pragma unroll
     for (int qi = 0; qi < Q; ++qi)
-        for (int li = 0; li < 32; ++li) {
-            const int i = 32 * qi + li;
-            if (i >= n) break;
-            double tn[Q];
+        for (int half = 0; half < 2; ++half) {
+            const int i0 = 32 * qi + QS_ROWS * half, rows = min(QS_ROWS, n - i0);
+            if (rows <= 0) break;
+            __syncthreads();
+            double t[QS_ROWS / 4][Q];         // every load of the panel in flight at once
 #pragma unroll
-            for (int q = qi; q < Q; ++q) {
-                const int kk = lane + 32 * q;
-                tn[q] = (i + 1 < n && kk > i && kk < n) ? T[(size_t)(i + 1) * ldt + kk] : 0.0;
-            }
-            const double x = __shfl_sync(0xffffffffu, b[qi], li) * rinv[i];
-            if (lane == li) b[qi] = x;
+            for (int w = 0; w < QS_ROWS / 4; ++w)
 #pragma unroll
-            for (int q = qi; q < Q; ++q) {
-                if (lane + 32 * q > i) b[q] = fma(-t[q], x, b[q]);
-                t[q] = tn[q];
+                for (int q = qi; q < Q; ++q) {
+                    const int i = (threadIdx.x >> 5) + 4 * w, kk = lane + 32 * q;
+                    t[w][q] = i < rows && kk > i0 + i && kk < n ? T[(size_t)(i0 + i) * ldt + kk] : 0.0;
+                }
+#pragma unroll
+            for (int w = 0; w < QS_ROWS / 4; ++w)
+#pragma unroll
+                for (int q = qi; q < Q; ++q) Ts[(threadIdx.x >> 5) + 4 * w][lane + 32 * q] = t[w][q];
+            if (threadIdx.x < rows) ri[threadIdx.x] = rinv[i0 + threadIdx.x];
+            __syncthreads();
+            for (int i = 0; i < rows; ++i) {
+                const int li = QS_ROWS * half + i;
+                const double x = __shfl_sync(0xffffffffu, b[qi], li) * ri[i];
+                if (lane == li) b[qi] = x;
+                // zeros of Ts leave the entries up to i0 + i alone
+#pragma unroll
+                for (int q = qi; q < Q; ++q)
+                    if (32 * q < n) {
+                        const int kk = lane + 32 * q;
+                        if (kk > i0 + i && kk < n) b[q] = fma(-Ts[i][kk], x, b[q]);
+                    }
             }
         }
 #pragma unroll
     for (int q = 0; q < Q; ++q) {
         const int i = lane + 32 * q;
-        if (i < r) X[(size_t)i * ldx + c] = b[q];
+        if (on && i < r) X[(size_t)i * ldx + c] = b[q];
     }
 }
 
 // Keep the rows j of X with nrm[j] > tol * max: To[a][rank] = X[j][a] sqrt(d[a]), d_out = 1,
 // k_out their count (d_out may alias d).
-__global__ void __launch_bounds__(256) qlp_select_kernel(const double* __restrict__ X, int ldx,
+__global__ void __launch_bounds__(1024) qlp_select_kernel(const double* __restrict__ X, int ldx,
                                                          const double* __restrict__ nrm, const int* __restrict__ k, int r,
                                                          double tol, const double* d, double* __restrict__ To, int ldt,
                                                          double* d_out, int* k_out) {
-    __shared__ double rs[LR_MAX_RANK], smax;
+    __shared__ double rs[LR_MAX_RANK];
     __shared__ int rank[LR_MAX_RANK], kept;
-    const int n = *k, tid = threadIdx.x;
-    for (int a = tid; a < r; a += blockDim.x) rs[a] = sqrt(d[a]);
-    if (tid == 0) {
+    const int n = *k, tid = threadIdx.x, lane = tid & 31;
+    if (tid < 32) {                       // the maximum, then the ranks, 32 rows at a time
         double m = 0.0;
-        for (int j = 0; j < n; ++j) m = fmax(m, nrm[j]);
-        smax = m;
+        for (int j = lane; j < n; j += 32) m = fmax(m, nrm[j]);
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, off));
         int c = 0;
-        for (int j = 0; j < n; ++j) rank[j] = nrm[j] > tol * m ? c++ : -1;
-        kept = c;
+        for (int j0 = 0; j0 < n; j0 += 32) {
+            const int j = j0 + lane;
+            const bool in = j < n && nrm[j] > tol * m;
+            const unsigned set = __ballot_sync(0xffffffffu, in);
+            if (j < n) rank[j] = in ? c + __popc(set & ((1u << lane) - 1)) : -1;
+            c += __popc(set);
+        }
+        if (lane == 0) kept = c;
+    } else {
+        for (int a = tid - 32; a < r; a += blockDim.x - 32) rs[a] = sqrt(d[a]);
     }
     __syncthreads();
     for (int e = tid; e < n * r; e += blockDim.x) {
@@ -721,7 +786,7 @@ dme_status launch_jacobi_eig(const double* G, int ldg, int r, double* Vt, int ld
     return DME_OK;
 }
 
-size_t chol_smem(int r) { return sizeof(double) * ((size_t)r * (r + 1) / 2 + 2 * (size_t)r) + sizeof(int) * (size_t)r; }
+size_t chol_smem(int r) { return sizeof(double) * ((size_t)r * (r + 1) / 2 + 3 * (size_t)r) + sizeof(int) * (size_t)r; }
 
 dme_status launch_chol_pivot(const double* G, int ldg, int r, const double* d, double tol, double* R, int ldr, int* k,
                              int* status, cudaStream_t st) {
@@ -749,7 +814,7 @@ dme_status launch_qlp_rows(const double* H, int ldh, int r, const double* R, int
 
 void launch_qlp_select(const double* X, int ldx, const double* nrm, const int* k, int r, double tol, const double* d,
                        double* T, int ldt, double* d_out, int* k_out, cudaStream_t st) {
-    qlp_select_kernel<<<1, 256, 0, st>>>(X, ldx, nrm, k, r, tol, d, T, ldt, d_out, k_out);
+    qlp_select_kernel<<<1, 1024, 0, st>>>(X, ldx, nrm, k, r, tol, d, T, ldt, d_out, k_out);
 }
 
 void launch_lr_select(const double* lam, const double* Vt, int ldv, int r, double tol, int inv_sqrt, double* T,
