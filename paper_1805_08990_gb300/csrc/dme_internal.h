@@ -196,7 +196,7 @@ void launch_spmm(const int* ptr, const int* idx, const double* val, int n, int r
 // (val holds the values of A^T already multiplied by invg = 1/g),
 // stopping after two consecutive terms with |d_k| |w_k|_F <= tol |p|_F (at most
 // `terms` - 1 terms), then v = scale p.  Y may be X.  Wa, Wb: n x r scratch
-// (ldw); part: 4 leja_grid_max() floats; sums: 4 floats; bar: 4 unsigned.
+// (ldw); part: 4 leja_grid_max() floats; bar: 4 unsigned, 8-byte aligned.
 struct LejaCall {
     const int* ptr;
     const int* idx;
@@ -214,8 +214,8 @@ struct LejaCall {
     const double* xi;    // host, `terms` Leja points
     const double* dd;    // host, `terms` divided differences
     double* part;
-    double* sums;
     unsigned* bar;
+    int row_nnz;         // most stored entries in a row of A^T
     int* status;         // DEV_TIMEOUT if a grid barrier wait ran out
 };
 int leja_grid_max();

@@ -62,11 +62,12 @@ struct dme_lr_s {
     int *s_ptr = nullptr, *s_idx = nullptr;   // sparse S (CSR, device), for T4
     double* s_val = nullptr;
     bool asym = false;               // sparse A: exactly symmetric
+    int row_nnz = 0;                 // sparse A: most stored entries in a row of A^T
     double lc = 0.0, lg = 0.0;       // A^T = lc I + lg X, spectrum of X in [-2, 2] (Gershgorin)
     std::vector<double> xi;          // Leja points
     std::vector<LejaTab> ltab;
     double *Wa = nullptr, *Wb = nullptr;   // Leja work (n x rcap)
-    double *lpart = nullptr, *lnorm = nullptr;  // per-block partial norms; norms and grid-barrier words
+    double *lpart = nullptr, *lbar = nullptr;   // per-block partial norms; grid-barrier words
     int n = 0, m = 0, p = 0, rcap = 0, q = 7;
     double tol = 1e-13;
     double *L = nullptr, *L2 = nullptr, *d = nullptr, *d2 = nullptr;   // n x rcap, rcap
@@ -471,8 +472,8 @@ dme_status leja_apply(dme_lr_t lr, const double* X, int ldx, int k, double* Y, i
     c.xi = lr->xi.data();
     c.dd = tb.dd.data();
     c.part = lr->lpart;
-    c.sums = lr->lnorm;
-    c.bar = reinterpret_cast<unsigned*>(lr->lnorm + 4);
+    c.bar = reinterpret_cast<unsigned*>(lr->lbar);
+    c.row_nnz = lr->row_nnz;
     c.status = lr->status;
     DME_TRY(launch_leja_apply(c, st));
     DME_CUDA_TRY(cudaGetLastError());
@@ -944,6 +945,7 @@ dme_status dme_lr_plan_csr(const dme_plan_desc* desc, int nnz, const int* rowptr
         }
         lr->lc = 0.5 * (a + b);
         lr->lg = 0.25 * (b - a);
+        for (int i = 0; i < n; ++i) lr->row_nnz = std::max(lr->row_nnz, tptr[i + 1] - tptr[i]);
         lr->asym = true;
         for (int i = 0; i < n && lr->asym; ++i) {        // rows of A against rows of A^T, in any stored order
             std::vector<std::pair<int, double>> ra, rt;
@@ -1025,7 +1027,7 @@ dme_status dme_lr_plan_csr(const dme_plan_desc* desc, int nnz, const int* rowptr
         DME_TRY(lr_alloc(lr.get(), &lr->Wa, (size_t)n * rc));
         DME_TRY(lr_alloc(lr.get(), &lr->Wb, (size_t)n * rc));
         DME_TRY(lr_alloc(lr.get(), &lr->lpart, 4 * (size_t)leja_grid_max()));
-        DME_TRY(lr_alloc(lr.get(), &lr->lnorm, 8));   // 4 sums, then the barrier words
+        DME_TRY(lr_alloc(lr.get(), &lr->lbar, 2));
         DME_TRY(lr_check(lr.get(), "dme_lr_plan_csr"));
         *out = lr.release();
         return DME_OK;
