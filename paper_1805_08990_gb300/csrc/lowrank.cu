@@ -238,10 +238,11 @@ dme_status compress(dme_lr_t lr, double*& L, double*& L2, double* d, int ld, int
     return DME_OK;
 }
 
-// The same factor with fewer or as many columns as `compress` keeps and up to a few more,
-// for the compressions that another one of the same solve follows: pivoted QLP instead
-// of the eigen-decomposition (launch_chol_pivot), L <- Lt X_k^T, d <- 1.
-dme_status compress_qlp(dme_lr_t lr) {
+// The same factor with as many columns as `compress` keeps and up to a few more, for the
+// compressions that another one of the same solve follows: pivoted QLP instead of the
+// eigen-decomposition (launch_chol_pivot), L <- Lt X_k^T, d <- 1, without the columns
+// whose squared norm is at most `drop` times the largest.
+dme_status compress_qlp(dme_lr_t lr, double drop) {
     int& r = lr->r;
     if (r == 0) return DME_OK;
     cudaStream_t st = lr->st;
@@ -255,7 +256,7 @@ dme_status compress_qlp(dme_lr_t lr) {
     // one Newton-Schulz step: the rows of X orthonormal to rounding
     DME_TRY(gemm(lr, mk(r, r, r, X, rc, 0, X, rc, 1, H, rc, 1.0, 1), st));
     DME_TRY(gemm(lr, mk(r, r, r, H, rc, 0, X, rc, 0, R, rc, -0.5, 0, X, 1.5), st));
-    launch_qlp_select(R, rc, nrm, lr->k0dev, r, lr->tol, lr->d, lr->T, rc, lr->d, lr->kdev, st);
+    launch_qlp_select(R, rc, nrm, lr->k0dev, r, drop, lr->d, lr->T, rc, lr->d, lr->kdev, st);
     int k = 0;
     DME_CUDA_TRY(cudaMemcpyAsync(&k, lr->kdev, sizeof(int), cudaMemcpyDeviceToHost, st));
     DME_CUDA_TRY(cudaStreamSynchronize(st));
@@ -269,7 +270,12 @@ dme_status compress_qlp(dme_lr_t lr) {
 // After an appending flow: `last` for the last compression of a solve, whose factor is the
 // eigen-decomposition of P.
 dme_status compress_state(dme_lr_t lr, bool last) {
-    if (!last) return compress_qlp(lr);
+    if (!last) return compress_qlp(lr, lr->tol);
+    // QLP first, dropping a hundredth of what the eigen-decomposition will: fewer columns
+    // (n = 3600: 122 -> 60) and a graded Gram matrix near its eigenbasis, on which both
+    // Jacobi passes take fewer sweeps (3.27 + 0.71 ms -> 1.07 + 0.3; r = 57: 1.15 + 0.58 ->
+    // 0.75 + 0.30) for 0.2 ms
+    if (lr->r >= 16) DME_TRY(compress_qlp(lr, 0.01 * lr->tol));
     lr->loose = false;
     return compress(lr, lr->L, lr->L2, lr->d, lr->rcap, lr->r);
 }
