@@ -385,123 +385,133 @@ __device__ __forceinline__ double cl_ld_f64(uint32_t a) {
     asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(a) : "memory");
     return v;
 }
-__device__ __forceinline__ int cl_ld_s32(uint32_t a) {
-    int v;
-    asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
-    return v;
-}
 // Every thread of every CTA of the cluster; orders shared-memory writes before it
 // with reads after it, across the cluster.
 __device__ __forceinline__ void cl_sync() {
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
+__device__ __forceinline__ int4 cl_ld_v4(uint32_t a) {
+    int4 v;
+    asm volatile("ld.shared::cluster.v4.b32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+                 : "r"(a)
+                 : "memory");
+    return v;
+}
+
+// A pivot candidate of a column: (high word, low word) of |value| and the row; no candidate:
+// high word -1.  The order is gj_better's, by integer reductions (FP64 compares of a lone
+// warp take about 65 cycles each, and a column's chain had 30).
+__device__ __forceinline__ int4 gjp_candidate(double v, int row) {
+    if ((__double2hiint(v) & 0x7FF00000) == 0x7FF00000 && (__double_as_longlong(v) << 12) != 0) v = 0.0;   // NaN
+    return make_int4(__double2hiint(v) & 0x7FFFFFFF, __double2loint(v), row, 0);
+}
+__device__ __forceinline__ int4 gjp_warp_best(int4 c) {
+    const int hi = __reduce_max_sync(0xffffffffu, c.x);
+    const unsigned lo = __reduce_max_sync(0xffffffffu, c.x == hi ? (unsigned)c.y : 0u);
+    const int row = __reduce_min_sync(0xffffffffu, c.x == hi && (unsigned)c.y == lo ? c.z : 0x7fffffff);
+    return make_int4(hi, (int)lo, row, 0);
+}
+__device__ __forceinline__ int4 gjp_better(int4 a, int4 b) {
+    const bool take = b.x > a.x || (b.x == a.x && ((unsigned)b.y > (unsigned)a.y || (b.y == a.y && b.z < a.z)));
+    return take ? b : a;
+}
+
 // Factor panel [k0, k0 + nbk) of rows 0..n-1: CTA `rank` of the cluster holds rows
-// [rank * rows_per, ...) of the panel in shared memory.  Column c: each CTA's best
-// unused row, one cluster barrier, every CTA reads all candidates and the winning
-// row's entries from its owner (distributed shared memory) and eliminates column c
-// from its own rows with the scaled pivot row; the owner writes the pivot row's
-// scaled entries after the next barrier (other CTAs may still be reading them).
+// [rank * rows_per, ...) of the panel in shared memory.  Column c: each warp's best unused
+// row, one cluster barrier, every CTA reads all candidates and the winning row's entries
+// from its owner (distributed shared memory) and eliminates column c from its own rows
+// with the scaled pivot row, 256 / rows_per threads a row, the first of which forms the
+// row's candidate for the next column; the owner writes the pivot row's scaled entries
+// after the next barrier (other CTAs may still be reading them).
+// Bound: the chain of a column.  As few rows a CTA as eight CTAs allow: an elimination of
+// 128 rows is 1000 cycles of one SM's FP64 pipe (n = 65 .. 350, panels of 32 columns: 60 - 69 us
+// with FP64 compares and 128 rows a CTA, 31 now).
 __global__ void __launch_bounds__(GJ_THREADS) gj_panel_kernel(const GJPanelArgs a) {
     extern __shared__ double sP[];                       // [rows_per][GJP_LD], then used flags
     int* sU = reinterpret_cast<int*>(sP + (size_t)a.rows_per * GJP_LD);
-    __shared__ double s_cv[2];                           // this CTA's candidate, by column parity
-    __shared__ int s_ci[2];
-    __shared__ double s_wv[GJ_WARPS];
-    __shared__ int s_wi[GJ_WARPS];
+    __shared__ int4 s_cand[2][GJ_WARPS];                 // this CTA's candidates, by column parity
     __shared__ double s_raw[GJ_NB];                      // the pivot row's panel entries
     __shared__ double s_sc[GJ_NB];                       // ... scaled right of the pivot
     __shared__ double s_pend[GJ_NB];                     // deferred write of this CTA's last pivot row
-    __shared__ int s_p, s_pend_r, s_pend_c;
+    __shared__ int s_p;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int rank = (int)cl_rank(), ncl = (int)cl_nrank();
     const int n = a.n, nbk = a.nbk, k0 = a.k0;
     const int r0 = rank * a.rows_per;
     const int nr = max(0, min(a.rows_per, n - r0));
+    // span threads over the rows (whole warps), GJ_THREADS / span on a row
+    const int span = a.rows_per <= 32 ? 32 : a.rows_per <= 64 ? 64 : a.rows_per <= 128 ? 128 : 256;
+    const int group = threadIdx.x / span, groups = GJ_THREADS / span, first = threadIdx.x % span;
+    const int cwarps = span / 32;                        // warps that hold candidates (group 0)
     for (int e = threadIdx.x; e < nr * nbk; e += GJ_THREADS) {
         const int r = e / nbk, c = e % nbk;
         sP[r * GJP_LD + c] = __ldcg(a.M + (size_t)(r0 + r) * a.ldm + k0 + c);
     }
     for (int r = threadIdx.x; r < nr; r += GJ_THREADS) sU[r] = __ldcg(a.used + r0 + r);
-    if (threadIdx.x == 0) s_pend_r = -1;
+    int pend_r = -1, pend_c = 0;                         // warp 0
     __syncthreads();
+    if (group == 0) {
+        int4 best = make_int4(-1, 0, 0x7fffffff, 0);
+        for (int r = first; r < nr; r += span)
+            if (!sU[r]) best = gjp_better(best, gjp_candidate(sP[r * GJP_LD], r0 + r));
+        best = gjp_warp_best(best);
+        if (lane == 0) s_cand[0][warp] = best;
+    }
     for (int c = 0; c < nbk; ++c) {
-        double best = -1.0;
-        int bi = n;
-        for (int r = threadIdx.x; r < nr; r += GJ_THREADS) {
-            if (sU[r]) continue;
-            double v = fabs(sP[r * GJP_LD + c]);
-            if (!(v == v)) v = 0.0;                      // NaN: a zero pivot if nothing better
-            if (gj_better(v, r0 + r, best, bi)) {
-                best = v;
-                bi = r0 + r;
-            }
-        }
-        gj_warp_best(best, bi);
-        if (lane == 0) {
-            s_wv[warp] = best;
-            s_wi[warp] = bi;
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            for (int w = 1; w < GJ_WARPS; ++w)
-                if (gj_better(s_wv[w], s_wi[w], best, bi)) {
-                    best = s_wv[w];
-                    bi = s_wi[w];
-                }
-            s_cv[c & 1] = best;
-            s_ci[c & 1] = bi;
-        }
+        __syncwarp();
         cl_sync();
-        // the previous column's pivot row (owned here) takes its scaled entries before
-        // this column eliminates it (no other CTA reads that row any more)
-        if (s_pend_r >= 0 && threadIdx.x < nbk && threadIdx.x >= s_pend_c)
-            sP[s_pend_r * GJP_LD + threadIdx.x] = s_pend[threadIdx.x];
-        __syncthreads();
-        // the pivot over the cluster, then its row's entries from its owner
         if (warp == 0) {
-            double v = -1.0;
-            int p = n;
-            if (lane < ncl) {
-                v = cl_ld_f64(cl_map(&s_cv[c & 1], lane));
-                p = cl_ld_s32(cl_map(&s_ci[c & 1], lane));
-            }
-            gj_warp_best(v, p);
-            const bool singular = !(v > 0.0);
-            if (p >= n) p = n - 1;                       // cannot happen: an unused row remains
+            // the previous column's pivot row (owned here) takes its scaled entries before
+            // this column eliminates it (no other CTA reads that row any more)
+            if (pend_r >= 0 && lane < nbk && lane >= pend_c) sP[pend_r * GJP_LD + lane] = s_pend[lane];
+            // the pivot over the cluster, then its row's entries from its owner
+            int4 best = make_int4(-1, 0, 0x7fffffff, 0);
+            for (int w = lane; w < ncl * cwarps; w += 32)
+                best = gjp_better(best, cl_ld_v4(cl_map(&s_cand[c & 1][w % cwarps], w / cwarps)));
+            best = gjp_warp_best(best);
+            const bool singular = best.x < 0 || (best.x | best.y) == 0;
+            const int p = best.x < 0 ? n - 1 : best.z;   // (an unused row always remains)
             const int owner = p / a.rows_per, pl = p - owner * a.rows_per;
             if (lane < nbk) s_raw[lane] = cl_ld_f64(cl_map(&sP[pl * GJP_LD + lane], owner));
             __syncwarp();
             const double piv = singular ? 0.0 : s_raw[c];
-            const double rp = piv != 0.0 ? 1.0 / piv : 0.0;
-            if (lane < nbk) s_sc[lane] = lane > c ? s_raw[lane] * rp : 0.0;
-            if (owner == rank && lane < nbk) s_pend[lane] = lane > c ? s_raw[lane] * rp : (lane == c ? piv : 0.0);
+            const double rp = singular ? 0.0 : 1.0 / piv;
+            const double sc = lane < nbk && lane > c ? s_raw[lane] * rp : 0.0;
+            if (lane < nbk) s_sc[lane] = sc;
+            pend_r = owner == rank ? pl : -1;
+            pend_c = c;
+            if (pend_r >= 0 && lane < nbk) s_pend[lane] = lane == c ? piv : sc;
             if (lane == 0) {
                 s_p = p;
-                s_pend_r = owner == rank ? pl : -1;
-                s_pend_c = c;
                 if (singular && rank == 0) atomicOr(a.status, DEV_SINGULAR);
                 if (owner == rank) {
                     sU[pl] = 1;
                     a.pr[k0 + c] = p;
                 }
             }
+            __syncwarp();
         }
         __syncthreads();
         // eliminate column c from this CTA's rows other than the pivot row
         const int p = s_p;
-        for (int r = threadIdx.x; r < nr; r += GJ_THREADS) {
-            if (r0 + r == p) continue;
+        int4 best = make_int4(-1, 0, 0x7fffffff, 0);
+        for (int r = first; r < nr; r += span) {
             double* row = sP + r * GJP_LD;
             const double f = row[c];
-            if (f == 0.0) continue;
-            for (int c2 = c + 1; c2 < nbk; ++c2) row[c2] = fma(-f, s_sc[c2], row[c2]);
+            if (r0 + r != p && (__double_as_longlong(f) << 1) != 0)
+                for (int c2 = c + 1 + group; c2 < nbk; c2 += groups) row[c2] = fma(-f, s_sc[c2], row[c2]);
+            if (group == 0 && c + 1 < nbk && !sU[r]) best = gjp_better(best, gjp_candidate(row[c + 1], r0 + r));
         }
-        __syncthreads();
+        if (group == 0 && c + 1 < nbk) {
+            best = gjp_warp_best(best);
+            if (lane == 0) s_cand[(c + 1) & 1][warp] = best;
+        }
     }
+    __syncwarp();
     cl_sync();                                           // nobody reads this CTA's rows any more
-    if (s_pend_r >= 0 && threadIdx.x < nbk && threadIdx.x >= s_pend_c)
-        sP[s_pend_r * GJP_LD + threadIdx.x] = s_pend[threadIdx.x];
+    if (warp == 0 && pend_r >= 0 && lane < nbk && lane >= pend_c) sP[pend_r * GJP_LD + lane] = s_pend[lane];
     __syncthreads();
     for (int e = threadIdx.x; e < nr * nbk; e += GJ_THREADS) {
         const int r = e / nbk, c = e % nbk;
@@ -704,7 +714,7 @@ size_t gj_work_doubles(int n, int nrhs) {
 // update; finally the gather of the solution rows.
 static dme_status gj_solve_panels(double* M, int n, int ldm, double* B, int nrhs, int ldb, double* V, int* used,
                                   int* pr, double* X, int* status, cudaStream_t st) {
-    const int cl = std::max(1, std::min(8, (n + 127) / 128));
+    const int cl = std::max(1, std::min(8, (n + 31) / 32));
     const int rows_per = (n + cl - 1) / cl;
     const size_t smem = (size_t)rows_per * GJP_LD * sizeof(double) + (size_t)rows_per * sizeof(int);
     static const cudaError_t attr = cudaFuncSetAttribute(
