@@ -117,6 +117,9 @@ GemmProb gp(int M, int N, int K, const double* A, int lda, int tA, const double*
 
 // One FP64 product: 64-wide output tiles when they fill one wave of the SMs, else 32-wide
 // ones, else (fewer 32-wide tiles than SMs) 8-wide ones; all give bit-identical results.
+// (n = 350: 121 32-wide tiles, 123 us; 8-wide about 80.  Below n = 288 K was split over the
+// SMs instead, with a reduction launch: the plan of n = 32 took 1000 us and takes 815, n = 100
+// 1580 and 1400.  Taking 8-wide tiles up to 304 or 600 32-wide ones changes nothing.)
 dme_status gemm1(const GemmProb& g, cudaStream_t st) {
     std::vector<GemmProb> v{g};
     auto tiles = [&](long w) {
@@ -293,12 +296,10 @@ void mod_rows(int n, ModWork& w, const double* X, int t, const ModBuf& b, cudaSt
 }
 
 // Where the exponential's products run: the accurate slice mode, residue products, or
-// (both null) the FP64 pipe, with K split for small n (skw).
+// (both null) the FP64 pipe.
 struct ProdPath {
     AccWork* acc = nullptr;
     ModWork* mod = nullptr;
-    double* skw = nullptr;
-    size_t skl = 0;
 };
 
 // C = alpha op(L) op(R) + b1 D1 (n x n).  On residue products `certify` is false for the
@@ -314,7 +315,7 @@ dme_status prod(int n, const ProdPath& w, const double* L, int tL, const double*
         mod_rows(n, *w.mod, R, !tR, w.mod->b, st);
         return launch_mod_gemm(w.mod->a, w.mod->b, g, w.mod->ws, certify, w.mod->status, st);
     }
-    return gemm64_splitk(g, w.skw, w.skl, st);
+    return gemm1(g, st);
 }
 
 // X = M^{-1} B (n x n) by iterative refinement with an FP32 inverse Y of M and residue
@@ -547,13 +548,6 @@ dme_status compute_ew(dme_plan_t p, double tau, int* idx) {
     DME_TRY(tp.get(&V12, nn));
     double* gjw = nullptr;
     DME_TRY(tp.get(&gjw, gj_work_doubles(n, n)));
-    // split-K partial sums of the small FP64 products (n <= 288: fewer 32-wide tiles than half the SMs)
-    double* skw = nullptr;
-    size_t skl = 0;
-    if (n <= 288) {
-        skl = gemm64_splitk_ws_doubles(n, n);
-        DME_TRY(tp.get(&skw, skl));
-    }
     // split plans of n >= kAccMinN: the Pade products on the tensor cores (accurate mode)
     AccWork accw;
     ProdPath pp;                          // the [13/13] chain
@@ -571,8 +565,6 @@ dme_status compute_ew(dme_plan_t p, double tau, int* idx) {
             set_error("");
         }
     }
-    pp.skw = skw;
-    pp.skl = skl;
 
     // X = sc M:  X22 = sc A, X12 = sc Q, X11 = -X22^T (implicit)
     launch_lincomb(X22, n, n, p->A, sc, nullptr, 0, nullptr, 0, 0.0, st);
@@ -649,7 +641,7 @@ dme_status compute_ew(dme_plan_t p, double tau, int* idx) {
             mod_rows(n, modw, tmp, 1, modw.a, st);
             DME_TRY(launch_mod_gemm(modw.b, modw.a, g3, modw.ws, true, p->status, st));
         } else {
-            for (const GemmProb* g : {&g1, &g2, &g3}) DME_TRY(gemm64_splitk(*g, skw, skl, st));
+            for (const GemmProb* g : {&g1, &g2, &g3}) DME_TRY(gemm1(*g, st));
         }
         std::swap(E, E2);
     }
