@@ -50,7 +50,11 @@ typedef enum { DME_DLE = 0, DME_DRE = 1, DME_GDLE = 2, DME_GDRE = 3 } dme_eq;
 /* sub-flows T1, T2, T12, T3, T4 of §2 */
 typedef enum { DME_F1 = 1, DME_F2 = 2, DME_F12 = 3, DME_F3 = 4, DME_F4 = 5 } dme_flow;
 typedef enum { DME_LIE = 1, DME_STRANG = 2 } dme_comp;
-/* DME_FP64: every product in float64 on the FP64 pipe.
+/* DME_FP64: every product to float64 accuracy.  From n = 192 the n x n products
+ *   of the steps and of the exponential are exact residue products of integer
+ *   rows on the tensor cores, rounded once, each entry certified to the error
+ *   bound of a float64 sum (K u sum |a b|) or recomputed as one; smaller ones,
+ *   served requests and the rest run on the FP64 pipe.
  * DME_SPLIT_TF32: reserved; not built.  A TF32 slice carries an 11-bit digit,
  *   so the fp32 tensor-core sum of K products of two such digits is exact
  *   only for K <= 4; plans asking for it fail with DME_EINVAL and say so in
@@ -100,7 +104,10 @@ typedef struct dme_server_s* dme_server_t;
  * and, for every step length t the scheme uses in T1/T12, E_t = e^{tA} and
  * W_t (Eq. full) by [13/13] Pade scaling and squaring of the Van Loan matrix
  * t[[-A^T, Q],[0, A]] (its 1-norm sets the squarings; the exponential is
- * built from its n x n blocks, see dme_expm).
+ * built from its n x n blocks, see dme_expm).  From n = 192 on a balanced A (row
+ * and column sums within 2^8 of one another) the denominator systems are solved
+ * by iterative refinement from a float32 inverse, with exact residuals; any other,
+ * and one whose corrections do not shrink, by Gauss-Jordan elimination.
  *   A: n x n.  QorC: n x n or p x n.  B: n x m (NULL unless DRE/GDRE).
  *   R: m x m SPD (NULL unless DRE/GDRE).  S: n x n (NULL unless GDLE/GDRE).
  *   cuda_stream: a cudaStream_t, or NULL for a plan-owned stream.
@@ -217,11 +224,13 @@ dme_status dme_plan_destroy(dme_plan_t plan);
  * The state is kept as P = L diag(d) L^T (L n x r, d > 0) and never formed
  * during the steps: T1 maps L to E_t^T L, T2 appends C^T with weights t,
  * T12 maps L and appends the compressed Gauss-Legendre factor of W_t (Alg. 2),
- * T3 updates the factor through an m x m eigenproblem ((I + t D L^T B R^-1 B^T L)^-1 D
+ * T3 updates the factor through an m x m Cholesky root ((I + t D L^T B R^-1 B^T L)^-1 D
  * of §2.2 in square-root form), T4 appends sqrt(t) S L and sqrt(t/2) S (sqrt(t) S L)
  * (midpoint) or sqrt(t) S L (Euler).  After every flow that appends columns the
- * factor is compressed: the eigen-decomposition of P on the span of L (a Gram
- * matrix and a Jacobi eigensolver), keeping eigenvalues > tol * max.  E_t is
+ * factor is compressed: by a pivoted QLP factorisation that drops what is below
+ * tol * max within a solve, and at its end (or where the capacity asks for it) to
+ * the eigen-decomposition of P on the span of L (a Gram matrix and a Jacobi
+ * eigensolver), keeping eigenvalues > tol * max.  E_t is
  * the dense exponential of the plan (n <= 16384; n <= 4096 with DME_SPLIT_BF16,
  * which runs the products with E_t and S on the tensor cores and the rest in
  * FP64).  P0 must be PSD. */
@@ -244,9 +253,9 @@ dme_status dme_lr_plan(const dme_plan_desc* desc, const double* A, const double*
  * (p x n) and, for a DRE / GDRE, B and R as in dme_plan.  e^{t A^T} L is applied by
  * Newton interpolation at Leja points (the action the paper computes with
  * `expleja`, §3): a Gershgorin interval [a, b] of A^T, A^T = c I + g X with
- * X's spectrum in [-2, 2], substeps of length t with t g <= 4, at most 80
+ * X's spectrum in [-2, 2], substeps of length t with t g <= 4 (10 for a symmetric A), at most 80
  * Leja points per substep, and the series stopped after two terms below
- * 1e-15 times the partial sum (Frobenius norms).  For GDLE / GDRE, S (of the
+ * 1e-15 times the partial sum (Frobenius norms; one more term is added).  For GDLE / GDRE, S (of the
  * S P S^T term, Eq. lyapGen; n x n) is given in CSR too (nnz_s, s_rowptr,
  * s_colidx, s_vals, same conventions and checks; ignored for DLE / DRE) and
  * T4 forms S L and S^2 L by a sparse product (§2.3).  desc: q_is_factor = 1,

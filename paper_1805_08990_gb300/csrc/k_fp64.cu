@@ -1,12 +1,11 @@
-// FP64 kernels of libdme: grouped GEMM with a symmetric-triangle mode and a
-// fused additive epilogue, the elementwise helpers of the plan step, dense LU
-// with partial pivoting and its triangular sweeps, and the small m x m
-// Cholesky used for R.
+// FP64-pipe kernels of libdme: grouped GEMM with a symmetric-triangle mode and
+// a fused additive epilogue (32- and 64-wide tiles), 8-wide tiles for products
+// of fewer tiles than SMs, the elementwise helpers of the plan step, and the
+// small m x m Cholesky used for R.
 //
-// GB300 executes FP64 on a narrow pipe (about 1.25 TFLOP/s for the whole
-// chip), so these kernels are ALU-bound: the GEMM keeps a 4 x 4 register
-// tile per thread fed from shared memory and spends its effort on coalesced
-// tile loads, not on latency hiding.
+// GB300 executes FP64 on a narrow pipe (about 1.25 TFLOP/s for the whole chip,
+// two FMAs a cycle and SM), so these kernels are ALU-bound and what counts is
+// that every SM has its share.
 #include "dme_internal.h"
 #include "gemm64_tile.cuh"
 #include "pdl.cuh"

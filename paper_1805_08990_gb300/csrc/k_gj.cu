@@ -426,7 +426,7 @@ __device__ __forceinline__ int4 gjp_better(int4 a, int4 b) {
 // row's candidate for the next column; the owner writes the pivot row's scaled entries
 // after the next barrier (other CTAs may still be reading them).
 // Bound: the chain of a column.  As few rows a CTA as eight CTAs allow: an elimination of
-// 128 rows is 1000 cycles of one SM's FP64 pipe (n = 65 .. 350, panels of 32 columns: 60 - 69 us
+// 128 rows is 1000 cycles of one SM's FP64 pipe (n = 65 .. 350, panels of 16 columns: 60 - 69 us
 // with FP64 compares and 128 rows a CTA, 31 now).
 __global__ void __launch_bounds__(GJ_THREADS) gj_panel_kernel(const GJPanelArgs a) {
     extern __shared__ double sP[];                       // [rows_per][GJP_LD], then used flags

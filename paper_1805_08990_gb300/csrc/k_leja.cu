@@ -19,7 +19,8 @@
 //    while every thread has at most two entries;
 //  - the norms are formed in fp32 from the top bits of the entries: in FP64 the shuffles
 //    and block sums alone were 830 FP64 warp instructions per SM and term.
-// (n = 3600, r = 56: LEJA_FIG.)
+// (n = 3600, r = 18 .. 60, 82 terms: 790 us an action with the terms in global memory and the last
+// arriving block summing the norms, 395 now.)
 #include "dme_internal.h"
 
 #include <algorithm>

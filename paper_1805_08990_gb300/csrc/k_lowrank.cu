@@ -1,9 +1,9 @@
-// Kernels of the low-rank (LDL^T) path: a one-CTA parallel Jacobi
-// eigensolver for the small symmetric systems of the column compression and
-// of the factored Riccati flow, the eigenvalue selection that builds the
-// compressed basis, and column scaling / copying helpers.
+// Kernels of the low-rank (LDL^T) path: the pivoted QLP factorisation of the
+// compressions within a solve, a one-CTA parallel Jacobi eigensolver for the
+// last one, the selections that build the compressed basis, the m x m root of
+// the factored Riccati flow, and column scaling / copying helpers.
 //
-// The compression only needs the eigen-decomposition of an r x r Gram matrix
+// The last compression needs the eigen-decomposition of an r x r Gram matrix
 // (r <= 224), so one CTA holds its upper triangle packed in shared memory and
 // applies r/2 disjoint rotations per sub-sweep (round-robin pairing); the
 // eigenvector matrix is accumulated transposed (rows p, q of V^T change per

@@ -298,7 +298,8 @@ struct ModGemmArgs {
 // MMA in a 128 x 128 tile, 512 in a pair's, and loads came back 3900 cycles after they were
 // issued at K = 2048 (six stages of the former: 690 cycles per K block; 128 x 256 tiles in
 // clusters of four with a multicast B, four stages of 48 KB: 970 per 512 of MMA; pairs,
-// seven stages: 860, and 800 with no load at all, where cuBLAS runs at 640).
+// seven stages: 860 with the MMAs issued by one diverged lane, 700 from uniform registers, where
+// cuBLAS runs at 640).
 template <int BN_, bool PAIR_>
 struct ModCfg {
     static constexpr int BN = BN_, CL = PAIR_ ? 2 : 1;
@@ -884,7 +885,7 @@ dme_status launch_mod_gemm(const ModBuf& A, const ModBuf& B, const GemmProb& g, 
                       : (mod_gemm_launch<64, false, false>(A.t128, B.t64, a, mod_sms(), st)));
     } else {
         // the shape with the shorter run: waves x measured cycles per K block of 64 (pairs:
-        // 860 in the steady state, less by what the first and last waves overlap).  Below
+        // 600 to 700, less the longer the run; the smaller tile 690).  Below
         // K = 512 a unit is all latency and the smaller tile is faster (n = 256: 8.4 us
         // against 12.1)
         const int np = mod_pairs();

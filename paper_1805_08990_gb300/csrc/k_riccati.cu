@@ -6,9 +6,10 @@
 // which only needs the small SPD matrix M = I_m + t Bt^T P Bt (the dense
 // counterpart of the r x r solve of §2.2).  With M = L L^T and Y = Z L^{-T}:
 //     T3(t) P = P - t Y Y^T.
-// Four kernels: (1) Z = P Bt with per-block partial Gram sums Bt^T Z,
-// (2) M from the partials (deterministic reduction order), its Cholesky and
-// L^{-1} (FP64), (3) Y = Z L^{-T}, (4) the rank-m update P <- P - t Y Y^T (+ q Q).
+// Kernels: (1) Z = P Bt with per-block partial Gram sums Bt^T Z, (2) M from the
+// partials (deterministic reduction order), its Cholesky and L^{-1} (FP64; in
+// registers for m <= 8), (3) Y = Z L^{-T}, (4) the rank-m update
+// P <- P - t Y Y^T (+ q Q); for m <= 8 (4) forms the rows of Y it needs by itself.
 // Each kernel takes a batch of independent problems (grouped launch): the
 // blocks of every problem are laid end to end and each block finds its
 // problem by a binary search over the per-problem block offsets, so a

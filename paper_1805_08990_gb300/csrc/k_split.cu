@@ -15,12 +15,13 @@
 // epilogue combines the levels as a two-float (hi = level 0, lo = the rest)
 // and scales by sigma_A,i sigma_B,j.
 //
-// Kernel shape: persistent, one CTA per SM, 10 warps, 128 x 128 output tiles:
+// Kernel shape: persistent, one CTA per SM, 10 warps, 128 x 128 output tiles (128 x 64 or
+// 128 x 32, with 64 K a stage, for products of fewer tiles than SMs):
 //   warp 0  TMA producer (one thread): a ring of STAGES stages, each holding
 //           the SA slices of a 128 x 32 A tile and the SB slices of a 128 x 32
 //           B tile (64-byte swizzled rows; one 3-D box per operand and stage,
 //           {32 k, 128 rows, planes}, the planes 8 KB apart),
-//   warp 1  TMEM allocator + MMA issuer (one thread): 2 x pairs tcgen05.mma
+//   warp 1  TMEM allocator + MMA issuer (one elected lane): 2 x pairs tcgen05.mma
 //           per stage into the four accumulators (512 TMEM columns),
 //   warps 2-9 epilogue, two warps per TMEM lane quadrant, each on 64 columns:
 //           they copy the accumulators into registers and release TMEM at
@@ -46,7 +47,6 @@ namespace dme {
 using namespace tc;
 
 constexpr int OZ_BM = 128, OZ_BN = 128, OZ_BK = 32;
-constexpr int OZ_SLICE_BYTES = OZ_BM * OZ_BK * 2;                 // 8 KB per slice tile
 constexpr uint64_t OZ_TIMEOUT_NS = 2000000000ull;                 // 2 s per wait
 constexpr int OZ_EPI_WARPS = 8;                                  // two per TMEM lane quadrant
 constexpr int OZ_THREADS = 64 + 32 * OZ_EPI_WARPS;               // producer + MMA warps + epilogue

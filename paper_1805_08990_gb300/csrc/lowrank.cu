@@ -13,7 +13,9 @@
 //            L (I + t D L^T B R^{-1} B^T L)^{-1} D L^T by the push-through identity
 //   T_4(t):  L <- [L, sqrt(t) S L, sqrt(t/2) S (sqrt(t) S L)], d <- [d, d, d] (midpoint)
 //            or [L, sqrt(t) S L], [d, d] (Euler), then compression
-//   compression: Lt = L diag(d)^{1/2}; Lt^T Lt = V Lambda V^T (Jacobi);
+//   compression, within a solve: Lt = L diag(d)^{1/2}, L <- Lt X_k^T with the orthonormal
+//            rows X of a pivoted QLP factorisation of Lt^T Lt, d <- 1;
+//   compression, last of a solve: Lt^T Lt = V Lambda V^T (Jacobi);
 //            L <- Lt V_k Lambda_k^{-1/2}, d <- lambda_k for lambda > tol * max lambda,
 //            i.e. the eigen-decomposition of P restricted to its numerical range
 //            (the paper's reduced SVD followed by the small diagonalisation).

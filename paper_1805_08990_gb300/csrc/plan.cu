@@ -11,8 +11,8 @@
 //    (X11 = -X22^T, so an even power has (1,1) = (2,2)^T and an odd one
 //    (1,1) = -(2,2)^T); a product therefore costs three n x n GEMMs;
 //  * the Pade denominator q = V - U has q11 = p22^T, so q R = p splits into
-//    R22 = q22^{-1} p22 and R12 = p22^{-T} (p12 - q12 R22): two n x n LU
-//    solves in FP64;
+//    R22 = q22^{-1} p22 and R12 = p22^{-T} (p12 - q12 R22): two n x n solves to
+//    FP64 rounding (refined from an FP32 inverse, or Gauss-Jordan elimination);
 //  * squaring the block matrix is the semigroup law of T12 (Eq. full):
 //    E_{2t} = E_t^2, W_{2t} = W_t + E_t^T W_t E_t.
 #include "plan_internal.h"

@@ -195,3 +195,31 @@ def test_leja_action_of_large_blocks_matches_sine_transform(n, k):
     EL = scipy.fft.idst(np.exp(lam)[:, None] * scipy.fft.dst(L0, 1, axis=0, norm="ortho"), 1, axis=0, norm="ortho")
     X = np.random.default_rng(1).standard_normal((n, 4))
     assert np.linalg.norm(P @ X - EL @ (EL.T @ X)) <= 3e-12 * np.linalg.norm(L0, 2) ** 2 * np.linalg.norm(X)
+
+
+# a symmetric A is recognised in any stored order, and one that only its values make
+# unsymmetric is not; entries stored twice are added either way
+@pytest.mark.parametrize("form", ["sorted", "reversed", "twice", "perturbed"])
+def test_leja_action_of_stored_orders(form):
+    n, k, t = 130, 6, 25.0
+    off = np.ones(n - 1)
+    A = sp.csr_matrix(sp.diags([off, -2.0 * np.ones(n), off], [-1, 0, 1])) * t
+    if form == "perturbed":
+        A[3, 4] = 0.5 * t
+    cols = [list(A.indices[A.indptr[i]:A.indptr[i + 1]]) for i in range(n)]
+    vals = [list(A.data[A.indptr[i]:A.indptr[i + 1]]) for i in range(n)]
+    if form == "reversed":
+        cols, vals = [c[::-1] for c in cols], [v[::-1] for v in vals]
+    if form == "twice":
+        cols, vals = [c + c[:1] for c in cols], [[0.5 * v[0]] + v[1:] + [0.5 * v[0]] for v in vals]
+
+    class Csr:
+        shape = (n, n)
+        indptr = np.concatenate([[0], np.cumsum([len(c) for c in cols])]).astype(np.int32)
+        indices = np.concatenate(cols).astype(np.int32)
+        data = np.concatenate(vals).astype(np.float64)
+
+    L0 = np.random.default_rng(2).standard_normal((n, k))
+    P = _t1(Csr(), L0, 1.0)
+    EL = scipy.linalg.expm(A.T.toarray()) @ L0
+    assert np.linalg.norm(P - EL @ EL.T) <= 3e-12 * np.linalg.norm(L0 @ L0.T, 2) * np.sqrt(n)
