@@ -469,7 +469,14 @@ dme_status split_cong(dme_plan_t p, const double* P, const SliceBuf& G, double* 
     return launch_ozaki_gemm(G, p->usl, b, st);
 }
 
-// T3 on the split path for n > 1536: Z^T = Bt^T P (P symmetric) on the tensor
+// Whether T3 of a split plan runs its products on the tensor cores.  That costs a slicing
+// of P whatever m is, the FP64 kernels 3 n^2 m flops (us, tensor / FP64: n = 1600, m = 1 86 / 31,
+// m = 4 93 / 63, m = 8 104 / 120; n = 2025, m = 4 105 / 95, m = 6 109 / 150; n = 3600, m = 4
+// 217 / 216; n = 4096, m = 2 260 / 187, m = 4 266 / 286, m = 8 281 / 620).  Below 1537 serving,
+// which uses the FP64 kernels, stays bit-identical to single plans.
+bool tensor_riccati(int n, int m) { return n > 1536 && (m > 4 || (m == 4 && n > 3600)); }
+
+// T3 on the split path (tensor_riccati): Z^T = Bt^T P (P symmetric) on the tensor
 // cores (Bt^T with 5 slices as the fixed operand, P with 4), then the m x m
 // part in FP64 (Gram partials, M = I + t Bt^T Z, Cholesky, Y = Z L^{-T}), then
 // P <- P - t Y Y^T (+ q Q) as a triangle tensor GEMM with K = m and the FP64
@@ -1339,19 +1346,15 @@ dme_status dme::plan_create(const dme_plan_desc* d, const double* A, const doubl
             DME_TRY(palloc_t(p, &p->kcnt, (size_t)OZ_SPLIT_MAX_TAIL));
             DME_CUDA_TRY(cudaMemsetAsync(p->kcnt, 0, sizeof(int) * OZ_SPLIT_MAX_TAIL, st));
         }
-        if (n > 1536) {
-            if (ric) {
-                // the Riccati products on the tensor cores (below 1537 the FP64 kernels are
-                // cheap, and serving, which uses them, stays bit-identical to single plans)
-                const int m = p->m;
-                p->tric = true;
-                DME_TRY(palloc_t(p, &p->Zt, (size_t)m * n));
-                DME_TRY(alloc_slices(p, &p->btsl, m, n, OZ_SLICES_FIXED));
-                DME_TRY(alloc_slices(p, &p->ysla, n, m, OZ_SLICES_FIXED));
-                DME_TRY(alloc_slices(p, &p->yslb, n, m, OZ_SLICES_STEP));
-                launch_transpose(p->Bt, p->Zt, n, m, m, n, st);
-                launch_slice_rows_f64(p->Zt, m, n, n, p->btsl, st);
-            }
+        if (ric && tensor_riccati(n, p->m)) {
+            const int m = p->m;
+            p->tric = true;
+            DME_TRY(palloc_t(p, &p->Zt, (size_t)m * n));
+            DME_TRY(alloc_slices(p, &p->btsl, m, n, OZ_SLICES_FIXED));
+            DME_TRY(alloc_slices(p, &p->ysla, n, m, OZ_SLICES_FIXED));
+            DME_TRY(alloc_slices(p, &p->yslb, n, m, OZ_SLICES_STEP));
+            launch_transpose(p->Bt, p->Zt, n, m, m, n, st);
+            launch_slice_rows_f64(p->Zt, m, n, n, p->btsl, st);
         }
         if (gen) {
             DME_TRY(alloc_slices(p, &p->Ssl, n, n, OZ_SLICES_FIXED));

@@ -60,6 +60,26 @@ def test_riccati_flow_matches_oracle(n, m):
     assert torch.equal(P, P.T)
 
 
+# T3 of split plans: FP64 kernels or tensor products, by n and m
+@pytest.mark.parametrize("n,m", [(1536, 5), (1537, 3), (1537, 4), (1537, 5), (1601, 9), (3600, 4), (3601, 4)])
+def test_riccati_flow_of_split_plans_matches_formula(n, m):
+    g = torch.Generator(device="cuda")
+    g.manual_seed(n + m)
+    B = torch.randn(n, m, generator=g, dtype=torch.float64, device="cuda")
+    R = torch.diag(0.5 + torch.rand(m, generator=g, dtype=torch.float64, device="cuda"))
+    G = torch.randn(n, 8, generator=g, dtype=torch.float64, device="cuda")
+    P0 = G @ G.T / n
+    plan = dme.Plan(-torch.eye(n, dtype=torch.float64, device="cuda"),
+                    C=torch.ones(1, n, dtype=torch.float64, device="cuda"), h=0.1, flows=["F3"], comp="lie", B=B, R=R,
+                    prec="split_bf16")
+    P = P0.clone()
+    plan.apply("F3", 0.1, P)
+    Z = P0 @ B
+    ref = P0 - 0.1 * Z @ torch.linalg.solve(R + 0.1 * B.T @ Z, Z.T)
+    assert (torch.linalg.norm(P - ref) / torch.linalg.norm(ref)).item() < SPLIT_TOL
+    assert torch.equal(P, P.T)
+
+
 # split-precision products in 128, 64 and 32 wide tiles (the width follows from the number of
 # tiles), whole and cut at the right and lower edges, odd and even multiples of 32 along K
 @pytest.mark.parametrize("pairs", [10, 13, 14])
