@@ -69,10 +69,12 @@ def test_riccati_flow_of_split_plans_matches_formula(n, m):
     R = torch.diag(0.5 + torch.rand(m, generator=g, dtype=torch.float64, device="cuda"))
     G = torch.randn(n, 8, generator=g, dtype=torch.float64, device="cuda")
     P0 = G @ G.T / n
-    plan = dme.Plan(-torch.eye(n, dtype=torch.float64, device="cuda"),
-                    C=torch.ones(1, n, dtype=torch.float64, device="cuda"), h=0.1, flows=["F3"], comp="lie", B=B, R=R,
+    A, C = -torch.eye(n, dtype=torch.float64, device="cuda"), torch.ones(1, n, dtype=torch.float64, device="cuda")
+    torch.cuda.synchronize()                     # the plan works on a stream of its own
+    plan = dme.Plan(A, C=C, h=0.1, flows=["F3"], comp="lie", B=B, R=R,
                     prec="split_bf16")
     P = P0.clone()
+    torch.cuda.synchronize()
     plan.apply("F3", 0.1, P)
     Z = P0 @ B
     ref = P0 - 0.1 * Z @ torch.linalg.solve(R + 0.1 * B.T @ Z, Z.T)
@@ -153,7 +155,7 @@ def test_factored_ranks_match_dense_schemes(p, m, prec, tol):
     plan.solve(0.1, 5, P_out=P)
     full = dme.Plan(dev(A), C=dev(C), h=0.02, flows=flows, B=dev(B), R=dev(R))
     ref = torch.empty(n, n, dtype=torch.float64, device="cuda")
-    full.solve(torch.zeros_like(ref), 0.1, 5, ref)
+    full.solve(np.zeros((n, n)), 0.1, 5, ref)
     assert rel(P, host(ref)) < tol
 
 
