@@ -62,8 +62,8 @@ typedef enum { DME_LIE = 1, DME_STRANG = 2 } dme_comp;
  * DME_SPLIT_BF16: congruences (T1, T12, T4) as error-free bf16 slice products
  *   on tcgen05 tensor cores accumulated in fp32, exactly for the leading
  *   level (Ozaki splitting), combined in fp64; n <= 4096.  The Riccati m x m
- *   solve, the Pade denominator solve and the squarings of the exponential
- *   stay fp64. */
+ *   solve (and all of T3 up to m = 4), the Pade denominator solve and the
+ *   squarings of the exponential keep float64 accuracy. */
 typedef enum { DME_FP64 = 0, DME_SPLIT_TF32 = 1, DME_SPLIT_BF16 = 2 } dme_prec;
 /* T4 rule; AUTO = midpoint for Strang, explicit Euler for Lie (§2.3). */
 typedef enum { DME_T4_AUTO = 0, DME_T4_MIDPOINT = 1, DME_T4_EULER = 2 } dme_t4_rule;
@@ -126,7 +126,8 @@ typedef struct dme_server_s* dme_server_t;
  * dme_plan_split_probe report the choice and its inputs.  Above n = 511 the
  * Pade products of the exponential run on the tensor cores too, in an
  * accurate mode (21 slice products with the exact sums of 512-wide K chunks
- * combined in fp64); the denominator solves and the squarings stay FP64.
+ * combined in fp64); the denominator solves and the squarings keep float64
+ * accuracy.
  * Errors: DME_EINVAL (inconsistent desc), DME_ENOTSPD (R), DME_ENOMEM,
  * DME_ECUDA.  On error *out is NULL. */
 dme_status dme_plan(const dme_plan_desc* desc, const double* A, const double* QorC,
