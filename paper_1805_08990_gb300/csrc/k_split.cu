@@ -768,14 +768,6 @@ __device__ __forceinline__ void oz_store_chunk_half(const OzParams& p, uint32_t 
     }
 }
 
-// L2 prefetch of the whole 16-byte units of x[0 .. len) (rows of an odd leading dimension
-// start between them).
-__device__ __forceinline__ void oz_prefetch_row(const double* x, int len) {
-    const uintptr_t a = (reinterpret_cast<uintptr_t>(x) + 15) & ~uintptr_t(15);
-    const uintptr_t e = reinterpret_cast<uintptr_t>(x + len) & ~uintptr_t(15);
-    if (len > 0 && e > a) prefetch_l2_bulk(reinterpret_cast<const void*>(a), (uint32_t)(e - a));
-}
-
 // The persistent loop.  Every role walks the same unit sequence
 // u = blockIdx.x, blockIdx.x + gridDim.x, ...; `resolve(u, unit)` maps a unit
 // index to its problem, tile and K range.
@@ -849,20 +841,21 @@ __device__ __forceinline__ void oz_persistent(int units, Resolve resolve) {
                     issued |= 1u << s;
                     last_ph = (last_ph & ~(1u << s)) | (ph << s);
                     // pull the epilogue's addend rows into L2: spread over the K loop, and all
-                    // of them at the last k block of a short one (the 16-byte units inside a
-                    // row's segment; transposed for tri outputs)
-                    if (!Cfg::ACC && p.mode == OZ_OUT_F64 && (p.D1 || p.D2)) {
+                    // of them at the last k block of a short one (full 128-column segments
+                    // only, 16-byte aligned; transposed for tri outputs)
+                    if (!Cfg::ACC && p.mode == OZ_OUT_F64 && (p.ldc % 2) == 0 && (p.D1 || p.D2)) {
                         // rows of the addend tile (transposed for tri outputs) and their length
                         const int nr = p.tri ? Cfg::BN : OZ_BM, seg = p.tri ? OZ_BM : Cfg::BN;
                         const int r0 = it, r1 = (it == w.nk - 1) ? nr : min(it + 1, nr);
                         for (int rr = r0; rr < r1; ++rr) {
                             const int ra = (p.tri ? n0 : m0) + rr, ca = p.tri ? m0 : n0;
                             const int rmax = p.tri ? p.N : p.M, cmax = p.tri ? p.M : p.N;
-                            if (ra >= rmax) break;
+                            if (ra >= rmax || ca + seg > cmax) continue;
                             const size_t off = (size_t)ra * p.ldc + ca;
-                            const int len = min(seg, cmax - ca);
-                            if (p.D1) oz_prefetch_row(p.D1 + off, len);
-                            if (p.D2) oz_prefetch_row(p.D2 + off, len);
+                            if (p.D1 && ((reinterpret_cast<uintptr_t>(p.D1 + off) & 15) == 0))
+                                prefetch_l2_bulk(p.D1 + off, seg * sizeof(double));
+                            if (p.D2 && ((reinterpret_cast<uintptr_t>(p.D2 + off) & 15) == 0))
+                                prefetch_l2_bulk(p.D2 + off, seg * sizeof(double));
                         }
                     }
                 }
