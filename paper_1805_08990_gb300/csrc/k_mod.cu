@@ -46,7 +46,6 @@ namespace {
 using u128 = unsigned __int128;
 
 // ------------------------------------------------------------------ constants
-constexpr int kModuli[MOD_NM] = {256, 255, 253, 251, 247, 241, 239, 233, 229, 227, 223, 217, 211, 199, 197, 193};
 constexpr int MOD_NORM = 61;                  // log2 of a row's largest 2-norm in integer units
 constexpr int MOD_MAX_EXP = 400;              // rows with larger exponents (of either sign) go to FP64
 constexpr int MOD_CHUNK = 1024;               // K per exact fp32 sum
@@ -105,6 +104,14 @@ constexpr ModConst make_mod_const() {
 
 __constant__ ModConst c_mod = make_mod_const();
 static_assert(mod_product() >> 125 != 0 && mod_product() >> 126 == 0, "2^122 < P / 8: the quotient is never ambiguous");
+
+// The bytes of an odd modulus hold every residue that mod_centred returns: p (1/2 + 2^-8) < 128.
+constexpr bool mod_residues_fit() {
+    for (int m = 1; m < MOD_NM; ++m)
+        if (kModuli[m] * 129 >= 128 * 256) return false;
+    return kModuli[0] == 256;
+}
+static_assert(mod_residues_fit(), "a residue of 128 is only legitimate modulo 256");
 
 // ------------------------------------------------------------------ 1. convert
 // |x| / 2^E as a float rounded towards zero (20 mantissa bits), from the bits of x.
@@ -347,14 +354,7 @@ __device__ __forceinline__ void mod_tile(const ModGemmArgs& p, int t, int& tm, i
     }
 }
 
-// The centred residue of an integer |x| <= 2^24 in fp32: in [-128, 127] for every modulus
-// but 256, and [-128, 128] there (the fma's only error is 1 / p's own rounding).
-__device__ __forceinline__ float mod_centred(float x, float p, float inv) {
-    const float q = fmaf(x, inv, 12582912.0f) - 12582912.0f;
-    return fmaf(-q, p, x);
-}
-
-// Bits whose low byte (low half for sums) is r + 128 (a residue 128 modulo 256 wraps to 0).
+// Bits whose low byte (low half for sums) is r + 128 (modulo 256 a residue 128 wraps to 0, i.e. -128).
 __device__ __forceinline__ uint32_t mod_bits(float r) { return __float_as_uint(r + 8388736.0f); }
 
 // Persistent, one CTA per SM: a unit is one tile (TM x BN) of one plane, worked on by the

@@ -6,10 +6,10 @@
 #include <cuda_runtime.h>
 
 #include "dme_internal.h"
+#include "mod_arith.h"
 
 namespace dme {
 
-constexpr int MOD_NM = 16;            // moduli
 constexpr int MOD_PLANES = 17;        // residues, then the magnitudes |x| / 2^E
 constexpr int MOD_BK = 64;            // K per stage (one 128-byte swizzle row of bf16)
 

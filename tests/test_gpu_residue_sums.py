@@ -1,0 +1,38 @@
+"""FP64 products whose residue sums are as large as they get: rows of one constant, so that
+every term of a sum has the same residue and sign."""
+import numpy as np
+import pytest
+import torch
+
+import paper_1805_08990_gb300 as dme
+from gpu_util import dev, host, require_gpu
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(autouse=True, scope="module")
+def _gpu():
+    require_gpu()
+
+
+# (n, a, b): n a b has a residue sum near -2^24 modulo 255 in integers of 61 - log2 |row| bits
+CASES = [(577, 0.8251856099188752, 0.358081198534387), (577, -0.6743668325837577, 0.6942725357276607),
+         (853, 0.6257815933973978, 0.7864648019957695), (853, -0.10328771224131583, 0.3026237893873138),
+         (1021, 0.4778152288085107, 0.6773822806304568), (1021, -0.7731704195343296, 0.1677869334346773),
+         (1024, -0.31116594213485516, 0.37246532836315493), (1024, -0.8688898331736545, 0.9979833558848721),
+         (1024, 0.9051924950571193, 0.873609794533183), (1024, 0.25091920048512395, 0.6978108688532659)]
+
+
+@pytest.mark.parametrize("n,a,b", CASES)
+def test_constant_rows(n, a, b):
+    """T4 (Euler) with S = a 1 1^T on P = b 1 1^T: every entry is b + t n^2 a^2 b, each of the two
+    products within K u of its sum."""
+    t = 0.25
+    A = -np.eye(n)
+    plan = dme.Plan(dev(A), C=dev(np.ones((1, n))), h=t, flows=["F12", "F4"], comp="lie", S=dev(np.full((n, n), a)),
+                    t4_rule=dme.DME_T4_EULER)
+    P = dev(np.full((n, n), b))
+    torch.cuda.synchronize()
+    plan.apply("F4", t, P)
+    want = b + t * n * n * a * a * b
+    assert np.abs(host(P) - want).max() <= (2 * n + 8) * 2.0 ** -53 * abs(want)
