@@ -658,13 +658,14 @@ __device__ __forceinline__ void oz_store_direct(const OzParams& p, int n0, int i
 // in the staging buffer T (16 columns of the two warps of a lane quadrant, so
 // T holds 32 tile columns).  Phase 2: the 256 epilogue threads write the 128
 // staged row segments (i, j) coalesced (non-triangle F64 outputs add their
-// addends here, read at (i, j)).  Two named-barrier syncs per round.
+// addends here, read at (i, j)).  Two named-barrier syncs per round.  (T is not
+// __restrict__: phase 2 reads what other threads wrote, ordered by the barrier alone.)
 // (EC: columns held; EW: columns per warp, the distance of the two warps' columns; o0: the
 // round's first column within the warp's.)
 template <int EC, int EW>
 __device__ __forceinline__ void oz_store_staged_at(const OzParams& p, int m0, int n0, int il, int c0, int h0, int o0,
                                                 bool diag, const OzColScale<EC>& sc, const uint32_t (&h)[EC],
-                                                const uint32_t (&l)[EC], uint64_t* __restrict__ T, int ew, int lane) {
+                                                const uint32_t (&l)[EC], uint64_t* T, int ew, int lane) {
     const int i = m0 + il;
     const int slot = (ew / 4) * 16;                        // T columns of this warp pair: 0..15 or 16..31
     const float sA = i < p.M ? p.sa[i] : 0.0f;
