@@ -117,10 +117,10 @@ static_assert(mod_residues_fit(), "a residue of 128 is only legitimate modulo 25
 // |x| / 2^E as a float rounded towards zero (20 mantissa bits), from the bits of x.
 __device__ __forceinline__ float mag_scaled(unsigned long long b, int E) {
     const int ex = (int)((b >> 52) & 0x7FF) - 1023 - E;       // |x| / 2^E in [2^ex, 2^(ex+1)), ex <= -1
-    if (((b >> 52) & 0x7FF) == 0) return 0.0f;
-    // entries below 2^-60 of the row's largest are raised to it: far too small to pass the
-    // certificate, and a product of nonzero entries stays distinguishable from zero
-    if (ex < -60) return __int_as_float((127 - 60) << 23);
+    // entries below 2^-60 of the row's largest (subnormal ones always are: E >= -399) are raised
+    // to it: far too small to pass the certificate, and a product of nonzero entries stays
+    // distinguishable from zero
+    if (ex < -60) return (b << 1) ? __int_as_float((127 - 60) << 23) : 0.0f;
     return __int_as_float(((ex + 127) << 23) | (int)((b >> 29) & 0x7FFFFF));
 }
 

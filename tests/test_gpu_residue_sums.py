@@ -36,3 +36,24 @@ def test_constant_rows(n, a, b):
     plan.apply("F4", t, P)
     want = b + t * n * n * a * a * b
     assert np.abs(host(P) - want).max() <= (2 * n + 8) * 2.0 ** -53 * abs(want)
+
+
+@pytest.mark.parametrize("n", [192, 1025])
+def test_products_of_subnormal_entries(n):
+    """An output whose only nonzero product has a subnormal factor is that product: S P S^T with
+    S[i, k] = 2^-1060 beside an entry 1, P = 2^390 e_k e_k^T."""
+    i, j, k = n // 3, n - 2, n // 2
+    S = np.zeros((n, n))
+    S[i, 5] = S[j, k] = 1.0
+    S[i, k] = 2.0 ** -1060
+    P0 = np.zeros((n, n))
+    P0[k, k] = 2.0 ** 390
+    plan = dme.Plan(dev(-np.eye(n)), C=dev(np.ones((1, n))), h=0.5, flows=["F12", "F4"], comp="lie", S=dev(S),
+                    t4_rule=dme.DME_T4_EULER)
+    P = dev(P0)
+    torch.cuda.synchronize()
+    plan.apply("F4", 0.5, P)
+    want = P0.copy()
+    want[j, j] += 0.5 * 2.0 ** 390
+    want[i, j] = want[j, i] = 0.5 * 2.0 ** -670
+    assert np.array_equal(host(P), want)
