@@ -254,7 +254,8 @@ dme_status dme_lr_plan(const dme_plan_desc* desc, const double* A, const double*
  * (p x n) and, for a DRE / GDRE, B and R as in dme_plan.  e^{t A^T} L is applied by
  * Newton interpolation at Leja points (the action the paper computes with
  * `expleja`, §3): a Gershgorin interval [a, b] of A^T, A^T = c I + g X with
- * X's spectrum in [-2, 2], substeps of length t with t g <= 4 (10 for a symmetric A), at most 80
+ * X's spectrum in [-2, 2], substeps of length t with t g <= 4 (10 for a
+ * symmetric A whose largest eigenvalue is within 0.15 g of b), at most 80
  * Leja points per substep, and the series stopped after two terms below
  * 1e-15 times the partial sum (Frobenius norms; one more term is added).  For GDLE / GDRE, S (of the
  * S P S^T term, Eq. lyapGen; n x n) is given in CSR too (nnz_s, s_rowptr,

@@ -63,7 +63,7 @@ struct dme_lr_s {
     double* at_val = nullptr;   // values of A^T / g
     int *s_ptr = nullptr, *s_idx = nullptr;   // sparse S (CSR, device), for T4
     double* s_val = nullptr;
-    bool asym = false;               // sparse A: exactly symmetric
+    double lrho = 0.0;               // sparse A: largest t g of a substep
     int row_nnz = 0;                 // sparse A: most stored entries in a row of A^T
     double lc = 0.0, lg = 0.0;       // A^T = lc I + lg X, spectrum of X in [-2, 2] (Gershgorin)
     std::vector<double> xi;          // Leja points
@@ -341,13 +341,17 @@ void gauss_legendre(int q, double t, std::vector<double>& s, std::vector<double>
 
 // ---------------------------------------------------------------- Leja action (sparse A)
 constexpr int kLejaTerms = 80;        // interpolation points per substep
-// Largest t g per substep.  A symmetric A has its spectrum inside the Gershgorin interval and
-// no hump: the interpolation error is that on the interval, and the terms grow to
-// e^{2 t g} of the result's bound before they fall.  At 10 the action takes 0.58 of the
-// terms of 4 (82 instead of 141 at t g = 18.6) with less error than squared tables had
-// at 4 (2e-15 against 3e-15 for smooth and random blocks); 20 would take 57 with five
-// times the error of 10 on rough ones.  Any other A keeps 4.
-constexpr double kLejaRho = 4.0, kLejaRhoSym = 10.0;
+// Largest t g per substep.  The partial sums of a substep reach e^{2 t g} of the substep's
+// input (the function at the right end of the interval), its result e^{x t g}, x the rightmost
+// eigenvalue of X that the input has: rounding is amplified by e^{(2 - x) t g}.  A symmetric A
+// (no hump) whose spectrum reaches the right end of its Gershgorin interval takes substeps of
+// 10 (0.58 of the terms: 82 instead of 141 at t g = 18.6): kLejaGapSym bounds 2 - x there.
+// Errors with tables in double at 4 (before) / in double-double at 4 / at 10, banded symmetric
+// matrices, random blocks: 2 - x = 0: 1e-14 / 9e-16 / 3e-15, 0.05: 1e-14 / 2e-15 / 7e-15, 0.1:
+// 2e-14 / 2e-15 / 1e-14, 0.15: 2e-14 / 2e-15 / 2e-14, 0.35: 2e-14 / 4e-15 / 6e-14, 1.1 (the
+// square of a Laplacian): 9e-14 / 2e-14 / 4e-11, 1.4 (random signs): 2e-13 / 4e-14 / 1e-9.
+// 20 would take 57 terms with five times the error of 10.  Any other A keeps 4.
+constexpr double kLejaRho = 4.0, kLejaRhoSym = 10.0, kLejaGapSym = 0.15;
 constexpr double kLejaTol = 1e-15;    // series stops after two terms below tol |p|
 constexpr int kLejaGrid = 20001;      // candidate points for the greedy Leja sequence
 
@@ -436,12 +440,37 @@ std::vector<double> dd_exp_host(const std::vector<double>& x, DD a) {
     return col;
 }
 
+// An upper bound of 2 - x, x the rightmost eigenvalue of X = (A - c I) / g, for a symmetric A
+// (CSR) of Gershgorin interval [a, b]: (b - v^T A v / v^T v) / g with v = 1 (`mean` its
+// quotient: Laplacians reach the bound up to their boundary, 0.07 on 30 x 30 nodes), then, if
+// that is near, up to eight steps of power iteration with A - a I (10 x 10 nodes: 0.20, 0.14 after two).
+double leja_gap(int n, const std::vector<int>& ptr, const std::vector<int>& idx, const std::vector<double>& val, double a,
+                double b, double g, double mean) {
+    double gap = (b - mean) / g;
+    if (!(gap > kLejaGapSym && gap <= 0.5)) return gap;
+    std::vector<double> v(n, 1.0 / std::sqrt((double)n)), w(n);
+    for (int it = 0; it <= 8 && gap > kLejaGapSym; ++it) {
+        double q = 0.0, nrm = 0.0;
+        for (int i = 0; i < n; ++i) {
+            double y = 0.0;
+            for (int e = ptr[i]; e < ptr[i + 1]; ++e) y += val[e] * v[idx[e]];
+            q += v[i] * y;
+            w[i] = y - a * v[i];
+            nrm += w[i] * w[i];
+        }
+        gap = std::min(gap, (b - q) / g);
+        if (!(nrm > 0.0)) break;
+        for (int i = 0; i < n; ++i) v[i] = w[i] / std::sqrt(nrm);
+    }
+    return gap;
+}
+
 const LejaTab& leja_table(dme_lr_t lr, double tau) {
     for (auto& t : lr->ltab)
         if (t.tau == tau) return t;
     LejaTab t;
     t.tau = tau;
-    t.s = std::max(1, (int)std::ceil(tau * lr->lg / (lr->asym ? kLejaRhoSym : kLejaRho)));
+    t.s = std::max(1, (int)std::ceil(tau * lr->lg / lr->lrho));
     t.scale = dd_exp(dd_div(dd_prod(tau, lr->lc), t.s));
     t.dd = dd_exp_host(lr->xi, dd_div(dd_prod(tau, lr->lg), t.s));
     lr->ltab.push_back(t);
@@ -941,10 +970,11 @@ dme_status dme_lr_plan_csr(const dme_plan_desc* desc, int nnz, const int* rowptr
         lr->sparse = true;
         lr->nnz = nnz;
         // Gershgorin interval of A^T (rows of A^T): A^T = c I + g X, X's spectrum in [-2, 2]
-        double a = 0.0, b = 0.0;
+        double a = 0.0, b = 0.0, total = 0.0;
         for (int i = 0; i < n; ++i) {
             double di = 0.0, ri = 0.0;
             for (int e = tptr[i]; e < tptr[i + 1]; ++e) {
+                total += tval[e];
                 if (tidx[e] == i) di += tval[e];
                 else ri += std::fabs(tval[e]);
             }
@@ -954,15 +984,17 @@ dme_status dme_lr_plan_csr(const dme_plan_desc* desc, int nnz, const int* rowptr
         lr->lc = 0.5 * (a + b);
         lr->lg = 0.25 * (b - a);
         for (int i = 0; i < n; ++i) lr->row_nnz = std::max(lr->row_nnz, tptr[i + 1] - tptr[i]);
-        lr->asym = true;
-        for (int i = 0; i < n && lr->asym; ++i) {        // rows of A against rows of A^T, in any stored order
+        bool sym = true;
+        for (int i = 0; i < n && sym; ++i) {        // rows of A against rows of A^T, in any stored order
             std::vector<std::pair<int, double>> ra, rt;
             for (int e = ptr[i]; e < ptr[i + 1]; ++e) ra.emplace_back(idx[e], val[e]);
             for (int e = tptr[i]; e < tptr[i + 1]; ++e) rt.emplace_back(tidx[e], tval[e]);
             std::sort(ra.begin(), ra.end());
             std::sort(rt.begin(), rt.end());
-            lr->asym = ra == rt;
+            sym = ra == rt;
         }
+        const bool wide = sym && leja_gap(n, tptr, tidx, tval, a, b, lr->lg, total / n) <= kLejaGapSym;
+        lr->lrho = wide ? kLejaRhoSym : kLejaRho;
         lr->xi = leja_points_host(kLejaTerms);
         // the device copy of A^T holds A^T / g (the Leja recurrence's operator up to the shift)
         if (lr->lg > 0.0)
