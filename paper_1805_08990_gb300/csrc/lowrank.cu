@@ -63,7 +63,7 @@ struct dme_lr_s {
     double* at_val = nullptr;   // values of A^T / g
     int *s_ptr = nullptr, *s_idx = nullptr;   // sparse S (CSR, device), for T4
     double* s_val = nullptr;
-    double lrho = 0.0;               // sparse A: largest t g of a substep
+    double lrho = 0.0;               // sparse A: largest t g of a substep (0: not decided yet)
     int row_nnz = 0;                 // sparse A: most stored entries in a row of A^T
     double lc = 0.0, lg = 0.0;       // A^T = lc I + lg X, spectrum of X in [-2, 2] (Gershgorin)
     std::vector<double> xi;          // Leja points
@@ -440,41 +440,115 @@ std::vector<double> dd_exp_host(const std::vector<double>& x, DD a) {
     return col;
 }
 
-// An upper bound of 2 - x, x the rightmost eigenvalue of X = (A - c I) / g, for a symmetric A
-// (CSR) of Gershgorin interval [a, b]: (b - v^T A v / v^T v) / g with v = 1 (`mean` its
-// quotient: Laplacians reach the bound up to their boundary, 0.07 on 30 x 30 nodes), then, if
-// that is near, up to eight steps of power iteration with A - a I (10 x 10 nodes: 0.20, 0.14 after two).
-double leja_gap(int n, const std::vector<int>& ptr, const std::vector<int>& idx, const std::vector<double>& val, double a,
-                double b, double g, double mean) {
-    double gap = (b - mean) / g;
-    if (!(gap > kLejaGapSym && gap <= 0.5)) return gap;
+// The transpose of a CSR matrix, rows by increasing column (a counting sort by column).
+void csr_transpose(int n, const std::vector<int>& ptr, const std::vector<int>& idx, const std::vector<double>& val,
+                   std::vector<int>& tptr, std::vector<int>& tidx, std::vector<double>& tval) {
+    tptr.assign(n + 1, 0);
+    tidx.resize(idx.size());
+    tval.resize(idx.size());
+    for (int c : idx) tptr[c + 1]++;
+    for (int i = 0; i < n; ++i) tptr[i + 1] += tptr[i];
+    std::vector<int> fill(tptr.begin(), tptr.end() - 1);
+    for (int i = 0; i < n; ++i)
+        for (int e = ptr[i]; e < ptr[i + 1]; ++e) {
+            const int dst = fill[idx[e]]++;
+            tidx[dst] = i;
+            tval[dst] = val[e];
+        }
+}
+
+// Whether a CSR matrix of sorted rows equals its transpose (also sorted); entries stored
+// twice may come in another order.
+bool csr_symmetric(int n, const std::vector<int>& ptr, const std::vector<int>& idx, const std::vector<double>& val,
+                   const std::vector<int>& tptr, const std::vector<int>& tidx, const std::vector<double>& tval) {
+    if (ptr != tptr || idx != tidx) return false;
+    if (val == tval) return true;
+    std::vector<double> ra, rt;
+    for (int i = 0; i < n; ++i)
+        for (int e = ptr[i], f = e; e < ptr[i + 1]; e = f) {
+            while (f < ptr[i + 1] && idx[f] == idx[e]) ++f;
+            if (f - e == 1) {
+                if (!(val[e] == tval[e])) return false;
+                continue;
+            }
+            ra.assign(val.begin() + e, val.begin() + f);
+            rt.assign(tval.begin() + e, tval.begin() + f);
+            for (double v : ra)
+                if (!std::isfinite(v)) return false;
+            for (double v : rt)
+                if (!std::isfinite(v)) return false;
+            std::sort(ra.begin(), ra.end());
+            std::sort(rt.begin(), rt.end());
+            if (ra != rt) return false;
+        }
+    return true;
+}
+
+// An upper bound of 2 - x, x the rightmost eigenvalue of X = M - c / g, for a symmetric M = A / g
+// (CSR) of Gershgorin interval [lo, hi]: hi - v^T M v / v^T v with v = 1 (Laplacians reach the
+// bound up to their boundary, 0.07 on 30 x 30 nodes), then, if that is near, after up to eight
+// steps of power iteration with M - lo I (10 x 10 nodes: 0.20, 0.14 after two).
+double leja_gap(int n, const std::vector<int>& ptr, const std::vector<int>& idx, const std::vector<double>& val, double lo,
+                double hi) {
     std::vector<double> v(n, 1.0 / std::sqrt((double)n)), w(n);
-    for (int it = 0; it <= 8 && gap > kLejaGapSym; ++it) {
+    double gap = HUGE_VAL;
+    for (int it = 0; it <= 8; ++it) {
         double q = 0.0, nrm = 0.0;
         for (int i = 0; i < n; ++i) {
             double y = 0.0;
             for (int e = ptr[i]; e < ptr[i + 1]; ++e) y += val[e] * v[idx[e]];
             q += v[i] * y;
-            w[i] = y - a * v[i];
+            w[i] = y - lo * v[i];
             nrm += w[i] * w[i];
         }
-        gap = std::min(gap, (b - q) / g);
-        if (!(nrm > 0.0)) break;
+        gap = std::min(gap, hi - q);
+        if (!(gap > kLejaGapSym && gap <= 0.5 && nrm > 0.0)) break;
         for (int i = 0; i < n; ++i) v[i] = w[i] / std::sqrt(nrm);
     }
     return gap;
 }
 
-const LejaTab& leja_table(dme_lr_t lr, double tau) {
+// The largest t g of a substep: decided by the first application that is longer than the
+// shorter one, from the device's A^T / g.  (In the plan, symmetry and quotient cost 10 of 46 ms at
+// n = 10^6 with sorted arrays compared as they lie, 140 with every row sorted, for applications
+// that may all take one substep.)
+dme_status leja_rho(dme_lr_t lr) {
+    if (lr->lrho > 0.0) return DME_OK;
+    const int n = lr->n;
+    std::vector<int> ptr(n + 1), idx(lr->nnz), tptr, tidx;
+    std::vector<double> val(lr->nnz), tval;
+    DME_CUDA_TRY(cudaMemcpyAsync(ptr.data(), lr->at_ptr, sizeof(int) * ptr.size(), cudaMemcpyDeviceToHost, lr->st));
+    if (lr->nnz) {
+        DME_CUDA_TRY(cudaMemcpyAsync(idx.data(), lr->at_idx, sizeof(int) * idx.size(), cudaMemcpyDeviceToHost, lr->st));
+        DME_CUDA_TRY(cudaMemcpyAsync(val.data(), lr->at_val, sizeof(double) * val.size(), cudaMemcpyDeviceToHost, lr->st));
+    }
+    DME_CUDA_TRY(cudaStreamSynchronize(lr->st));
+    csr_transpose(n, ptr, idx, val, tptr, tidx, tval);
+    const double mid = lr->lc / lr->lg;
+    const bool wide = csr_symmetric(n, ptr, idx, val, tptr, tidx, tval) &&
+                      leja_gap(n, ptr, idx, val, mid - 2.0, mid + 2.0) <= kLejaGapSym;
+    lr->lrho = wide ? kLejaRhoSym : kLejaRho;
+    return DME_OK;
+}
+
+dme_status leja_table(dme_lr_t lr, double tau, const LejaTab** out) {
     for (auto& t : lr->ltab)
-        if (t.tau == tau) return t;
+        if (t.tau == tau) {
+            *out = &t;
+            return DME_OK;
+        }
     LejaTab t;
     t.tau = tau;
-    t.s = std::max(1, (int)std::ceil(tau * lr->lg / lr->lrho));
+    t.s = 1;
+    if (tau * lr->lg > kLejaRho) {
+        DME_TRY(leja_rho(lr));
+        t.s = (int)std::ceil(tau * lr->lg / lr->lrho);
+    }
     t.scale = dd_exp(dd_div(dd_prod(tau, lr->lc), t.s));
     t.dd = dd_exp_host(lr->xi, dd_div(dd_prod(tau, lr->lg), t.s));
     lr->ltab.push_back(t);
-    return lr->ltab.back();
+    *out = &lr->ltab.back();
+    return DME_OK;
 }
 
 // Y (n x k, ldy) = e^{tau A^T} X (n x k, ldx) by Leja interpolation; Y may be X.
@@ -486,7 +560,9 @@ dme_status leja_apply(dme_lr_t lr, const double* X, int ldx, int k, double* Y, i
         launch_copy_cols(Y, ldy, X, ldx, n, k, std::exp(tau * lr->lc), nullptr, st);
         return DME_OK;
     }
-    const LejaTab& tb = leja_table(lr, tau);
+    const LejaTab* tab = nullptr;
+    DME_TRY(leja_table(lr, tau, &tab));
+    const LejaTab& tb = *tab;
     LejaCall c;
     c.ptr = lr->at_ptr;
     c.idx = lr->at_idx;
@@ -954,47 +1030,29 @@ dme_status dme_lr_plan_csr(const dme_plan_desc* desc, int nnz, const int* rowptr
             if (ptr[i + 1] < ptr[i]) return set_error("CSR: rowptr must be non-decreasing"), DME_EINVAL;
         for (int e = 0; e < nnz; ++e)
             if (idx[e] < 0 || idx[e] >= n) return set_error("CSR: column index out of range"), DME_EINVAL;
-        // A^T in CSR (a counting sort by column)
-        std::vector<int> tptr(n + 1, 0), tidx(nnz);
-        std::vector<double> tval(nnz);
-        for (int e = 0; e < nnz; ++e) tptr[idx[e] + 1]++;
-        for (int i = 0; i < n; ++i) tptr[i + 1] += tptr[i];
-        std::vector<int> fill(tptr.begin(), tptr.end() - 1);
-        for (int i = 0; i < n; ++i)
-            for (int e = ptr[i]; e < ptr[i + 1]; ++e) {
-                const int dst = fill[idx[e]]++;
-                tidx[dst] = i;
-                tval[dst] = val[e];
-            }
+        // A^T in CSR
+        std::vector<int> tptr, tidx;
+        std::vector<double> tval;
+        csr_transpose(n, ptr, idx, val, tptr, tidx, tval);
         std::unique_ptr<dme_lr_s, void (*)(dme_lr_t)> lr(new dme_lr_s(), lr_free);
         lr->sparse = true;
         lr->nnz = nnz;
         // Gershgorin interval of A^T (rows of A^T): A^T = c I + g X, X's spectrum in [-2, 2]
-        double a = 0.0, b = 0.0, total = 0.0;
+        double a = 0.0, b = 0.0;
+        int widest = 0;
         for (int i = 0; i < n; ++i) {
             double di = 0.0, ri = 0.0;
             for (int e = tptr[i]; e < tptr[i + 1]; ++e) {
-                total += tval[e];
                 if (tidx[e] == i) di += tval[e];
                 else ri += std::fabs(tval[e]);
             }
             if (i == 0 || di - ri < a) a = di - ri;
             if (i == 0 || di + ri > b) b = di + ri;
+            widest = std::max(widest, tptr[i + 1] - tptr[i]);
         }
+        lr->row_nnz = widest;
         lr->lc = 0.5 * (a + b);
         lr->lg = 0.25 * (b - a);
-        for (int i = 0; i < n; ++i) lr->row_nnz = std::max(lr->row_nnz, tptr[i + 1] - tptr[i]);
-        bool sym = true;
-        for (int i = 0; i < n && sym; ++i) {        // rows of A against rows of A^T, in any stored order
-            std::vector<std::pair<int, double>> ra, rt;
-            for (int e = ptr[i]; e < ptr[i + 1]; ++e) ra.emplace_back(idx[e], val[e]);
-            for (int e = tptr[i]; e < tptr[i + 1]; ++e) rt.emplace_back(tidx[e], tval[e]);
-            std::sort(ra.begin(), ra.end());
-            std::sort(rt.begin(), rt.end());
-            sym = ra == rt;
-        }
-        const bool wide = sym && leja_gap(n, tptr, tidx, tval, a, b, lr->lg, total / n) <= kLejaGapSym;
-        lr->lrho = wide ? kLejaRhoSym : kLejaRho;
         lr->xi = leja_points_host(kLejaTerms);
         // the device copy of A^T holds A^T / g (the Leja recurrence's operator up to the shift)
         if (lr->lg > 0.0)
