@@ -27,7 +27,6 @@
 // blocks that combine.
 //
 // Bound: tensor pipe for n >= 1024 (17 bf16 products), launch latency below.
-#include "gemm64_tile.cuh"
 #include "mod_internal.h"
 #include "split_internal.h"
 #include "tc_ptx.cuh"
@@ -642,45 +641,96 @@ __device__ __forceinline__ double int_scaled(__int128 v, int e) {
     return __longlong_as_double((long long)b);
 }
 
-// FP64 sums of a 32 x 32 tile from the operands (k in increasing order, fma).
-__device__ __noinline__ void mod_native_tile(const GemmProb& pb, int row0, int col0, double (*As)[33], double (*Bs)[33],
-                                             double (*sS)[33]) {
-    double acc[2][2];
-    gemm64_accum<32>(pb, row0, col0, 0, pb.K, reinterpret_cast<double(&)[G64_BK][33]>(*As),
-                     reinterpret_cast<double(&)[G64_BK][33]>(*Bs), acc);
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+// A block of the combine: MC_ROWS rows of a 32 x 32 tile, four outputs a thread.
+constexpr int MC_ROWS = 8, MC_THREADS = 8 * MC_ROWS;
+// Most outputs of a strip (256) recomputed one by one, a warp each; more, and the whole strip is.
+// The list's time grows with its length: 64, 128, 192 outputs against the strip at n = 256 93, 118,
+// 143 / 122 us, n = 576 210, 319, 428 / 453, n = 1024 714, 1256, 1781 / 1968 (S P S^T, two products,
+// all strips alike).  Where strips differ, the longest list decides: a localised state at
+// n = 225 takes 136 us with lists of up to 8, 197 with up to 128.
+constexpr int MC_LIST = 64;
+
+// FP64 sums of a strip from the operands (k in increasing order, fma), four outputs a thread;
+// the next 16 k are loaded beside the FMAs.
+__device__ __noinline__ void mod_native_strip(const GemmProb& pb, int row0, int col0, double (*As)[MC_ROWS + 1],
+                                              double (*Bs)[33], double (*sS)[33]) {
+    constexpr int NT = MC_THREADS, ROWS = MC_ROWS, NB = 16 * 32 / NT;
+    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+    double a[2], b[NB];
+    auto load = [&](int k0) {
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const int e = tid + NT * q, r = row0 + (pb.transA ? e % ROWS : e >> 4), k = k0 + (pb.transA ? e / ROWS : e & 15);
+            a[q] = r < pb.M && k < pb.K ? (pb.transA ? pb.A[(size_t)k * pb.lda + r] : pb.A[(size_t)r * pb.lda + k]) : 0.0;
+        }
+#pragma unroll
+        for (int q = 0; q < NB; ++q) {
+            const int e = tid + NT * q, c = col0 + (pb.transB ? e >> 4 : e & 31), k = k0 + (pb.transB ? e & 15 : e >> 5);
+            b[q] = c < pb.N && k < pb.K ? (pb.transB ? pb.B[(size_t)c * pb.ldb + k] : pb.B[(size_t)k * pb.ldb + c]) : 0.0;
+        }
+    };
+    double acc[2][2] = {};
+    load(0);
+    for (int k0 = 0; k0 < pb.K; k0 += 16) {
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const int e = tid + NT * q;
+            As[pb.transA ? e / ROWS : e & 15][pb.transA ? e % ROWS : e >> 4] = a[q];
+        }
+#pragma unroll
+        for (int q = 0; q < NB; ++q) {
+            const int e = tid + NT * q;
+            Bs[pb.transB ? e & 15 : e >> 5][pb.transB ? e >> 4 : e & 31] = b[q];
+        }
+        __syncthreads();
+        if (k0 + 16 < pb.K) load(k0 + 16);
+#pragma unroll
+        for (int k = 0; k < 16; ++k) {
+            const double a0 = As[k][ty], a1 = As[k][ty + ROWS / 2], b0 = Bs[k][tx], b1 = Bs[k][tx + 16];
+            acc[0][0] = fma(a0, b0, acc[0][0]);
+            acc[0][1] = fma(a0, b1, acc[0][1]);
+            acc[1][0] = fma(a1, b0, acc[1][0]);
+            acc[1][1] = fma(a1, b1, acc[1][1]);
+        }
+    }
 #pragma unroll
     for (int i = 0; i < 2; ++i)
 #pragma unroll
-        for (int j = 0; j < 2; ++j) sS[ty + 16 * i][tx + 16 * j] = acc[i][j];
+        for (int j = 0; j < 2; ++j) sS[ty + ROWS / 2 * i][tx + 16 * j] = acc[i][j];
 }
 
-// One 32 x 32 tile per block: four outputs a thread from their 16 residues (one word
-// per plane), the sums staged in shared memory; outputs without a certificate replaced
-// by FP64 sums (a warp each, or the whole tile when they are many); then the product's
-// epilogue, coalesced (and its mirror for a triangle).
-constexpr int MC_LIST = 32;
-__global__ void __launch_bounds__(256) mod_combine_kernel(const __grid_constant__ GemmProb pb,
-                                                          const uint8_t* __restrict__ R, size_t plane, int ldr,
-                                                          const ModRow* __restrict__ ra, const ModRow* __restrict__ rb,
-                                                          int certify, int tiles_n) {
-    __shared__ double sS[32][33];
-    __shared__ double As[G64_BK][33], Bs[G64_BK][33];
+// Four outputs a thread from their 16 residues (one word per plane), the sums staged in shared
+// memory; outputs without a certificate replaced by FP64 sums (a warp each, or the whole
+// strip); then the product's epilogue, coalesced (and its mirror for a triangle).
+// Strips of 8 rows: where most outputs fail (a state localised around one node, P0 = 0) the FP64
+// pipe bounds the product, and blocks of a whole tile left SMs idle.  T12 step of such a state /
+// of a dense one, us: n = 196 123 / 34 (tiles of 32 rows, 33 outputs sending the tile to FP64:
+// 174 / 35; the FP64 pipe alone 145), n = 256 144 / 34 (204 / 36; 174), n = 576 604 / 64 (836 / 66;
+// 781), n = 1024 2695 / 111 (3016 / 113; 3168), n = 2025 19090 / 424 (21290 / 426; 22760).  Eight
+// factored steps from one node's C: n = 1024 2.1 ms (5.4; 2.1), n = 2304 4.6 (12.8; 12.1).
+__global__ void __launch_bounds__(MC_THREADS) mod_combine_kernel(const __grid_constant__ GemmProb pb,
+                                                                 const uint8_t* __restrict__ R, size_t plane, int ldr,
+                                                                 const ModRow* __restrict__ ra, const ModRow* __restrict__ rb,
+                                                                 int certify, int tiles_n) {
+    constexpr int ROWS = MC_ROWS, STRIPS = 32 / ROWS, WARPS = MC_THREADS / 32;
+    __shared__ double sS[ROWS][33];
+    __shared__ double As[16][ROWS + 1], Bs[16][33];
     __shared__ int s_cnt;
     __shared__ int s_list[MC_LIST];
+    const int tile = blockIdx.x / STRIPS;
     int ti, tj;
     if (pb.tri) {
         // tile t of the upper triangle, column by column: tj (tj + 1) / 2 <= t
-        const int t = blockIdx.x;
-        tj = (int)((sqrtf(8.0f * (float)t + 1.0f) - 1.0f) * 0.5f);
-        while ((tj + 1) * (tj + 2) / 2 <= t) ++tj;
-        while (tj * (tj + 1) / 2 > t) --tj;
-        ti = t - tj * (tj + 1) / 2;
+        tj = (int)((sqrtf(8.0f * (float)tile + 1.0f) - 1.0f) * 0.5f);
+        while ((tj + 1) * (tj + 2) / 2 <= tile) ++tj;
+        while (tj * (tj + 1) / 2 > tile) --tj;
+        ti = tile - tj * (tj + 1) / 2;
     } else {
-        ti = blockIdx.x / tiles_n;
-        tj = blockIdx.x % tiles_n;
+        ti = tile / tiles_n;
+        tj = tile % tiles_n;
     }
-    const int i0 = ti * 32, j0 = tj * 32;
+    const int i0 = ti * 32 + (blockIdx.x % STRIPS) * ROWS, j0 = tj * 32;
     if (threadIdx.x == 0) s_cnt = 0;
     __syncthreads();
     {
@@ -722,11 +772,11 @@ __global__ void __launch_bounds__(256) mod_combine_kernel(const __grid_constant_
     __syncthreads();
     const int cnt = s_cnt;
     if (cnt > MC_LIST) {
-        mod_native_tile(pb, i0, j0, As, Bs, sS);
+        mod_native_strip(pb, i0, j0, As, Bs, sS);
         __syncthreads();
     } else if (cnt > 0) {
         const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-        for (int e = warp; e < cnt; e += 8) {
+        for (int e = warp; e < cnt; e += WARPS) {
             const int i = i0 + s_list[e] / 32, j = j0 + s_list[e] % 32;
             double a = 0.0;
             for (int k = lane; k < pb.K; k += 32) {
@@ -743,7 +793,7 @@ __global__ void __launch_bounds__(256) mod_combine_kernel(const __grid_constant_
     const int cc = threadIdx.x & 31;
 #pragma unroll
     for (int h = 0; h < 4; ++h) {
-        const int r = (threadIdx.x >> 5) + 8 * h, i = i0 + r, j = j0 + cc;
+        const int r = (threadIdx.x >> 5) + WARPS * h, i = i0 + r, j = j0 + cc;
         if (i < pb.M && j < pb.N && !(pb.tri && i > j)) {
             const size_t off = (size_t)i * pb.ldd + j;
             double v = sS[r][cc];
@@ -759,9 +809,9 @@ __global__ void __launch_bounds__(256) mod_combine_kernel(const __grid_constant_
     __syncthreads();
 #pragma unroll
     for (int h = 0; h < 4; ++h) {
-        // the mirror: row j0 + r of the lower triangle, column i0 + cc
-        const int r = (threadIdx.x >> 5) + 8 * h, j = j0 + r, i = i0 + cc;
-        if (j < pb.N && i < pb.M && i < j) pb.C[(size_t)j * pb.ldc + i] = sS[cc][r];
+        // the mirror: row j0 + r of the lower triangle, column i0 + ic
+        const int ic = threadIdx.x % ROWS, r = threadIdx.x / ROWS + 8 * h, j = j0 + r, i = i0 + ic;
+        if (j < pb.N && i < pb.M && i < j) pb.C[(size_t)j * pb.ldc + i] = sS[ic][r];
     }
 }
 
@@ -902,8 +952,8 @@ dme_status launch_mod_gemm(const ModBuf& A, const ModBuf& B, const GemmProb& g, 
         }
     }
     const int tn = (g.N + 31) / 32, tm = (g.M + 31) / 32;
-    const int blocks = g.tri ? tn * (tn + 1) / 2 : tm * tn;
-    mod_combine_kernel<<<blocks, 256, 0, st>>>(g, a.R, a.plane, a.ldr, a.ra, a.rb, certify ? 1 : 0, tn);
+    const int strips = (g.tri ? tn * (tn + 1) / 2 : tm * tn) * (32 / MC_ROWS);
+    mod_combine_kernel<<<strips, MC_THREADS, 0, st>>>(g, a.R, a.plane, a.ldr, a.ra, a.rb, certify ? 1 : 0, tn);
     DME_CUDA_TRY(cudaGetLastError());
     return DME_OK;
 }

@@ -57,3 +57,33 @@ def test_products_of_subnormal_entries(n):
     want[j, j] += 0.5 * 2.0 ** 390
     want[i, j] = want[j, i] = 0.5 * 2.0 ** -670
     assert np.array_equal(host(P), want)
+
+
+@pytest.mark.parametrize("n", [192, 231, 416])
+@pytest.mark.parametrize("c", [1, 7, 8, 9, 32])
+def test_outputs_without_certificate(n, c):
+    """c columns of each 32 of P have no entry where the rows of S are large, so that 8 c of a
+    strip's 256 outputs fail the certificate (recomputed one by one up to 64, as a strip
+    beyond).  Bound: two chained FP64 products of length n, entrywise."""
+    r = np.random.default_rng(n + c)
+    S = r.standard_normal((n, n)) * 2.0 ** -30
+    S[:, 0] = 1.0
+    G = r.standard_normal((n, 8))
+    P0 = G @ G.T + 3.0
+    J = np.arange(n) % 32 >= 32 - c
+    J[0] = False
+    P0[0, J] = P0[J, 0] = 0.0
+    t = 0.5
+    plan = dme.Plan(dev(-np.eye(n)), C=dev(np.ones((1, n))), h=t, flows=["F12", "F4"], comp="lie", S=dev(S),
+                    t4_rule=dme.DME_T4_EULER)
+    P = dev(P0)
+    torch.cuda.synchronize()
+    plan.apply("F4", t, P)
+    got = host(P)
+    assert np.array_equal(got, got.T)
+    q = np.longdouble
+    rows = np.arange(0, n, 5)
+    ref = P0[rows] + t * ((S[rows].astype(q) @ P0.astype(q)) @ S.T.astype(q))
+    mag = np.abs(P0[rows]) + t * ((np.abs(S[rows]) @ np.abs(P0)) @ np.abs(S.T))
+    err = np.abs((got[rows] - ref).astype(np.float64))
+    assert np.all(err <= (2 * n + 6) * 2.0 ** -53 * mag)
