@@ -892,7 +892,9 @@ int mod_tile_count(int M, int N, int tri, int tm, int bn) {
 
 }  // namespace
 
-dme_status mod_make_maps(ModBuf& b) {
+dme_status mod_place(ModBuf& b, void* mem) {
+    b.data = static_cast<__nv_bfloat16*>(mem);
+    b.row = reinterpret_cast<ModRow*>(static_cast<char*>(mem) + mod_plane_bytes(b.rows, b.k));
     DME_TRY(mod_map(b, 64, &b.t64));
     return mod_map(b, 128, &b.t128);
 }

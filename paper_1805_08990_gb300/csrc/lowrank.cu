@@ -81,12 +81,12 @@ struct dme_lr_s {
     int* kdev = nullptr;
     bool split = false;            // the products with E_t and S on the tensor cores
     SliceBuf xsl;                  // split: slices of X^T for M X (rows = rmax, k = n)
-    double* Xtr = nullptr;         // split: X^T (rmax x n)
+    double* Xtr = nullptr;         // X^T (rmax x n)
     double* ws = nullptr;          // split-K partial products
     size_t ws_doubles = 0;
     GemmProb* wsdesc = nullptr;    // their descriptors (kSplitMax)
     std::vector<WFactor> wf;
-    std::vector<void*> allocs;
+    std::vector<void*> allocs, opt;   // (opt: the residue products' buffers)
     int r = 0;
     bool loose = false;            // the factor's last compression was a QLP one
     int* k0dev = nullptr;
@@ -99,8 +99,26 @@ struct dme_lr_s {
 
 namespace {
 
+// Give back the residue products' buffers, the dense plan's included (the products stay on the
+// FP64 pipe from then on).  False if there were none.
+bool lr_release_mod(dme_lr_t lr) {
+    const bool planes = lr->P && plan_release_planes(lr->P);
+    if (lr->opt.empty()) return planes;
+    cudaGetLastError();
+    cudaStreamSynchronize(lr->st);
+    for (void* q : lr->opt) cudaFree(q);
+    lr->opt.clear();
+    lr->mod = false;
+    lr->ml.data = lr->ms.data = nullptr;
+    lr->mws = nullptr;
+    lr->Xtr = nullptr;
+    return true;
+}
+
 dme_status lr_alloc(dme_lr_t lr, double** out, size_t count) {
-    cudaError_t e = cudaMalloc(reinterpret_cast<void**>(out), std::max<size_t>(count, 1) * sizeof(double));
+    const size_t bytes = std::max<size_t>(count, 1) * sizeof(double);
+    cudaError_t e = cudaMalloc(reinterpret_cast<void**>(out), bytes);
+    if (e != cudaSuccess && lr_release_mod(lr)) e = cudaMalloc(reinterpret_cast<void**>(out), bytes);
     if (e != cudaSuccess) {
         cudaGetLastError();
         set_error(std::string("low-rank plan: cudaMalloc: ") + cudaGetErrorString(e));
@@ -108,6 +126,14 @@ dme_status lr_alloc(dme_lr_t lr, double** out, size_t count) {
     }
     lr->allocs.push_back(*out);
     return DME_OK;
+}
+
+// E_t of the dense plan, for which the residue products' buffers make room.
+dme_status lr_ew(dme_lr_t lr, double tau, int* idx) {
+    const dme_status s = plan_ew(lr->P, tau, idx);
+    if (s != DME_ENOMEM || !lr_release_mod(lr)) return s;
+    set_error("");
+    return plan_ew(lr->P, tau, idx);
 }
 
 GemmProb mk(int M, int N, int K, const double* A, int lda, int tA, const double* B, int ldb, int tB, double* C,
@@ -631,7 +657,7 @@ dme_status wfactor(dme_lr_t lr, double tau, const WFactor** out) {
             DME_TRY(leja_apply(lr, lr->LQ, p, p, WL + (size_t)k * p, lr->rcap, s[k]));                 // e^{s A^T} C^T
         } else {
             int idx;
-            DME_TRY(plan_ew(lr->P, s[k], &idx));
+            DME_TRY(lr_ew(lr, s[k], &idx));
             const double* E = lr->P->ew[idx].E;
             DME_TRY(gemm(lr, mk(n, p, n, E, n, 1, lr->LQ, p, 0, WL + (size_t)k * p, lr->rcap, 1.0), st));   // E_s^T C^T
         }
@@ -696,7 +722,7 @@ dme_status lr_T1(dme_lr_t lr, double tau) {
         return DME_OK;
     }
     int idx;
-    DME_TRY(plan_ew(lr->P, tau, &idx));
+    DME_TRY(lr_ew(lr, tau, &idx));
     const EWEntry& e = lr->P->ew[idx];
     if (lr->mod) DME_TRY(plan_mod_planes(lr->P, idx));
     const ModBuf& Gm = lr->P->ew[idx].Gm;
@@ -801,7 +827,8 @@ dme_status lr_apply(dme_lr_t lr, int flow, double tau, bool last) {
 void lr_free(dme_lr_t lr) {
     if (!lr) return;
     if (lr->st) cudaStreamSynchronize(lr->st);
-    for (void* q : lr->allocs) cudaFree(q);
+    for (auto* v : {&lr->allocs, &lr->opt})
+        for (void* q : *v) cudaFree(q);
     if (lr->P) free_plan(lr->P);
     if (lr->own_st && lr->st) cudaStreamDestroy(lr->st);
     delete lr;
@@ -854,33 +881,30 @@ dme_status lr_opts(const dme_lr_opts* opts, int* q, int* rmax, double* tol) {
 // Planes of L^T (and of S) and the workspace of E_t^T L on residue products; without them
 // (not enough memory) the products stay on the FP64 pipe.
 dme_status lr_mod_setup(dme_lr_t lr, int n, int rc) {
+    auto get = [&](size_t bytes) -> void* {
+        void* q = nullptr;
+        if (cudaMalloc(&q, bytes) != cudaSuccess) {
+            cudaGetLastError();
+            return nullptr;
+        }
+        lr->opt.push_back(q);
+        return q;
+    };
     auto planes = [&](ModBuf* b, int rows) -> bool {
-        double *pl = nullptr, *rw = nullptr;
         b->rows = rows;
         b->k = n;
         b->Kp = mod_kpad(n);
-        if (lr_alloc(lr, &pl, mod_plane_bytes(rows, n) / 8 + 1) != DME_OK ||
-            lr_alloc(lr, &rw, mod_row_bytes(rows) / 8 + 1) != DME_OK)
-            return false;
-        b->data = reinterpret_cast<__nv_bfloat16*>(pl);
-        b->row = reinterpret_cast<ModRow*>(rw);
-        return mod_make_maps(*b) == DME_OK;
+        void* q = get(mod_buf_bytes(rows, n));
+        return q && mod_place(*b, q) == DME_OK;
     };
-    double* ws = nullptr;
-    if (!planes(&lr->ml, rc) || lr_alloc(lr, &ws, mod_ws_bytes(n, rc) / 8 + 1) != DME_OK ||
-        lr_alloc(lr, &lr->Xtr, (size_t)rc * n) != DME_OK) {
-        set_error("");
+    lr->mws = static_cast<uint8_t*>(get(mod_ws_bytes(n, rc)));
+    lr->Xtr = static_cast<double*>(get(sizeof(double) * rc * n));
+    lr->mod = planes(&lr->ml, rc) && lr->mws && lr->Xtr;
+    if (!lr->mod) {
+        lr_release_mod(lr);
         return DME_OK;
     }
-    lr->mws = reinterpret_cast<uint8_t*>(ws);
-    lr->mod = true;
-    if (lr->P->S) {
-        if (planes(&lr->ms, n)) launch_mod_convert(lr->P->S, n, n, n, lr->ms, lr->st);
-        else {
-            lr->ms.data = nullptr;
-            set_error("");
-        }
-    }
+    if (lr->P->S && planes(&lr->ms, n)) launch_mod_convert(lr->P->S, n, n, n, lr->ms, lr->st);
     return DME_OK;
 }
 
@@ -934,7 +958,6 @@ dme_status lr_setup(dme_lr_t lr, const dme_plan_desc* desc, const double* C, int
         DME_CUDA_TRY(cudaMemsetAsync(xs, 0, sizeof(float) * rc, st));
         DME_TRY(make_slice_tmaps(lr->xsl));
     }
-    if (!lr->split && lr->P && lr->P->mod_ew) DME_TRY(lr_mod_setup(lr, (int)n, (int)rc));
     double* kd = nullptr;
     DME_TRY(lr_alloc(lr, &kd, 1));
     lr->kdev = reinterpret_cast<int*>(kd);
@@ -943,6 +966,7 @@ dme_status lr_setup(dme_lr_t lr, const dme_plan_desc* desc, const double* C, int
     DME_TRY(lr_alloc(lr, &Cd, (size_t)desc->p * n));
     DME_CUDA_TRY(cudaMemcpyAsync(Cd, C, sizeof(double) * desc->p * n, cudaMemcpyDefault, st));
     launch_transpose(Cd, lr->LQ, desc->p, (int)n, (int)n, desc->p, st);
+    if (lr->P && lr->P->mod_planes) DME_TRY(lr_mod_setup(lr, (int)n, (int)rc));
     DME_CUDA_TRY(cudaStreamSynchronize(st));
     return DME_OK;
 }

@@ -33,13 +33,14 @@ struct ModBuf {
 
 inline int mod_kpad(int k) { return (k + MOD_BK - 1) / MOD_BK * MOD_BK; }
 inline size_t mod_plane_bytes(int rows, int k) { return (size_t)MOD_PLANES * rows * mod_kpad(k) * 2; }
-inline size_t mod_row_bytes(int rows) { return (size_t)rows * sizeof(ModRow); }
+// One allocation: the planes (a multiple of 128 bytes), then the rows' scales.
+inline size_t mod_buf_bytes(int rows, int k) { return mod_plane_bytes(rows, k) + (size_t)rows * sizeof(ModRow); }
 // Workspace of an M x N product: a byte per residue and output, and the certificate.
 inline int mod_ldr(int N) { return (N + 255) / 256 * 256; }
 inline size_t mod_ws_bytes(int M, int N) { return (size_t)MOD_PLANES * M * mod_ldr(N); }
 
-// Encode the tensor maps of buf (data, rows, k, Kp set).
-dme_status mod_make_maps(ModBuf& buf);
+// Put buf (rows, k, Kp set) into mod_buf_bytes of memory and encode its tensor maps.
+dme_status mod_place(ModBuf& buf, void* mem);
 // Residue planes of the rows of X (rows x k, leading dimension ld; rows <= buf.rows).
 void launch_mod_convert(const double* X, int rows, int k, int ld, const ModBuf& buf, cudaStream_t st);
 // g (C = alpha op(A) op(B) + addends, triangle mode as gemm64_grouped) from the residue

@@ -52,6 +52,7 @@ dme_status palloc(dme_plan_t p, void** out, size_t bytes) {
     *out = nullptr;
     if (bytes == 0) bytes = 16;
     cudaError_t e = cudaMallocAsync(out, bytes, p->st);
+    if (e != cudaSuccess && plan_release_planes(p)) e = cudaMallocAsync(out, bytes, p->st);
     if (e != cudaSuccess) {
         cudaGetLastError();
         set_error(std::string("cudaMalloc(") + std::to_string(bytes) + "): " + cudaGetErrorString(e));
@@ -62,21 +63,39 @@ dme_status palloc(dme_plan_t p, void** out, size_t bytes) {
     return DME_OK;
 }
 
+// A buffer the plan can do without (in p->opt); null, and no error, if it does not fit.
+void* palloc_opt(dme_plan_t p, size_t bytes) {
+    void* q = nullptr;
+    if (cudaMallocAsync(&q, bytes, p->st) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    p->opt.push_back(q);
+    return q;
+}
+
 template <typename T>
 dme_status palloc_t(dme_plan_t p, T** out, size_t count) {
     return palloc(p, reinterpret_cast<void**>(out), count * sizeof(T));
 }
 
-// Temporary device buffers released at scope exit (plan-time only), stream ordered.
+// Temporary device buffers released at scope exit (plan-time only), stream ordered.  With a
+// plan, its residue planes make room for them.
 struct TmpPool {
     cudaStream_t st;
+    dme_plan_t p = nullptr;
     std::vector<void*> v;
     explicit TmpPool(cudaStream_t s) : st(s) {}
-    ~TmpPool() {
+    explicit TmpPool(dme_plan_t plan) : st(plan->st), p(plan) {}
+    ~TmpPool() { clear(); }
+    void clear() {
         for (void* q : v) cudaFreeAsync(q, st);
+        v.clear();
     }
     dme_status get(double** out, size_t count) {
-        cudaError_t e = cudaMallocAsync(reinterpret_cast<void**>(out), std::max<size_t>(count, 2) * sizeof(double), st);
+        const size_t bytes = std::max<size_t>(count, 2) * sizeof(double);
+        cudaError_t e = cudaMallocAsync(reinterpret_cast<void**>(out), bytes, st);
+        if (e != cudaSuccess && p && plan_release_planes(p)) e = cudaMallocAsync(reinterpret_cast<void**>(out), bytes, st);
         if (e != cudaSuccess) {
             cudaGetLastError();
             set_error(std::string("cudaMalloc (temporary): ") + cudaGetErrorString(e));
@@ -84,6 +103,16 @@ struct TmpPool {
         }
         v.push_back(*out);
         return DME_OK;
+    }
+};
+
+// Frees what the plan has allocated since (beyond the first n) unless n is moved on.
+struct AllocMark {
+    dme_plan_t p;
+    size_t n;
+    explicit AllocMark(dme_plan_t plan) : p(plan), n(plan->allocs.size()) {}
+    ~AllocMark() {
+        for (; p->allocs.size() > n; p->allocs.pop_back()) cudaFreeAsync(p->allocs.back(), p->st);
     }
 };
 
@@ -143,14 +172,9 @@ dme_status mod_alloc(dme_plan_t p, ModBuf* b, int rows, int k, bool* ok) {
     b->rows = rows;
     b->k = k;
     b->Kp = mod_kpad(k);
-    *ok = palloc(p, reinterpret_cast<void**>(&b->data), mod_plane_bytes(rows, k)) == DME_OK &&
-          palloc(p, reinterpret_cast<void**>(&b->row), mod_row_bytes(rows)) == DME_OK;
-    if (!*ok) {
-        b->data = nullptr;
-        set_error("");
-        return DME_OK;
-    }
-    return mod_make_maps(*b);
+    void* q = palloc_opt(p, mod_buf_bytes(rows, k));
+    *ok = q != nullptr;
+    return q ? mod_place(*b, q) : DME_OK;
 }
 
 // cong64 by residue products: with G = op(Gp) (its planes in G), X = G P^T and
@@ -271,15 +295,12 @@ struct ModWork {
 
 dme_status mod_setup(TmpPool& tp, int n, int* status, ModWork* w) {
     for (ModBuf* b : {&w->a, &w->b, &w->c}) {
-        double *pl, *rw;
-        DME_TRY(tp.get(&pl, mod_plane_bytes(n, n) / 8 + 1));
-        DME_TRY(tp.get(&rw, mod_row_bytes(n) / 8 + 1));
-        b->data = reinterpret_cast<__nv_bfloat16*>(pl);
-        b->row = reinterpret_cast<dme::ModRow*>(rw);
+        double* q;
+        DME_TRY(tp.get(&q, mod_buf_bytes(n, n) / 8 + 1));
         b->rows = n;
         b->k = n;
         b->Kp = mod_kpad(n);
-        DME_TRY(mod_make_maps(*b));
+        DME_TRY(mod_place(*b, q));
     }
     double* ws;
     DME_TRY(tp.get(&ws, mod_ws_bytes(n, n) / 8 + 1));
@@ -534,7 +555,8 @@ dme_status compute_ew(dme_plan_t p, double tau, int* idx) {
     if (nrm > kTheta13) s = (int)std::ceil(std::log2(nrm / kTheta13));
     const double sc = std::ldexp(tau, -s);
 
-    TmpPool tp(st);
+    TmpPool tp(p), tmod(st);
+    AllocMark kept(p);
     double *X22, *X12, *A22, *A12, *B22, *B12, *C22, *C12, *Y22, *Y12, *T22, *T12, *U22, *U12, *V22, *V12;
     double *LUq, *LUp, *R22, *R12;
     DME_TRY(tp.get(&X22, nn));
@@ -562,13 +584,20 @@ dme_status compute_ew(dme_plan_t p, double tau, int* idx) {
         DME_TRY(acc_setup(tp, n, p->status, &accw));
         pp.acc = &accw;
     }
+    // what the plan keeps, before what it can do without
+    EWEntry ent;
+    ent.tau = tau;
+    ent.s = s;
+    DME_TRY(palloc_t(p, &ent.E, nn));
+    DME_TRY(palloc_t(p, &ent.W, nn));
     // residue products, if their planes fit in memory
     ModWork modw;
     if (p->mod_ew) {
-        if (mod_setup(tp, n, p->status, &modw) == DME_OK) {
+        if (mod_setup(tmod, n, p->status, &modw) == DME_OK) {
             modw.balanced = p->balanced;
             pp.mod = &modw;
         } else {
+            tmod.clear();
             set_error("");
         }
     }
@@ -652,11 +681,6 @@ dme_status compute_ew(dme_plan_t p, double tau, int* idx) {
         }
         std::swap(E, E2);
     }
-    EWEntry ent;
-    ent.tau = tau;
-    ent.s = s;
-    DME_TRY(palloc_t(p, &ent.E, nn));
-    DME_TRY(palloc_t(p, &ent.W, nn));
     DME_CUDA_TRY(cudaMemcpyAsync(ent.E, E, nn * sizeof(double), cudaMemcpyDeviceToDevice, st));
     DME_CUDA_TRY(cudaMemcpyAsync(ent.W, Wm, nn * sizeof(double), cudaMemcpyDeviceToDevice, st));
     if (p->split) {
@@ -667,6 +691,7 @@ dme_status compute_ew(dme_plan_t p, double tau, int* idx) {
     DME_CUDA_TRY(cudaGetLastError());
     DME_TRY(check_status(p, "dme_expm"));
     p->ew.push_back(ent);
+    kept.n = p->allocs.size();
     *idx = (int)p->ew.size() - 1;
     return DME_OK;
 }
@@ -1030,18 +1055,30 @@ void drop_graph(GraphSlot& g) {
 
 dme_status dme::plan_mod_planes(dme_plan_t p, int idx) {
     EWEntry& e = p->ew[idx];
-    if (!p->mod_ew || e.Gm.data) return DME_OK;
+    if (!p->mod_planes || e.Gm.data) return DME_OK;
     const int n = p->n;
     bool ok = false;
     DME_TRY(mod_alloc(p, &e.Gm, n, n, &ok));
     if (!ok) return DME_OK;
-    TmpPool tp(p->st);
-    double* Et = nullptr;
-    DME_TRY(tp.get(&Et, (size_t)n * n));
-    launch_transpose(e.E, Et, n, n, n, n, p->st);
-    launch_mod_convert(Et, n, n, n, e.Gm, p->st);
+    launch_transpose(e.E, p->X, n, n, n, n, p->st);           // (X: scratch of a congruence)
+    launch_mod_convert(p->X, n, n, n, e.Gm, p->st);
     DME_CUDA_TRY(cudaGetLastError());
     return DME_OK;
+}
+
+bool dme::plan_release_planes(dme_plan_t p) {
+    p->mod_planes = false;
+    if (p->opt.empty()) return false;
+    cudaGetLastError();
+    p->mod = false;
+    for (GraphSlot* g : {&p->g_step, &p->g_head, &p->g_body, &p->g_tail}) drop_graph(*g);
+    for (void* q : p->opt) cudaFreeAsync(q, p->st);
+    p->opt.clear();
+    for (ModBuf* b : {&p->mstep, &p->mS}) b->data = nullptr;
+    for (EWEntry& e : p->ew) e.Gm.data = nullptr;
+    p->mws = nullptr;
+    cudaStreamSynchronize(p->st);                             // (the pool gives the memory back)
+    return true;
 }
 
 // Compile one step of size h into ops (and, with fsal, its head / interior /
@@ -1232,7 +1269,8 @@ void dme::free_plan(dme_plan_t p) {
         cudaEventDestroy(r.b);
     }
     for (cudaEvent_t e : p->evpool) cudaEventDestroy(e);
-    for (void* q : p->allocs) cudaFreeAsync(q, p->st);
+    for (auto* v : {&p->allocs, &p->opt})
+        for (void* q : *v) cudaFreeAsync(q, p->st);
     if (p->st) cudaStreamSynchronize(p->st);
     if (p->own_st && p->st) cudaStreamDestroy(p->st);
     delete p;
@@ -1361,19 +1399,21 @@ dme_status dme::plan_create(const dme_plan_desc* d, const double* A, const doubl
             launch_slice_rows_f64(p->S, n, n, n, p->Ssl, st);
         }
     }
-    if (!p->split && !serving && dense_steps && n >= kModMinN) {
+    p->mod_ew = !serving && n >= kModMinN;
+    p->mod_planes = p->mod_ew && !p->split;
+    if (p->mod_planes && dense_steps) {
         bool ok = false, oks = true;
         DME_TRY(mod_alloc(p, &p->mstep, n, n, &ok));
-        if (ok) ok = palloc_t(p, &p->mws, mod_ws_bytes(n, n)) == DME_OK;
-        if (ok && gen) DME_TRY(mod_alloc(p, &p->mS, n, n, &oks));
-        if (ok && gen && oks) launch_mod_convert(p->S, n, n, n, p->mS, st);
-        p->mod = ok;
-        if (!ok) set_error("");
+        if (ok) p->mws = static_cast<uint8_t*>(palloc_opt(p, mod_ws_bytes(n, n)));
+        p->mod = p->mws != nullptr;
+        if (!p->mod) plan_release_planes(p);
+        if (p->mod && gen) DME_TRY(mod_alloc(p, &p->mS, n, n, &oks));
+        if (p->mod && gen && oks) launch_mod_convert(p->S, n, n, n, p->mS, st);
     }
     // ||[[-A^T, Q], [0, A]]||_1 for the scaling of every t
     double norms[2] = {0.0, 0.0};
     {
-        TmpPool tp(st);
+        TmpPool tp(p);
         double* work = nullptr;
         DME_TRY(tp.get(&work, block_norm1_work_doubles(n)));
         launch_block_norm1(p->A, p->Q, n, work, p->small, st);
@@ -1382,7 +1422,6 @@ dme_status dme::plan_create(const dme_plan_desc* d, const double* A, const doubl
     DME_CUDA_TRY(cudaStreamSynchronize(st));
     p->normM = norms[0];
     p->balanced = norms[1] <= 8.0;
-    p->mod_ew = !serving && n >= kModMinN;
     DME_TRY(build_ops(p, d->h));
     DME_TRY(check_status(p, "dme_plan"));
     DME_TRY(choose_pairs(p));

@@ -86,6 +86,8 @@ struct dme_plan_s {
     // operand, P or G P; of S; and the products' workspace)
     bool mod = false;          // the steps' products
     bool mod_ew = false;       // the exponential's products (its transients fit no serving budget)
+    bool mod_planes = false;   // planes may be held (until memory for something else runs out)
+    std::vector<void*> opt;    // their allocations
     bool balanced = false;     // A's row and column sums agree within 2^8 at every index
     ModBuf mstep, mS;
     uint8_t* mws = nullptr;
@@ -110,7 +112,7 @@ namespace dme {
 // Build a plan (validated descriptor; pointers host or device).  A serving plan
 // (grouped launches, which never split K: at the server's loads splitting only adds
 // units and tail work to launches that are already full) holds no split-K workspace
-// and no residue planes; nor has the plan under a factored path (dense_steps = false).
+// and no residue planes; the plan under a factored path (dense_steps = false) holds only E_t's.
 dme_status plan_create(const dme_plan_desc* d, const double* A, const double* QorC, const double* B,
                        const double* R, const double* S, void* stream, dme_plan_t* out, bool serving = false,
                        bool dense_steps = true);
@@ -127,6 +129,10 @@ dme_status plan_ew(dme_plan_t p, double t, int* idx);
 // Residue planes of E_t^T of p->ew[idx] (FP64 plans on residue products; none if they do
 // not fit in memory: the products with this E then stay on the FP64 pipe).
 dme_status plan_mod_planes(dme_plan_t p, int idx);
+// Give back every residue plane and their workspace (the products stay on the FP64 pipe from
+// then on; captured steps are captured again): called when an allocation fails.  False if
+// there was none.
+bool plan_release_planes(dme_plan_t p);
 // Report (and clear) the plan's device status word after synchronising its stream.
 dme_status plan_check(dme_plan_t p, const char* where);
 // The descriptor and pointer checks of dme_plan.
