@@ -698,7 +698,6 @@ dme_status apply_split(dme_lr_t lr, const SliceBuf& Msl, const double* X, int ld
     p.alpha = alpha;
     p.status = lr->status;
     p.ws = lr->P->kws;
-    p.ws_cnt = lr->P->kcnt;
     return launch_ozaki_gemm(Msl, lr->xsl, p, st);
 }
 

@@ -345,13 +345,14 @@ dme_status prod(int n, const ProdPath& w, const double* L, int tL, const double*
 // residual is exact to 2^-56 of its operands' rows, so X is accurate to rounding, more than
 // an elimination's.  *ok = false when the corrections do not shrink tenfold each, or M is
 // not one for FP32 at all: the caller then eliminates (launch_gj_solve).  t1 .. t4: n x n
-// scratch, t4 at least inv32_floats(n) floats.  Synchronises st.
+// scratch (t3 the inverse's work and the norms, t4 its floats).  Synchronises st.
 // n = 1024: 1.7 ms against 9.0 for the elimination (64 panels of 68 us, each a chain of 16
 // pivots over a cluster, and an FP64 rank-16 update of 60 us each).
 dme_status refined_solve(int n, ModWork& w, const double* M, const double* B, double* X, double* t1, double* t2, double* t3,
                          double* t4, cudaStream_t st, bool* ok) {
     *ok = false;
     const size_t nn = (size_t)n * n;
+    if (inv32_floats(n) > 2 * nn || inv32_work_floats(n) > 2 * nn || refine_work_doubles() > nn) return DME_OK;
     double* Y = t1;
     double* R = t2;
     double* work = t3;
@@ -461,7 +462,6 @@ dme_status split_cong(dme_plan_t p, const double* P, const SliceBuf& G, double* 
     a.Cp = p->U;
     a.status = p->status;
     a.ws = p->kws;
-    a.ws_cnt = p->kcnt;
     {
         ProfScope ps(p, DME_KIND_SPLIT_GEMM);
         DME_TRY(launch_ozaki_gemm(G, p->psl, a, st));
@@ -485,7 +485,6 @@ dme_status split_cong(dme_plan_t p, const double* P, const SliceBuf& G, double* 
     b.b3 = b3;
     b.status = p->status;
     b.ws = p->kws;
-    b.ws_cnt = p->kcnt;
     ProfScope ps(p, DME_KIND_SPLIT_GEMM);
     return launch_ozaki_gemm(G, p->usl, b, st);
 }
@@ -516,7 +515,6 @@ dme_status split_riccati(dme_plan_t p, double* P, double tau, double qcoef) {
     a.alpha = 1.0;
     a.status = p->status;
     a.ws = p->kws;
-    a.ws_cnt = p->kcnt;
     DME_TRY(launch_ozaki_gemm(p->btsl, p->psl, a, st));
     launch_transpose(p->Zt, Z, m, n, n, m, st);
     DME_TRY(launch_riccati_from_z(p->Bt, n, m, tau, p->rwork, p->status, st));
@@ -1381,8 +1379,6 @@ dme_status dme::plan_create(const dme_plan_desc* d, const double* A, const doubl
             // (n <= 1024 here), or the last partial wave of one with more tiles than SMs
             // (n > 1536; the plan's own tensor Riccati products need it in serving too)
             DME_TRY(palloc_t(p, &p->kws, OZ_SPLIT_WS_FLOAT2));
-            DME_TRY(palloc_t(p, &p->kcnt, (size_t)OZ_SPLIT_MAX_TAIL));
-            DME_CUDA_TRY(cudaMemsetAsync(p->kcnt, 0, sizeof(int) * OZ_SPLIT_MAX_TAIL, st));
         }
         if (ric && tensor_riccati(n, p->m)) {
             const int m = p->m;

@@ -81,7 +81,6 @@ struct dme_plan_s {
     SliceBuf psl, usl, Ssl;    // split path: slices of P, of U = G P, and of S
     float2* U = nullptr;       // split path: G P as normalised (hi, lo) pairs
     float2* kws = nullptr;     // split path: split-K workspace of the tail tiles
-    int* kcnt = nullptr;       // split path: split-K arrival counters
     // FP64 path from kModMinN on: products as residue products (planes of the per-step
     // operand, P or G P; of S; and the products' workspace)
     bool mod = false;          // the steps' products

@@ -83,7 +83,6 @@ struct OzParams {
     // level sums to ws, and a second kernel adds them in part order and runs the
     // epilogue.  ws: [tail tile][part][128 columns][128 rows] (level 0, levels >= 1).
     float2* ws;
-    int* ws_cnt;          // unused (kept for the layout of the grouped descriptors)
     int split_first;      // set by the launcher
     int split_parts;      // set by the launcher (1: no split)
     // accurate mode: [chunk][M][N] doubles of the per-chunk products (chunks of
