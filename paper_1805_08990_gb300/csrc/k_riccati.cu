@@ -9,7 +9,7 @@
 // Kernels: (1) Z = P Bt with per-block partial Gram sums Bt^T Z, (2) M from the
 // partials (deterministic reduction order), its Cholesky and L^{-1} (FP64; in
 // registers for m <= 8), (3) Y = Z L^{-T}, (4) the rank-m update
-// P <- P - t Y Y^T (+ q Q); for m <= 8 (4) forms the rows of Y it needs by itself.
+// P <- P - t Y Y^T (+ q Q); where that is little work (4) forms the rows of Y it needs itself.
 // Each kernel takes a batch of independent problems (grouped launch): the
 // blocks of every problem are laid end to end and each block finds its
 // problem by a binary search over the per-problem block offsets, so a
@@ -25,18 +25,28 @@
 
 namespace dme {
 
-constexpr int RZ_ROWS = 4;      // rows of P per block in kernel (1): two warps each
 constexpr int RZ_MB = 8;        // columns of Bt per pass
+constexpr int RZ_DIRECT = 4;    // most columns of Bt read as they lie
+constexpr int RZ_WIDE = 1700;   // kernel (1) takes eight rows a block from this n on, if it stages Bt
 constexpr int RU_TILE = 32;     // update tile
-constexpr int RU_FUSE = 8;      // largest m whose Y the update forms itself
+constexpr int RS_SUM = 8;       // largest m whose partial Gram sums one block adds
+// Whether the update forms the rows of Y it needs from Z and L^{-1} (n^2 m (m + 1) / 64 FMAs
+// more) or reads those of a launch of its own (5 to 8 us).  T3, us, formed / read: n = 625, m = 8
+// 49.1 / 49.9; n = 1024, m = 5 49.3 / 49.8, m = 8 72.3 / 68.3; n = 1500, m = 4 61.9 / 60.3, m = 8 111 / 102;
+// n = 2025, m = 3 72.3 / 72.3, m = 4 95.5 / 91.8; n = 4096, m = 2 188 / 185, m = 8 588 / 490.
+inline bool ru_fused(int n, int m) { return m <= 8 && (long long)n * n * (m * (m + 1)) <= 50000000; }
 
 constexpr int RZ_PARTS = 608;   // most blocks of kernel (1), and so most partial Gram matrices
-__host__ __device__ __forceinline__ int rz_groups(int n) { return (n + RZ_ROWS - 1) / RZ_ROWS; }
-__host__ __device__ __forceinline__ int rz_blocks(int n) { return rz_groups(n) < RZ_PARTS ? rz_groups(n) : RZ_PARTS; }
+// Rows of P per block and step in kernel (1): four with two warps each, or eight with one.
+inline int rz_rows(int n, int m) { return m > RZ_DIRECT && n >= RZ_WIDE ? 8 : 4; }
+inline int rz_groups(int n, int m) { return (n + rz_rows(n, m) - 1) / rz_rows(n, m); }
+inline int rz_blocks(int n, int m) {
+    return rz_groups(n, m) < RZ_PARTS ? rz_groups(n, m) : RZ_PARTS;
+}
 
 size_t riccati_work_doubles(int n, int m) {
     // Z (n m) | Y (n m) | Gpart (blocks m m) | Linv (m m)
-    return (size_t)2 * n * m + (size_t)rz_blocks(n) * m * m + (size_t)m * m + 8;
+    return (size_t)2 * n * m + (size_t)rz_blocks(n, m) * m * m + (size_t)m * m + 8;
 }
 
 // One problem of a (possibly grouped) Riccati update; the block-prefix fields
@@ -53,7 +63,17 @@ struct RicDesc {
     int n, m;
     int* status;
     int sz, sy, su;     // first block of this problem in the z, y and update grids
+    unsigned short parts;           // rz_blocks, rz_rows, ru_fused (ric_shape)
+    unsigned char rows, fused;
 };
+
+static void ric_shape(RicDesc& d, int n, int m) {
+    d.n = n;
+    d.m = m;
+    d.parts = (unsigned short)rz_blocks(n, m);
+    d.rows = (unsigned char)rz_rows(n, m);
+    d.fused = ru_fused(n, m);
+}
 
 constexpr int kRicLocal = 8;
 struct RicBatch {
@@ -77,28 +97,30 @@ __device__ __forceinline__ int ric_find(const RicDesc* d, int nd, int blk) {
     return lo;
 }
 
-// (1) Z[r][c] = sum_k P[r][k] Bt[k][c], four rows at a time (row groups b, b + gridDim, ...),
-// two warps a row (each half of the row's 64-column steps, the halves added in order), and
-// the block's partial Gram sums Gpart[b][i][c] = sum_{its rows} Bt[r][i] Z[r][c], one entry
-// a thread, in a fixed order (deterministic, no atomics).  MB columns per pass.
+// (1) Z[r][c] = sum_k P[r][k] Bt[k][c], four or eight rows at a time (rz_rows; row groups b,
+// b + gridDim, ...), two warps or one a row (each of two on half of the row's 64-column steps,
+// the halves added in order), and the block's partial Gram sums Gpart[b][i][c] =
+// sum_{its rows} Bt[r][i] Z[r][c], one entry a thread, in a fixed order (deterministic, no
+// atomics).  MB columns per pass.
 // Bound: the FP64 pipe (two FMAs per SM and cycle): n^2 m FMAs, so a pass computes no
 // column that is not there, and four rows a block give n / 4 blocks; at most RZ_PARTS of
 // them, since one block adds the partial sums (n = 4096, m = 8, 1024 of them: 16 us of its FP64 pipe).
 // Up to four columns of Bt are read as they lie; more of them, at a stride of m doubles per
 // lane, would keep L1 busier than the FP64 pipe (n = 4096, m = 8: 535 us), so they are staged
-// column by column in pairs: sB[c][k / 2] = (Bt[k][c], Bt[k + 1][c]) (344 us; the FP64
-// pipe alone 223).
-constexpr int RZ_KC = 512;
+// column by column in pairs: sB[c][k / 2] = (Bt[k][c], Bt[k + 1][c]).  Eight rows then share a
+// staging, where there are blocks enough (T3, m = 8, four rows / eight: n = 1500 115 / 123 us, 1700
+// 131 / 138, 1849 178 / 152, 2025 206 / 171, 4096 626 / 612; m = 32: n = 1500 535 / 505, 2025 717 / 700).
+constexpr int RZ_KC = 512, RZ_SB = RZ_KC / 2 + 1;    // (+ 1: the columns' stores in different banks)
 
-template <int MB, bool STAGED>
-__device__ __forceinline__ void riccati_z_row(const RicDesc& d, int row, int half, int lane, int c0, int kbeg, int kend,
-                                              const double2 (*sB)[RZ_KC / 2], double (&acc)[RZ_MB]) {
+template <int MB, bool STAGED, int KSTEP>
+__device__ __forceinline__ void riccati_z_row(const RicDesc& d, int row, int kfirst, int c0, int kbeg, int kend,
+                                              const double2 (*sB)[RZ_SB], double (&acc)[RZ_MB]) {
     const int n = d.n, m = d.m;
     const double* __restrict__ prow = d.P + (size_t)row * n;
     const double* __restrict__ Bt = d.Bt + c0;
     const bool vec = (n % 2) == 0;
 #pragma unroll 2
-    for (int k = kbeg + 2 * lane + 64 * half; k < kend; k += 128) {
+    for (int k = kbeg + kfirst; k < kend; k += KSTEP) {
         const bool two = k + 1 < kend;
         double p0, p1 = 0.0;
         if (vec) {
@@ -125,36 +147,41 @@ __device__ __forceinline__ void riccati_z_row(const RicDesc& d, int row, int hal
     }
 }
 
+// WIDE: eight rows a block, a warp each; else four with two warps each.  A batch of both kinds
+// takes two launches, in which the other kind's blocks return at once.
+template <bool WIDE>
 __global__ void __launch_bounds__(256) riccati_z_kernel(const __grid_constant__ RicBatch batch) {
     pdl_trigger();
     pdl_wait();
-    __shared__ double2 sB[RZ_MB][RZ_KC / 2];
-    __shared__ double sH[2 * RZ_ROWS][RZ_MB];
-    __shared__ double sZ[RZ_ROWS][RZ_MB];
+    __shared__ double2 sB[RZ_MB][RZ_SB];
+    __shared__ double sH[8][RZ_MB], sZ[WIDE ? 8 : 4][RZ_MB];
     const RicDesc* ds = ric_descs(batch);
     const int ip = ric_find<0>(ds, batch.nd, blockIdx.x);
     const RicDesc& d = ds[ip];
     const int lb = blockIdx.x - d.sz;
     const int n = d.n, m = d.m;
+    constexpr int ROWS = WIDE ? 8 : 4, KSTEP = WIDE ? 64 : 128;
+    if (d.rows != ROWS) return;
     const double* __restrict__ Bt = d.Bt;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, tid = threadIdx.x;
-    const int parts = rz_blocks(n), groups = rz_groups(n);
+    const int parts = d.parts, groups = (n + ROWS - 1) / ROWS;
+    const int kfirst = 2 * lane + (WIDE ? 0 : 64 * (warp & 1));
     for (int c0 = 0; c0 < m; c0 += RZ_MB) {
         const int mb = min(RZ_MB, m - c0);
         const int gi = tid / mb, gj = tid % mb;               // this thread's Gram entry (m mb <= 256)
         double gram = 0.0;
         for (int g = lb; g < groups; g += parts) {
-            const int row = g * RZ_ROWS + (warp >> 1);
+            const int row = g * ROWS + (WIDE ? warp : warp >> 1);
             double acc[RZ_MB];
 #pragma unroll
             for (int c = 0; c < RZ_MB; ++c) acc[c] = 0.0;
-            if (mb <= 4) {
+            if (mb <= RZ_DIRECT) {
                 if (row < n) {
                     switch (mb) {
-                        case 1: riccati_z_row<1, false>(d, row, warp & 1, lane, c0, 0, n, sB, acc); break;
-                        case 2: riccati_z_row<2, false>(d, row, warp & 1, lane, c0, 0, n, sB, acc); break;
-                        case 3: riccati_z_row<3, false>(d, row, warp & 1, lane, c0, 0, n, sB, acc); break;
-                        default: riccati_z_row<4, false>(d, row, warp & 1, lane, c0, 0, n, sB, acc); break;
+                        case 1: riccati_z_row<1, false, KSTEP>(d, row, kfirst, c0, 0, n, sB, acc); break;
+                        case 2: riccati_z_row<2, false, KSTEP>(d, row, kfirst, c0, 0, n, sB, acc); break;
+                        case 3: riccati_z_row<3, false, KSTEP>(d, row, kfirst, c0, 0, n, sB, acc); break;
+                        default: riccati_z_row<4, false, KSTEP>(d, row, kfirst, c0, 0, n, sB, acc); break;
                     }
                 }
             } else {
@@ -171,10 +198,10 @@ __global__ void __launch_bounds__(256) riccati_z_kernel(const __grid_constant__ 
                     if (row >= n) continue;
                     const int kend = min(n, k0 + RZ_KC);
                     switch (mb) {
-                        case 5: riccati_z_row<5, true>(d, row, warp & 1, lane, c0, k0, kend, sB, acc); break;
-                        case 6: riccati_z_row<6, true>(d, row, warp & 1, lane, c0, k0, kend, sB, acc); break;
-                        case 7: riccati_z_row<7, true>(d, row, warp & 1, lane, c0, k0, kend, sB, acc); break;
-                        default: riccati_z_row<8, true>(d, row, warp & 1, lane, c0, k0, kend, sB, acc); break;
+                        case 5: riccati_z_row<5, true, KSTEP>(d, row, kfirst, c0, k0, kend, sB, acc); break;
+                        case 6: riccati_z_row<6, true, KSTEP>(d, row, kfirst, c0, k0, kend, sB, acc); break;
+                        case 7: riccati_z_row<7, true, KSTEP>(d, row, kfirst, c0, k0, kend, sB, acc); break;
+                        default: riccati_z_row<8, true, KSTEP>(d, row, kfirst, c0, k0, kend, sB, acc); break;
                     }
                 }
             }
@@ -187,16 +214,20 @@ __global__ void __launch_bounds__(256) riccati_z_kernel(const __grid_constant__ 
                 if (lane == 0) sH[warp][c] = v;
             }
             __syncthreads();
-            if (tid < RZ_ROWS * mb) {
-                const int r = tid / mb, c = tid % mb, rr = g * RZ_ROWS + r;
-                const double v = rr < n ? sH[2 * r][c] + sH[2 * r + 1][c] : 0.0;
+            if (tid < ROWS * mb) {
+                const int r = tid / mb, c = tid % mb, rr = g * ROWS + r;
+                double v = 0.0;
+                if (rr < n) {
+                    if constexpr (WIDE) v = sH[r][c];
+                    else v = sH[2 * r][c] + sH[2 * r + 1][c];
+                }
                 sZ[r][c] = v;
                 if (rr < n) d.Z[(size_t)rr * m + c0 + c] = v;
             }
             __syncthreads();
             if (gi < m)
-                for (int r = 0; r < RZ_ROWS; ++r) {
-                    const int rr = g * RZ_ROWS + r;
+                for (int r = 0; r < ROWS; ++r) {
+                    const int rr = g * ROWS + r;
                     if (rr < n) gram = fma(Bt[(size_t)rr * m + gi], sZ[r][gj], gram);
                 }
         }
@@ -205,11 +236,37 @@ __global__ void __launch_bounds__(256) riccati_z_kernel(const __grid_constant__ 
     }
 }
 
+// (1c) For m > RS_SUM: the partial sums added over the whole chip, 32 entries a block, a warp
+// per eighth of the parts, into part 0; in one block their m^2 FP64 adds a part kept that SM's pipe
+// busy for 0.27 us each (n = 2025, m = 32: 254 us with the factor, 70 with this launch).
+__global__ void __launch_bounds__(256) riccati_gsum_kernel(const __grid_constant__ RicBatch batch) {
+    pdl_trigger();
+    pdl_wait();
+    __shared__ double sums[8][32];
+    const RicDesc& d = ric_descs(batch)[blockIdx.y];
+    const int E = d.m * d.m, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, e = blockIdx.x * 32 + lane;
+    if (d.m <= RS_SUM || blockIdx.x * 32 >= E) return;
+    const int parts = d.parts;
+    double s = 0.0;
+    if (e < E) {
+#pragma unroll 8
+        for (int b = warp; b < parts; b += 8) s += d.Gpart[(size_t)b * E + e];
+    }
+    sums[warp][lane] = s;
+    __syncthreads();
+    if (warp == 0 && e < E) {
+        for (int w = 1; w < 8; ++w) s += sums[w][lane];
+        d.Gpart[e] = s;
+    }
+}
+
 // Threads of riccati_small_kernel for a problem: few partial sums leave most of 1024 threads
 // nothing but the tree over them; many need the loads in flight (n = 4096, m = 8: 35 us with
 // 256 threads, 20 with 1024).  The order of the sums follows from it, not from the launch's
 // size, so a problem gives the same bits alone and in a batch.
-__host__ __device__ __forceinline__ int rs_threads(int n, int m) { return m <= 16 && rz_blocks(n) * m * m <= 4096 ? 256 : 1024; }
+__host__ __device__ __forceinline__ int rs_threads(int parts, int m) {
+    return m <= 16 && (m > RS_SUM ? 1 : parts) * m * m <= 4096 ? 256 : 1024;
+}
 
 // M = I + t (G + G^T) / 2 for m <= RS_MAX, its Cholesky and L^{-1} in one warp: row `lane` of
 // M in registers, the pivot row handed out by shuffles (through shared memory, with the
@@ -258,10 +315,10 @@ __global__ void __launch_bounds__(1024) riccati_small_kernel(const __grid_consta
     __shared__ double L[32][33];
     const RicDesc& d = ric_descs(batch)[blockIdx.x];
     const int m = d.m;
-    const int nblocks = rz_blocks(d.n);
+    const int nblocks = m > RS_SUM ? 1 : d.parts;
     const double t = d.t;
     const int E = m * m;
-    const int G = max(1, rs_threads(d.n, m) / E);
+    const int G = max(1, rs_threads(nblocks, m) / E);
     const int tid = threadIdx.x;
     const int e = tid % E, g = tid / E;
     double sacc = 0.0;
@@ -329,13 +386,13 @@ __global__ void riccati_gpart_kernel(const __grid_constant__ RicBatch batch) {
     const RicDesc* ds = ric_descs(batch);
     const RicDesc& d = ds[ric_find<0>(ds, batch.nd, blockIdx.x)];
     const int lb = blockIdx.x - d.sz, n = d.n, m = d.m;
-    const int parts = rz_blocks(n), groups = rz_groups(n);
+    const int parts = d.parts, rows = d.rows, groups = (n + rows - 1) / rows;
     for (int e = threadIdx.x; e < m * m; e += blockDim.x) {
         const int i = e / m, c = e % m;
         double sacc = 0.0;
         for (int g = lb; g < groups; g += parts)
-            for (int r = 0; r < RZ_ROWS; ++r) {
-                const int rr = g * RZ_ROWS + r;
+            for (int r = 0; r < rows; ++r) {
+                const int rr = g * rows + r;
                 if (rr < n) sacc = fma(d.Bt[(size_t)rr * m + i], d.Z[(size_t)rr * m + c], sacc);
             }
         d.Gpart[(size_t)lb * m * m + e] = sacc;
@@ -367,8 +424,8 @@ __global__ void riccati_y_kernel(const __grid_constant__ RicBatch batch) {
 // the 32 x 32 tiles on or above the diagonal are computed: each reads its
 // upper block of P, writes it, and for an off-diagonal tile also writes the
 // transposed block below the diagonal from a shared-memory copy (coalesced).
-// Half of the FP64 work and of the traffic on P of a full update.  Problems of
-// m <= RU_FUSE form the Y rows of the tile from Z and Linv here (m (m + 1) FMAs per
+// Half of the FP64 work and of the traffic on P of a full update.  Fused problems
+// (ru_fused) form the Y rows of the tile from Z and Linv here (m (m + 1) FMAs per
 // row against 32 m of the tile's own), which saves them a launch.  The tile's entries
 // of P (and Q) are loaded together before the first is stored: one by one, each load
 // waited behind the store before it (64-wide tiles, n = 81: 16 us).
@@ -400,7 +457,7 @@ __global__ void __launch_bounds__(256) riccati_update_kernel(const __grid_consta
         pv[h] = in ? d.P[off] : 0.0;
         qv[h] = in && d.Qadd ? d.Qadd[off] : 0.0;
     }
-    const bool fuse = m <= RU_FUSE;
+    const bool fuse = d.fused != 0;
     for (int e = threadIdx.x; e < RU_TILE * m; e += blockDim.x) {
         const int r = e / m, c = e % m;
         const int gi = i0 + r, gj = j0 + r;
@@ -440,13 +497,13 @@ dme_status launch_riccati_from_z(const double* Bt, int n, int m, double t, doubl
     d.Z = work;
     d.Y = d.Z + (size_t)n * m;
     d.Gpart = d.Y + (size_t)n * m;
-    d.Linv = d.Gpart + (size_t)rz_blocks(n) * m * m;
+    d.Linv = d.Gpart + (size_t)rz_blocks(n, m) * m * m;
     d.t = t;
-    d.n = n;
-    d.m = m;
+    ric_shape(d, n, m);
     d.status = status;
-    DME_CUDA_TRY(pdl_launch(riccati_gpart_kernel, rz_blocks(n), 64, 0, st, b));
-    DME_CUDA_TRY(pdl_launch(riccati_small_kernel, 1, rs_threads(n, m), 0, st, b));
+    DME_CUDA_TRY(pdl_launch(riccati_gpart_kernel, rz_blocks(n, m), 64, 0, st, b));
+    if (m > RS_SUM) DME_CUDA_TRY(pdl_launch(riccati_gsum_kernel, (m * m + 31) / 32, 256, 0, st, b));
+    DME_CUDA_TRY(pdl_launch(riccati_small_kernel, 1, rs_threads(d.parts, m), 0, st, b));
     DME_CUDA_TRY(pdl_launch(riccati_y_kernel, (n + 127) / 128, 128, 0, st, b));
     return DME_OK;
 }
@@ -480,17 +537,16 @@ dme_status launch_riccati_grouped(const std::vector<RicItem>& items, void* dev_d
         d.Z = it.work;
         d.Y = d.Z + (size_t)n * m;
         d.Gpart = d.Y + (size_t)n * m;
-        d.Linv = d.Gpart + (size_t)rz_blocks(n) * m * m;
+        d.Linv = d.Gpart + (size_t)rz_blocks(n, m) * m * m;
         d.Qadd = it.Qadd;
         d.t = it.t;
         d.q = it.q;
-        d.n = n;
-        d.m = m;
+        ric_shape(d, n, m);
         d.status = it.status;
         d.sz = sz;
         d.sy = sy;
         d.su = su;
-        sz += rz_blocks(n);
+        sz += rz_blocks(n, m);
         sy += (n + 127) / 128;
         const int tn = (n + RU_TILE - 1) / RU_TILE;
         su += tn * (tn + 1) / 2;
@@ -515,13 +571,18 @@ dme_status launch_riccati_grouped(const std::vector<RicItem>& items, void* dev_d
         b.dev = reinterpret_cast<const RicDesc*>(dev_desc);
     }
     int mmax = 0, threads = 256;
+    bool y = false, wide = false, narrow = false;
     for (const RicItem& it : items) {
+        (rz_rows(it.n, it.m) == 8 ? wide : narrow) = true;
         mmax = std::max(mmax, it.m);
-        threads = std::max(threads, rs_threads(it.n, it.m));
+        y = y || !ru_fused(it.n, it.m);
+        threads = std::max(threads, rs_threads(rz_blocks(it.n, it.m), it.m));
     }
-    DME_CUDA_TRY(pdl_launch(riccati_z_kernel, sz, 256, 0, st, b));
+    if (narrow) DME_CUDA_TRY(pdl_launch(riccati_z_kernel<false>, sz, 256, 0, st, b));
+    if (wide) DME_CUDA_TRY(pdl_launch(riccati_z_kernel<true>, sz, 256, 0, st, b));
+    if (mmax > RS_SUM) DME_CUDA_TRY(pdl_launch(riccati_gsum_kernel, dim3((mmax * mmax + 31) / 32, b.nd), 256, 0, st, b));
     DME_CUDA_TRY(pdl_launch(riccati_small_kernel, b.nd, threads, 0, st, b));
-    if (mmax > RU_FUSE) DME_CUDA_TRY(pdl_launch(riccati_y_kernel, sy, 128, 0, st, b));
+    if (y) DME_CUDA_TRY(pdl_launch(riccati_y_kernel, sy, 128, 0, st, b));
     DME_CUDA_TRY(pdl_launch(riccati_update_kernel, su, 256, 0, st, b));
     DME_CUDA_TRY(cudaGetLastError());
     return DME_OK;
@@ -566,6 +627,11 @@ __global__ void lqr_gain_hist_kernel(const double* __restrict__ Z, const double*
 
 __global__ void counter_inc_kernel(int* ctr) { *ctr += 1; }
 
+static void launch_z(const RicBatch& b, int n, int m, cudaStream_t st) {
+    if (rz_rows(n, m) == 8) riccati_z_kernel<true><<<rz_blocks(n, m), 256, 0, st>>>(b);
+    else riccati_z_kernel<false><<<rz_blocks(n, m), 256, 0, st>>>(b);
+}
+
 dme_status launch_lqr_gain_hist(const double* P, const double* Bt, const double* LR, int n, int m, double* work,
                                 double* Kbase, int* ctr, int cap, cudaStream_t st) {
     RicBatch b;
@@ -576,10 +642,9 @@ dme_status launch_lqr_gain_hist(const double* P, const double* Bt, const double*
     d.Z = work;
     d.Y = d.Z + (size_t)n * m;
     d.Gpart = d.Y + (size_t)n * m;
-    d.n = n;
-    d.m = m;
+    ric_shape(d, n, m);
     b.nd = 1;
-    riccati_z_kernel<<<rz_blocks(n), 256, 0, st>>>(b);       // Z = P Bt (P is only read)
+    launch_z(b, n, m, st);                                   // Z = P Bt (P is only read)
     lqr_gain_hist_kernel<<<(n + 127) / 128, 128, 0, st>>>(d.Z, LR, Kbase, n, m, ctr, cap);
     counter_inc_kernel<<<1, 1, 0, st>>>(ctr);
     DME_CUDA_TRY(cudaGetLastError());
@@ -596,10 +661,9 @@ dme_status launch_lqr_gain(const double* P, const double* Bt, const double* LR, 
     d.Z = work;
     d.Y = d.Z + (size_t)n * m;
     d.Gpart = d.Y + (size_t)n * m;
-    d.n = n;
-    d.m = m;
+    ric_shape(d, n, m);
     b.nd = 1;
-    riccati_z_kernel<<<rz_blocks(n), 256, 0, st>>>(b);       // Z = P Bt (P is only read)
+    launch_z(b, n, m, st);                                   // Z = P Bt (P is only read)
     lqr_gain_kernel<<<(n + 127) / 128, 128, 0, st>>>(d.Z, LR, K, n, m);
     DME_CUDA_TRY(cudaGetLastError());
     return DME_OK;
