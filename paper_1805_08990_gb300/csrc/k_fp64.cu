@@ -194,10 +194,19 @@ __device__ __forceinline__ void gemm64_load8(const GemmProb& pb, int row0, int c
     }
 }
 
+// Overlapped starts pay while a launch is about as short as its start (plan of n = 100, s = 17
+// doublings, overlapped / not: 1700 / 1885 us, n = 128, 256 blocks, 1992 / 2093); the early blocks of
+// larger grids slow the one they wait for (n = 150, 361 blocks, 2727 / 2476; n = 191, 576
+// blocks, 4048 / 3031).
+constexpr int G8_PDL_BLOCKS = 304;
+
+template <bool OVERLAP>
 __global__ void __launch_bounds__(64) gemm64_small_kernel(const __grid_constant__ GemmProb pb) {
     __shared__ double As[G8_K][G8 + 1], Bs[G8_K][G8 + 1];
-    pdl_trigger();
-    pdl_wait();
+    if (OVERLAP) {
+        pdl_trigger();
+        pdl_wait();
+    }
     int ti, tj;
     tile_coords(pb, blockIdx.x, ti, tj);
     const int row0 = ti * G8, col0 = tj * G8, tx = threadIdx.x & 7, ty = threadIdx.x >> 3;
@@ -233,7 +242,13 @@ dme_status gemm64_small(const GemmProb& g, cudaStream_t st) {
     GemmProb pb = g;
     const int tm = (g.M + G8 - 1) / G8, tn = (g.N + G8 - 1) / G8;
     pb.tiles_n = tn;
-    DME_CUDA_TRY(pdl_launch(gemm64_small_kernel, g.tri ? tn * (tn + 1) / 2 : tm * tn, 64, 0, st, pb));
+    const int blocks = g.tri ? tn * (tn + 1) / 2 : tm * tn;
+    if (blocks <= G8_PDL_BLOCKS) {
+        DME_CUDA_TRY(pdl_launch(gemm64_small_kernel<true>, blocks, 64, 0, st, pb));
+    } else {
+        gemm64_small_kernel<false><<<blocks, 64, 0, st>>>(pb);
+        DME_CUDA_TRY(cudaGetLastError());
+    }
     return DME_OK;
 }
 

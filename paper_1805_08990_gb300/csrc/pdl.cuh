@@ -5,7 +5,7 @@
 // that one waited too, everything before it).  pdl_trigger lets the successor begin
 // launching; after a plain launch both are no-ops.  The chains of a composition step are a
 // few microseconds per kernel, of which launch latency and block start-up are a part (DRE
-// n = 81: 47.6 -> 44.3 us a step).  Used for the small FP64 products and T3 only: in the
+// n = 81: 47.6 -> 44.3 us a step).  Used for T3 and the FP64 products of few blocks only: in the
 // chains of the tensor kernels the early blocks cost more than they saved (DRE n = 1024
 // split, 64 steps: 11.8 -> 13.5 ms; DLE n = 256 FP64, 100 steps: 6.3 -> 6.8 ms).
 #pragma once
