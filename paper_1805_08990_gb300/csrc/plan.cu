@@ -280,8 +280,17 @@ dme_status acc_setup(TmpPool& tp, int n, int* status, AccWork* w) {
 
 // Plans from this size on run their FP64 products as residue products (k_mod.cu): the
 // steps' of an FP64 plan, and the exponential's (squarings included) of any plan that is
-// not built inside a serving budget.
+// not built inside a serving budget.  T12 step / whole plan, us, residues against the FP64 pipe: n = 144
+// 34 / 26 and (160) 1741 / 1933, n = 169 34 / 33, n = 196 34 / 39 and (192) 1751 / 2301, n = 256 34 / 59 and
+// 1853 / 3109.  (A state localised around one node, whose products are recomputed on the FP64 pipe,
+// takes 123 us at n = 196, 144 at 256, 272 at 400; n = 400 is 360 on the FP64 pipe alone.)
 constexpr int kModMinN = 192;
+// An unbalanced A's exponential, whose solves eliminate and whose products are all certified and
+// then often recomputed, takes residues where its products no longer fit the 8-wide tiles of
+// gemm1.  Plans of graded A (row against column sums 2^16 / 2^40 apart), residues / FP64 pipe, us:
+// n = 192 4510 / 2852 and 9047 / 3973, n = 300 6355 / 5552 and 13278 / 8724, n = 350 7156 / 7597 and
+// 16092 / 12455, n = 400 8263 / 14600 and 19608 / 26184.
+constexpr int kModMinUnbalanced = 385;
 
 // The exponential's residue products: planes of the left and the right operand,
 // transpose scratch, workspace.
@@ -490,10 +499,12 @@ dme_status split_cong(dme_plan_t p, const double* P, const SliceBuf& G, double* 
 }
 
 // Whether T3 of a split plan runs its products on the tensor cores.  That costs a slicing
-// of P whatever m is, the FP64 kernels 3 n^2 m flops (us, tensor / FP64: n = 1600, m = 1 86 / 31,
-// m = 4 93 / 63, m = 8 104 / 120; n = 2025, m = 4 105 / 95, m = 6 109 / 150; n = 3600, m = 4
-// 217 / 216; n = 4096, m = 2 260 / 187, m = 4 266 / 286, m = 8 281 / 620).  Below 1537 serving,
-// which uses the FP64 kernels, stays bit-identical to single plans.
+// of P whatever m is, the FP64 kernels 3 n^2 m flops (us, tensor / FP64: n = 1600, m = 4 93 / 64,
+// m = 5 97 / 76, m = 6 99 / 89, m = 8 103 / 108; n = 2025, m = 4 105 / 96, m = 5 109 / 105, m = 6 109 / 125;
+// n = 3000, m = 4 155 / 155, m = 5 159 / 193; n = 3600, m = 4 215 / 216; n = 4096, m = 3 265 / 216, m = 4 267 /
+// 268 to 285, m = 8 281 / 511).  m = 5 .. 7 below n of about 2000 would gain up to 20 us of a step of a
+// millisecond on the FP64 kernels; the line is by m alone.  Up to n = 1536 single plans and
+// served ones take the same T3 kernels.
 bool tensor_riccati(int n, int m) { return n > 1536 && (m > 4 || (m == 4 && n > 3600)); }
 
 // T3 on the split path (tensor_riccati): Z^T = Bt^T P (P symmetric) on the tensor
@@ -590,7 +601,7 @@ dme_status compute_ew(dme_plan_t p, double tau, int* idx) {
     DME_TRY(palloc_t(p, &ent.W, nn));
     // residue products, if their planes fit in memory
     ModWork modw;
-    if (p->mod_ew) {
+    if (p->mod_ew && (p->balanced || n >= kModMinUnbalanced)) {
         if (mod_setup(tmod, n, p->status, &modw) == DME_OK) {
             modw.balanced = p->balanced;
             pp.mod = &modw;
