@@ -54,7 +54,13 @@ typedef enum { DME_LIE = 1, DME_STRANG = 2 } dme_comp;
  *   of the steps and of the exponential are exact residue products of integer
  *   rows on the tensor cores, rounded once, each entry certified to the error
  *   bound of a float64 sum (K u sum |a b|) or recomputed as one; smaller ones,
- *   served requests and the rest run on the FP64 pipe.
+ *   the exponential of an unbalanced A (dme_plan) up to n = 384, served requests
+ *   and the rest run on the FP64 pipe.  Not certified are the powers and squares
+ *   of a balanced A's exponential and the products of its refined solves: E_t is
+ *   then accurate in norm, and an entry far below its row's and column's largest
+ *   holds fewer digits (as after an elimination).  Residue planes are held only
+ *   while memory allows: a plan that runs out of it gives them back and keeps its
+ *   products on the FP64 pipe.
  * DME_SPLIT_TF32: reserved; not built.  A TF32 slice carries an 11-bit digit,
  *   so the fp32 tensor-core sum of K products of two such digits is exact
  *   only for K <= 4; plans asking for it fail with DME_EINVAL and say so in

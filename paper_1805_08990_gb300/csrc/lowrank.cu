@@ -187,7 +187,9 @@ dme_status gemm(dme_lr_t lr, const GemmProb& g, cudaStream_t st) {
     }
     const long tiles64 = (long)((g.M + 63) / 64) * ((g.N + 63) / 64);
     if (tiles64 <= 16 && g.K >= 1024) return gemm_ws(lr, g, st);
-    // few 32-wide tiles (the r x r products): 8-wide ones, over all SMs
+    // few 32-wide tiles (the r x r products): 8-wide ones, over all SMs (whole solves, us, never / up
+    // to 76 / 152 / 304 tiles: n = 400, rank 50 8380 / 4608 / 4600 / 4592; n = 2304, rank 49 6549 / 5732 / 5742 /
+    // 5712; rank 120 17079 / 14085 / 14086 / 13572)
     if ((long)((g.M + 31) / 32) * ((g.N + 31) / 32) <= 76) return gemm64_small(g, st);
     std::vector<GemmProb> v{g};
     return gemm64_grouped(v, nullptr, st, nullptr, g.N <= 64 ? 32 : 64);
@@ -303,6 +305,8 @@ dme_status compress_state(dme_lr_t lr, bool last) {
     // (n = 3600: 122 -> 60) and a graded Gram matrix near its eigenbasis, on which both
     // Jacobi passes take fewer sweeps (3.27 + 0.71 ms -> 1.07 + 0.3; r = 57: 1.15 + 0.58 ->
     // 0.75 + 0.30) for 0.2 ms
+    // (solve of one or two steps, n = 1024, us, always / from 16 columns on / never: final rank 1
+    // 253 / 205 / 206, rank 8 644 / 663 / 654, rank 12 771 / 767 / 890, rank 16 903 / 911 / 1022)
     if (lr->r >= 16) DME_TRY(compress_qlp(lr, 0.01 * lr->tol));
     lr->loose = false;
     return compress(lr, lr->L, lr->L2, lr->d, lr->rcap, lr->r);
