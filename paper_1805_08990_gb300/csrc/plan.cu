@@ -59,6 +59,7 @@ dme_status palloc(dme_plan_t p, void** out, size_t bytes) {
         return DME_ENOMEM;
     }
     p->allocs.push_back(*out);
+    p->sizes.push_back(bytes);
     p->bytes += bytes;
     return DME_OK;
 }
@@ -71,6 +72,7 @@ void* palloc_opt(dme_plan_t p, size_t bytes) {
         return nullptr;
     }
     p->opt.push_back(q);
+    p->opt_bytes += bytes;
     return q;
 }
 
@@ -112,7 +114,10 @@ struct AllocMark {
     size_t n;
     explicit AllocMark(dme_plan_t plan) : p(plan), n(plan->allocs.size()) {}
     ~AllocMark() {
-        for (; p->allocs.size() > n; p->allocs.pop_back()) cudaFreeAsync(p->allocs.back(), p->st);
+        for (; p->allocs.size() > n; p->allocs.pop_back(), p->sizes.pop_back()) {
+            cudaFreeAsync(p->allocs.back(), p->st);
+            p->bytes -= p->sizes.back();
+        }
     }
 };
 
@@ -1083,6 +1088,7 @@ bool dme::plan_release_planes(dme_plan_t p) {
     for (GraphSlot* g : {&p->g_step, &p->g_head, &p->g_body, &p->g_tail}) drop_graph(*g);
     for (void* q : p->opt) cudaFreeAsync(q, p->st);
     p->opt.clear();
+    p->opt_bytes = 0;
     for (ModBuf* b : {&p->mstep, &p->mS}) b->data = nullptr;
     for (EWEntry& e : p->ew) e.Gm.data = nullptr;
     p->mws = nullptr;
@@ -1767,7 +1773,7 @@ dme_status dme_solve(dme_plan_t plan, const double* P0, double T, int nsteps, do
     });
 }
 
-size_t dme_plan_bytes(dme_plan_t plan) { return plan ? plan->bytes : 0; }
+size_t dme_plan_bytes(dme_plan_t plan) { return plan ? plan->bytes + plan->opt_bytes : 0; }
 
 dme_status dme_plan_destroy(dme_plan_t plan) {
     free_plan(plan);

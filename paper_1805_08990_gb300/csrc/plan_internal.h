@@ -71,6 +71,7 @@ struct dme_plan_s {
     double* xacc = nullptr;    // extrapolated scheme: accumulator state (n x n)
     double* xwork = nullptr;   // extrapolated scheme with q >= 3: work state (n x n)
     std::vector<void*> allocs;
+    std::vector<size_t> sizes;   // of allocs
     size_t bytes = 0;
     GraphSlot g_step, g_head, g_body, g_tail;
     bool split = false;
@@ -87,6 +88,7 @@ struct dme_plan_s {
     bool mod_ew = false;       // the exponential's products (its transients fit no serving budget)
     bool mod_planes = false;   // planes may be held (until memory for something else runs out)
     std::vector<void*> opt;    // their allocations
+    size_t opt_bytes = 0;
     bool balanced = false;     // A's row and column sums agree within 2^8 at every index
     ModBuf mstep, mS;
     uint8_t* mws = nullptr;

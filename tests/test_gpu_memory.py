@@ -61,3 +61,27 @@ def test_plan_fits_without_planes(kind, free_mb):
         del fill
         torch.cuda.empty_cache()
     assert rel(got, want) < 1e-12
+
+
+def test_plan_bytes_count_the_planes():
+    """dme_plan_bytes: A, Q, X, E_t, W_t and, beside them, 34 bytes an entry for the planes of
+    E_t^T and of the step operand and 17 for the workspace; less once they have made room."""
+    n = N
+    A, C, _ = _data(n)
+    plan = dme.Plan(A, C=C, h=0.1, flows=["F12"], comp="lie")
+    full = dme.dme_plan_bytes(plan.handle)
+    assert (5 * 8 + 2 * 34 + 17) * n * n <= full <= (5 * 8 + 2 * 34 + 17) * n * n * 1.05
+    plan.apply("F12", 0.1, torch.zeros(n, n, dtype=torch.float64, device="cuda"))
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    fill = torch.empty(torch.cuda.mem_get_info()[0] - 500 * MB, dtype=torch.uint8, device="cuda")
+    P = torch.zeros(n, n, dtype=torch.float64, device="cuda")
+    torch.cuda.synchronize()
+    try:
+        plan.apply("F12", 0.2, P)      # another E_t and W_t: 20 blocks of 32 MB beside the planes' 11
+    finally:
+        del fill
+        torch.cuda.empty_cache()
+    held = dme.dme_plan_bytes(plan.handle)
+    assert 7 * 8 * n * n <= held <= 7 * 8 * n * n * 1.05
+    plan.close()
